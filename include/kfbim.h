@@ -166,11 +166,11 @@ typedef struct {
 } kfbim_options;
 
 /* Kernels of the FP32 transforms of MIXED contexts.
- * The Schur CG (Sec. 4.2, the dominant cost) runs, for N = 32, 64 and 128, as
- * four kernels per iteration: the transforms along z of the CG direction, one
- * CTA per (x, y) plane for the rest of the three spectral terms in shared
- * memory, the inverse transforms along z with the first dot product, and the
- * vector update (the "slab" iteration).  The other FP32 transforms (Schur
+ * The Schur CG (Sec. 4.2, the dominant cost) runs, for N = 32, 64, 96 and 128,
+ * as three kernels per iteration: the pending vector update and the transforms
+ * along z of the CG direction, one CTA per spectral term and (x, y) plane for
+ * the rest of the three terms in shared memory, and the inverse transforms along
+ * z with the dot products (the "slab" iteration).  The other FP32 transforms (Schur
  * right-hand side, velocity recovery) run as one-axis passes: four-step FFT
  * passes on the CUDA cores, or, for N = 128, a dense 3xTF32
  * transform-matrix GEMM on the tensor cores (tcgen05).  FP64 passes are
@@ -349,7 +349,7 @@ int kfbim_solve_adjoint(kfbim_ctx* ctx, const double* ubar_dev, double* gbar_dev
  * and CG iteration per instance).
  * MIXED contexts run the instances in lockstep: every FFT stage is one launch
  * for all instances still iterating, each Schur CG of the batch (N = 32, 64,
- * 128) is one launch of a CUDA graph whose conditional while loop runs the
+ * 96, 128) is one launch of a CUDA graph whose conditional while loop runs the
  * three slab kernels of every instance until all are done, and GMRES reads
  * its host scalars once per iteration for the whole batch.  FP64 contexts solve the instances one
  * after another.  The first call with a larger B than before allocates the
@@ -378,8 +378,8 @@ typedef enum {
   KFBIM_KCLASS_TRANSFORM_FP32 = 1,  /* one-axis transform passes, FP32 (FFT or tensor core) */
   KFBIM_KCLASS_CG_ZFWD = 2,         /* slab CG: the previous iteration's x, r update, d = r + beta d,
                                        z transforms (9 N^3 floats) */
-  KFBIM_KCLASS_CG_XY = 3,           /* slab CG: xy planes of the three terms (4 N^3 floats) */
-  KFBIM_KCLASS_CG_ZINV = 4,         /* slab CG: inverse z transforms, d.q, r.r, r.q, q.q (5 N^3 floats) */
+  KFBIM_KCLASS_CG_XY = 3,           /* slab CG: xy planes of the three terms (6 N^3 floats) */
+  KFBIM_KCLASS_CG_ZINV = 4,         /* slab CG: inverse z transforms, d.q, r.r, r.q, q.q (6 N^3 floats) */
   KFBIM_KCLASS_CG_UPDATE = 5,       /* slab CG: the x update still pending when a run stops
                                        (3 N^3 floats, once per CG run) */
   KFBIM_KCLASS_CG_VECTOR = 6,       /* staged CG: the three vector kernels (14 N^3 values) */

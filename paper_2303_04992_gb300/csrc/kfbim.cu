@@ -570,11 +570,12 @@ struct CgWs {
 CgWs<double> ws64(kfbim_ctx* c) { return {c->p, c->rres, c->cd, c->cq, c->q2, c->q3, c->T6}; }
 CgWs<float> ws32(kfbim_ctx* c) { return {c->fx, c->fr, c->fd, c->fq, c->fq2, c->fq3, c->fT6}; }
 
-// The slab CG of a single run on the FP32 workspace.
-SlabCg slab_run(kfbim_ctx* c, const CgWs<float>& w) {
+// The slab CG of a single run on the FP32 workspace (q2, an output of the
+// Schur right-hand side, is free during the run and holds x in slab order).
+SlabCg slab_run(kfbim_ctx* c, const CgWs<float>& w, const float* b = nullptr) {
   const int64_t n = c->N3;
-  return {c->N, w.x, w.r, w.d, w.q, w.T6, w.T6 + n, c->d_twc32, c->d_q32, c->d_s2f, (float)(1.0 / c->mu),
-          c->cgs, c->partial};
+  return {c->N, b, w.x, w.q2, w.r, w.d, w.q, w.T6, w.T6 + n, w.T6 + 2 * n, w.T6 + 3 * n, c->d_twc32, c->d_q32,
+          c->d_s2f, (float)(1.0 / c->mu), c->cgs, c->partial};
 }
 
 // One CG iteration: q = S d (5 staged launches), then the three fused
@@ -595,7 +596,7 @@ void cg_iteration(kfbim_ctx* c, const CgWs<T>& w, cudaStream_t s) {
           prof_end(c, s, at, KFBIM_KCLASS_CG_ZFWD + k, 1, (double)kSlabValues[k] * n * sizeof(float));
         }
       } else {
-        g_launches += slab_cg_iteration(a, s);
+        g_launches += slab_cg_iteration(&a, 1, s);
       }
       check_launch();
       return;
@@ -689,13 +690,23 @@ int cg_loop(kfbim_ctx* c, const T* b, const CgWs<T>& w, double tol, int maxit, c
   const bool graphs = c->use_graphs && !c->prof;
   cudaGraphExec_t exec = graphs ? cg_graph<T>(c, w) : nullptr;
   CK(cudaMemsetAsync(c->cgs, 0, sizeof(CGScalars), s));
-  CK(cudaMemsetAsync(w.x, 0, n * sizeof(T), s));
-  CK(cudaMemcpyAsync(w.r, b, n * sizeof(T), cudaMemcpyDeviceToDevice, s));
-  CK(cudaMemcpyAsync(w.d, b, n * sizeof(T), cudaMemcpyDeviceToDevice, s));
   const double rank1 = c->navier ? 0.0 : 1.0 / (c->mu * (double)n);
-  k_cg_init<T><<<RED_BLOCKS, RED_THREADS, 0, s>>>(b, n, c->cgs, tol * tol, rank1, c->cpen,
-                                                   c->partial);
-  ++g_launches;
+  bool started = false;
+  if constexpr (std::is_same<T, float>::value) {
+    if (c->slab) {
+      const SlabCg a = slab_run(c, w, b);
+      const double tol2 = tol * tol;
+      g_launches += slab_cg_start(&a, 1, &tol2, rank1, c->cpen, s);
+      started = true;
+    }
+  }
+  if (!started) {
+    CK(cudaMemsetAsync(w.x, 0, n * sizeof(T), s));
+    CK(cudaMemcpyAsync(w.r, b, n * sizeof(T), cudaMemcpyDeviceToDevice, s));
+    CK(cudaMemcpyAsync(w.d, b, n * sizeof(T), cudaMemcpyDeviceToDevice, s));
+    k_cg_init<T><<<RED_BLOCKS, RED_THREADS, 0, s>>>(b, n, c->cgs, tol * tol, rank1, c->cpen, c->partial);
+    ++g_launches;
+  }
   check_launch();
   const bool loop = graphs && c->cg_loop[Slot<T>::v];
   if (loop) CK(cudaGraphLaunch(exec, s));
@@ -728,7 +739,8 @@ int cg(kfbim_ctx* c, const T* b, const CgWs<T>& w, double tol, int maxit, cudaSt
   if constexpr (std::is_same<T, float>::value) {
     if (c->slab) {
       const int at = prof_begin(c, s);
-      g_launches += slab_cg_finish(slab_run(c, w), s);
+      const SlabCg a = slab_run(c, w);
+      g_launches += slab_cg_finish(&a, 1, s);
       prof_end(c, s, at, KFBIM_KCLASS_CG_UPDATE, 1, (double)kSlabValues[3] * c->N3 * sizeof(float));
       check_launch();
     }
@@ -1649,8 +1661,8 @@ std::vector<SlabCg> slab_batch_runs(kfbim_ctx* c, const std::vector<int>& slots)
   std::vector<SlabCg> runs;
   for (int b : slots) {
     const kfbim_ctx::Slot& w = c->bs[b];
-    runs.push_back({c->N, w.x, w.r, w.d, w.q, w.T6, w.T6 + n, c->d_twc32, c->d_q32, c->d_s2f,
-                    (float)(1.0 / c->mu), &c->bcgs[b], c->bpartial + (size_t)kRunPartials * b});
+    runs.push_back({c->N, w.fu, w.x, w.q2, w.r, w.d, w.q, w.T6, w.T6 + n, w.T6 + 2 * n, w.T6 + 3 * n, c->d_twc32,
+                    c->d_q32, c->d_s2f, (float)(1.0 / c->mu), &c->bcgs[b], c->bpartial + (size_t)kRunPartials * b});
   }
   return runs;
 }
@@ -1684,7 +1696,7 @@ cudaGraphExec_t cg_batch_graph(kfbim_ctx* c, const std::vector<SlabCg>& all) {
   c->bcg_tried = true;
   CK(cudaStreamSynchronize(c->cap_stream));
   const int64_t before = g_launches;
-  slab_cg_iteration_batch(all.data(), (int)all.size(), c->cap_stream);
+  slab_cg_iteration(all.data(), (int)all.size(), c->cap_stream);
   CK(cudaStreamSynchronize(c->cap_stream));
   const int64_t per_iter = g_launches - before;
   g_launches = before;
@@ -1708,7 +1720,7 @@ cudaGraphExec_t cg_batch_graph(kfbim_ctx* c, const std::vector<SlabCg>& all) {
   }
   cudaGraph_t body = np.conditional.phGraph_out[0];
   CK(cudaStreamBeginCaptureToGraph(c->cap_stream, body, nullptr, nullptr, 0, cudaStreamCaptureModeThreadLocal));
-  slab_cg_iteration_batch(all.data(), (int)all.size(), c->cap_stream);
+  slab_cg_iteration(all.data(), (int)all.size(), c->cap_stream);
   k_cg_cond_batch<<<1, 1, 0, c->cap_stream>>>(h, c->bcgs, (int)all.size(), std::max(1, c->opt.cg_max));
   CK(cudaStreamEndCapture(c->cap_stream, &body));
   g_launches = before;
@@ -1741,14 +1753,23 @@ void cg_batch(kfbim_ctx* c, const std::vector<int>& act, double tol, cudaStream_
   CK(cudaMemsetAsync(c->bcgs, 0, sizeof(CGScalars) * c->bcap, s));
   k_cg_mark_idle<<<1, 64, 0, s>>>(c->bcgs, c->bcap, mask);
   ++g_launches;
+  // each slot's tolerance, relaxed with its refinement tolerance as in grid_solve_mixed
+  std::vector<double> tol2;
   for (int b : act) {
+    const double tb = std::max(tol, relaxed_inner_tol(c, c->b_refine_tol[b]));
+    tol2.push_back(tb * tb);
+  }
+  if (c->slab && !act.empty()) {
+    const std::vector<SlabCg> runs = slab_batch_runs(c, act);
+    g_launches += slab_cg_start(runs.data(), (int)runs.size(), tol2.data(), rank1, c->cpen, s);
+  }
+  for (size_t k = 0; k < act.size() && !c->slab; ++k) {
+    const int b = act[k];
     const kfbim_ctx::Slot& w = c->bs[b];
     CK(cudaMemsetAsync(w.x, 0, n * sizeof(float), s));
     CK(cudaMemcpyAsync(w.r, w.fu, n * sizeof(float), cudaMemcpyDeviceToDevice, s));
     CK(cudaMemcpyAsync(w.d, w.fu, n * sizeof(float), cudaMemcpyDeviceToDevice, s));
-    // the slot's tolerance, relaxed with its refinement tolerance as in grid_solve_mixed
-    const double tb = std::max(tol, relaxed_inner_tol(c, c->b_refine_tol[b]));
-    k_cg_init<float><<<RED_BLOCKS, RED_THREADS, 0, s>>>(w.fu, n, &c->bcgs[b], tb * tb, rank1, c->cpen,
+    k_cg_init<float><<<RED_BLOCKS, RED_THREADS, 0, s>>>(w.fu, n, &c->bcgs[b], tol2[k], rank1, c->cpen,
                                                          c->partial);
     ++g_launches;
   }
@@ -1792,7 +1813,7 @@ void cg_batch(kfbim_ctx* c, const std::vector<int>& act, double tol, cudaStream_
       // iteration (blockIdx.y = instance; the single-run arithmetic)
       const std::vector<SlabCg> runs = slab_batch_runs(c, run);
       for (int it = 0; it < kCgGraphIters; ++it) {
-        g_launches += slab_cg_iteration_batch(runs.data(), (int)runs.size(), s);
+        g_launches += slab_cg_iteration(runs.data(), (int)runs.size(), s);
         check_launch();
       }
     } else {
@@ -1810,7 +1831,7 @@ void cg_batch(kfbim_ctx* c, const std::vector<int>& act, double tol, cudaStream_
   if (c->slab && !act.empty()) {
     // the update each run left pending when it stopped
     const std::vector<SlabCg> runs = slab_batch_runs(c, act);
-    g_launches += slab_cg_finish_batch(runs.data(), (int)runs.size(), s);
+    g_launches += slab_cg_finish(runs.data(), (int)runs.size(), s);
     check_launch();
   }
   for (int b : act) {
@@ -2418,20 +2439,16 @@ int kfbim_poisson(kfbim_ctx* c, int comp, const double* r, double* u, void* stre
 int kfbim_schur_apply_f32(kfbim_ctx* c, const float* d, float* q, void* stream) {
   return guarded(c, [&]() -> int {
     if (!d || !q || d == q) return fail(c, KFBIM_E_INVALID, "kfbim_schur_apply_f32: bad pointers");
-    if (!c->slab) return fail(c, KFBIM_E_INVALID, "kfbim_schur_apply_f32: no slab CG on this context");
+    if (!c->slab || c->N == 96)
+      return fail(c, KFBIM_E_INVALID, "kfbim_schur_apply_f32: needs the slab CG at N = 32, 64 or 128");
     cudaStream_t s = (cudaStream_t)stream;
-    const int64_t n = c->N3;
     const CgWs<float> w = ws32(c);
     // scalars of a fresh run: beta = 0 (so d = r), not done, the Navier c p block
     CGScalars h{};
     h.cdiag = c->cpen;
     std::memcpy(c->pinned, &h, sizeof(CGScalars));
     CK(cudaMemcpyAsync(c->cgs, c->pinned, sizeof(CGScalars), cudaMemcpyHostToDevice, s));
-    CK(cudaMemcpyAsync(w.r, d, n * sizeof(float), cudaMemcpyDeviceToDevice, s));
-    CK(cudaMemsetAsync(w.d, 0, n * sizeof(float), s));
-    SlabCg a{c->N, w.x, w.r, w.d, q, w.T6, w.T6 + n, c->d_twc32, c->d_q32, c->d_s2f, (float)(1.0 / c->mu),
-             c->cgs, c->partial};
-    g_launches += slab_schur_apply(a, s);
+    g_launches += slab_schur_apply(slab_run(c, w), d, q, s);
     check_launch();
     CK(cudaStreamSynchronize(s));   // the pinned scalars are reused by the next call
     return KFBIM_OK;
