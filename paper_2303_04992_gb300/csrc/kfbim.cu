@@ -144,7 +144,7 @@ struct kfbim_ctx {
   CGScalars* bcgs = nullptr;   // one per slot, contiguous
   double* bscal = nullptr;     // 8 per slot, contiguous
   double* bgh = nullptr;       // (bm + 1) per slot, contiguous (slot.gh points into it)
-  double* bpartial = nullptr;  // kRunPartials reduction partials per slot (batched CG kernels)
+  double* bpartial = nullptr;  // run_partials() reduction partials per slot (batched CG kernels)
   void* bpinned = nullptr;     // host staging of bcgs / bscal / bgh
   int bcap = 0, bm = 0;
   std::vector<int> b_cg, b_sweeps, b_isolves;   // per-slot counters of the current call
@@ -274,8 +274,11 @@ struct Tw<float> {
 };
 
 // Reduction partials per batch slot: RED_BLOCKS for the staged CG kernels,
-// four per block of the slab iteration's k_cg_zinv (4 x 512 at N = 128).
-constexpr int kRunPartials = 2 * RED_BLOCKS;
+// four per block of the slab iteration's k_cg_zinv (4 x 512 at N = 128, 4 x 2048
+// at N = 256).
+size_t run_partials(const kfbim_ctx* c) {
+  return std::max((size_t)2 * RED_BLOCKS, (size_t)c->N * c->N / 8);
+}
 constexpr int kMaxJobs = kPass2BatchJobs;   // jobs per batched launch: 3 per instance, 16 instances
 
 template <typename Tin, typename T, typename Tout, int N, int MAXJ>
@@ -1585,7 +1588,7 @@ void batch_alloc(kfbim_ctx* c, int B) {
   }
   c->bcgs = dalloc<CGScalars>(c, B);
   c->bscal = dalloc<double>(c, 8 * (size_t)B);
-  c->bpartial = dalloc<double>(c, (size_t)kRunPartials * B);
+  c->bpartial = dalloc<double>(c, run_partials(c) * B);
   if (c->bpinned) CK(cudaFreeHost(c->bpinned));
   c->bpinned = nullptr;
   const size_t pin = std::max({sizeof(CGScalars) * B, sizeof(double) * 8 * B,
@@ -1662,7 +1665,7 @@ std::vector<SlabCg> slab_batch_runs(kfbim_ctx* c, const std::vector<int>& slots)
   for (int b : slots) {
     const kfbim_ctx::Slot& w = c->bs[b];
     runs.push_back({c->N, w.fu, w.x, w.q2, w.r, w.d, w.q, w.T6, w.T6 + n, w.T6 + 2 * n, w.T6 + 3 * n, c->d_twc32,
-                    c->d_q32, c->d_s2f, (float)(1.0 / c->mu), &c->bcgs[b], c->bpartial + (size_t)kRunPartials * b});
+                    c->d_q32, c->d_s2f, (float)(1.0 / c->mu), &c->bcgs[b], c->bpartial + run_partials(c) * b});
   }
   return runs;
 }
@@ -1805,7 +1808,7 @@ void cg_batch(kfbim_ctx* c, const std::vector<int>& act, double tol, cudaStream_
       A.q2[k] = w.q2;
       A.q3[k] = w.q3;
       A.s[k] = &c->bcgs[run[k]];
-      A.partial[k] = c->bpartial + (size_t)kRunPartials * run[k];
+      A.partial[k] = c->bpartial + run_partials(c) * run[k];
     }
     const dim3 grid(RED_BLOCKS, (unsigned)run.size());
     if (c->slab) {
@@ -2439,7 +2442,7 @@ int kfbim_poisson(kfbim_ctx* c, int comp, const double* r, double* u, void* stre
 int kfbim_schur_apply_f32(kfbim_ctx* c, const float* d, float* q, void* stream) {
   return guarded(c, [&]() -> int {
     if (!d || !q || d == q) return fail(c, KFBIM_E_INVALID, "kfbim_schur_apply_f32: bad pointers");
-    if (!c->slab || c->N == 96)
+    if (!c->slab || c->N == 96 || c->N == 256)
       return fail(c, KFBIM_E_INVALID, "kfbim_schur_apply_f32: needs the slab CG at N = 32, 64 or 128");
     cudaStream_t s = (cudaStream_t)stream;
     const CgWs<float> w = ws32(c);

@@ -37,6 +37,7 @@
 // resident CTAs run as fast as 127 with two.
 #pragma once
 
+#include <cooperative_groups.h>
 #include <cuda_runtime.h>
 #include <stdint.h>
 
@@ -51,14 +52,19 @@ namespace plane {
 // pairs at M consecutive x are one contiguous run of 64 numbers.
 template <int N>
 struct Shape {
-  static constexpr int R = N == 128 ? 16 : (N == 96 ? 24 : 8);   // values per lane
+  static constexpr int R = N >= 128 ? 16 : (N == 96 ? 24 : 8);   // values per lane
   static constexpr int M = N / R;                                // lanes per FFT
   static constexpr int NS = R / M;                               // DFT_M per lane
   static constexpr int H = R / 2;
   static constexpr int LINES = N / 2;
-  static constexpr int ROUNDS = N == 128 ? 2 : 1;                // FFTs per team and axis step
-  static constexpr int TEAMS = LINES / ROUNDS;
-  static constexpr int THREADS = TEAMS * M;                      // 256, 192, 256, 64
+  // CTAs per plane: the 256 KB of a plane at N = 256 take two CTAs of a cluster,
+  // each with half of the lines, half of the row pairs and the other's lines
+  // through distributed shared memory
+  static constexpr int CL = N == 256 ? 2 : 1;
+  static constexpr int LL = LINES / CL;                          // lines and row pairs per CTA
+  static constexpr int ROUNDS = N >= 128 ? 2 : 1;                // FFTs per team and axis step
+  static constexpr int TEAMS = LL / ROUNDS;
+  static constexpr int THREADS = TEAMS * M;                      // 512, 256, 192, 256, 64
   static constexpr int YB = 2 * (32 / M);                        // y positions of one warp's row pairs
   static_assert(R % M == 0, "four-step split");
 };
@@ -209,7 +215,8 @@ __device__ __forceinline__ void dft(C2<T>* v) {
 // teams, lines 0 and 1 of an exchange, lines 0..3 of a column pair.
 template <int M>
 __device__ __forceinline__ int line_sw(int l) {
-  if constexpr (M == 8) return ((l & 3) << 2) | ((l >> 1) & 2);
+  if constexpr (M == 16) return (l & 7) << 1;   // a half warp is one team: 8 lines of a column pair
+  else if constexpr (M == 8) return ((l & 3) << 2) | ((l >> 1) & 2);
   else return ((l & 1) << 3) | ((l & 2) << 1);
 }
 
@@ -225,6 +232,12 @@ struct XSlots {   // along x
     const int line = s * (S::M / 2) + (w >> 1);
     return line * N + ((col + (w & 1)) ^ line_sw<S::M>(line));
   }
+};
+template <int N>
+struct XScratch {   // along x on two CTAs, whose columns are not whole: a buffer of the team
+  using S = Shape<N>;
+  int base;
+  __device__ __forceinline__ int at(int s, int v) const { return base + s * S::M + (v ^ (s & (S::M - 1))); }
 };
 template <int N>
 struct YSlots {   // along y
@@ -346,7 +359,8 @@ struct LineW {
 template <int N, typename T>
 struct Smem {
   using S = Shape<N>;
-  static constexpr size_t field = sizeof(C2<T>) * S::LINES * N;
+  static constexpr size_t scratch = S::CL > 1 ? sizeof(C2<T>) * S::TEAMS * N : 0;
+  static constexpr size_t field = sizeof(C2<T>) * S::LL * N + scratch;
   static constexpr size_t tables = sizeof(C2<T>) * (N + 2 * S::LINES) + sizeof(T) * S::LINES;
   static constexpr size_t bytes = field + tables;
 };
@@ -357,14 +371,14 @@ struct Smem {
 // instead the signs of `signs` (so that two terms can share an input).
 // az: the plane's 4 sin^2 along z; sc: 1 / (mu N^2).
 // twg: exp(-pi i t / N), t < 2N; qg: exp(-pi i k / 2N); s2: 4 sin^2(pi a / 2N), a < N.
-// Called by all threads of the CTA.
+// Called by all threads of the CTA (of both CTAs of the cluster; rank: this one's).
 template <int N, typename T>
 __device__ __forceinline__ void term_plane(const T* in, T* out, const Term term, const Term signs, T az, T sc,
                                            C2<T>* P, const C2<T>* __restrict__ twg, const C2<T>* __restrict__ qg,
-                                           const T* __restrict__ s2) {
+                                           const T* __restrict__ s2, int rank = 0) {
   using S = Shape<N>;
   constexpr int M = S::M, R = S::R, H = S::H;
-  C2<T>* tws = P + S::LINES * N;        // FFT twiddles [s][m]
+  C2<T>* tws = P + Smem<N, T>::field / sizeof(C2<T>);   // FFT twiddles [s][m]
   C2<T>* qh = tws + N;                  // q_k / 2, k < N/2
   C2<T>* cy = qh + S::LINES;            // exp(i pi k / N), k < N/2
   T* sg = reinterpret_cast<T*>(cy + S::LINES);   // 4 sin^2(pi k / 2N), k < N/2
@@ -378,6 +392,24 @@ __device__ __forceinline__ void term_plane(const T* in, T* out, const Term term,
   const int t = threadIdx.x / M, m = threadIdx.x % M;
   const int lane = threadIdx.x & 31;
   const int partner = (lane & ~(M - 1)) | ((M - m) & (M - 1));
+  // the lines of CTA c of the cluster (all lines without one)
+  C2<T>* lines[S::CL];
+  if constexpr (S::CL > 1) {
+#pragma unroll
+    for (int c = 0; c < S::CL; ++c) lines[c] = cooperative_groups::this_cluster().map_shared_rank(P, c);
+  } else {
+    lines[0] = P;
+  }
+  auto sync = [] {
+    if constexpr (S::CL > 1) cooperative_groups::this_cluster().sync();
+    else __syncthreads();
+  };
+  // the column pair n0, n0 + 1 of line l = m + M j
+  auto pair_at = [&](int j, int n0) -> C2<T>* {
+    const int l = m + M * j;
+    if constexpr (S::CL > 1) return lines[M * j / S::LL] + ((l % S::LL) * N + (n0 ^ line_sw<M>(l)));
+    else return P + (l * N + (n0 ^ line_sw<M>(l)));
+  };
   C2<T> v[R];
   // One copy of the code of an FFT along x serves the forward and the inverse
   // step (likewise along y): with a copy per step the warps wait for instructions.
@@ -386,31 +418,30 @@ __device__ __forceinline__ void term_plane(const T* in, T* out, const Term term,
 #pragma unroll 1
     for (int rd = 0; rd < S::ROUNDS; ++rd) {
       // the rows of Makhoul positions 2p, 2p + 1 along y <-> columns 2p, 2p + 1
-      const int n0 = 2 * (t + S::TEAMS * rd);
+      const int n0 = 2 * (rank * S::LL + t + S::TEAMS * rd);
       const int64_t at0 = (n0 / S::YB) * (N * S::YB) + m * S::YB + n0 % S::YB;
       if (!back) {
         const C2<T>* ra = reinterpret_cast<const C2<T>*>(in + at0);
         const T fl = (n0 >= N / 2 && term.ys != signs.ys) ? T(-1) : T(1), fh = term.xs != signs.xs ? -fl : fl;
 #pragma unroll
         for (int r = 0; r < R; ++r) v[r] = cscale(ldc(ra + r * (M * S::YB / 2)), r < H ? fl : fh);
-        if (rd == 0) __syncthreads();   // tables
+        if (rd == 0) sync();   // tables (and the other CTA runs before its lines are written)
       } else {
         // conj Z'_k = q conj(A + i B), conj Z'_(N-k) = conj(q) (A - i B)
         C2<T> up[H];
 #pragma unroll
         for (int j = 0; j < H; ++j) {
-          const int l = m + M * j;
-          const int at = l * N + (n0 ^ line_sw<M>(l));
+          const C2<T>* at = pair_at(j, n0);
           C2<T> a, b;
           if constexpr (sizeof(T) == 4) {
-            const float4 f = *reinterpret_cast<const float4*>(P + at);
+            const float4 f = *reinterpret_cast<const float4*>(at);
             a = {f.x, f.y};
             b = {f.z, f.w};
           } else {
-            a = P[at];
-            b = P[at + 1];
+            a = at[0];
+            b = at[1];
           }
-          const C2<T> q = ldc(qh + l);
+          const C2<T> q = ldc(qh + m + M * j);
           C2<T> lo = cmul(q, C2<T>{a.x - b.y, -(a.y + b.x)}), hi = cmul(conjg(q), C2<T>{a.x + b.y, a.y - b.x});
           if (j == 0 && m == 0) {
             lo = {T(0.5) * a.x, T(-0.5) * b.x};
@@ -421,8 +452,8 @@ __device__ __forceinline__ void term_plane(const T* in, T* out, const Term term,
         }
         mirror_put<N, T>(v, up, m);
       }
-      const XSlots<N> X{n0};
-      team_fft<N, T>(v, P, X, tws, m);
+      if constexpr (S::CL > 1) team_fft<N, T>(v, P, XScratch<N>{S::LL * N + t * N}, tws, m);
+      else team_fft<N, T>(v, P, XSlots<N>{n0}, tws, m);
       if (!back) {
 #pragma unroll
         for (int j = 0; j < H; ++j) {
@@ -433,13 +464,12 @@ __device__ __forceinline__ void term_plane(const T* in, T* out, const Term term,
             a = {z.x, g.x};
             b = {z.y, g.y};
           }
-          const int l = m + M * j;
-          const int at = l * N + (n0 ^ line_sw<M>(l));   // the swizzle keeps pairs 2p, 2p + 1 together
+          C2<T>* at = pair_at(j, n0);   // the swizzle keeps pairs 2p, 2p + 1 together
           if constexpr (sizeof(T) == 4) {
-            *reinterpret_cast<float4*>(P + at) = make_float4(a.x, a.y, b.x, b.y);
+            *reinterpret_cast<float4*>(at) = make_float4(a.x, a.y, b.x, b.y);
           } else {
-            P[at] = a;
-            P[at + 1] = b;
+            at[0] = a;
+            at[1] = b;
           }
         }
       } else {
@@ -449,14 +479,14 @@ __device__ __forceinline__ void term_plane(const T* in, T* out, const Term term,
       }
     }
     if (back) break;
-    __syncthreads();
+    sync();
     // y: transform, weight and inverse transform of line l in place
 #pragma unroll 1
     for (int rd = 0; rd < S::ROUNDS; ++rd) {
       const int tt = t + S::TEAMS * rd;
       // the two teams of 8 lanes of a half warp take lines that differ in bit 1
-      const int l = M == 8 ? ((tt & ~3) | ((tt & 1) << 1) | ((tt >> 1) & 1)) : tt;
-      const YSlots<N> Y{l * N, line_sw<M>(l)};
+      const int ll = M == 8 ? ((tt & ~3) | ((tt & 1) << 1) | ((tt >> 1) & 1)) : tt, l = rank * S::LL + ll;
+      const YSlots<N> Y{ll * N, line_sw<M>(l)};
 #pragma unroll
       for (int r = 0; r < R; ++r) v[r] = ldc(P + (Y.base + ((m + M * r) ^ Y.sw)));
 #pragma unroll 1
@@ -503,8 +533,9 @@ __device__ __forceinline__ void term_plane(const T* in, T* out, const Term term,
 #pragma unroll
       for (int j = 0; j < R; ++j) stc(P + (Y.base + ((m + M * j) ^ Y.sw)), conjg(v[j]));
     }
-    __syncthreads();
+    sync();
   }
+  if constexpr (S::CL > 1) sync();   // the other CTA may still read this one's lines
 }
 
 }  // namespace plane

@@ -6,7 +6,7 @@
 
 namespace kfbim {
 
-bool slab_supported(int N) { return N == 32 || N == 64 || N == 96 || N == 128; }
+bool slab_supported(int N) { return N == 32 || N == 64 || N == 96 || N == 128 || N == 256; }
 
 namespace {
 
@@ -17,7 +17,9 @@ cudaError_t raise(K kern, size_t bytes) {
 
 template <int N, int MAXB>
 cudaError_t prepare_nb() {
-  cudaError_t e = raise(slab::k_cg_terms<N, MAXB>, plane::Smem<N, float>::bytes);
+  cudaError_t e;
+  if constexpr (plane::Shape<N>::CL > 1) e = raise(slab::k_cg_terms_cl<N, MAXB>, plane::Smem<N, float>::bytes);
+  else e = raise(slab::k_cg_terms<N, MAXB>, plane::Smem<N, float>::bytes);
   if (e == cudaSuccess) e = raise(slab::k_cg_zfwd<N, MAXB>, slab::ZShape<N>::bytes);
   if (e == cudaSuccess) e = raise(slab::k_cg_zinv<N, MAXB>, slab::ZShape<N>::bytes);
   if (e == cudaSuccess) e = raise(slab::k_cg_start<N, MAXB>, slab::Conv<N>::bytes);
@@ -65,8 +67,12 @@ void launch_nb(int which, const slab::SlabArgs<MAXB>& args, const SlabCg& t, int
       slab::k_cg_zfwd<N, MAXB><<<dim3(Z::BLOCKS, nrun), Z::THREADS, Z::bytes, st>>>(args, t.tw, t.qN);
       break;
     case 1:
-      slab::k_cg_terms<N, MAXB><<<dim3(3 * N, nrun), plane::Shape<N>::THREADS, plane::Smem<N, float>::bytes, st>>>(
-          args, t.tw, t.qN, t.s2, t.inv_mu);
+      if constexpr (plane::Shape<N>::CL > 1)
+        slab::k_cg_terms_cl<N, MAXB><<<dim3(2 * 3 * N, nrun), plane::Shape<N>::THREADS,
+                                       plane::Smem<N, float>::bytes, st>>>(args, t.tw, t.qN, t.s2, t.inv_mu);
+      else
+        slab::k_cg_terms<N, MAXB><<<dim3(3 * N, nrun), plane::Shape<N>::THREADS, plane::Smem<N, float>::bytes, st>>>(
+            args, t.tw, t.qN, t.s2, t.inv_mu);
       break;
     case 2:
       slab::k_cg_zinv<N, MAXB><<<dim3(Z::BLOCKS, nrun), Z::THREADS, Z::bytes, st>>>(args, t.tw, t.qN);
@@ -114,6 +120,7 @@ void schur_n(const SlabCg& a, const float* d, float* q, cudaStream_t st) {
 // CALL(N) for a supported grid size, returning n; else 0.
 #define KFBIM_SLAB_SWITCH(N_, CALL, n) \
   switch (N_) {                        \
+    case 256: CALL(256); return n;     \
     case 128: CALL(128); return n;     \
     case 96: CALL(96); return n;       \
     case 64: CALL(64); return n;       \
@@ -125,6 +132,7 @@ void schur_n(const SlabCg& a, const float* d, float* q, cudaStream_t st) {
 
 cudaError_t slab_prepare(int N) {
   switch (N) {
+    case 256: return prepare_n<256>();
     case 128: return prepare_n<128>();
     case 96: return prepare_n<96>();
     case 64: return prepare_n<64>();

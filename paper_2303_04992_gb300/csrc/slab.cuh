@@ -1,5 +1,5 @@
 // FP32 Schur-complement CG iteration in three kernels (Sec. 4.2, Eq. linearS1
-// and items i-iii), for N = 32, 64, 96, 128.
+// and items i-iii), for N = 32, 64, 96, 128, 256.
 //
 // The Schur operator is applied in spectral form,
 //   S d = (1/mu) sum_c B_c^-1 Lambda_c B_c d (+ rank-one / c d terms),
@@ -64,7 +64,7 @@ struct ZShape {
   static constexpr size_t tile = sizeof(float) * N * TILE;
   static constexpr size_t bytes = 2 * tile + sizeof(C2<float>) * (N + S::LINES);
   // resident CTAs per SM asked of the compiler (64 registers; 100 at N = 96, 24 values per lane)
-  static constexpr int OCC = THREADS == 256 ? 4 : (N == 96 ? 5 : 8);
+  static constexpr int OCC = THREADS == 512 ? 2 : (THREADS == 256 ? 4 : (N == 96 ? 5 : 8));
 };
 
 // Element (z mode k, column l) of a tile at k TILE + (l ^ tile_sw(k)): the lanes of
@@ -73,7 +73,8 @@ struct ZShape {
 template <int N>
 __device__ __forceinline__ int tile_at(int k, int l) {
   constexpr int M = plane::Shape<N>::M, TILE = ZShape<N>::TILE;
-  const int sw = TILE == 32 ? (k & (M - 1)) * (32 / M) : ((k >> 1) & (M / 2 - 1)) * (32 / M);
+  const int sw = M == 16 ? ((k >> 1) & 7) * 4   // modes 2i, 2i + 1 share banks (two-way): groups of four stay whole
+                 : TILE == 32 ? (k & (M - 1)) * (32 / M) : ((k >> 1) & (M / 2 - 1)) * (32 / M);
   return k * TILE + (l ^ sw);
 }
 
@@ -81,7 +82,7 @@ __device__ __forceinline__ int tile_at(int k, int l) {
 // that the teams of a half warp (adjacent lines) use distinct banks.
 template <int N>
 __device__ __forceinline__ plane::YSlots<N> z_slots(int t) {
-  return {t * N, plane::Shape<N>::M == 8 ? (t & 1) << 3 : (t & 3) << 2};
+  return {t * N, plane::Shape<N>::M == 16 ? 0 : (plane::Shape<N>::M == 8 ? (t & 1) << 3 : (t & 3) << 2)};
 }
 
 // The buffers of up to MAXB independent CG runs on one grid (blockIdx.y
@@ -228,23 +229,40 @@ k_cg_zfwd(const __grid_constant__ SlabArgs<MAXB> args, const C2<float>* __restri
     s->sumd = sum[0];
 }
 
-// One term of the Schur operator on one plane (plane.cuh): blockIdx.x = term N +
-// plane.  Z1 carries the signs of the DST-II along y, Z3 those along x and y.
+// One term of the Schur operator on one plane (plane.cuh), plane-major so that
+// terms 1 and 2 of a plane read Z1 close in time.  Z1 carries the signs of the
+// DST-II along y, Z3 those along x and y.
 template <int N, int MAXB>
-__global__ void __launch_bounds__(plane::Shape<N>::THREADS, 2)
-k_cg_terms(const __grid_constant__ SlabArgs<MAXB> args, const C2<float>* __restrict__ twg,
-           const C2<float>* __restrict__ qg, const float* __restrict__ s2g, float inv_mu) {
+__device__ __forceinline__ void terms_body(const SlabArgs<MAXB>& args, int unit, int rank,
+                                           const C2<float>* __restrict__ twg, const C2<float>* __restrict__ qg,
+                                           const float* __restrict__ s2g, float inv_mu) {
   const int b = blockIdx.y;
   if (args.s[b]->done) return;
   extern __shared__ __align__(16) unsigned char smx[];
-  const int term = blockIdx.x / N, k = blockIdx.x % N;
+  const int term = unit % 3, k = unit / 3;
   const int64_t off = (int64_t)k * N * N;
   const float* in = (term == 2 ? args.z3[b] : args.z1[b]) + off;
   float* out = (term == 0 ? args.w1[b] : (term == 1 ? args.w2[b] : args.z3[b])) + off;
   // 4 sin^2 along z: DCT-II mode k (term 3), DST-II mode N - 1 - k (terms 1, 2)
   const float az = term == 2 ? s2g[k] : s2g[2 * N - 1 - k];
   plane::term_plane<N, float>(in, out, plane::term_of(term), plane::term_of(term == 2 ? 2 : 0), az,
-                              inv_mu * (1.0f / ((float)N * N)), reinterpret_cast<C2<float>*>(smx), twg, qg, s2g);
+                              inv_mu * (1.0f / ((float)N * N)), reinterpret_cast<C2<float>*>(smx), twg, qg, s2g,
+                              rank);
+}
+template <int N, int MAXB>
+__global__ void __launch_bounds__(plane::Shape<N>::THREADS, 2)
+k_cg_terms(const __grid_constant__ SlabArgs<MAXB> args, const C2<float>* __restrict__ twg,
+           const C2<float>* __restrict__ qg, const float* __restrict__ s2g, float inv_mu) {
+  terms_body<N, MAXB>(args, blockIdx.x, 0, twg, qg, s2g, inv_mu);
+}
+// The same with a plane on a cluster of two CTAs (N = 256): 270 us, bound by
+// issue and shared memory with its 16 warps per SM; the five one-axis stages it
+// replaces took 1.16 ms of a staged CG iteration of 1.32 ms (now 0.47 ms).
+template <int N, int MAXB>
+__global__ void __cluster_dims__(2, 1, 1) __launch_bounds__(plane::Shape<N>::THREADS, 1)
+k_cg_terms_cl(const __grid_constant__ SlabArgs<MAXB> args, const C2<float>* __restrict__ twg,
+              const C2<float>* __restrict__ qg, const float* __restrict__ s2g, float inv_mu) {
+  terms_body<N, MAXB>(args, blockIdx.x / 2, blockIdx.x % 2, twg, qg, s2g, inv_mu);
 }
 
 // q = DST-III_z (W1 + W2) + DCT-III_z W3 + cdiag d + rank1 sumd; d.q, r.r, r.q,

@@ -34,7 +34,7 @@ struct SlabCg {
 constexpr int kSlabBatchMax = 64;
 
 // Grids the slab iteration covers: N / 2 complex lines of N numbers (a whole
-// plane) fit in one CTA's shared memory.
+// plane) fit in the shared memory of one CTA, at N = 256 of a cluster of two.
 bool slab_supported(int N);
 // Raises the kernels' dynamic shared-memory limits on the current device.
 cudaError_t slab_prepare(int N);
