@@ -211,7 +211,7 @@ def measured_peaks():
     return 6800.0, "fallback"
 
 
-PASS_SOURCES = {"fft": ("transforms.cuh", "transforms2.cuh"),
+PASS_SOURCES = {"fft": ("transforms.cuh", "plane.cuh", "lines.cuh"),
                  "tensor": ("transforms.cuh", "transforms2.cuh", "tc_pass.cuh")}
 
 
@@ -260,7 +260,7 @@ def ncu_traffic_slab(workload):
         return None
     txt = open(p).read()
     h = hashlib.sha256()
-    for f in ("slab.cuh", "cg_common.cuh", "transforms2.cuh"):
+    for f in ("slab.cuh", "cg_common.cuh", "plane.cuh"):
         h.update(open(os.path.join(ROOT, "paper_2303_04992_gb300", "csrc", f), "rb").read())
     m = re.search(r"kernel_source_sha256_12:\s*([0-9a-f]+)", txt)
     t = re.search(r"dram_bytes_per_launch:\s*([0-9.eE+]+)", txt)
@@ -538,7 +538,7 @@ def large_fp32_leg(args, flush, stream, dev, peak, peak_kind):
     return {"workload": "star256 (r = 0.5 + 0.1 sin 3theta cos 4phi, 256^3, [-1,1]^3)", "precision": "fp32",
             "solves_per_s": round(1e3 / ms, 4), "ms_per_solve": round(ms, 2), "setup_s": round(setup_s, 2),
             "gmres_iters": st["gmres_iters"], "cg_iters": st["cg_iters"],
-            "transform_roofline": {"bound": "hbm", "kernel": "k_axis_pass2 (N = 256)", "launches": n_x,
+            "transform_roofline": {"bound": "hbm", "kernel": "k_lines (N = 256)", "launches": n_x,
                                    "avg_launch_us": round(ms_x / n_x * 1e3, 2),
                                    "bytes_per_launch": round(b_x / n_x), "achieved": round(achieved, 1),
                                    "peak": peak, "unit": "GB/s", "frac": round(achieved / peak, 4),

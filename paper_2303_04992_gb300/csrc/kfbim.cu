@@ -29,7 +29,7 @@
 #include "kernels.cuh"
 #include "transforms.cuh"
 #include "transforms2.cuh"
-#include "pass2.h"
+#include "lines.h"
 #include "tc_pass.cuh"
 #include "slab.h"
 
@@ -279,13 +279,6 @@ struct Tw<float> {
 size_t run_partials(const kfbim_ctx* c) {
   return std::max((size_t)2 * RED_BLOCKS, (size_t)c->N * c->N / 8);
 }
-constexpr int kMaxJobs = kPass2BatchJobs;   // jobs per batched launch: 3 per instance, 16 instances
-
-template <typename Tin, typename T, typename Tout, int N, int MAXJ>
-void launch_pass2(kfbim_ctx* c, const PassJobs<Tin, Tout, MAXJ>& jobs, int njobs, cudaStream_t s) {
-  CK((pass2_launch<N, Tin, T, Tout, MAXJ>(jobs, njobs, Tw<T>::twc(c), Tw<T>::q(c), Tw<T>::s2(c), s)));
-}
-
 // One transform pass of a stage: input, output, axis, first transform,
 // second transform, spectral weight, weight component, accumulate flag, and
 // the done flag of the CG run the pass belongs to (nullable).
@@ -316,21 +309,50 @@ PassJob<Tin, Tout> make_job(kfbim_ctx* c, const Job& j, const int* skip) {
   return {static_cast<const Tin*>(j.in), static_cast<Tout*>(j.out), a};
 }
 
+// The operation of a pass with transforms t0, t1 (lines::Op); -1: none.
+int line_op(int t0, int t1) {
+  const bool f2 = t0 == X_DCT2F || t0 == X_DST2F, i2 = t0 == X_DCT2I || t0 == X_DST2I;
+  if (t1 == X_NONE) return f2 ? lines::OP_F2 : (i2 ? lines::OP_I2 : (t0 == X_DST1F ? lines::OP_F1 : lines::OP_I1));
+  if (t0 == X_DCT2F && t1 == X_DCT2I) return lines::OP_F2I2;
+  if (t0 == X_DST1F && t1 == X_DST1I) return lines::OP_F1I1;
+  if (t0 == X_DST1F && t1 == X_DCT2I) return lines::OP_F1I2;
+  return -1;
+}
+
 template <typename Tin, typename T, typename Tout, int MAXJ>
 void launch_jobs(kfbim_ctx* c, const Job* list, int nj, cudaStream_t s, const int* skip) {
-  PassJobs<Tin, Tout, MAXJ> jobs{};
-  for (int k = 0; k < nj; ++k) jobs.j[k] = make_job<Tin, Tout>(c, list[k], skip);
-  if (c->N == 128) launch_pass2<Tin, T, Tout, 128, MAXJ>(c, jobs, nj, s);
-  else if (c->N == 256) launch_pass2<Tin, T, Tout, 256, MAXJ>(c, jobs, nj, s);
-  else if (c->N == 96) launch_pass2<Tin, T, Tout, 96, MAXJ>(c, jobs, nj, s);
-  else if (c->N == 64) launch_pass2<Tin, T, Tout, 64, MAXJ>(c, jobs, nj, s);
-  else launch_pass2<Tin, T, Tout, 32, MAXJ>(c, jobs, nj, s);
+  lines::Jobs<Tin, Tout, MAXJ> jobs{};
+  for (int k = 0; k < nj; ++k) {
+    const Job& j = list[k];
+    lines::Job<Tin, Tout>& o = jobs.j[k];
+    o.in = static_cast<const Tin*>(j.in);
+    o.out = static_cast<Tout*>(j.out);
+    o.skip = j.skip ? j.skip : skip;
+    o.axis = (int8_t)j.axis;
+    o.dst = j.t0 == X_DST2F || j.t0 == X_DST2I;
+    o.wmode = (int8_t)j.wmode;
+    o.wc = (int8_t)j.wc;
+    // vectors of two numbers need both fields aligned (a caller's may not be)
+    o.vec = reinterpret_cast<uintptr_t>(j.in) % (2 * sizeof(Tin)) == 0 &&
+            reinterpret_cast<uintptr_t>(j.out) % (2 * sizeof(Tout)) == 0;
+  }
+  const int op = line_op(list[0].t0, list[0].t1);
+  const T h = T(c->h), im = T(1.0 / c->mu);
+  const auto *tw = Tw<T>::twc(c), *q = Tw<T>::q(c);
+  const T* s2 = Tw<T>::s2(c);
+  switch (c->N) {
+    case 256: CK((lines_launch<256, Tin, T, Tout, MAXJ>(op, jobs, nj, h, im, tw, q, s2, s))); break;
+    case 128: CK((lines_launch<128, Tin, T, Tout, MAXJ>(op, jobs, nj, h, im, tw, q, s2, s))); break;
+    case 96: CK((lines_launch<96, Tin, T, Tout, MAXJ>(op, jobs, nj, h, im, tw, q, s2, s))); break;
+    case 64: CK((lines_launch<64, Tin, T, Tout, MAXJ>(op, jobs, nj, h, im, tw, q, s2, s))); break;
+    default: CK((lines_launch<32, Tin, T, Tout, MAXJ>(op, jobs, nj, h, im, tw, q, s2, s)));
+  }
   ++g_launches;
 }
 
-// Launch a list of independent passes: up to 3 jobs per launch on the
-// compile-time-N kernel (48 for longer, batched lists), one launch per job on
-// the runtime-N kernel.
+// Launch a list of independent passes (all of the same transforms): up to 3 jobs
+// per launch on the compile-time-N kernel (48 for longer, batched lists), one
+// launch per job on the runtime-N kernel.
 // Tensor-core passes of one stage: all jobs share the first transform; a
 // fused job (second transform) becomes a weighted pass into its output and an
 // in-place pass of the second transform.  Returns the kernel launches.
@@ -395,13 +417,15 @@ void stage_list(kfbim_ctx* c, const std::vector<Job>& list, cudaStream_t s, cons
     launches = tc_passes(c, list, s, skip, &bytes);
   } else if (c->N == 256 || c->N == 128 || c->N == 96 || c->N == 64 || c->N == 32) {
     for (const Job& j : list) bytes += (double)c->N3 * (sizeof(Tin) + sizeof(Tout) * (j.acc ? 2 : 1));
-    if (nj <= 3) {
-      launch_jobs<Tin, T, Tout, 3>(c, list.data(), nj, s, skip);
-    } else {
-      for (int k0 = 0; k0 < nj; k0 += kMaxJobs)
-        launch_jobs<Tin, T, Tout, kMaxJobs>(c, list.data() + k0, std::min(kMaxJobs, nj - k0), s, skip);
+    // FP32 batches go by kLineBatchJobs jobs per launch, the rest by three
+    constexpr int kMost = sizeof(T) == 4 ? kLineBatchJobs : kLineJobs;
+    launches = 0;
+    for (int k0 = 0; k0 < nj; ++launches) {
+      const int n = std::min(nj - k0, nj <= kLineJobs ? kLineJobs : kMost);
+      if (nj <= kLineJobs) launch_jobs<Tin, T, Tout, kLineJobs>(c, list.data() + k0, n, s, skip);
+      else launch_jobs<Tin, T, Tout, kMost>(c, list.data() + k0, n, s, skip);
+      k0 += n;
     }
-    launches = nj <= 3 ? 1 : (nj + kMaxJobs - 1) / kMaxJobs;
   } else {
     const size_t smem = pass_smem_bytes(c->N, sizeof(T));
     auto kern = k_axis_pass<Tin, T, Tout>;

@@ -1,0 +1,440 @@
+// One-axis transform pass: the real transforms of transforms.cuh (DCT-II/III,
+// DST-II/III, DST-I) of every line of an N^3 field along one axis, optionally
+// followed by the spectral weight and an inverse transform along the same axis
+// in the same registers.  N = 32, 64, 96, 128, 256; FP32 and FP64.
+//
+// A team of M lanes (plane.cuh) transforms a pair of adjacent lines: DCT-II and
+// DST-II of the two real lines as one complex FFT in Makhoul's order (a DST-II is
+// the DCT-II with the odd elements negated, its mode a at DCT index N - 1 - a),
+// DST-I one line at a time: the odd extension y of the line (length 2N) packed as
+// z_n = y_2n + i y_(2n+1) is one complex FFT of length N, and with
+// a, b = (Z_k +- conj Z_(N-k)) / 2, w = exp(-i pi k / N) its modes are
+//   X_k, X_(N-k) = (Re(w b) -+ Im a) / 2;
+// backwards Z_k = (c s, s' s + d), Z_(N-k) = (-c s, s' s - d) with c + i s' =
+// exp(i pi k / N), s = X_k + X_(N-k), d = X_(N-k) - X_k, and the inverse FFT is
+// z_n = x_2n + i x_(2n+1).  A lane ends a forward transform holding modes k and
+// N - k of its lines for k = m + M j < N/2, which is what the inverse starts from,
+// so the weight of a fused pass costs no exchange.
+//
+// Lines go from global memory straight into the FFT registers and back: along y
+// and z a pair of lines is one vector per element and a warp's teams fill 32- to
+// 64-byte sectors; along x a lane reads (x_2n, x_(2n+1)) as one vector and hands
+// the odd element to its mirror lane by a shuffle.  Shared memory holds the FFT
+// exchange (N complex numbers per team) and the twiddles; the teams of a CTA do
+// not wait for one another.
+#pragma once
+
+#include <cuda_runtime.h>
+#include <stdint.h>
+
+#include "fastcvt.h"
+#include "plane.cuh"
+#include "transforms.cuh"
+
+namespace kfbim {
+namespace lines {
+
+// What a pass does.  F2, I2: forward / inverse of the DCT-II and DST-II family;
+// F1, I1: DST-I; the others forward, weight, inverse.
+enum Op : int { OP_F2 = 0, OP_I2, OP_F1, OP_I1, OP_F2I2, OP_F1I1, OP_F1I2 };
+__host__ __device__ constexpr bool op_fwd1(int op) { return op == OP_F1 || op == OP_F1I1 || op == OP_F1I2; }
+__host__ __device__ constexpr bool op_fwd2(int op) { return op == OP_F2 || op == OP_F2I2; }
+__host__ __device__ constexpr bool op_inv1(int op) { return op == OP_I1 || op == OP_F1I1; }
+__host__ __device__ constexpr bool op_inv2(int op) { return op == OP_I2 || op == OP_F2I2 || op == OP_F1I2; }
+
+// One pass of one field.  vec: in and out are aligned for vectors of two numbers.
+template <typename Tin, typename Tout>
+struct Job {
+  const Tin* in;
+  Tout* out;
+  const int* skip;   // nullable: the pass does nothing when *skip != 0
+  int8_t axis;       // 0 x, 1 y, 2 z
+  int8_t dst;        // F2, I2: 1 for the DST-II family
+  int8_t wmode, wc;  // weight mode (transforms.cuh), component axis of the weight
+  int8_t vec;
+};
+template <typename Tin, typename Tout, int MAXJ>
+struct Jobs {
+  Job<Tin, Tout> j[MAXJ];
+};
+
+template <int N, typename T>
+struct LShape {
+  using S = plane::Shape<N>;
+  static constexpr int TEAMS = 128 / S::M;                 // line pairs per CTA
+  static constexpr int THREADS = 128;
+  static constexpr int BLOCKS = (N * N / 2 + TEAMS - 1) / TEAMS;
+  static constexpr size_t bytes = sizeof(C2<T>) * ((size_t)TEAMS * N + N);
+  // CTAs per SM asked of the compiler: 96 registers in FP32, 128 for the fused passes (168 at
+  // N = 96, 24 values per lane), 255 in FP64
+  static constexpr int occ(bool fused) { return sizeof(T) == 8 ? 2 : (N == 96 ? 3 : (fused ? 4 : 5)); }
+};
+
+template <typename T, typename Tin>
+__device__ __forceinline__ T to_work(Tin v) {
+  if constexpr (sizeof(T) == 4 && sizeof(Tin) == 8) return f64_to_f32(v);   // integer operations: fastcvt.h
+  else return T(v);
+}
+
+// Two adjacent numbers p[0], p[1].
+template <typename T, typename Tin>
+__device__ __forceinline__ C2<T> ld2(const Tin* p, bool vec) {
+  if (vec) {
+    if constexpr (sizeof(Tin) == 4) {
+      const float2 v = *reinterpret_cast<const float2*>(p);
+      return {to_work<T>(v.x), to_work<T>(v.y)};
+    } else {
+      const double2 v = *reinterpret_cast<const double2*>(p);
+      return {to_work<T>(v.x), to_work<T>(v.y)};
+    }
+  }
+  return {to_work<T>(p[0]), to_work<T>(p[1])};
+}
+template <typename T, typename Tout>
+__device__ __forceinline__ void st2(Tout* p, T a, T b, bool vec) {
+  if (vec) {
+    if constexpr (sizeof(Tout) == 4) *reinterpret_cast<float2*>(p) = make_float2(a, b);
+    else *reinterpret_cast<double2*>(p) = make_double2(a, b);
+  } else {
+    p[0] = a;
+    p[1] = b;
+  }
+}
+
+// The exchange slots of a team: as plane.cuh's along y, each team its own line.
+template <int N>
+__device__ __forceinline__ plane::YSlots<N> slots(int t) {
+  constexpr int M = plane::Shape<N>::M;
+  return {t * N, M == 16 ? 0 : (M == 8 ? (t & 1) << 3 : (t & 3) << 2)};
+}
+
+// Weights of a pass (the factors of spectral_weight2): 4 sin^2 of the line's two
+// other modes, of the mode along the pass's axis, and the numerator.
+template <typename T, int N>
+struct Weights {
+  const T* __restrict__ s2;
+  T rest;       // 4 sin^2 of the modes across the line, summed
+  T num;        // numerator, where it is not that of the pass's axis
+  int kind;     // 0: the pass's axis takes DCT / DST-I modes, 1: DST-II modes
+  int wmode;
+  bool own;     // the weight's component axis is the pass's axis
+  T h, inv_mu;
+  // numerator for component mode value v = 4 sin^2 (zero for mode 0 of a face basis)
+  __device__ __forceinline__ T numer(T v, bool zero) const {
+    if (wmode == W_SCHUR) return v * inv_mu;
+    if (zero) return T(0);
+    if (wmode == W_POISSON) return h * h * inv_mu;
+    return -h * inv_mu * sqrt(v);   // -2 h sin(a), v = 4 sin^2(a)
+  }
+  __device__ __forceinline__ T at(int a, T& den) const {
+    const T v = s2[kind * N + a];
+    den = rest + v;
+    return own ? numer(v, a == 0) : num;
+  }
+};
+
+template <typename Tin, typename T, typename Tout, int N, int OP, int MAXJ>
+__global__ void __launch_bounds__(128, (LShape<N, T>::occ(OP >= OP_F2I2)))
+k_lines(const __grid_constant__ Jobs<Tin, Tout, MAXJ> jobs, T h, T inv_mu, const C2<T>* __restrict__ twg,
+        const C2<T>* __restrict__ qg, const T* __restrict__ s2) {
+  using S = plane::Shape<N>;
+  using L = LShape<N, T>;
+  constexpr int M = S::M, R = S::R, H = S::H;
+  const Job<Tin, Tout>& job = jobs.j[blockIdx.y];
+  if (job.skip && *job.skip) return;
+  extern __shared__ __align__(16) unsigned char sml[];
+  C2<T>* P = reinterpret_cast<C2<T>*>(sml);
+  C2<T>* tws = P + L::TEAMS * N;
+  for (int e = threadIdx.x; e < N; e += L::THREADS) tws[e] = twg[2 * (e / M) * (e % M)];
+  __syncthreads();
+  const int t = threadIdx.x / M, m = threadIdx.x % M, lane = threadIdx.x & 31;
+  const int partner = (lane & ~(M - 1)) | ((M - m) & (M - 1));
+  const int pair = blockIdx.x * L::TEAMS + t;   // N^2 / 2 is a multiple of the CTA's teams
+  const int line = 2 * pair;
+  const int axis = job.axis;
+  const bool vec = job.vec, dst = job.dst;
+  // lines: x: line = k N + j (contiguous); y: (k, i); z: (j, i); ls, es: strides of lines and elements
+  const int64_t base = axis == 0 ? (int64_t)line * N : (axis == 1 ? (int64_t)(line / N) * N * N + line % N : line);
+  const int64_t ls = axis == 0 ? N : 1, es = axis == 0 ? 1 : (axis == 1 ? N : (int64_t)N * N);
+  const Tin* in = job.in + base;
+  Tout* out = job.out + base;
+  const auto X = slots<N>(t);
+  constexpr T half = T(0.5), r2 = T(1.41421356237309504880), ir2 = T(0.70710678118654752440);
+  // modes (k, N - k) of the two lines, k = m + M j; slot (0, N/2) for k = 0
+  C2<T> A[H], B[H];
+  auto k2 = [&](int j) { return (j == 0 && m == 0) ? N / 2 : N - (m + M * j); };
+  auto mode = [&](int k) { return dst ? N - 1 - k : k; };   // array index of DCT index k (F2, I2)
+
+  // ------------------------------------------------------------- forward
+  if constexpr (op_fwd2(OP)) {
+    C2<T> v[R];
+    const T sg = dst ? T(-1) : T(1);
+    if (axis == 0) {
+#pragma unroll
+      for (int r = 0; r < H; ++r) {
+        const int n = m + M * r;
+        const C2<T> a = ld2<T>(in + 2 * n, vec), b = ld2<T>(in + N + 2 * n, vec);
+        v[r] = {a.x, b.x};
+        // element 2n + 1 is position N - 1 - n: lane M - 1 - m, register R - 1 - r
+        v[R - 1 - r] = {sg * __shfl_xor_sync(0xffffffffu, a.y, M - 1), sg * __shfl_xor_sync(0xffffffffu, b.y, M - 1)};
+      }
+    } else {
+#pragma unroll
+      for (int r = 0; r < R; ++r) {
+        const int n = m + M * r;
+        const int i = r < H ? 2 * n : 2 * (N - 1 - n) + 1;
+        v[r] = ld2<T>(in + (int64_t)i * es, vec);
+        if (r >= H) v[r] = plane::cscale(v[r], sg);
+      }
+    }
+    plane::team_fft<N, T>(v, P, X, tws, m);
+#pragma unroll
+    for (int j = 0; j < H; ++j) {
+      const C2<T> g = plane::mirror_fetch<N, T>(v, j, m, partner);
+      const C2<T> z = v[j], q0 = qg[m + M * j];
+      const C2<T> q = {half * q0.x, half * q0.y};
+      C2<T> a = cmul(q, C2<T>{z.x + g.x, z.y - g.y}), b = cmul(q, C2<T>{z.y + g.y, g.x - z.x});
+      if (j == 0 && m == 0) {
+        a = {z.x, -(ir2 * g.x)};
+        b = {z.y, -(ir2 * g.y)};
+      }
+      A[j] = {a.x, -a.y};   // X_k, X_(N-k)
+      B[j] = {b.x, -b.y};
+    }
+  } else if constexpr (op_fwd1(OP)) {
+#pragma unroll 1
+    for (int ab = 0; ab < 2; ++ab) {
+      const Tin* x = in + ab * ls;
+      C2<T> v[R];
+      // z_n = x_2n + i x_(2n+1) (x_0 is the wall: 0), z_(N-n) = -x_2n - i x_(2n-1)
+#pragma unroll
+      for (int r = 0; r < H; ++r) {
+        const int n = m + M * r;
+        C2<T> a;
+        if (axis == 0) a = ld2<T>(x + 2 * n, vec);
+        else a = {to_work<T>(x[(int64_t)(2 * n) * es]), to_work<T>(x[(int64_t)(2 * n + 1) * es])};
+        if (r == 0 && m == 0) a.x = T(0);
+        v[r] = a;
+      }
+#pragma unroll
+      for (int r = 0; r < H; ++r) {
+        // position n = m + M (R - 1 - r): x_2n' of n' = N - n at lane M - m, register r (lane 0:
+        // register r + 1, zero for n' = N/2), x_(2n'-1) at lane M - 1 - m, register r
+        const T nx = r + 1 < H ? v[r + 1].x : T(0);
+        const T re = __shfl_sync(0xffffffffu, m ? v[r].x : nx, partner);
+        const T im = __shfl_xor_sync(0xffffffffu, v[r].y, M - 1);
+        v[R - 1 - r] = {-re, -im};
+      }
+      plane::team_fft<N, T>(v, P, X, tws, m);
+#pragma unroll
+      for (int j = 0; j < H; ++j) {
+        const C2<T> g = plane::mirror_fetch<N, T>(v, j, m, partner);
+        const C2<T> z = v[j], w = twg[m + M * j];
+        // twice a and b: a = (.., z.y - g.y), b = (z.x - g.x, z.y + g.y)
+        const T ia = T(0.25) * (z.y - g.y), wb = T(0.25) * (w.x * (z.x - g.x) - w.y * (z.y + g.y));
+        C2<T> f = {wb - ia, wb + ia};
+        if (j == 0 && m == 0) f = {T(0), half * g.y};   // modes 0 and N/2
+        if (ab) B[j] = f;
+        else A[j] = f;
+      }
+    }
+  } else {   // inverse only: the modes come from memory
+#pragma unroll
+    for (int j = 0; j < H; ++j) {
+      int ka = m + M * j, kb = k2(j);
+      if constexpr (OP == OP_I2) {
+        ka = mode(ka);
+        kb = mode(kb);
+      }
+      C2<T> a, b;
+      if (axis == 0) {
+        a = {to_work<T>(in[ka]), to_work<T>(in[kb])};
+        b = {to_work<T>(in[N + ka]), to_work<T>(in[N + kb])};
+      } else {
+        const C2<T> e = ld2<T>(in + (int64_t)ka * es, vec), f = ld2<T>(in + (int64_t)kb * es, vec);
+        a = {e.x, f.x};
+        b = {e.y, f.y};
+      }
+      if (OP == OP_I1 && j == 0 && m == 0) a.x = b.x = T(0);   // DST-I has no mode 0
+      A[j] = a;
+      B[j] = b;
+    }
+  }
+
+  // -------------------------------------------------------------- weight
+  Weights<T, N> WA, WB;
+  constexpr bool fused = OP == OP_F2I2 || OP == OP_F1I1 || OP == OP_F1I2;
+  if (fused || job.wmode != W_NONE) {
+    auto setup = [&](int ln) {
+      Weights<T, N> w;
+      w.s2 = s2;
+      w.h = h;
+      w.inv_mu = inv_mu;
+      w.wmode = job.wmode;
+      w.own = job.wc == axis;
+      w.kind = w.own ? 0 : 1;
+      // the two other axes' mode indices and their kinds (component axis 0, else 1)
+      const int hi = ln / N, lo = ln % N;
+      const int ax1 = axis == 0 ? 1 : 0, ax2 = axis == 2 ? 1 : 2;   // lo runs along ax1, hi along ax2
+      const T v1 = s2[(job.wc == ax1 ? 0 : 1) * N + lo], v2 = s2[(job.wc == ax2 ? 0 : 1) * N + hi];
+      w.rest = v1 + v2;
+      w.num = w.own ? T(0) : (job.wc == ax1 ? w.numer(v1, lo == 0) : w.numer(v2, hi == 0));
+      return w;
+    };
+    WA = setup(line);
+    WB = setup(line + 1);
+  }
+  // the weights of modes a1, a2 of both lines: one reciprocal for the four (products of
+  // 4 sin^2 sums, 1e-4 .. 12 each)
+  auto weigh = [&](int a1, int a2, T& w1, T& w2, T& u1, T& u2) {
+    T d1, d2, e1, e2;
+    const T n1 = WA.at(a1, d1), n2 = WA.at(a2, d2), o1 = WB.at(a1, e1), o2 = WB.at(a2, e2);
+    if constexpr (sizeof(T) == 4) {
+      w1 = n1 * plane::rcp(d1);
+      w2 = n2 * plane::rcp(d2);
+      u1 = o1 * plane::rcp(e1);
+      u2 = o2 * plane::rcp(e2);
+    } else {
+      const T d = d1 * d2, e = e1 * e2, r = T(1) / (d * e), rd = e * r, re = d * r;
+      w1 = n1 * (d2 * rd);
+      w2 = n2 * (d1 * rd);
+      u1 = o1 * (e2 * re);
+      u2 = o2 * (e1 * re);
+    }
+  };
+  if constexpr (fused) {
+#pragma unroll
+    for (int j = 0; j < H; ++j) {
+      int ka = m + M * j, kb = k2(j);
+      if constexpr (OP == OP_F2I2) {
+        ka = mode(ka);
+        kb = mode(kb);
+      }
+      T w1, w2, u1, u2;
+      weigh(ka, kb, w1, w2, u1, u2);
+      A[j] = {A[j].x * w1, A[j].y * w2};
+      B[j] = {B[j].x * u1, B[j].y * u2};
+    }
+  }
+
+  // ------------------------------------------------------------- inverse
+  if constexpr (op_inv2(OP)) {
+    // both lines in one FFT: conj Z_k = q conj(a + i b), conj Z_(N-k) = conj(q) (a - i b)
+    // with a = X_k - i X_(N-k) of line A, b of line B
+    C2<T> v[R], up[H];
+#pragma unroll
+    for (int j = 0; j < H; ++j) {
+      const C2<T> a = {A[j].x, -A[j].y}, b = {B[j].x, -B[j].y}, q = qg[m + M * j];
+      C2<T> lo = cmul(q, C2<T>{a.x - b.y, -(a.y + b.x)});
+      C2<T> hi = cmul(plane::conjg(q), C2<T>{a.x + b.y, a.y - b.x});
+      if (j == 0 && m == 0) {
+        lo = {a.x, -b.x};
+        hi = {r2 * A[0].y, -(r2 * B[0].y)};
+      }
+      v[j] = lo;
+      up[j] = {__shfl_sync(0xffffffffu, hi.x, partner), __shfl_sync(0xffffffffu, hi.y, partner)};
+    }
+    plane::mirror_put<N, T>(v, up, m);
+    plane::team_fft<N, T>(v, P, X, tws, m);
+    const T sc = T(1) / T(N), so = (OP == OP_I2 || OP == OP_F2I2) && dst ? -sc : sc;
+    const bool weighted = OP == OP_I2 && job.wmode != W_NONE;
+#pragma unroll
+    for (int j = 0; j < H; ++j) {
+      const int n = m + M * j;
+      // v holds the conjugate: line A in the real, minus line B in the imaginary part;
+      // element 2n here, element 2n + 1 at position N - 1 - n
+      C2<T> e = {sc * v[j].x, -(sc * v[j].y)};
+      if (axis == 0) {
+        C2<T> o = {so * __shfl_xor_sync(0xffffffffu, v[R - 1 - j].x, M - 1),
+                   -(so * __shfl_xor_sync(0xffffffffu, v[R - 1 - j].y, M - 1))};
+        if (weighted) {
+          T w1, w2, u1, u2;
+          weigh(2 * n, 2 * n + 1, w1, w2, u1, u2);
+          e = {e.x * w1, e.y * u1};
+          o = {o.x * w2, o.y * u2};
+        }
+        st2<T>(out + 2 * n, e.x, o.x, vec);
+        st2<T>(out + N + 2 * n, e.y, o.y, vec);
+      } else {
+        C2<T> o = {so * v[R - 1 - j].x, -(so * v[R - 1 - j].y)};
+        const int io = 2 * ((M - 1 - m) + M * j) + 1;   // register R - 1 - j: position N - 1 - (io / 2)
+        if (weighted) {
+          T w1, w2, u1, u2;
+          weigh(2 * n, io, w1, w2, u1, u2);
+          e = {e.x * w1, e.y * u1};
+          o = {o.x * w2, o.y * u2};
+        }
+        st2<T>(out + (int64_t)(2 * n) * es, e.x, e.y, vec);
+        st2<T>(out + (int64_t)io * es, o.x, o.y, vec);
+      }
+    }
+  } else if constexpr (op_inv1(OP)) {
+#pragma unroll 1
+    for (int ab = 0; ab < 2; ++ab) {
+      C2<T> v[R], up[H];
+#pragma unroll
+      for (int j = 0; j < H; ++j) {
+        const C2<T> f = ab ? B[j] : A[j], w = twg[m + M * j];   // exp(-i pi k / N)
+        const T s = f.x + f.y, d = f.y - f.x, cs = w.x * s, ss = -(w.y * s);
+        C2<T> lo = {cs, -(ss + d)}, hi = {-cs, d - ss};   // conjugated
+        if (j == 0 && m == 0) {
+          lo = {T(0), T(0)};
+          hi = {T(0), T(-2) * f.y};
+        }
+        v[j] = lo;
+        up[j] = {__shfl_sync(0xffffffffu, hi.x, partner), __shfl_sync(0xffffffffu, hi.y, partner)};
+      }
+      plane::mirror_put<N, T>(v, up, m);
+      plane::team_fft<N, T>(v, P, X, tws, m);
+      Tout* x = out + ab * ls;
+      const T sc = T(1) / T(N);
+      const bool weighted = OP == OP_I1 && job.wmode != W_NONE;
+#pragma unroll
+      for (int j = 0; j < H; ++j) {
+        const int n = m + M * j;
+        T e = sc * v[j].x, o = -(sc * v[j].y);
+        if (j == 0 && m == 0) e = T(0);
+        if (weighted) {
+          T w1, w2, u1, u2;
+          weigh(2 * n, 2 * n + 1, w1, w2, u1, u2);
+          e *= ab ? u1 : w1;
+          o *= ab ? u2 : w2;
+        }
+        if (axis == 0) {
+          st2<T>(x + 2 * n, e, o, vec);
+        } else {
+          x[(int64_t)(2 * n) * es] = e;
+          x[(int64_t)(2 * n + 1) * es] = o;
+        }
+      }
+    }
+  } else {   // forward only: the modes go to memory
+#pragma unroll
+    for (int j = 0; j < H; ++j) {
+      int ka = m + M * j, kb = k2(j);
+      if constexpr (OP == OP_F2) {
+        ka = mode(ka);
+        kb = mode(kb);
+      }
+      C2<T> a = A[j], b = B[j];
+      if (job.wmode != W_NONE) {
+        T w1, w2, u1, u2;
+        weigh(ka, kb, w1, w2, u1, u2);
+        a = {a.x * w1, a.y * w2};
+        b = {b.x * u1, b.y * u2};
+      }
+      if (axis == 0) {
+        out[ka] = a.x;
+        out[kb] = a.y;
+        out[N + ka] = b.x;
+        out[N + kb] = b.y;
+      } else {
+        st2<T>(out + (int64_t)ka * es, a.x, b.x, vec);
+        st2<T>(out + (int64_t)kb * es, a.y, b.y, vec);
+      }
+    }
+  }
+}
+
+}  // namespace lines
+}  // namespace kfbim
