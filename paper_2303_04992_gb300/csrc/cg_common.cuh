@@ -36,8 +36,27 @@ struct CGScalars {
   double rr, bb, stop, dq, alpha, beta, sumd, rank1, cdiag;
   int done, iters;
   unsigned int ticket[3];
-  int trips;   // iterations run by the device-side loop of a conditional graph
 };
+
+// Device-side loop of a CG run captured as a conditional graph: the loop's
+// condition, the number of runs still iterating and the iteration cap.  The last
+// block of an iteration's last kernel ends the loop itself (a kernel of its own
+// for that took 3 us per iteration).  active == nullptr: no device-side loop.
+struct CgLoop {
+  cudaGraphConditionalHandle handle;
+  int* active;
+  int maxit;
+};
+// Called by one thread of a run once its iteration is complete.
+__device__ __forceinline__ void loop_step(const CgLoop& loop, bool done, int iters) {
+  if (loop.active && (done || iters >= loop.maxit) && atomicSub(loop.active, 1) == 1)
+    cudaGraphSetConditional(loop.handle, 0u);
+}
+// Called by one thread of a run that had nothing to do in this iteration (it was
+// done from the start): ends the loop when no run is iterating.
+__device__ __forceinline__ void loop_idle(const CgLoop& loop) {
+  if (loop.active && *(volatile int*)loop.active <= 0) cudaGraphSetConditional(loop.handle, 0u);
+}
 
 // Sum of the gridDim.x partials by the last block; returns true in that block.
 __device__ __forceinline__ bool last_block_sum(double v, double* __restrict__ partial,

@@ -402,10 +402,13 @@ __global__ void k_cg_update(T* __restrict__ x, T* __restrict__ r, const T* __res
 // d = r + beta d; sumd = sum d; done once rr <= stop
 template <typename T>
 __global__ void k_cg_direction(T* __restrict__ d, const T* __restrict__ r, int64_t n, CGScalars* s,
-                               double* __restrict__ partial) {
+                               double* __restrict__ partial, const CgLoop loop) {
   __shared__ double sh[32];
   __shared__ double total;
-  if (s->done) return;
+  if (s->done) {
+    if (blockIdx.x == 0 && threadIdx.x == 0) loop_idle(loop);
+    return;
+  }
   const T b = T(s->beta);
   CgAcc<T> acc;
   for (int64_t e = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; e < n;
@@ -416,7 +419,9 @@ __global__ void k_cg_direction(T* __restrict__ d, const T* __restrict__ r, int64
   }
   if (last_block_sum(acc.value(), partial, &s->ticket[2], sh, &total) && threadIdx.x == 0) {
     s->sumd = total;
-    if (!(s->rr > s->stop)) s->done = 1;
+    const bool done = !(s->rr > s->stop);
+    if (done) s->done = 1;
+    loop_step(loop, done, s->iters);
   }
 }
 
@@ -509,7 +514,7 @@ __global__ void k_cg_direction_b(const __grid_constant__ CgBatchArgs<T> A, int64
 // initial scalars: rr = bb = b.b, sumd = sum b, stop = tol^2 bb
 template <typename T>
 __global__ void k_cg_init(const T* __restrict__ b, int64_t n, CGScalars* s, double tol2, double rank1,
-                          double cdiag, double* __restrict__ partial) {
+                          double cdiag, double* __restrict__ partial, int* active) {
   double s0 = 0.0, s1 = 0.0;
   bool last;
   if constexpr (sizeof(T) == 4) {
@@ -567,6 +572,7 @@ __global__ void k_cg_init(const T* __restrict__ b, int64_t n, CGScalars* s, doub
     s->cdiag = cdiag;
     s->done = (s0 > s->stop) ? 0 : 1;
     s->iters = 0;
+    if (active && !s->done) atomicAdd(active, 1);   // the runs of a device-side loop
   }
 }
 

@@ -609,7 +609,7 @@ SlabCg slab_run(kfbim_ctx* c, const CgWs<float>& w, const float* b = nullptr) {
 // scalar/vector kernels; or the three slab kernels.  All of it is a no-op
 // once cgs->done is set.
 template <typename T>
-void cg_iteration(kfbim_ctx* c, const CgWs<T>& w, cudaStream_t s) {
+void cg_iteration(kfbim_ctx* c, const CgWs<T>& w, cudaStream_t s, const CgLoop& loop = CgLoop{}) {
   const int64_t n = c->N3;
   if constexpr (std::is_same<T, float>::value) {
     if (c->slab) {
@@ -623,7 +623,7 @@ void cg_iteration(kfbim_ctx* c, const CgWs<T>& w, cudaStream_t s) {
           prof_end(c, s, at, KFBIM_KCLASS_CG_ZFWD + k, 1, (double)kSlabValues[k] * n * sizeof(float));
         }
       } else {
-        g_launches += slab_cg_iteration(&a, 1, s);
+        g_launches += slab_cg_iteration(&a, 1, loop, s);
       }
       check_launch();
       return;
@@ -633,7 +633,7 @@ void cg_iteration(kfbim_ctx* c, const CgWs<T>& w, cudaStream_t s) {
   const int at = prof_begin(c, s);
   k_cg_alpha<T><<<RED_BLOCKS, RED_THREADS, 0, s>>>(w.d, w.q, w.q2, w.q3, n, c->cgs, c->partial); ++g_launches;
   k_cg_update<T><<<RED_BLOCKS, RED_THREADS, 0, s>>>(w.x, w.r, w.d, w.q, n, c->cgs, c->partial); ++g_launches;
-  k_cg_direction<T><<<RED_BLOCKS, RED_THREADS, 0, s>>>(w.d, w.r, n, c->cgs, c->partial); ++g_launches;
+  k_cg_direction<T><<<RED_BLOCKS, RED_THREADS, 0, s>>>(w.d, w.r, n, c->cgs, c->partial, loop); ++g_launches;
   // values moved: alpha 5 N^3 (d, q, q2, q3 read, q written), update 6, direction 3
   prof_end(c, s, at, KFBIM_KCLASS_CG_VECTOR, 3, 14.0 * n * sizeof(T));
   check_launch();
@@ -646,18 +646,15 @@ struct Slot<double> { static constexpr int v = 0; };
 template <>
 struct Slot<float> { static constexpr int v = 1; };
 
-// Device side of the CG loop of a conditional graph: counts the trip and
-// keeps the loop going while the run is neither converged (done) nor at its
-// iteration cap, so the loop always ends after at most maxit trips.
-__global__ void k_cg_cond(cudaGraphConditionalHandle h, CGScalars* s, int maxit) {
-  const int t = ++s->trips;
-  cudaGraphSetConditional(h, (!s->done && t < maxit) ? 1u : 0u);
-}
+// Runs still iterating in the device-side loop, behind the single run's scalars
+// and behind the batch slots' (zeroed with them).
+int* cg_active(kfbim_ctx* c) { return reinterpret_cast<int*>(c->cgs + 1); }
+int* batch_active(kfbim_ctx* c) { return reinterpret_cast<int*>(c->bcgs + c->bcap); }
 
 // The CG graph of this precision, captured once per context (every pointer
 // it uses is a fixed workspace buffer): a conditional while node whose body is
-// one CG iteration and k_cg_cond, so that a whole CG run is one graph launch
-// and one read of the scalars; where conditional nodes are not available,
+// one CG iteration, whose last kernel ends the loop (CgLoop), so that a whole CG
+// run is one graph launch and one read of the scalars; where conditional nodes are not available,
 // kCgGraphIters iterations in a row, launched until the run is done.
 template <typename T>
 cudaGraphExec_t cg_graph(kfbim_ctx* c, const CgWs<T>& w) {
@@ -688,8 +685,7 @@ cudaGraphExec_t cg_graph(kfbim_ctx* c, const CgWs<T>& w) {
       cudaGraph_t body = np.conditional.phGraph_out[0];
       CK(cudaStreamBeginCaptureToGraph(c->cap_stream, body, nullptr, nullptr, 0,
                                        cudaStreamCaptureModeThreadLocal));
-      cg_iteration<T>(c, w, c->cap_stream);
-      k_cg_cond<<<1, 1, 0, c->cap_stream>>>(h, c->cgs, std::max(1, c->opt.cg_max));
+      cg_iteration<T>(c, w, c->cap_stream, CgLoop{h, cg_active(c), std::max(1, c->opt.cg_max)});
       CK(cudaStreamEndCapture(c->cap_stream, &body));
     }
   }
@@ -704,7 +700,7 @@ cudaGraphExec_t cg_graph(kfbim_ctx* c, const CgWs<T>& w) {
   CK(cudaGraphInstantiate(&c->cg_exec[slot], graph, 0));
   CK(cudaGraphDestroy(graph));
   c->cg_loop[slot] = loop;
-  c->cg_graph_kernels[slot] = loop ? per_iter + 1 : per_iter * kCgGraphIters;
+  c->cg_graph_kernels[slot] = loop ? per_iter : per_iter * kCgGraphIters;
   return c->cg_exec[slot];
 }
 
@@ -716,14 +712,14 @@ int cg_loop(kfbim_ctx* c, const T* b, const CgWs<T>& w, double tol, int maxit, c
   const int64_t n = c->N3;
   const bool graphs = c->use_graphs && !c->prof;
   cudaGraphExec_t exec = graphs ? cg_graph<T>(c, w) : nullptr;
-  CK(cudaMemsetAsync(c->cgs, 0, sizeof(CGScalars), s));
+  CK(cudaMemsetAsync(c->cgs, 0, 2 * sizeof(CGScalars), s));   // the scalars and the count of running runs
   const double rank1 = c->navier ? 0.0 : 1.0 / (c->mu * (double)n);
   bool started = false;
   if constexpr (std::is_same<T, float>::value) {
     if (c->slab) {
       const SlabCg a = slab_run(c, w, b);
       const double tol2 = tol * tol;
-      g_launches += slab_cg_start(&a, 1, &tol2, rank1, c->cpen, s);
+      g_launches += slab_cg_start(&a, 1, &tol2, rank1, c->cpen, cg_active(c), s);
       started = true;
     }
   }
@@ -731,7 +727,7 @@ int cg_loop(kfbim_ctx* c, const T* b, const CgWs<T>& w, double tol, int maxit, c
     CK(cudaMemsetAsync(w.x, 0, n * sizeof(T), s));
     CK(cudaMemcpyAsync(w.r, b, n * sizeof(T), cudaMemcpyDeviceToDevice, s));
     CK(cudaMemcpyAsync(w.d, b, n * sizeof(T), cudaMemcpyDeviceToDevice, s));
-    k_cg_init<T><<<RED_BLOCKS, RED_THREADS, 0, s>>>(b, n, c->cgs, tol * tol, rank1, c->cpen, c->partial);
+    k_cg_init<T><<<RED_BLOCKS, RED_THREADS, 0, s>>>(b, n, c->cgs, tol * tol, rank1, c->cpen, c->partial, cg_active(c));
     ++g_launches;
   }
   check_launch();
@@ -745,7 +741,7 @@ int cg_loop(kfbim_ctx* c, const T* b, const CgWs<T>& w, double tol, int maxit, c
     CGScalars h;
     std::memcpy(&h, c->pinned, sizeof(CGScalars));
     *iters = h.iters;
-    if (loop) g_launches += (int64_t)h.trips * c->cg_graph_kernels[Slot<T>::v];
+    if (loop) g_launches += (int64_t)std::max(1, h.iters) * c->cg_graph_kernels[Slot<T>::v];   // one trip at least
     if (!std::isfinite(h.rr)) return KFBIM_E_NONFINITE;
     if (h.done) return KFBIM_OK;
     if (loop || launched >= maxit) return KFBIM_E_NOCONV;
@@ -1353,7 +1349,7 @@ void fill_tables(kfbim_ctx* c) {
   CK(cudaMemsetAsync(c->zero_phi, 0, std::max<int64_t>(1, t.n_prim) * sizeof(double), c->setup_stream));
   c->partial = dalloc<double>(c, (size_t)RED_BLOCKS * 256);
   c->scal = dalloc<double>(c, 64);
-  c->cgs = dalloc<CGScalars>(c, 1);
+  c->cgs = dalloc<CGScalars>(c, 2);   // the scalars, and the count of running runs behind them
   c->q2 = dalloc<double>(c, N3);
   c->q3 = dalloc<double>(c, N3);
   c->T6 = dalloc<double>(c, 6 * N3);
@@ -1610,7 +1606,7 @@ void batch_alloc(kfbim_ctx* c, int B) {
     sl.fu = dalloc<float>(c, 3 * N3);
     c->bs.push_back(sl);
   }
-  c->bcgs = dalloc<CGScalars>(c, B);
+  c->bcgs = dalloc<CGScalars>(c, B + 1);
   c->bscal = dalloc<double>(c, 8 * (size_t)B);
   c->bpartial = dalloc<double>(c, run_partials(c) * B);
   if (c->bpinned) CK(cudaFreeHost(c->bpinned));
@@ -1701,18 +1697,6 @@ __global__ void k_cg_mark_idle(CGScalars* s, int nslot, unsigned long long activ
   if (b < nslot && !((active >> b) & 1ull)) s[b].done = 1;
 }
 
-// Device side of the batched CG loop: counts the trip (in every slot) and
-// keeps the loop going while any slot is running and the cap is not reached.
-__global__ void k_cg_cond_batch(cudaGraphConditionalHandle h, CGScalars* s, int nslot, int maxit) {
-  bool any = false;
-  int t = 0;
-  for (int b = 0; b < nslot; ++b) {
-    t = ++s[b].trips;
-    any = any || !s[b].done;
-  }
-  cudaGraphSetConditional(h, (any && t < maxit) ? 1u : 0u);
-}
-
 // The batched slab CG of all bcap slots as a conditional while loop: one
 // graph launch runs every slot's CG to its end (slots already done return
 // at once).  Captured on first use after the slot scalars are reset with
@@ -1723,7 +1707,7 @@ cudaGraphExec_t cg_batch_graph(kfbim_ctx* c, const std::vector<SlabCg>& all) {
   c->bcg_tried = true;
   CK(cudaStreamSynchronize(c->cap_stream));
   const int64_t before = g_launches;
-  slab_cg_iteration(all.data(), (int)all.size(), c->cap_stream);
+  slab_cg_iteration(all.data(), (int)all.size(), CgLoop{}, c->cap_stream);
   CK(cudaStreamSynchronize(c->cap_stream));
   const int64_t per_iter = g_launches - before;
   g_launches = before;
@@ -1747,13 +1731,13 @@ cudaGraphExec_t cg_batch_graph(kfbim_ctx* c, const std::vector<SlabCg>& all) {
   }
   cudaGraph_t body = np.conditional.phGraph_out[0];
   CK(cudaStreamBeginCaptureToGraph(c->cap_stream, body, nullptr, nullptr, 0, cudaStreamCaptureModeThreadLocal));
-  slab_cg_iteration(all.data(), (int)all.size(), c->cap_stream);
-  k_cg_cond_batch<<<1, 1, 0, c->cap_stream>>>(h, c->bcgs, (int)all.size(), std::max(1, c->opt.cg_max));
+  slab_cg_iteration(all.data(), (int)all.size(), CgLoop{h, batch_active(c), std::max(1, c->opt.cg_max)},
+                    c->cap_stream);
   CK(cudaStreamEndCapture(c->cap_stream, &body));
   g_launches = before;
   CK(cudaGraphInstantiate(&c->bcg_exec, graph, 0));
   CK(cudaGraphDestroy(graph));
-  c->bcg_kernels = per_iter + 1;
+  c->bcg_kernels = per_iter;
   return c->bcg_exec;
 }
 
@@ -1767,7 +1751,7 @@ void cg_batch(kfbim_ctx* c, const std::vector<int>& act, double tol, cudaStream_
   const bool graphs = c->slab && c->use_graphs && !c->prof;
   if (graphs && !c->bcg_tried) {
     // the capture stream's warm-up iteration must see every slot done
-    CK(cudaMemsetAsync(c->bcgs, 0, sizeof(CGScalars) * c->bcap, s));
+    CK(cudaMemsetAsync(c->bcgs, 0, sizeof(CGScalars) * (c->bcap + 1), s));
     k_cg_mark_idle<<<1, 64, 0, s>>>(c->bcgs, c->bcap, 0ull);
     ++g_launches;
     check_launch();
@@ -1777,7 +1761,7 @@ void cg_batch(kfbim_ctx* c, const std::vector<int>& act, double tol, cudaStream_
   cudaGraphExec_t exec = graphs ? c->bcg_exec : nullptr;
   unsigned long long mask = 0ull;
   for (int b : act) mask |= 1ull << b;
-  CK(cudaMemsetAsync(c->bcgs, 0, sizeof(CGScalars) * c->bcap, s));
+  CK(cudaMemsetAsync(c->bcgs, 0, sizeof(CGScalars) * (c->bcap + 1), s));
   k_cg_mark_idle<<<1, 64, 0, s>>>(c->bcgs, c->bcap, mask);
   ++g_launches;
   // each slot's tolerance, relaxed with its refinement tolerance as in grid_solve_mixed
@@ -1788,7 +1772,7 @@ void cg_batch(kfbim_ctx* c, const std::vector<int>& act, double tol, cudaStream_
   }
   if (c->slab && !act.empty()) {
     const std::vector<SlabCg> runs = slab_batch_runs(c, act);
-    g_launches += slab_cg_start(runs.data(), (int)runs.size(), tol2.data(), rank1, c->cpen, s);
+    g_launches += slab_cg_start(runs.data(), (int)runs.size(), tol2.data(), rank1, c->cpen, batch_active(c), s);
   }
   for (size_t k = 0; k < act.size() && !c->slab; ++k) {
     const int b = act[k];
@@ -1797,7 +1781,7 @@ void cg_batch(kfbim_ctx* c, const std::vector<int>& act, double tol, cudaStream_
     CK(cudaMemcpyAsync(w.r, w.fu, n * sizeof(float), cudaMemcpyDeviceToDevice, s));
     CK(cudaMemcpyAsync(w.d, w.fu, n * sizeof(float), cudaMemcpyDeviceToDevice, s));
     k_cg_init<float><<<RED_BLOCKS, RED_THREADS, 0, s>>>(w.fu, n, &c->bcgs[b], tol2[k], rank1, c->cpen,
-                                                         c->partial);
+                                                         c->partial, nullptr);
     ++g_launches;
   }
   check_launch();
@@ -1813,7 +1797,11 @@ void cg_batch(kfbim_ctx* c, const std::vector<int>& act, double tol, cudaStream_
     CK(cudaStreamSynchronize(s));
     if (c->prof_used) prof_collect(c);
     std::memcpy(h.data(), c->bpinned, sizeof(CGScalars) * c->bcap);
-    if (exec) g_launches += (int64_t)h[0].trips * c->bcg_kernels;
+    if (exec) {
+      int trips = 1;
+      for (int b : act) trips = std::max(trips, h[b].iters);
+      g_launches += (int64_t)trips * c->bcg_kernels;
+    }
     std::vector<int> run;
     for (int b : act) {
       if (!std::isfinite(h[b].rr)) throw CudaError{"non-finite CG residual in a batched solve", KFBIM_E_NONFINITE};
@@ -1840,7 +1828,7 @@ void cg_batch(kfbim_ctx* c, const std::vector<int>& act, double tol, cudaStream_
       // iteration (blockIdx.y = instance; the single-run arithmetic)
       const std::vector<SlabCg> runs = slab_batch_runs(c, run);
       for (int it = 0; it < kCgGraphIters; ++it) {
-        g_launches += slab_cg_iteration(runs.data(), (int)runs.size(), s);
+        g_launches += slab_cg_iteration(runs.data(), (int)runs.size(), CgLoop{}, s);
         check_launch();
       }
     } else {

@@ -59,7 +59,8 @@ slab::SlabArgs<MAXB> make_args(const SlabCg* runs, int nrun) {
 // Kernel `which` of the iteration: 0 k_cg_zfwd, 1 k_cg_terms, 2 k_cg_zinv; 3 is
 // k_cg_fin, the update still pending when a run stops.
 template <int N, int MAXB>
-void launch_nb(int which, const slab::SlabArgs<MAXB>& args, const SlabCg& t, int nrun, cudaStream_t st) {
+void launch_nb(int which, const slab::SlabArgs<MAXB>& args, const SlabCg& t, int nrun, const CgLoop& loop,
+               cudaStream_t st) {
   using Z = slab::ZShape<N>;
   using V = slab::Conv<N>;
   switch (which) {
@@ -75,7 +76,7 @@ void launch_nb(int which, const slab::SlabArgs<MAXB>& args, const SlabCg& t, int
             args, t.tw, t.qN, t.s2, t.inv_mu);
       break;
     case 2:
-      slab::k_cg_zinv<N, MAXB><<<dim3(Z::BLOCKS, nrun), Z::THREADS, Z::bytes, st>>>(args, t.tw, t.qN);
+      slab::k_cg_zinv<N, MAXB><<<dim3(Z::BLOCKS, nrun), Z::THREADS, Z::bytes, st>>>(args, t.tw, t.qN, loop);
       break;
     default:
       slab::k_cg_fin<N, MAXB><<<dim3(V::BLOCKS, nrun), V::THREADS, V::bytes, st>>>(args);
@@ -84,28 +85,30 @@ void launch_nb(int which, const slab::SlabArgs<MAXB>& args, const SlabCg& t, int
 
 // `count` kernels of the iteration from `first` on, for nrun runs.
 template <int N>
-void launch_n(int first, int count, const SlabCg* runs, int nrun, cudaStream_t st) {
+void launch_n(int first, int count, const SlabCg* runs, int nrun, const CgLoop& loop, cudaStream_t st) {
   if (nrun == 1) {
     const slab::SlabArgs<1> args = make_args<1>(runs, 1);
-    for (int k = first; k < first + count; ++k) launch_nb<N, 1>(k, args, runs[0], 1, st);
+    for (int k = first; k < first + count; ++k) launch_nb<N, 1>(k, args, runs[0], 1, loop, st);
   } else {
     const slab::SlabArgs<kSlabBatchMax> args = make_args<kSlabBatchMax>(runs, nrun);
-    for (int k = first; k < first + count; ++k) launch_nb<N, kSlabBatchMax>(k, args, runs[0], nrun, st);
+    for (int k = first; k < first + count; ++k) launch_nb<N, kSlabBatchMax>(k, args, runs[0], nrun, loop, st);
   }
 }
 
 template <int N>
-void start_n(const SlabCg* runs, int nrun, const double* tol2, double rank1, double cdiag, cudaStream_t st) {
+void start_n(const SlabCg* runs, int nrun, const double* tol2, double rank1, double cdiag, int* active,
+             cudaStream_t st) {
   using V = slab::Conv<N>;
   slab::Tol2<1> t1{};
   if (nrun == 1) {
     t1.v[0] = tol2[0];
-    slab::k_cg_start<N, 1><<<dim3(V::BLOCKS, 1), V::THREADS, V::bytes, st>>>(make_args<1>(runs, 1), t1, rank1, cdiag);
+    slab::k_cg_start<N, 1><<<dim3(V::BLOCKS, 1), V::THREADS, V::bytes, st>>>(make_args<1>(runs, 1), t1, rank1, cdiag,
+                                                                                      active);
   } else {
     slab::Tol2<kSlabBatchMax> t{};
     for (int k = 0; k < nrun; ++k) t.v[k] = tol2[k];
     slab::k_cg_start<N, kSlabBatchMax><<<dim3(V::BLOCKS, nrun), V::THREADS, V::bytes, st>>>(
-        make_args<kSlabBatchMax>(runs, nrun), t, rank1, cdiag);
+        make_args<kSlabBatchMax>(runs, nrun), t, rank1, cdiag, active);
   }
 }
 
@@ -113,7 +116,7 @@ template <int N>
 void schur_n(const SlabCg& a, const float* d, float* q, cudaStream_t st) {
   using V = slab::Conv<N>;
   slab::k_to_slab<N><<<V::BLOCKS, V::THREADS, V::bytes, st>>>(d, a.r);
-  launch_n<N>(0, 3, &a, 1, st);
+  launch_n<N>(0, 3, &a, 1, CgLoop{}, st);
   slab::k_from_slab<N><<<V::BLOCKS, V::THREADS, V::bytes, st>>>(a.q, q);
 }
 
@@ -141,30 +144,31 @@ cudaError_t slab_prepare(int N) {
   }
 }
 
-int slab_cg_start(const SlabCg* runs, int nrun, const double* tol2, double rank1, double cdiag, cudaStream_t st) {
+int slab_cg_start(const SlabCg* runs, int nrun, const double* tol2, double rank1, double cdiag, int* active,
+                  cudaStream_t st) {
   if (nrun < 1 || nrun > kSlabBatchMax) return 0;
-#define KFBIM_CALL(N) start_n<N>(runs, nrun, tol2, rank1, cdiag, st)
+#define KFBIM_CALL(N) start_n<N>(runs, nrun, tol2, rank1, cdiag, active, st)
   KFBIM_SLAB_SWITCH(runs[0].N, KFBIM_CALL, 1)
 #undef KFBIM_CALL
 }
 
-int slab_cg_iteration(const SlabCg* runs, int nrun, cudaStream_t st) {
+int slab_cg_iteration(const SlabCg* runs, int nrun, const CgLoop& loop, cudaStream_t st) {
   if (nrun < 1 || nrun > kSlabBatchMax) return 0;
-#define KFBIM_CALL(N) launch_n<N>(0, 3, runs, nrun, st)
+#define KFBIM_CALL(N) launch_n<N>(0, 3, runs, nrun, loop, st)
   KFBIM_SLAB_SWITCH(runs[0].N, KFBIM_CALL, 3)
 #undef KFBIM_CALL
 }
 
 int slab_cg_finish(const SlabCg* runs, int nrun, cudaStream_t st) {
   if (nrun < 1 || nrun > kSlabBatchMax) return 0;
-#define KFBIM_CALL(N) launch_n<N>(3, 1, runs, nrun, st)
+#define KFBIM_CALL(N) launch_n<N>(3, 1, runs, nrun, CgLoop{}, st)
   KFBIM_SLAB_SWITCH(runs[0].N, KFBIM_CALL, 1)
 #undef KFBIM_CALL
 }
 
 int slab_launch(int which, const SlabCg& a, cudaStream_t st) {
   if (which < 0 || which > 3) return 0;
-#define KFBIM_CALL(N) launch_n<N>(which, 1, &a, 1, st)
+#define KFBIM_CALL(N) launch_n<N>(which, 1, &a, 1, CgLoop{}, st)
   KFBIM_SLAB_SWITCH(a.N, KFBIM_CALL, 1)
 #undef KFBIM_CALL
 }

@@ -223,10 +223,19 @@ k_cg_zfwd(const __grid_constant__ SlabArgs<MAXB> args, const C2<float>* __restri
     *reinterpret_cast<float4*>(z1 + g) = *reinterpret_cast<const float4*>(O1 + tile_at<N>(k, c4));
     *reinterpret_cast<float4*>(z3 + g) = *reinterpret_cast<const float4*>(O3 + tile_at<N>(k, c4));
   }
-  double sum[1];
-  if (last_block_merge<1>(acc, reinterpret_cast<float2*>(args.partial[b]), &s->ticket[2], sh, sum) &&
-      threadIdx.x == 0)
-    s->sumd = sum[0];
+  // the block's part of sum(d); k_cg_terms merges the parts
+  block_merge<1>(acc, sh);
+  if (threadIdx.x == 0) reinterpret_cast<float2*>(args.partial[b])[blockIdx.x] = make_float2(acc[0].s, acc[0].c);
+}
+
+// sum(d) from the blocks' parts of k_cg_zfwd, in block order, by one CTA.
+template <int N, int THREADS>
+__device__ __forceinline__ void merge_sumd(const float2* __restrict__ part, CGScalars* s) {
+  __shared__ float2 sh[32];
+  CgAcc<float> g[1];
+  for (int e = threadIdx.x; e < ZShape<N>::BLOCKS; e += THREADS) g[0].merge(part[e].x, part[e].y);
+  block_merge<1>(g, sh);
+  if (threadIdx.x == 0) s->sumd = g[0].value();
 }
 
 // One term of the Schur operator on one plane (plane.cuh), plane-major so that
@@ -239,6 +248,8 @@ __device__ __forceinline__ void terms_body(const SlabArgs<MAXB>& args, int unit,
   const int b = blockIdx.y;
   if (args.s[b]->done) return;
   extern __shared__ __align__(16) unsigned char smx[];
+  if (unit == 3 * N - 1 && rank == 0)
+    merge_sumd<N, plane::Shape<N>::THREADS>(reinterpret_cast<const float2*>(args.partial[b]), args.s[b]);
   const int term = unit % 3, k = unit / 3;
   const int64_t off = (int64_t)k * N * N;
   const float* in = (term == 2 ? args.z3[b] : args.z1[b]) + off;
@@ -271,14 +282,17 @@ k_cg_terms_cl(const __grid_constant__ SlabArgs<MAXB> args, const C2<float>* __re
 template <int N, int MAXB>
 __global__ void __launch_bounds__(ZShape<N>::THREADS, ZShape<N>::OCC)
 k_cg_zinv(const __grid_constant__ SlabArgs<MAXB> args, const C2<float>* __restrict__ twg,
-          const C2<float>* __restrict__ qg) {
+          const C2<float>* __restrict__ qg, const CgLoop loop) {
   using S = plane::Shape<N>;
   using Z = ZShape<N>;
   constexpr int M = S::M, R = S::R, H = S::H, TILE = Z::TILE;
   __shared__ float2 sh[4 * 32];
   const int b = blockIdx.y;
   CGScalars* s = args.s[b];
-  if (s->done) return;
+  if (s->done) {
+    if (blockIdx.x == 0 && threadIdx.x == 0) loop_idle(loop);
+    return;
+  }
   extern __shared__ __align__(16) unsigned char smi[];
   C2<float>* P = reinterpret_cast<C2<float>*>(smi);
   float* O3 = reinterpret_cast<float*>(smi);
@@ -390,8 +404,11 @@ k_cg_zinv(const __grid_constant__ SlabArgs<MAXB> args, const C2<float>* __restri
     s->alpha = al;
     s->beta = (rr != 0.0) ? rr1 / rr : 0.0;
     s->rr = rr1;
-    s->iters += 1;
-    if (!(rr1 > s->stop)) s->done = 1;
+    const int its = s->iters + 1;
+    const bool done = !(rr1 > s->stop);
+    s->iters = its;
+    if (done) s->done = 1;
+    loop_step(loop, done, its);
   }
 }
 
@@ -447,12 +464,13 @@ struct Tol2 {
 };
 
 // Start of a run on (S + rank one) x = b from x = 0: r = b in slab order, and
-// the scalars rr = b.b, stop = tol2 b.b (compensated FP32 sums, cg_common.cuh).
+// the scalars rr = b.b, stop = tol2 b.b (compensated FP32 sums, cg_common.cuh);
+// *active counts the runs that iterate.
 // x and d need no start values: the first iterations do not read them.
 template <int N, int MAXB>
 __global__ void __launch_bounds__(Conv<N>::THREADS)
 k_cg_start(const __grid_constant__ SlabArgs<MAXB> args, const __grid_constant__ Tol2<MAXB> tol2, double rank1,
-           double cdiag) {
+           double cdiag, int* active) {
   using V = Conv<N>;
   extern __shared__ float smc[];
   __shared__ float2 sh[32];
@@ -479,8 +497,8 @@ k_cg_start(const __grid_constant__ SlabArgs<MAXB> args, const __grid_constant__ 
     s->rank1 = rank1;
     s->cdiag = cdiag;
     s->iters = 0;
-    s->trips = 0;
     s->done = (sum[0] > s->stop) ? 0 : 1;
+    if (active && !s->done) atomicAdd(active, 1);
   }
 }
 

@@ -8,6 +8,7 @@
 namespace kfbim {
 
 struct CGScalars;
+struct CgLoop;
 template <typename T>
 struct C2;
 
@@ -43,15 +44,18 @@ cudaError_t slab_prepare(int N);
 //
 // Start of `nrun` independent runs on one grid (blockIdx.y = run; only
 // runs[0]'s N, tables and inv_mu are read): r = b, scalars of
-// (S + rank1 1 1^T + cdiag I) x = b, stop at tol2[k] |b_k|^2.  The scalars' memory
-// must have been zeroed.
-int slab_cg_start(const SlabCg* runs, int nrun, const double* tol2, double rank1, double cdiag, cudaStream_t st);
+// (S + rank1 1 1^T + cdiag I) x = b, stop at tol2[k] |b_k|^2; *active (nullable)
+// counts the runs that iterate.  The memory of the scalars and of *active must
+// have been zeroed.
+int slab_cg_start(const SlabCg* runs, int nrun, const double* tol2, double rank1, double cdiag, int* active,
+                  cudaStream_t st);
 // One CG iteration of the runs (a no-op on the device for a run whose s->done is
 // set); each run's arithmetic and reduction order are those of a single run.
 // Each iteration leaves its own vector update (x += alpha d, r -= alpha q)
 // pending for the next one, so a run that has stopped needs slab_cg_finish
 // before x is read.
-int slab_cg_iteration(const SlabCg* runs, int nrun, cudaStream_t st);
+// loop: the device-side loop the iteration is the body of (captured graphs).
+int slab_cg_iteration(const SlabCg* runs, int nrun, const CgLoop& loop, cudaStream_t st);
 // x = xs + alpha d in natural order, the update still pending when the run
 // stopped (whether by done or by an iteration cap).
 int slab_cg_finish(const SlabCg* runs, int nrun, cudaStream_t st);
