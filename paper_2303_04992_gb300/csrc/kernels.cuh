@@ -204,9 +204,8 @@ __global__ void k_pressure_trace(const double* __restrict__ p, const double* __r
 // --------------------------------------------------------- MAC stencils
 
 // r^(c) = f^(c) - G_c p   (face grid c; wall faces 0)
-template <typename Tp, typename Tout>
-__global__ void k_f_minus_gp(const double* __restrict__ f, const Tp* __restrict__ p, GridIx gx, double h,
-                             Tout* __restrict__ r) {
+__global__ void k_f_minus_gp(const double* __restrict__ f, const double* __restrict__ p, GridIx gx, double h,
+                             double* __restrict__ r) {
   const int64_t N3 = gx.n3();
   const double ih = 1.0 / h;
   for (int64_t e = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; e < 3 * N3;
@@ -216,33 +215,23 @@ __global__ void k_f_minus_gp(const double* __restrict__ f, const Tp* __restrict_
     int id[3];
     gx.unflat(x, id[0], id[1], id[2]);
     const int nrm = c == 0 ? id[0] : (c == 1 ? id[1] : id[2]);
-    if constexpr (sizeof(Tout) == 4 && sizeof(Tp) == 4) {
-      // FP32 result (the MIXED correction): FP32 arithmetic, f rounded by
-      // integer operations (no FP64 instruction per element)
-      float v = 0.f;
-      if (nrm > 0) {
-        const int64_t st = gx.stride(c);
-        v = f64_to_f32(f[e]) - (float(p[x]) - float(p[x - st])) * float(ih);
-      }
-      r[e] = Tout(v);
-    } else {
-      double v = 0.0;
-      if (nrm > 0) {
-        const int64_t st = gx.stride(c);
-        v = f[e] - (double(p[x]) - double(p[x - st])) * ih;
-      }
-      r[e] = Tout(v);
-    }
+    r[e] = nrm > 0 ? f[e] - (p[x] - p[x - gx.stride(c)]) * ih : 0.0;
   }
 }
 
 // FP64 residual of the corrected MAC system (Eq. MAC with the lambda_h
 // projection): rf = f - (-mu Lap u + G p), rg = g - mean(g) - D u - c p
-// (Stokes: c = 0; Navier: the mean is 0 and c = 1/(lambda + mu)).
+// (Stokes: c = 0; Navier: the mean is 0 and c = 1/(lambda + mu)), and its norm
+// r2 = |rf|^2 + |rg|^2 for the refinement's stopping test (compensated FP32 squares
+// of the values rounded to FP32: about 1e-7 relative), which a pass of its own over
+// the stored residual took 17 us for at N = 128.
 __global__ void k_mac_residual(const double* __restrict__ f, const double* __restrict__ g,
                                const double* __restrict__ gmean, const double* __restrict__ u,
                                const double* __restrict__ p, GridIx gx, double h, double mu, double cpen,
-                               double* __restrict__ rf, double* __restrict__ rg) {
+                               double* __restrict__ rf, double* __restrict__ rg, double* __restrict__ partial,
+                               unsigned int* ticket, double* __restrict__ r2) {
+  __shared__ float2 sh[32];
+  CgAcc<float> acc[1];
   const int N = gx.N;
   const int64_t N3 = gx.n3();
   const double ih = 1.0 / h, c_lap = -mu / (h * h);
@@ -280,7 +269,10 @@ __global__ void k_mac_residual(const double* __restrict__ f, const double* __res
       // rf = f - dp / h - c_lap (sum - 6 u0)
       const double lap = fma(-6.0, u0, (pair[0] + pair[1]) + pair[2]);
       const double dp = p[x] - p[x - gx.stride(c)];
-      rf[e] = fma(-c_lap, lap, fma(-ih, dp, f[e]));
+      const double v = fma(-c_lap, lap, fma(-ih, dp, f[e]));
+      rf[e] = v;
+      const float vf = f64_to_f32(v);
+      acc[0].add_prod(vf, vf);
     } else {
       double dif[3];
 #pragma unroll
@@ -292,8 +284,32 @@ __global__ void k_mac_residual(const double* __restrict__ f, const double* __res
         const double hi = (ib + 1 <= N - 1) ? ub[x + st] : 0.0;
         dif[b] = hi - lo;
       }
-      rg[x] = fma(-ih, (dif[0] + dif[1]) + dif[2], fma(-cpen, p[x], g[x] - gm));
+      const double v = fma(-ih, (dif[0] + dif[1]) + dif[2], fma(-cpen, p[x], g[x] - gm));
+      rg[x] = v;
+      const float vf = f64_to_f32(v);
+      acc[0].add_prod(vf, vf);
     }
+  }
+  double sum[1];
+  if (last_block_merge<1>(acc, reinterpret_cast<float2*>(partial), ticket, sh, sum) && threadIdx.x == 0) *r2 = sum[0];
+}
+
+// After a correction solve of the MIXED refinement: the FP32 right-hand side
+// rf - G dp of the velocity recovery, and p = dp (first) or p += dp.
+__global__ void k_recover(const double* __restrict__ rf, const float* __restrict__ dp, GridIx gx, float ih, int first,
+                          float* __restrict__ r, double* __restrict__ p) {
+  const int64_t N3 = gx.n3();
+  for (int64_t e = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; e < 3 * N3;
+       e += (int64_t)gridDim.x * blockDim.x) {
+    int64_t x;
+    const int c = gx.field(e, x);
+    int id[3];
+    gx.unflat(x, id[0], id[1], id[2]);
+    const int nrm = c == 0 ? id[0] : (c == 1 ? id[1] : id[2]);
+    const float px = dp[x];
+    // FP32 arithmetic, rf rounded by integer operations (no FP64 instruction per element)
+    r[e] = nrm > 0 ? f64_to_f32(rf[e]) - (px - dp[x - gx.stride(c)]) * ih : 0.f;
+    if (c == 0) p[x] = first ? f32_to_f64(px) : p[x] + f32_to_f64(px);
   }
 }
 
@@ -311,29 +327,62 @@ __global__ void k_dot_partial(const Ta* __restrict__ x, const Tb* __restrict__ y
   if (threadIdx.x == 0) partial[blockIdx.x] = s;
 }
 
-// partial[b] = this block's compensated FP32 sum of x[e]^2 over a grid-stride
-// range of FP64 values rounded to FP32 by integer operations: a norm for the
-// refinement's stopping test (relative accuracy about 1e-7) without FP64
-// instructions per element.  Finished by k_merge_partials.
-__global__ void k_norm2_partial(const double* __restrict__ x, int64_t n, float2* __restrict__ partial) {
-  __shared__ float2 sh[32];
+// Mean of g and norm of the right-hand side [f (3 N^3) | g (N^3)] of a MIXED grid
+// solve in one pass: gmean = mean(g) (0 unless `stokes`), ref2 = |f|^2 + |g - gmean|^2.
+// |f|^2 sums compensated FP32 squares of the values rounded to FP32 by integer
+// operations (about 1e-7 relative, without FP64 instructions per element); the
+// two moments of g are FP64.  The last block merges the blocks' parts in order.
+constexpr int MOMENT_DOUBLES = 3;   // partial doubles per block
+__global__ void k_rhs_moments(const double* __restrict__ rhs, int64_t n3, int stokes, double* __restrict__ partial,
+                              unsigned int* ticket, double* __restrict__ gmean, double* __restrict__ ref2) {
+  __shared__ float2 shf[32];
+  __shared__ double sh[32];
+  __shared__ bool is_last;
   CgAcc<float> a[1];
-  for (int64_t e = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; e < n;
-       e += (int64_t)gridDim.x * blockDim.x) {
-    const float v = f64_to_f32(x[e]);
+  double s1 = 0.0, s2 = 0.0;
+  const int64_t t0 = (int64_t)blockIdx.x * blockDim.x + threadIdx.x, step = (int64_t)gridDim.x * blockDim.x;
+  for (int64_t e = t0; e < 3 * n3; e += step) {
+    const float v = f64_to_f32(rhs[e]);
     a[0].add_prod(v, v);
   }
-  block_merge<1>(a, sh);
-  if (threadIdx.x == 0) partial[blockIdx.x] = make_float2(a[0].s, a[0].c);
-}
-
-// out = scale * the merged sum of nb compensated pairs (fixed order, one block)
-__global__ void k_merge_partials(const float2* __restrict__ partial, int nb, double scale, double* __restrict__ out) {
-  __shared__ float2 sh[32];
-  CgAcc<float> a[1];
-  for (int b = threadIdx.x; b < nb; b += blockDim.x) a[0].merge(partial[b].x, partial[b].y);
-  block_merge<1>(a, sh);
-  if (threadIdx.x == 0) out[0] = scale * a[0].value();
+  const double* __restrict__ g = rhs + 3 * n3;
+  for (int64_t e = t0; e < n3; e += step) {
+    const double v = g[e];
+    s1 += v;
+    s2 = fma(v, v, s2);
+  }
+  block_merge<1>(a, shf);
+  s1 = block_sum<double>(s1, sh);
+  s2 = block_sum<double>(s2, sh);
+  if (threadIdx.x == 0) {
+    double* p = partial + (size_t)MOMENT_DOUBLES * blockIdx.x;
+    reinterpret_cast<float2*>(p)[0] = make_float2(a[0].s, a[0].c);
+    p[1] = s1;
+    p[2] = s2;
+    __threadfence();
+    is_last = (atomicAdd(ticket, 1u) == gridDim.x - 1);
+  }
+  __syncthreads();
+  if (!is_last) return;
+  __threadfence();
+  CgAcc<float> t[1];
+  s1 = s2 = 0.0;
+  for (int b = threadIdx.x; b < (int)gridDim.x; b += blockDim.x) {
+    const double* p = partial + (size_t)MOMENT_DOUBLES * b;
+    const float2 f = __ldcg(reinterpret_cast<const float2*>(p));
+    t[0].merge(f.x, f.y);
+    s1 += __ldcg(p + 1);
+    s2 += __ldcg(p + 2);
+  }
+  block_merge<1>(t, shf);
+  s1 = block_sum<double>(s1, sh);
+  s2 = block_sum<double>(s2, sh);
+  if (threadIdx.x == 0) {
+    const double m = stokes ? s1 / (double)n3 : 0.0;
+    *gmean = m;
+    *ref2 = t[0].value() + fmax(s2 - m * s1, 0.0);
+    *ticket = 0u;
+  }
 }
 
 // out[j] = scale * sum_b partial[j * nb + b]  (fixed order, one block per j)
@@ -595,40 +644,43 @@ __global__ void k_sum3(const T* __restrict__ b1, const T* __restrict__ b2, const
     out[e] = b1[e] + b2[e] + b3[e];
 }
 
-// out = g + b1 + b2 + b3
-template <typename Ta, typename Tb>
-__global__ void k_sum4(const Ta* __restrict__ g, const Tb* __restrict__ b1, const Tb* __restrict__ b2,
-                       const Tb* __restrict__ b3, Tb* __restrict__ out, int64_t n) {
+// out = g - gmean + b1 + b2 + b3 (gmean nullable)
+template <typename Tb>
+__global__ void k_sum4(const double* __restrict__ g, const double* __restrict__ gmean, const Tb* __restrict__ b1,
+                       const Tb* __restrict__ b2, const Tb* __restrict__ b3, Tb* __restrict__ out, int64_t n) {
+  const double gm = gmean ? gmean[0] : 0.0;
   for (int64_t e = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; e < n;
-       e += (int64_t)gridDim.x * blockDim.x)
-  {
-    if constexpr (sizeof(Ta) == 8 && sizeof(Tb) == 4)
-      out[e] = f64_to_f32(g[e]) + b1[e] + b2[e] + b3[e];   // FP32 right-hand side, FP32 sums
+       e += (int64_t)gridDim.x * blockDim.x) {
+    if constexpr (sizeof(Tb) == 4)
+      out[e] = f64_to_f32(gmean ? g[e] - gm : g[e]) + b1[e] + b2[e] + b3[e];   // FP32 right-hand side, FP32 sums
     else
-      out[e] = Tb(double(g[e]) + double(b1[e]) + double(b2[e]) + double(b3[e]));
+      out[e] = Tb((g[e] - gm) + double(b1[e]) + double(b2[e]) + double(b3[e]));
   }
 }
 
-template <typename Ta, typename Tb>
-__global__ void k_convert(const Ta* __restrict__ a, Tb* __restrict__ b, int64_t n) {
-  for (int64_t e = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; e < n;
-       e += (int64_t)gridDim.x * blockDim.x)
-    b[e] = Tb(a[e]);
-}
-
+// b += a, or b = a (assign)
 template <typename Ta>
-__global__ void k_add_to(const Ta* __restrict__ a, double* __restrict__ b, int64_t n) {
+__global__ void k_add_to(const Ta* __restrict__ a, double* __restrict__ b, int64_t n, int assign = 0) {
   for (int64_t e = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; e < n;
        e += (int64_t)gridDim.x * blockDim.x)
   {
-    if constexpr (sizeof(Ta) == 4)
-      b[e] += f32_to_f64(a[e]);   // exact widening by integer operations, one FP64 add
-    else
-      b[e] += double(a[e]);
+    double v;
+    if constexpr (sizeof(Ta) == 4) v = f32_to_f64(a[e]);   // exact widening by integer operations
+    else v = double(a[e]);
+    b[e] = assign ? v : b[e] + v;
   }
 }
 
-// b[e] = a[e] + shift[0] * sc   (pressure gauge)
+// Pressure gauge: p += mu gmean - mean(p)
+__global__ void k_gauge(double* __restrict__ p, const double* __restrict__ mean, const double* __restrict__ gmean,
+                        double mu, int64_t n) {
+  const double m = mean[0], t = mu * gmean[0];
+  for (int64_t e = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; e < n;
+       e += (int64_t)gridDim.x * blockDim.x)
+    p[e] = (p[e] - m) + t;
+}
+
+// b[e] = a[e] + shift[0] * sc
 __global__ void k_shift(double* __restrict__ b, const double* __restrict__ shift, double sc, int64_t n) {
   for (int64_t e = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; e < n;
        e += (int64_t)gridDim.x * blockDim.x)

@@ -35,6 +35,19 @@
 
 using namespace kfbim;
 
+namespace kfbim {
+// Device scalars of a single grid solve, read by the host in one copy: the CG
+// run, the count of runs in its device-side loop, and of the MIXED refinement
+// the mean of g, the norms |[f | g - mean]|^2 and |residual|^2 and the ticket of
+// their reductions.
+struct GridScalars {
+  CGScalars cg;
+  int active;
+  unsigned int ticket;
+  double gmean, ref2, r2;
+};
+}  // namespace kfbim
+
 struct kfbim_ctx {
   kfbim_options opt{};
   std::string err;
@@ -95,7 +108,8 @@ struct kfbim_ctx {
   double *J = nullptr, *rhs = nullptr, *u = nullptr, *p = nullptr, *t1 = nullptr, *t2 = nullptr;
   double *cr = nullptr, *cd = nullptr, *cq = nullptr, *rres = nullptr, *zero_phi = nullptr;
   double *partial = nullptr, *scal = nullptr;   // reduction partials, scalars
-  CGScalars* cgs = nullptr;
+  GridScalars* gs = nullptr;
+  CGScalars* cgs = nullptr;                     // &gs->cg
   // FP32 workspace (mixed)
   float *f1 = nullptr, *f2 = nullptr, *fx = nullptr, *fr = nullptr, *fd = nullptr, *fq = nullptr,
         *fu = nullptr;
@@ -332,6 +346,7 @@ void launch_jobs(kfbim_ctx* c, const Job* list, int nj, cudaStream_t s, const in
     o.dst = j.t0 == X_DST2F || j.t0 == X_DST2I;
     o.wmode = (int8_t)j.wmode;
     o.wc = (int8_t)j.wc;
+    o.acc = (int8_t)j.acc;
     // vectors of two numbers need both fields aligned (a caller's may not be)
     o.vec = reinterpret_cast<uintptr_t>(j.in) % (2 * sizeof(Tin)) == 0 &&
             reinterpret_cast<uintptr_t>(j.out) % (2 * sizeof(Tout)) == 0;
@@ -505,12 +520,12 @@ void face_poisson(kfbim_ctx* c, int cax, const Tin* r, Tout* u, T* t1, T* t2, cu
 }
 
 // u^(c) = (1/mu) (-Delta_c)^{-1} r^(c) for c = 1..3 (r, u: 3 N^3, may alias);
-// T6 = six N^3 temporaries.
-template <typename T>
-void face_poisson3(kfbim_ctx* c, const T* r, T* u, T* T6, cudaStream_t s) {
+// T6 = six N^3 temporaries.  FP32 with an FP64 result: u = or, with acc, u += .
+template <typename T, typename Tout = T>
+void face_poisson3(kfbim_ctx* c, const T* r, Tout* u, T* T6, cudaStream_t s, int acc = 0) {
   const int64_t n = c->N3;
   const T *r1 = r, *r2 = r + n, *r3 = r + 2 * n;
-  T *u1 = u, *u2 = u + n, *u3 = u + 2 * n;
+  Tout *u1 = u, *u2 = u + n, *u3 = u + 2 * n;
   T *A = T6, *B = T6 + n, *C = T6 + 2 * n, *D = T6 + 3 * n, *E = T6 + 4 * n, *F = T6 + 5 * n;
   stage<T, T, T>(c, {{r1, A, 2, X_DST2F, X_NONE, W_NONE, 0, 0}, {r2, B, 2, X_DST2F, X_NONE, W_NONE, 1, 0},
                      {r3, C, 1, X_DST2F, X_NONE, W_NONE, 2, 0}}, s);
@@ -520,8 +535,8 @@ void face_poisson3(kfbim_ctx* c, const T* r, T* u, T* T6, cudaStream_t s) {
                      {F, C, 2, X_DST1F, X_DST1I, W_POISSON, 2, 0}}, s);
   stage<T, T, T>(c, {{A, D, 1, X_DST2I, X_NONE, W_NONE, 0, 0}, {B, E, 0, X_DST2I, X_NONE, W_NONE, 1, 0},
                      {C, F, 0, X_DST2I, X_NONE, W_NONE, 2, 0}}, s);
-  stage<T, T, T>(c, {{D, u1, 2, X_DST2I, X_NONE, W_NONE, 0, 0}, {E, u2, 2, X_DST2I, X_NONE, W_NONE, 1, 0},
-                     {F, u3, 1, X_DST2I, X_NONE, W_NONE, 2, 0}}, s);
+  stage<T, T, Tout>(c, {{D, u1, 2, X_DST2I, X_NONE, W_NONE, 0, acc}, {E, u2, 2, X_DST2I, X_NONE, W_NONE, 1, acc},
+                        {F, u3, 1, X_DST2I, X_NONE, W_NONE, 2, acc}}, s);
 }
 
 // b_c = (1/mu) G_c^T (-Delta_c)^{-1} f^(c) for c = 1..3 into b1, b2, b3
@@ -577,15 +592,6 @@ void dot(kfbim_ctx* c, const Ta* x, const Tb* y, int64_t n, double* out, double 
   check_launch();
 }
 
-// |x|^2 of an FP64 field for the refinement's stopping test (about 1e-7
-// relative; compensated FP32 sums of the values rounded to FP32).
-void norm2_fast(kfbim_ctx* c, const double* x, int64_t n, double* out, cudaStream_t s) {
-  float2* part = reinterpret_cast<float2*>(c->partial);
-  k_norm2_partial<<<RED_BLOCKS, RED_THREADS, 0, s>>>(x, n, part); ++g_launches;
-  k_merge_partials<<<1, RED_THREADS, 0, s>>>(part, RED_BLOCKS, 1.0, out); ++g_launches;
-  check_launch();
-}
-
 constexpr int kCgGraphIters = 4;
 
 // CG vectors and stage temporaries of one precision (fixed workspace buffers).
@@ -599,9 +605,9 @@ CgWs<float> ws32(kfbim_ctx* c) { return {c->fx, c->fr, c->fd, c->fq, c->fq2, c->
 
 // The slab CG of a single run on the FP32 workspace (q2, an output of the
 // Schur right-hand side, is free during the run and holds x in slab order).
-SlabCg slab_run(kfbim_ctx* c, const CgWs<float>& w, const float* b = nullptr) {
+SlabCg slab_run(kfbim_ctx* c, const CgWs<float>& w) {
   const int64_t n = c->N3;
-  return {c->N, b, w.x, w.q2, w.r, w.d, w.q, w.T6, w.T6 + n, w.T6 + 2 * n, w.T6 + 3 * n, c->d_twc32, c->d_q32,
+  return {c->N, w.x, w.q2, w.r, w.d, w.q, w.T6, w.T6 + n, w.T6 + 2 * n, w.T6 + 3 * n, c->d_twc32, c->d_q32,
           c->d_s2f, (float)(1.0 / c->mu), c->cgs, c->partial};
 }
 
@@ -646,9 +652,8 @@ struct Slot<double> { static constexpr int v = 0; };
 template <>
 struct Slot<float> { static constexpr int v = 1; };
 
-// Runs still iterating in the device-side loop, behind the single run's scalars
-// and behind the batch slots' (zeroed with them).
-int* cg_active(kfbim_ctx* c) { return reinterpret_cast<int*>(c->cgs + 1); }
+// Runs still iterating in the device-side loop of a batch: behind the slots'
+// scalars (zeroed with them).
 int* batch_active(kfbim_ctx* c) { return reinterpret_cast<int*>(c->bcgs + c->bcap); }
 
 // The CG graph of this precision, captured once per context (every pointer
@@ -685,7 +690,7 @@ cudaGraphExec_t cg_graph(kfbim_ctx* c, const CgWs<T>& w) {
       cudaGraph_t body = np.conditional.phGraph_out[0];
       CK(cudaStreamBeginCaptureToGraph(c->cap_stream, body, nullptr, nullptr, 0,
                                        cudaStreamCaptureModeThreadLocal));
-      cg_iteration<T>(c, w, c->cap_stream, CgLoop{h, cg_active(c), std::max(1, c->opt.cg_max)});
+      cg_iteration<T>(c, w, c->cap_stream, CgLoop{h, &c->gs->active, std::max(1, c->opt.cg_max)});
       CK(cudaStreamEndCapture(c->cap_stream, &body));
     }
   }
@@ -704,71 +709,85 @@ cudaGraphExec_t cg_graph(kfbim_ctx* c, const CgWs<T>& w) {
   return c->cg_exec[slot];
 }
 
+// A CG run's scalars as the host reads them: counters and status.
+int cg_result(kfbim_ctx* c, const CGScalars& h, int slot, bool loop) {
+  c->cg_iters += h.iters;
+  if (loop) g_launches += (int64_t)std::max(1, h.iters) * c->cg_graph_kernels[slot];   // one trip at least
+  if (!std::isfinite(h.rr)) return KFBIM_E_NONFINITE;
+  return h.done ? KFBIM_OK : KFBIM_E_NOCONV;
+}
+
+// The grid scalars in one copy (waits for the stream).
+GridScalars read_grid_scalars(kfbim_ctx* c, cudaStream_t s) {
+  CK(cudaMemcpyAsync(c->pinned, c->gs, sizeof(GridScalars), cudaMemcpyDeviceToHost, s));
+  CK(cudaStreamSynchronize(s));
+  if (c->prof_used) prof_collect(c);
+  GridScalars h;
+  std::memcpy(&h, c->pinned, sizeof(GridScalars));
+  return h;
+}
+
 // CG on (S + 1 1^T / (mu N^3)) x = b from x = 0, vectors of type T, FP64
-// scalars.  With a loop graph the host reads the scalars once per run; else
-// once per kCgGraphIters iterations.
+// scalars.  b: natural order, or for the slab iteration the parts of it (rhs).
+// With a loop graph the host need not wait: with `deferred` the call returns
+// once the run is enqueued, and the caller reads the scalars with its own
+// (cg_result).  Otherwise the host reads them once per kCgGraphIters iterations.
 template <typename T>
-int cg_loop(kfbim_ctx* c, const T* b, const CgWs<T>& w, double tol, int maxit, cudaStream_t s, int* iters) {
+int cg(kfbim_ctx* c, const T* b, const SlabRhs* rhs, const CgWs<T>& w, double tol, int maxit, cudaStream_t s,
+       bool* deferred = nullptr) {
   const int64_t n = c->N3;
+  const int slot = Slot<T>::v;
+  const bool slab = std::is_same<T, float>::value && c->slab;
   const bool graphs = c->use_graphs && !c->prof;
   cudaGraphExec_t exec = graphs ? cg_graph<T>(c, w) : nullptr;
-  CK(cudaMemsetAsync(c->cgs, 0, 2 * sizeof(CGScalars), s));   // the scalars and the count of running runs
+  CK(cudaMemsetAsync(c->gs, 0, offsetof(GridScalars, ticket), s));   // the run's scalars and the loop's count
   const double rank1 = c->navier ? 0.0 : 1.0 / (c->mu * (double)n);
-  bool started = false;
   if constexpr (std::is_same<T, float>::value) {
-    if (c->slab) {
-      const SlabCg a = slab_run(c, w, b);
-      const double tol2 = tol * tol;
-      g_launches += slab_cg_start(&a, 1, &tol2, rank1, c->cpen, cg_active(c), s);
-      started = true;
+    if (slab) {
+      const SlabCg a = slab_run(c, w);
+      g_launches += slab_cg_start(&a, 1, rhs, rank1, c->cpen, &c->gs->active, s);
     }
   }
-  if (!started) {
+  if (!slab) {
     CK(cudaMemsetAsync(w.x, 0, n * sizeof(T), s));
     CK(cudaMemcpyAsync(w.r, b, n * sizeof(T), cudaMemcpyDeviceToDevice, s));
     CK(cudaMemcpyAsync(w.d, b, n * sizeof(T), cudaMemcpyDeviceToDevice, s));
-    k_cg_init<T><<<RED_BLOCKS, RED_THREADS, 0, s>>>(b, n, c->cgs, tol * tol, rank1, c->cpen, c->partial, cg_active(c));
+    k_cg_init<T><<<RED_BLOCKS, RED_THREADS, 0, s>>>(b, n, c->cgs, tol * tol, rank1, c->cpen, c->partial,
+                                                     &c->gs->active);
     ++g_launches;
   }
   check_launch();
-  const bool loop = graphs && c->cg_loop[Slot<T>::v];
-  if (loop) CK(cudaGraphLaunch(exec, s));
-  int launched = 0;
-  while (true) {
-    CK(cudaMemcpyAsync(c->pinned, c->cgs, sizeof(CGScalars), cudaMemcpyDeviceToHost, s));
-    CK(cudaStreamSynchronize(s));
-    if (c->prof_used) prof_collect(c);
-    CGScalars h;
-    std::memcpy(&h, c->pinned, sizeof(CGScalars));
-    *iters = h.iters;
-    if (loop) g_launches += (int64_t)std::max(1, h.iters) * c->cg_graph_kernels[Slot<T>::v];   // one trip at least
-    if (!std::isfinite(h.rr)) return KFBIM_E_NONFINITE;
-    if (h.done) return KFBIM_OK;
-    if (loop || launched >= maxit) return KFBIM_E_NOCONV;
-    if (graphs) {
-      CK(cudaGraphLaunch(exec, s));
-      g_launches += c->cg_graph_kernels[Slot<T>::v];
-    } else {
-      for (int it = 0; it < kCgGraphIters; ++it) cg_iteration<T>(c, w, s);
-    }
-    launched += kCgGraphIters;
-  }
-}
-
-// The CG run, and for the slab iteration the update it left pending.
-template <typename T>
-int cg(kfbim_ctx* c, const T* b, const CgWs<T>& w, double tol, int maxit, cudaStream_t s, int* iters) {
-  const int st = cg_loop<T>(c, b, w, tol, maxit, s, iters);
-  if constexpr (std::is_same<T, float>::value) {
-    if (c->slab) {
+  // the update a slab run left pending when it stopped
+  auto finish = [&] {
+    if constexpr (std::is_same<T, float>::value) {
+      if (!slab) return;
       const int at = prof_begin(c, s);
       const SlabCg a = slab_run(c, w);
       g_launches += slab_cg_finish(&a, 1, s);
       prof_end(c, s, at, KFBIM_KCLASS_CG_UPDATE, 1, (double)kSlabValues[3] * c->N3 * sizeof(float));
       check_launch();
     }
+  };
+  const bool loop = graphs && c->cg_loop[slot];
+  if (loop) CK(cudaGraphLaunch(exec, s));
+  if (loop && deferred) {
+    *deferred = true;
+    finish();
+    return KFBIM_OK;
   }
-  return st;
+  for (int launched = 0;; launched += kCgGraphIters) {
+    const CGScalars h = read_grid_scalars(c, s).cg;
+    if (loop || !std::isfinite(h.rr) || h.done || launched >= maxit) {
+      finish();
+      return cg_result(c, h, slot, loop);
+    }
+    if (graphs) {
+      CK(cudaGraphLaunch(exec, s));
+      g_launches += c->cg_graph_kernels[slot];
+    } else {
+      for (int it = 0; it < kCgGraphIters; ++it) cg_iteration<T>(c, w, s);
+    }
+  }
 }
 
 // Solve the corrected MAC system for rhs = [f1|f2|f3|g] (FP64) -> u, p (FP64).
@@ -779,14 +798,12 @@ int grid_solve_fp64(kfbim_ctx* c, cudaStream_t s) {
   double* b = c->cr;   // Schur RHS; CG copies it into its residual
   const CgWs<double> w = ws64(c);
   schur_rhs3<double, double>(c, f, w.q, w.q2, w.q3, w.T6, s);
-  k_sum4<double, double><<<grid_for(N3), 256, 0, s>>>(g, w.q, w.q2, w.q3, b, N3); ++g_launches;
+  k_sum4<double><<<grid_for(N3), 256, 0, s>>>(g, nullptr, w.q, w.q2, w.q3, b, N3); ++g_launches;
   check_launch();
-  int it = 0;
-  int st = cg<double>(c, b, w, c->opt.cg_tol, c->opt.cg_max, s, &it);
-  c->cg_iters += it;
+  int st = cg<double>(c, b, nullptr, w, c->opt.cg_tol, c->opt.cg_max, s);
   if (st != KFBIM_OK && st != KFBIM_E_NOCONV) return st;
   // u^(c) = (1/mu)(-Delta)^{-1} (f^(c) - G_c p)
-  k_f_minus_gp<double, double><<<grid_for(3 * N3), 256, 0, s>>>(f, c->p, c->gix(), c->h, c->u); ++g_launches;
+  k_f_minus_gp<<<grid_for(3 * N3), 256, 0, s>>>(f, c->p, c->gix(), c->h, c->u); ++g_launches;
   check_launch();
   face_poisson3<double>(c, c->u, c->u, w.T6, s);
   return st;
@@ -794,73 +811,87 @@ int grid_solve_fp64(kfbim_ctx* c, cudaStream_t s) {
 
 double relaxed_inner_tol(const kfbim_ctx* c, double tol);
 
-// MIXED: FP32 transforms and CG inside FP64 iterative refinement.
-int grid_solve_mixed(kfbim_ctx* c, cudaStream_t s) {
+// Whether the last stage of the velocity recovery can add into the FP64 velocity
+// itself (the four-step passes; not the runtime-N and tensor-core ones).
+bool fused_velocity(const kfbim_ctx* c) { return c->N >= 32 && !c->xf_plain; }
+
+// u^(c) = or += (1/mu) (-Delta_c)^{-1} r^(c), FP32 with an FP64 result (r is overwritten).
+void recover_velocity(kfbim_ctx* c, float* r, double* u, float* T6, bool first, cudaStream_t s) {
+  const int64_t n = c->N3;
+  if (!fused_velocity(c)) {
+    face_poisson3<float>(c, r, r, T6, s);
+    k_add_to<float><<<grid_for(3 * n), 256, 0, s>>>(r, u, 3 * n, first); ++g_launches;
+    check_launch();
+    return;
+  }
+  face_poisson3<float, double>(c, r, u, T6, s, !first);
+}
+
+// MIXED: FP32 transforms and CG inside FP64 iterative refinement.  need_p: the
+// pressure is wanted with its gauge (the trace of a matvec reads the velocity only).
+int grid_solve_mixed(kfbim_ctx* c, cudaStream_t s, bool need_p) {
   const int64_t N3 = c->N3;
   double* f = c->rhs;
   double* g = c->rhs + 3 * N3;
   double* resf = c->t1;            // FP64 residual [rf (3 fields) | rg]
   double* resg = c->t1 + 3 * N3;
-  double* gmean = c->scal + 4;
-  double* sc = c->scal + 5;
-  CK(cudaMemsetAsync(c->u, 0, 3 * N3 * sizeof(double), s));
-  CK(cudaMemsetAsync(c->p, 0, N3 * sizeof(double), s));
-  if (c->navier) CK(cudaMemsetAsync(gmean, 0, sizeof(double), s));
-  else dot(c, g, (const double*)nullptr, N3, gmean, 1.0 / (double)N3, s);
-  // u = p = 0: the first residual is [f; g - mean g] (no stencil needed)
-  CK(cudaMemcpyAsync(resf, f, 3 * N3 * sizeof(double), cudaMemcpyDeviceToDevice, s));
-  CK(cudaMemcpyAsync(resg, g, N3 * sizeof(double), cudaMemcpyDeviceToDevice, s));
-  k_shift<<<grid_for(N3), 256, 0, s>>>(resg, gmean, -1.0, N3); ++g_launches;
+  double* gmean = &c->gs->gmean;
+  k_rhs_moments<<<RED_BLOCKS, RED_THREADS, 0, s>>>(c->rhs, N3, c->navier ? 0 : 1, c->partial, &c->gs->ticket, gmean,
+                                                    &c->gs->ref2); ++g_launches;
   check_launch();
-  norm2_fast(c, resf, 4 * N3, sc, s);
-  const double ref2 = read_scalar(c, sc, s);
-  if (!std::isfinite(ref2)) return KFBIM_E_NONFINITE;
   int status = KFBIM_OK;
+  const CgWs<float> w = ws32(c);
   for (int sweep = 0;; ++sweep) {
-    if (sweep > 0) {
-      if (c->fp32_only) break;   // FP32: one correction solve, no FP64 residual
+    ++c->refine_sweeps;
+    // FP32 correction solve: b = rg + (1/mu) sum G^T (-Delta)^{-1} rf; from u = p = 0
+    // the first residual is [f; g - mean g]
+    const bool first = sweep == 0;
+    const double* rf = first ? f : resf;
+    const double* rg = first ? g : resg;
+    const double* gm = first && !c->navier ? gmean : nullptr;
+    schur_rhs3<double, float>(c, rf, w.q, w.q2, w.q3, w.T6, s);
+    const double tol = relaxed_inner_tol(c, c->refine_tol_now);
+    const SlabRhs rhs{rg, gm, w.q, w.q2, w.q3, tol * tol};
+    float* b32 = c->fu;  // N3 floats (fu holds 3*N3)
+    if (!c->slab) {
+      k_sum4<float><<<grid_for(N3), 256, 0, s>>>(rg, gm, w.q, w.q2, w.q3, b32, N3); ++g_launches;
+      check_launch();
+    }
+    bool deferred = false;
+    if (cg<float>(c, b32, &rhs, w, tol, c->opt.cg_max, s, &deferred) == KFBIM_E_NONFINITE) return KFBIM_E_NONFINITE;
+    // p += dp; u += (1/mu)(-Delta)^{-1}(rf - G dp)
+    k_recover<<<grid_for(3 * N3), 256, 0, s>>>(rf, w.x, c->gix(), (float)(1.0 / c->h), first, c->fu, c->p); ++g_launches;
+    check_launch();
+    recover_velocity(c, c->fu, c->u, w.T6, first, s);
+    if (!c->fp32_only) {   // FP32: one correction solve, no FP64 residual
       const int at = prof_begin(c, s);
-      k_mac_residual<<<grid_for(4 * N3), 256, 0, s>>>(f, g, gmean, c->u, c->p, c->gix(), c->h, c->mu, c->cpen, resf, resg); ++g_launches;
+      k_mac_residual<<<grid_for(4 * N3), 256, 0, s>>>(f, g, gmean, c->u, c->p, c->gix(), c->h, c->mu, c->cpen, resf, resg,
+                                                       c->partial, &c->gs->ticket, &c->gs->r2); ++g_launches;
       // reads f, g, u, p (8 N^3 doubles), writes rf, rg (4 N^3)
       prof_end(c, s, at, KFBIM_KCLASS_MAC_RESIDUAL, 1, 12.0 * N3 * sizeof(double));
       check_launch();
-      norm2_fast(c, resf, 4 * N3, sc, s);
-      const double r2 = read_scalar(c, sc, s);
-      if (!std::isfinite(r2)) return KFBIM_E_NONFINITE;
-      if (r2 <= c->refine_tol_now * c->refine_tol_now * ref2 || ref2 == 0.0) break;
-      if (sweep >= c->opt.refine_max) { status = KFBIM_E_NOCONV; break; }
     }
-    ++c->refine_sweeps;
-    // FP32 correction solve: b = rg + (1/mu) sum G^T (-Delta)^{-1} rf
-    const CgWs<float> w = ws32(c);
-    float* b32 = c->fu;  // N3 floats (fu holds 3*N3)
-    schur_rhs3<double, float>(c, resf, w.q, w.q2, w.q3, w.T6, s);
-    k_sum4<double, float><<<grid_for(N3), 256, 0, s>>>(resg, w.q, w.q2, w.q3, b32, N3); ++g_launches;
-    check_launch();
-    int it = 0;
-    int st = cg<float>(c, b32, w, relaxed_inner_tol(c, c->refine_tol_now), c->opt.cg_max, s, &it);
-    c->cg_iters += it;
-    if (st == KFBIM_E_NONFINITE) return st;
-    // p += dp; u += (1/mu)(-Delta)^{-1}(rf - G dp)
-    k_add_to<float><<<grid_for(N3), 256, 0, s>>>(w.x, c->p, N3); ++g_launches;
-    k_f_minus_gp<float, float><<<grid_for(3 * N3), 256, 0, s>>>(resf, w.x, c->gix(), c->h, c->fu); ++g_launches;
-    check_launch();
-    face_poisson3<float>(c, c->fu, c->fu, w.T6, s);
-    k_add_to<float><<<grid_for(3 * N3), 256, 0, s>>>(c->fu, c->u, 3 * N3); ++g_launches;
-    check_launch();
+    // one wait per sweep: the CG run's outcome and the norms
+    const GridScalars h = read_grid_scalars(c, s);
+    if (deferred && cg_result(c, h.cg, Slot<float>::v, true) == KFBIM_E_NONFINITE) return KFBIM_E_NONFINITE;
+    if (!std::isfinite(h.ref2)) return KFBIM_E_NONFINITE;
+    if (c->fp32_only) break;
+    if (!std::isfinite(h.r2)) return KFBIM_E_NONFINITE;
+    if (h.r2 <= c->refine_tol_now * c->refine_tol_now * h.ref2 || h.ref2 == 0.0) break;
+    if (sweep + 1 >= c->opt.refine_max) { status = KFBIM_E_NOCONV; break; }
   }
-  if (c->navier) return status;
+  if (c->navier || !need_p) return status;
   // gauge: mean(p) = mu * mean(g)  (the lambda_h system with gamma = 1, alpha = mu N^3)
+  double* sc = c->scal + 5;
   dot(c, c->p, (const double*)nullptr, N3, sc, 1.0 / (double)N3, s);
-  k_shift<<<grid_for(N3), 256, 0, s>>>(c->p, sc, -1.0, N3); ++g_launches;
-  k_shift<<<grid_for(N3), 256, 0, s>>>(c->p, gmean, c->mu, N3); ++g_launches;
+  k_gauge<<<grid_for(N3), 256, 0, s>>>(c->p, sc, gmean, c->mu, N3); ++g_launches;
   check_launch();
   return status;
 }
 
 // Full interface solve: jumps -> RHS -> grid solve.  Leaves J, u, p in ctx.
 int interface_solve(kfbim_ctx* c, const double* phi, const double* fpts, const double* fgrid,
-                    cudaStream_t s) {
+                    cudaStream_t s, bool need_p = true) {
   const int64_t n = c->n_all;
   const int at = prof_begin(c, s);
   k_jumps<<<(unsigned)((n + JB - 1) / JB), 3 * JB, 0, s>>>(
@@ -880,7 +911,7 @@ int interface_solve(kfbim_ctx* c, const double* phi, const double* fpts, const d
     check_launch();
   }
   ++c->interface_solves;
-  return c->opt.precision == KFBIM_MIXED ? grid_solve_mixed(c, s) : grid_solve_fp64(c, s);
+  return c->opt.precision == KFBIM_MIXED ? grid_solve_mixed(c, s, need_p) : grid_solve_fp64(c, s);
 }
 
 void trace(kfbim_ctx* c, const double* u, const double* J, double* out, cudaStream_t s) {
@@ -890,7 +921,7 @@ void trace(kfbim_ctx* c, const double* u, const double* J, double* out, cudaStre
 }
 
 int apply_impl(kfbim_ctx* c, const double* phi, double* out, cudaStream_t s) {
-  int st = interface_solve(c, phi, nullptr, nullptr, s);
+  int st = interface_solve(c, phi, nullptr, nullptr, s, false);
   if (st != KFBIM_OK && st != KFBIM_E_NOCONV) return st;
   trace(c, c->u, c->J, out, s);
   return st;
@@ -1104,7 +1135,7 @@ void adjoint_tables(kfbim_ctx* c) {
 int adjoint_tail(kfbim_ctx* c, double* out, cudaStream_t s) {
   const int64_t N3 = c->N3, n = c->n_all;
   ++c->interface_solves;
-  int st = c->opt.precision == KFBIM_MIXED ? grid_solve_mixed(c, s) : grid_solve_fp64(c, s);
+  int st = c->opt.precision == KFBIM_MIXED ? grid_solve_mixed(c, s, true) : grid_solve_fp64(c, s);
   if (st != KFBIM_OK && st != KFBIM_E_NOCONV) return st;
   double* rbar = c->t1;   // [u' | -p'] (4 N^3)
   CK(cudaMemcpyAsync(rbar, c->u, 3 * N3 * sizeof(double), cudaMemcpyDeviceToDevice, s));
@@ -1349,7 +1380,9 @@ void fill_tables(kfbim_ctx* c) {
   CK(cudaMemsetAsync(c->zero_phi, 0, std::max<int64_t>(1, t.n_prim) * sizeof(double), c->setup_stream));
   c->partial = dalloc<double>(c, (size_t)RED_BLOCKS * 256);
   c->scal = dalloc<double>(c, 64);
-  c->cgs = dalloc<CGScalars>(c, 2);   // the scalars, and the count of running runs behind them
+  c->gs = dalloc<GridScalars>(c, 1);
+  CK(cudaMemsetAsync(c->gs, 0, sizeof(GridScalars), c->setup_stream));
+  c->cgs = &c->gs->cg;
   c->q2 = dalloc<double>(c, N3);
   c->q3 = dalloc<double>(c, N3);
   c->T6 = dalloc<double>(c, 6 * N3);
@@ -1575,7 +1608,7 @@ cudaError_t noalloc_pass(const NoAllocSymbols& d, int N, double h, const double*
 // instances with one batched matvec per iteration.
 namespace {
 
-void batch_alloc(kfbim_ctx* c, int B) {
+void batch_alloc(kfbim_ctx* c, int B, cudaStream_t s) {
   if (B <= c->bcap) return;
   if (c->bcg_exec) CK(cudaGraphExecDestroy(c->bcg_exec));   // it holds the old slot scalars
   c->bcg_exec = nullptr;
@@ -1608,6 +1641,7 @@ void batch_alloc(kfbim_ctx* c, int B) {
   }
   c->bcgs = dalloc<CGScalars>(c, B + 1);
   c->bscal = dalloc<double>(c, 8 * (size_t)B);
+  CK(cudaMemsetAsync(c->bscal, 0, 8 * (size_t)B * sizeof(double), s));   // the reductions' tickets
   c->bpartial = dalloc<double>(c, run_partials(c) * B);
   if (c->bpinned) CK(cudaFreeHost(c->bpinned));
   c->bpinned = nullptr;
@@ -1646,10 +1680,10 @@ void schur_apply_batch(kfbim_ctx* c, const std::vector<int>& act, cudaStream_t s
 
 // face-to-cell (W_RHS) or face-to-face (W_POISSON) transform of three face
 // fields per instance: src(b) -> dst(b) (component outputs at stride N^3)
-template <typename Tin>
+template <typename Tin, typename Tout>
 void face3_batch(kfbim_ctx* c, const std::vector<int>& act, const std::vector<const Tin*>& src,
-                 const std::vector<float*>& dst1, const std::vector<float*>& dst2,
-                 const std::vector<float*>& dst3, int wmode, cudaStream_t s) {
+                 const std::vector<Tout*>& dst1, const std::vector<Tout*>& dst2,
+                 const std::vector<Tout*>& dst3, int wmode, cudaStream_t s, int acc = 0) {
   const int64_t n = c->N3;
   const int t1 = wmode == W_RHS ? X_DCT2I : X_DST1I;
   std::vector<Job> L[5];
@@ -1670,12 +1704,13 @@ void face3_batch(kfbim_ctx* c, const std::vector<int>& act, const std::vector<co
     L[3].push_back({A, D, 1, X_DST2I, X_NONE, W_NONE, 0, 0});
     L[3].push_back({B, E, 0, X_DST2I, X_NONE, W_NONE, 1, 0});
     L[3].push_back({C, F, 0, X_DST2I, X_NONE, W_NONE, 2, 0});
-    L[4].push_back({D, dst1[q], 2, X_DST2I, X_NONE, W_NONE, 0, 0});
-    L[4].push_back({E, dst2[q], 2, X_DST2I, X_NONE, W_NONE, 1, 0});
-    L[4].push_back({F, dst3[q], 1, X_DST2I, X_NONE, W_NONE, 2, 0});
+    L[4].push_back({D, dst1[q], 2, X_DST2I, X_NONE, W_NONE, 0, acc});
+    L[4].push_back({E, dst2[q], 2, X_DST2I, X_NONE, W_NONE, 1, acc});
+    L[4].push_back({F, dst3[q], 1, X_DST2I, X_NONE, W_NONE, 2, acc});
   }
   stage_list<Tin, float, float>(c, L[0], s);
-  for (int k = 1; k < 5; ++k) stage_list<float, float, float>(c, L[k], s);
+  for (int k = 1; k < 4; ++k) stage_list<float, float, float>(c, L[k], s);
+  stage_list<float, float, Tout>(c, L[4], s);
 }
 
 // The slab CG runs of batch slots `slots`.
@@ -1684,7 +1719,7 @@ std::vector<SlabCg> slab_batch_runs(kfbim_ctx* c, const std::vector<int>& slots)
   std::vector<SlabCg> runs;
   for (int b : slots) {
     const kfbim_ctx::Slot& w = c->bs[b];
-    runs.push_back({c->N, w.fu, w.x, w.q2, w.r, w.d, w.q, w.T6, w.T6 + n, w.T6 + 2 * n, w.T6 + 3 * n, c->d_twc32,
+    runs.push_back({c->N, w.x, w.q2, w.r, w.d, w.q, w.T6, w.T6 + n, w.T6 + 2 * n, w.T6 + 3 * n, c->d_twc32,
                     c->d_q32, c->d_s2f, (float)(1.0 / c->mu), &c->bcgs[b], c->bpartial + run_partials(c) * b});
   }
   return runs;
@@ -1741,8 +1776,10 @@ cudaGraphExec_t cg_batch_graph(kfbim_ctx* c, const std::vector<SlabCg>& all) {
   return c->bcg_exec;
 }
 
-// Lockstep FP32 CG of the instances in `act` on (S + ...) x = b (b in fu[0:N3]).
-void cg_batch(kfbim_ctx* c, const std::vector<int>& act, double tol, cudaStream_t s) {
+// Lockstep FP32 CG of the instances in `act` on (S + ...) x = b, b = rg - gm + q +
+// q2 + q3 per slot (rg, gm per instance).
+void cg_batch(kfbim_ctx* c, const std::vector<int>& act, const std::vector<const double*>& rg,
+              const std::vector<const double*>& gm, double tol, cudaStream_t s) {
   const int64_t n = c->N3;
   const double rank1 = c->navier ? 0.0 : 1.0 / (c->mu * (double)n);
   std::vector<int> slots(c->bcap);
@@ -1765,22 +1802,25 @@ void cg_batch(kfbim_ctx* c, const std::vector<int>& act, double tol, cudaStream_
   k_cg_mark_idle<<<1, 64, 0, s>>>(c->bcgs, c->bcap, mask);
   ++g_launches;
   // each slot's tolerance, relaxed with its refinement tolerance as in grid_solve_mixed
-  std::vector<double> tol2;
-  for (int b : act) {
-    const double tb = std::max(tol, relaxed_inner_tol(c, c->b_refine_tol[b]));
-    tol2.push_back(tb * tb);
+  std::vector<SlabRhs> rhs;
+  for (size_t k = 0; k < act.size(); ++k) {
+    const kfbim_ctx::Slot& w = c->bs[act[k]];
+    const double tb = std::max(tol, relaxed_inner_tol(c, c->b_refine_tol[act[k]]));
+    rhs.push_back({rg[k], gm[k], w.q, w.q2, w.q3, tb * tb});
   }
   if (c->slab && !act.empty()) {
     const std::vector<SlabCg> runs = slab_batch_runs(c, act);
-    g_launches += slab_cg_start(runs.data(), (int)runs.size(), tol2.data(), rank1, c->cpen, batch_active(c), s);
+    g_launches += slab_cg_start(runs.data(), (int)runs.size(), rhs.data(), rank1, c->cpen, batch_active(c), s);
   }
   for (size_t k = 0; k < act.size() && !c->slab; ++k) {
     const int b = act[k];
     const kfbim_ctx::Slot& w = c->bs[b];
+    k_sum4<float><<<grid_for(n), 256, 0, s>>>(rg[k], gm[k], w.q, w.q2, w.q3, w.fu, n);
+    ++g_launches;
     CK(cudaMemsetAsync(w.x, 0, n * sizeof(float), s));
     CK(cudaMemcpyAsync(w.r, w.fu, n * sizeof(float), cudaMemcpyDeviceToDevice, s));
     CK(cudaMemcpyAsync(w.d, w.fu, n * sizeof(float), cudaMemcpyDeviceToDevice, s));
-    k_cg_init<float><<<RED_BLOCKS, RED_THREADS, 0, s>>>(w.fu, n, &c->bcgs[b], tol2[k], rank1, c->cpen,
+    k_cg_init<float><<<RED_BLOCKS, RED_THREADS, 0, s>>>(w.fu, n, &c->bcgs[b], rhs[k].tol2, rank1, c->cpen,
                                                          c->partial, nullptr);
     ++g_launches;
   }
@@ -1870,93 +1910,98 @@ std::vector<double> read_slots(kfbim_ctx* c, const std::vector<int>& act, int k,
 }
 
 // MIXED grid solve of the instances in `act` (rhs in slot.rhs -> slot.u, slot.p).
-void grid_solve_batch(kfbim_ctx* c, const std::vector<int>& act, cudaStream_t s) {
+void grid_solve_batch(kfbim_ctx* c, const std::vector<int>& act, cudaStream_t s, bool need_p) {
   const int64_t N3 = c->N3;
+  // slot scalars: 0 mean of g, 1 and 2 the norms, 3 mean of p, 6 the reductions' ticket
+  auto ticket = [&](int b) { return reinterpret_cast<unsigned int*>(c->bscal + 8 * b + 6); };
   for (int b : act) {
     const kfbim_ctx::Slot& w = c->bs[b];
-    double* g = w.rhs + 3 * N3;
-    double* gmean = c->bscal + 8 * b;
-    CK(cudaMemsetAsync(w.u, 0, 3 * N3 * sizeof(double), s));
-    CK(cudaMemsetAsync(w.p, 0, N3 * sizeof(double), s));
-    if (c->navier) CK(cudaMemsetAsync(gmean, 0, sizeof(double), s));
-    else dot(c, g, (const double*)nullptr, N3, gmean, 1.0 / (double)N3, s);
-    CK(cudaMemcpyAsync(w.res, w.rhs, 4 * N3 * sizeof(double), cudaMemcpyDeviceToDevice, s));
-    k_shift<<<grid_for(N3), 256, 0, s>>>(w.res + 3 * N3, gmean, -1.0, N3); ++g_launches;
-    norm2_fast(c, w.res, 4 * N3, c->bscal + 8 * b + 1, s);
+    k_rhs_moments<<<RED_BLOCKS, RED_THREADS, 0, s>>>(w.rhs, N3, c->navier ? 0 : 1, c->partial, ticket(b),
+                                                      c->bscal + 8 * b, c->bscal + 8 * b + 1);
+    ++g_launches;
   }
+  check_launch();
   const std::vector<double> ref2 = read_slots(c, act, 1, s);
   std::vector<int> live;
-  for (size_t q = 0; q < act.size(); ++q)
-    if (ref2[q] > 0.0) live.push_back(act[q]);
-  for (int sweep = 0; !live.empty(); ++sweep) {
-    if (sweep > 0) {
-      if (c->fp32_only) break;   // FP32: one correction solve, no FP64 residual
-      for (int b : live) {
-        const kfbim_ctx::Slot& w = c->bs[b];
-        k_mac_residual<<<grid_for(4 * N3), 256, 0, s>>>(w.rhs, w.rhs + 3 * N3, c->bscal + 8 * b, w.u, w.p,
-                                                        c->gix(), c->h, c->mu, c->cpen, w.res, w.res + 3 * N3);
-        ++g_launches;
-        norm2_fast(c, w.res, 4 * N3, c->bscal + 8 * b + 2, s);
-      }
-      check_launch();
-      const std::vector<double> r2 = read_slots(c, live, 2, s);
-      std::vector<int> keep;
-      for (size_t q = 0; q < live.size(); ++q) {
-        const double ref = ref2[std::find(act.begin(), act.end(), live[q]) - act.begin()];
-        const double tol = c->b_refine_tol[live[q]];
-        if (!(r2[q] <= tol * tol * ref)) keep.push_back(live[q]);
-      }
-      live.swap(keep);
-      if (live.empty() || sweep >= c->opt.refine_max) break;
+  for (size_t q = 0; q < act.size(); ++q) {
+    if (ref2[q] > 0.0) {
+      live.push_back(act[q]);
+    } else {
+      const kfbim_ctx::Slot& w = c->bs[act[q]];
+      CK(cudaMemsetAsync(w.u, 0, 3 * N3 * sizeof(double), s));
+      CK(cudaMemsetAsync(w.p, 0, N3 * sizeof(double), s));
     }
+  }
+  for (int sweep = 0; !live.empty(); ++sweep) {
+    const bool first = sweep == 0;
     c->refine_sweeps += (int)live.size();
     for (int b : live) ++c->b_sweeps[b];
-    std::vector<const double*> src;
+    std::vector<const double*> rf, rg, gm;
     std::vector<float*> d1, d2, d3;
     for (int b : live) {
       const kfbim_ctx::Slot& w = c->bs[b];
-      src.push_back(w.res);
+      rf.push_back(first ? w.rhs : w.res);
+      rg.push_back(rf.back() + 3 * N3);
+      gm.push_back(first && !c->navier ? c->bscal + 8 * b : nullptr);
       d1.push_back(w.q);
       d2.push_back(w.q2);
       d3.push_back(w.q3);
     }
-    face3_batch<double>(c, live, src, d1, d2, d3, W_RHS, s);
-    for (int b : live) {
-      const kfbim_ctx::Slot& w = c->bs[b];
-      k_sum4<double, float><<<grid_for(N3), 256, 0, s>>>(w.res + 3 * N3, w.q, w.q2, w.q3, w.fu, N3);
-      ++g_launches;
-    }
-    check_launch();
-    cg_batch(c, live, c->opt.inner_tol, s);
+    face3_batch<double, float>(c, live, rf, d1, d2, d3, W_RHS, s);
+    cg_batch(c, live, rg, gm, c->opt.inner_tol, s);
     std::vector<const float*> fsrc;
-    std::vector<float*> u1, u2, u3;
-    for (int b : live) {
-      const kfbim_ctx::Slot& w = c->bs[b];
-      k_add_to<float><<<grid_for(N3), 256, 0, s>>>(w.x, w.p, N3);
-      k_f_minus_gp<float, float><<<grid_for(3 * N3), 256, 0, s>>>(w.res, w.x, c->gix(), c->h, w.fu);
-      g_launches += 2;
+    std::vector<float*> v1, v2, v3;
+    std::vector<double*> u1, u2, u3;
+    for (size_t q = 0; q < live.size(); ++q) {
+      const kfbim_ctx::Slot& w = c->bs[live[q]];
+      k_recover<<<grid_for(3 * N3), 256, 0, s>>>(rf[q], w.x, c->gix(), (float)(1.0 / c->h), first, w.fu, w.p);
+      ++g_launches;
       fsrc.push_back(w.fu);
-      u1.push_back(w.fu);
-      u2.push_back(w.fu + N3);
-      u3.push_back(w.fu + 2 * N3);
+      v1.push_back(w.fu);
+      v2.push_back(w.fu + N3);
+      v3.push_back(w.fu + 2 * N3);
+      u1.push_back(w.u);
+      u2.push_back(w.u + N3);
+      u3.push_back(w.u + 2 * N3);
     }
     check_launch();
-    face3_batch<float>(c, live, fsrc, u1, u2, u3, W_POISSON, s);
+    if (fused_velocity(c)) {
+      face3_batch<float, double>(c, live, fsrc, u1, u2, u3, W_POISSON, s, !first);
+    } else {
+      face3_batch<float, float>(c, live, fsrc, v1, v2, v3, W_POISSON, s);
+      for (int b : live) {
+        const kfbim_ctx::Slot& w = c->bs[b];
+        k_add_to<float><<<grid_for(3 * N3), 256, 0, s>>>(w.fu, w.u, 3 * N3, first);
+        ++g_launches;
+      }
+      check_launch();
+    }
+    if (c->fp32_only) break;   // FP32: one correction solve, no FP64 residual
     for (int b : live) {
       const kfbim_ctx::Slot& w = c->bs[b];
-      k_add_to<float><<<grid_for(3 * N3), 256, 0, s>>>(w.fu, w.u, 3 * N3);
+      k_mac_residual<<<grid_for(4 * N3), 256, 0, s>>>(w.rhs, w.rhs + 3 * N3, c->bscal + 8 * b, w.u, w.p,
+                                                      c->gix(), c->h, c->mu, c->cpen, w.res, w.res + 3 * N3, c->partial,
+                                                      ticket(b), c->bscal + 8 * b + 2);
       ++g_launches;
     }
     check_launch();
+    const std::vector<double> r2 = read_slots(c, live, 2, s);
+    std::vector<int> keep;
+    for (size_t q = 0; q < live.size(); ++q) {
+      const double ref = ref2[std::find(act.begin(), act.end(), live[q]) - act.begin()];
+      const double tol = c->b_refine_tol[live[q]];
+      if (!(r2[q] <= tol * tol * ref)) keep.push_back(live[q]);
+    }
+    live.swap(keep);
+    if (sweep + 1 >= c->opt.refine_max) break;
   }
-  if (c->navier) return;
+  if (c->navier || !need_p) return;
   for (int b : act) {   // gauge mean(p) = mu mean(g)
     const kfbim_ctx::Slot& w = c->bs[b];
     double* sc = c->bscal + 8 * b + 3;
     dot(c, w.p, (const double*)nullptr, N3, sc, 1.0 / (double)N3, s);
-    k_shift<<<grid_for(N3), 256, 0, s>>>(w.p, sc, -1.0, N3);
-    k_shift<<<grid_for(N3), 256, 0, s>>>(w.p, c->bscal + 8 * b, c->mu, N3);
-    g_launches += 2;
+    k_gauge<<<grid_for(N3), 256, 0, s>>>(w.p, sc, c->bscal + 8 * b, c->mu, N3);
+    ++g_launches;
   }
   check_launch();
 }
@@ -1964,7 +2009,7 @@ void grid_solve_batch(kfbim_ctx* c, const std::vector<int>& act, cudaStream_t s)
 // Jumps, RHS and grid solve for the instances in `act`; phi/fpts/fgrid per instance.
 void interface_batch(kfbim_ctx* c, const std::vector<int>& act, const std::vector<const double*>& phi,
                      const std::vector<const double*>& fpts, const std::vector<const double*>& fgrid,
-                     cudaStream_t s) {
+                     cudaStream_t s, bool need_p) {
   const int64_t n = c->n_all;
   for (size_t q = 0; q < act.size(); ++q) {
     const kfbim_ctx::Slot& w = c->bs[act[q]];
@@ -1983,7 +2028,7 @@ void interface_batch(kfbim_ctx* c, const std::vector<int>& act, const std::vecto
   check_launch();
   c->interface_solves += (int)act.size();
   for (int b : act) ++c->b_isolves[b];
-  grid_solve_batch(c, act, s);
+  grid_solve_batch(c, act, s, need_p);
 }
 
 // Lockstep GMRES (Alg. 1 step 3) of the instances in `act` with right-hand
@@ -2039,7 +2084,7 @@ void gmres_batch(kfbim_ctx* c, const std::vector<int>& act, const std::vector<do
       phi.push_back(c->bs[b].V + (int64_t)(k - 1) * ld);
       c->b_refine_tol[b] = relaxed_refine_tol(c, resid[b]);
     }
-    interface_batch(c, live, phi, nul, nul, s);
+    interface_batch(c, live, phi, nul, nul, s, false);
     for (int b : live) {
       const kfbim_ctx::Slot& w = c->bs[b];
       k_trace<<<grid_for(c->n_prim), 256, 0, s>>>(w.u, w.J, c->n_all, c->n_prim, c->d_prim_of, c->N,
@@ -2501,7 +2546,7 @@ int kfbim_solve(kfbim_ctx* c, const double* g, const double* fpts, const double*
     const int64_t n = c->n_prim;
     CK(cudaMemcpyAsync(c->grhs, g, n * sizeof(double), cudaMemcpyDeviceToDevice, s));
     if (fpts || fgrid) {
-      int st = interface_solve(c, c->zero_phi, fpts, fgrid, s);
+      int st = interface_solve(c, c->zero_phi, fpts, fgrid, s, false);
       if (st != KFBIM_OK && st != KFBIM_E_NOCONV) return st;
       trace(c, c->u, c->J, c->gw, s);
       k_scale_copy<<<grid_for(n), 256, 0, s>>>(c->gw, -1.0, nullptr, c->gw, n); ++g_launches;
@@ -2555,7 +2600,7 @@ int kfbim_solve_batch(kfbim_ctx* c, int B, const double* g, const double* fpts, 
       }
       return worst;
     }
-    batch_alloc(c, B);
+    batch_alloc(c, B, (cudaStream_t)stream);
     reset_counters(c);
     c->b_cg.assign(c->bcap, 0);
     c->b_sweeps.assign(c->bcap, 0);
@@ -2576,7 +2621,7 @@ int kfbim_solve_batch(kfbim_ctx* c, int B, const double* g, const double* fpts, 
     }
     if (fpts || fgrid) {
       // g - G_v f: the interface solve with zero density and the forcing
-      interface_batch(c, all, zero, fp, fg, s);
+      interface_batch(c, all, zero, fp, fg, s, false);
       for (int b = 0; b < B; ++b) {
         const kfbim_ctx::Slot& w = c->bs[b];
         k_trace<<<grid_for(n), 256, 0, s>>>(w.u, w.J, na, n, c->d_prim_of, c->N, c->d_tr_comp, c->d_tr_node,
@@ -2590,7 +2635,7 @@ int kfbim_solve_batch(kfbim_ctx* c, int B, const double* g, const double* fpts, 
     std::vector<int> its(c->bcap, 0), st(c->bcap, KFBIM_OK);
     std::vector<double> res(c->bcap, 0.0);
     gmres_batch(c, all, x, its, res, st, s);
-    interface_batch(c, all, ph, fp, fg, s);
+    interface_batch(c, all, ph, fp, fg, s, true);
     for (int b = 0; b < B; ++b) {
       const kfbim_ctx::Slot& w = c->bs[b];
       if (u) CK(cudaMemcpyAsync(u + b * 3 * N3, w.u, 3 * N3 * sizeof(double), cudaMemcpyDeviceToDevice, s));

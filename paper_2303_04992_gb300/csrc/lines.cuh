@@ -52,6 +52,7 @@ struct Job {
   int8_t dst;        // F2, I2: 1 for the DST-II family
   int8_t wmode, wc;  // weight mode (transforms.cuh), component axis of the weight
   int8_t vec;
+  int8_t acc;        // FP64 output of an FP32 inverse pass: added to `out` instead of stored
 };
 template <typename Tin, typename Tout, int MAXJ>
 struct Jobs {
@@ -91,8 +92,17 @@ __device__ __forceinline__ C2<T> ld2(const Tin* p, bool vec) {
   return {to_work<T>(p[0]), to_work<T>(p[1])};
 }
 template <typename T, typename Tout>
-__device__ __forceinline__ void st2(Tout* p, T a, T b, bool vec) {
-  if (vec) {
+__device__ __forceinline__ void st2(Tout* p, T a, T b, bool vec, bool acc = false) {
+  if constexpr (sizeof(Tout) == 8 && sizeof(T) == 4) {   // exact widening by integer operations
+    double2 v = make_double2(f32_to_f64(a), f32_to_f64(b));
+    double2* q = reinterpret_cast<double2*>(p);          // a field of the library: aligned
+    if (acc) {
+      const double2 o = *q;
+      v.x += o.x;
+      v.y += o.y;
+    }
+    *q = v;
+  } else if (vec) {
     if constexpr (sizeof(Tout) == 4) *reinterpret_cast<float2*>(p) = make_float2(a, b);
     else *reinterpret_cast<double2*>(p) = make_double2(a, b);
   } else {
@@ -152,7 +162,7 @@ k_lines(const __grid_constant__ Jobs<Tin, Tout, MAXJ> jobs, T h, T inv_mu, const
   const int pair = blockIdx.x * L::TEAMS + t;   // N^2 / 2 is a multiple of the CTA's teams
   const int line = 2 * pair;
   const int axis = job.axis;
-  const bool vec = job.vec, dst = job.dst;
+  const bool vec = job.vec, dst = job.dst, acc = job.acc;
   // lines: x: line = k N + j (contiguous); y: (k, i); z: (j, i); ls, es: strides of lines and elements
   const int64_t base = axis == 0 ? (int64_t)line * N : (axis == 1 ? (int64_t)(line / N) * N * N + line % N : line);
   const int64_t ls = axis == 0 ? N : 1, es = axis == 0 ? 1 : (axis == 1 ? N : (int64_t)N * N);
@@ -353,8 +363,8 @@ k_lines(const __grid_constant__ Jobs<Tin, Tout, MAXJ> jobs, T h, T inv_mu, const
           e = {e.x * w1, e.y * u1};
           o = {o.x * w2, o.y * u2};
         }
-        st2<T>(out + 2 * n, e.x, o.x, vec);
-        st2<T>(out + N + 2 * n, e.y, o.y, vec);
+        st2<T>(out + 2 * n, e.x, o.x, vec, acc);
+        st2<T>(out + N + 2 * n, e.y, o.y, vec, acc);
       } else {
         C2<T> o = {so * v[R - 1 - j].x, -(so * v[R - 1 - j].y)};
         const int io = 2 * ((M - 1 - m) + M * j) + 1;   // register R - 1 - j: position N - 1 - (io / 2)
@@ -364,8 +374,8 @@ k_lines(const __grid_constant__ Jobs<Tin, Tout, MAXJ> jobs, T h, T inv_mu, const
           e = {e.x * w1, e.y * u1};
           o = {o.x * w2, o.y * u2};
         }
-        st2<T>(out + (int64_t)(2 * n) * es, e.x, e.y, vec);
-        st2<T>(out + (int64_t)io * es, o.x, o.y, vec);
+        st2<T>(out + (int64_t)(2 * n) * es, e.x, e.y, vec, acc);
+        st2<T>(out + (int64_t)io * es, o.x, o.y, vec, acc);
       }
     }
   } else if constexpr (op_inv1(OP)) {

@@ -20,7 +20,8 @@ cudaError_t raise_dynamic_smem(const void* kern, size_t bytes);
 // One launch of operation op (lines::Op) for grid N over njobs jobs (blockIdx.y =
 // job), with the FP32 or FP64 tables of the context.  (Tin, T, Tout) =
 // (double, double, double) with MAXJ = 3; (float, float, float) and, for
-// op = OP_F2 only, (double, float, float) with MAXJ = 3 and kLineBatchJobs;
+// op = OP_F2 only, (double, float, float), for OP_I2 only, (float, float, double),
+// with MAXJ = 3 and kLineBatchJobs;
 // cudaErrorInvalidValue for a combination that has no kernel (plain DST-I passes
 // of a batch).
 template <int N, typename Tin, typename T, typename Tout, int MAXJ>

@@ -22,7 +22,12 @@ cudaError_t lines_launch(int op, const lines::Jobs<Tin, Tout, MAXJ>& jobs, int n
                          const C2<T>* tw, const C2<T>* qN, const T* s2, cudaStream_t s) {
 #define KFBIM_LINES_OP(OP) \
   case OP: return lines_launch_op<N, OP, Tin, T, Tout, MAXJ>(jobs, njobs, h, inv_mu, tw, qN, s2, s)
-  if constexpr (sizeof(Tin) == sizeof(T)) {
+  if constexpr (sizeof(Tout) > sizeof(T)) {
+    switch (op) {
+      KFBIM_LINES_OP(lines::OP_I2);
+      default: break;
+    }
+  } else if constexpr (sizeof(Tin) == sizeof(T)) {
     switch (op) {
       KFBIM_LINES_OP(lines::OP_F2);
       KFBIM_LINES_OP(lines::OP_I2);
@@ -58,5 +63,7 @@ cudaError_t lines_launch(int op, const lines::Jobs<Tin, Tout, MAXJ>& jobs, int n
   KFBIM_LINES_INSTANTIATE_ONE(N, double, double, double, kfbim::kLineJobs)          \
   KFBIM_LINES_INSTANTIATE_ONE(N, double, float, float, kfbim::kLineJobs)            \
   KFBIM_LINES_INSTANTIATE_ONE(N, double, float, float, kfbim::kLineBatchJobs)       \
+  KFBIM_LINES_INSTANTIATE_ONE(N, float, float, double, kfbim::kLineJobs)            \
+  KFBIM_LINES_INSTANTIATE_ONE(N, float, float, double, kfbim::kLineBatchJobs)       \
   KFBIM_LINES_INSTANTIATE_ONE(N, float, float, float, kfbim::kLineJobs)             \
   KFBIM_LINES_INSTANTIATE_ONE(N, float, float, float, kfbim::kLineBatchJobs)

@@ -40,7 +40,6 @@ template <int MAXB>
 slab::SlabArgs<MAXB> make_args(const SlabCg* runs, int nrun) {
   slab::SlabArgs<MAXB> a{};
   for (int k = 0; k < nrun; ++k) {
-    a.b[k] = runs[k].b;
     a.x[k] = runs[k].x;
     a.xs[k] = runs[k].xs;
     a.r[k] = runs[k].r;
@@ -95,21 +94,28 @@ void launch_n(int first, int count, const SlabCg* runs, int nrun, const CgLoop& 
   }
 }
 
-template <int N>
-void start_n(const SlabCg* runs, int nrun, const double* tol2, double rank1, double cdiag, int* active,
-             cudaStream_t st) {
+template <int N, int MAXB>
+void start_nb(const SlabCg* runs, int nrun, const SlabRhs* rhs, double rank1, double cdiag, int* active,
+              cudaStream_t st) {
   using V = slab::Conv<N>;
-  slab::Tol2<1> t1{};
-  if (nrun == 1) {
-    t1.v[0] = tol2[0];
-    slab::k_cg_start<N, 1><<<dim3(V::BLOCKS, 1), V::THREADS, V::bytes, st>>>(make_args<1>(runs, 1), t1, rank1, cdiag,
-                                                                                      active);
-  } else {
-    slab::Tol2<kSlabBatchMax> t{};
-    for (int k = 0; k < nrun; ++k) t.v[k] = tol2[k];
-    slab::k_cg_start<N, kSlabBatchMax><<<dim3(V::BLOCKS, nrun), V::THREADS, V::bytes, st>>>(
-        make_args<kSlabBatchMax>(runs, nrun), t, rank1, cdiag, active);
+  slab::StartArgs<MAXB> a{};
+  for (int k = 0; k < nrun; ++k) {
+    a.g[k] = rhs[k].g;
+    a.gm[k] = rhs[k].gm;
+    a.b1[k] = rhs[k].b1;
+    a.b2[k] = rhs[k].b2;
+    a.b3[k] = rhs[k].b3;
+    a.tol2[k] = rhs[k].tol2;
   }
+  slab::k_cg_start<N, MAXB><<<dim3(V::BLOCKS, nrun), V::THREADS, V::bytes, st>>>(make_args<MAXB>(runs, nrun), a, rank1,
+                                                                                 cdiag, active);
+}
+
+template <int N>
+void start_n(const SlabCg* runs, int nrun, const SlabRhs* rhs, double rank1, double cdiag, int* active,
+             cudaStream_t st) {
+  if (nrun == 1) start_nb<N, 1>(runs, 1, rhs, rank1, cdiag, active, st);
+  else start_nb<N, kSlabBatchMax>(runs, nrun, rhs, rank1, cdiag, active, st);
 }
 
 template <int N>
@@ -144,10 +150,10 @@ cudaError_t slab_prepare(int N) {
   }
 }
 
-int slab_cg_start(const SlabCg* runs, int nrun, const double* tol2, double rank1, double cdiag, int* active,
+int slab_cg_start(const SlabCg* runs, int nrun, const SlabRhs* rhs, double rank1, double cdiag, int* active,
                   cudaStream_t st) {
   if (nrun < 1 || nrun > kSlabBatchMax) return 0;
-#define KFBIM_CALL(N) start_n<N>(runs, nrun, tol2, rank1, cdiag, active, st)
+#define KFBIM_CALL(N) start_n<N>(runs, nrun, rhs, rank1, cdiag, active, st)
   KFBIM_SLAB_SWITCH(runs[0].N, KFBIM_CALL, 1)
 #undef KFBIM_CALL
 }

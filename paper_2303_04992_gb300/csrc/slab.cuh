@@ -47,6 +47,7 @@
 #include <stdint.h>
 
 #include "cg_common.cuh"
+#include "fastcvt.h"
 #include "plane.cuh"
 
 namespace kfbim {
@@ -90,7 +91,6 @@ __device__ __forceinline__ plane::YSlots<N> z_slots(int t) {
 // run's arithmetic does not depend on the batch it is part of.
 template <int MAXB>
 struct SlabArgs {
-  const float* b[MAXB];   // right-hand side, natural order (k_cg_start)
   float* x[MAXB];         // solution, natural order (k_cg_fin)
   float* xs[MAXB];        // x, r, d, q in slab order
   float* r[MAXB];
@@ -457,10 +457,14 @@ __global__ void __launch_bounds__(Conv<N>::THREADS) k_from_slab(const float* __r
   for (int e = threadIdx.x; e < V::ROWS * N; e += V::THREADS) out[V::row(blk, e / N) + e % N] = smc[(e / N) * V::RS + e % N];
 }
 
-// Squared relative tolerances of up to MAXB runs.
+// Right-hand sides b = g - gm[0] + b1 + b2 + b3 (natural order; gm nullable) and
+// squared relative tolerances of up to MAXB runs.
 template <int MAXB>
-struct Tol2 {
-  double v[MAXB];
+struct StartArgs {
+  const double* g[MAXB];
+  const double* gm[MAXB];
+  const float *b1[MAXB], *b2[MAXB], *b3[MAXB];
+  double tol2[MAXB];
 };
 
 // Start of a run on (S + rank one) x = b from x = 0: r = b in slab order, and
@@ -469,17 +473,21 @@ struct Tol2 {
 // x and d need no start values: the first iterations do not read them.
 template <int N, int MAXB>
 __global__ void __launch_bounds__(Conv<N>::THREADS)
-k_cg_start(const __grid_constant__ SlabArgs<MAXB> args, const __grid_constant__ Tol2<MAXB> tol2, double rank1,
+k_cg_start(const __grid_constant__ SlabArgs<MAXB> args, const __grid_constant__ StartArgs<MAXB> st, double rank1,
            double cdiag, int* active) {
   using V = Conv<N>;
   extern __shared__ float smc[];
   __shared__ float2 sh[32];
   const int run = blockIdx.y, blk = blockIdx.x;
   CGScalars* s = args.s[run];
-  const float* __restrict__ in = args.b[run];
+  const double* __restrict__ g = st.g[run];
+  const double* __restrict__ gm = st.gm[run];
+  const float *__restrict__ b1 = st.b1[run], *__restrict__ b2 = st.b2[run], *__restrict__ b3 = st.b3[run];
   CgAcc<float> acc[1];
   for (int e = threadIdx.x; e < V::ROWS * N; e += V::THREADS) {
-    const float v = in[V::row(blk, e / N) + e % N];
+    const int64_t at = V::row(blk, e / N) + e % N;
+    // FP32 sums of the FP64 g rounded once (by integer operations)
+    const float v = f64_to_f32(gm ? g[at] - gm[0] : g[at]) + b1[at] + b2[at] + b3[at];
     smc[(e / N) * V::RS + e % N] = v;
     acc[0].add_prod(v, v);
   }
@@ -491,7 +499,7 @@ k_cg_start(const __grid_constant__ SlabArgs<MAXB> args, const __grid_constant__ 
       threadIdx.x == 0) {
     s->rr = sum[0];
     s->bb = sum[0];
-    s->stop = tol2.v[run] * sum[0];
+    s->stop = st.tol2[run] * sum[0];
     s->alpha = 0.0;
     s->beta = 0.0;
     s->rank1 = rank1;

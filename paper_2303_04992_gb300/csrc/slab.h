@@ -12,8 +12,7 @@ struct CgLoop;
 template <typename T>
 struct C2;
 
-// One CG run's buffers: the right-hand side b and the solution x in natural
-// order; xs, r, d, q (slab order), the z-transformed fields z1, z3 and the
+// One CG run's buffers: the solution x in natural order; xs, r, d, q (slab order), the z-transformed fields z1, z3 and the
 // term results w1, w2 (N^3 floats each); the FP32 transform tables (full-circle
 // twiddles exp(-2 pi i t / 2N), t < 2N; post-twiddles exp(-i pi k / 2N), k < N;
 // the eigenvalue table 4 sin^2 of the DCT (N) and DST (N) modes), 1/mu, the
@@ -21,7 +20,6 @@ struct C2;
 // eight bytes: k_cg_zinv stores four FP32 pairs per block).
 struct SlabCg {
   int N;
-  const float* b;
   float *x, *xs, *r, *d, *q, *z1, *z3, *w1, *w2;
   const C2<float>* tw;
   const C2<float>* qN;
@@ -42,12 +40,20 @@ cudaError_t slab_prepare(int N);
 
 // Every call below returns the number of kernels it enqueued.
 //
+// The right-hand side of a run, in natural order: b = g - gm[0] + b1 + b2 + b3 (gm
+// nullable: no shift; g FP64, rounded once); the run stops at |r|^2 <= tol2 |b|^2.
+struct SlabRhs {
+  const double* g;
+  const double* gm;
+  const float *b1, *b2, *b3;
+  double tol2;
+};
 // Start of `nrun` independent runs on one grid (blockIdx.y = run; only
 // runs[0]'s N, tables and inv_mu are read): r = b, scalars of
-// (S + rank1 1 1^T + cdiag I) x = b, stop at tol2[k] |b_k|^2; *active (nullable)
+// (S + rank1 1 1^T + cdiag I) x = b; *active (nullable)
 // counts the runs that iterate.  The memory of the scalars and of *active must
 // have been zeroed.
-int slab_cg_start(const SlabCg* runs, int nrun, const double* tol2, double rank1, double cdiag, int* active,
+int slab_cg_start(const SlabCg* runs, int nrun, const SlabRhs* rhs, double rank1, double cdiag, int* active,
                   cudaStream_t st);
 // One CG iteration of the runs (a no-op on the device for a run whose s->done is
 // set); each run's arithmetic and reduction order are those of a single run.
