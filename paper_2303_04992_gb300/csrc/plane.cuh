@@ -15,8 +15,8 @@
 //   V'_k = s_k V_k + t_k exp(i pi k / N) V_(N-k),  s, t = (w_k +- w_(N-k)) / 2
 // for a real line, and for the two real lines A, B of a complex one
 //   Z'_k = s Z_k + ds P* + c (t P + dt Z*),  P = Z_(N-k), c = exp(i pi k / N),
-// with s = (s_A + s_B) / 2, ds = (s_A - s_B) / 2 and t, dt alike; Z_(N-k) lies
-// with lane M - m of the FFT's team and comes by a shuffle.
+// with s = (s_A + s_B) / 2, ds = (s_A - s_B) / 2 and t, dt alike.  Where a lane
+// holds several residues of the index, Z_k and Z_(N-k) lie in the same lane.
 //
 // Shared memory: N/2 lines of N complex numbers, element n of line l at
 // l N + (n ^ line_sw(l)).  A team of M lanes computes one FFT, R = N / M values
@@ -28,13 +28,14 @@
 //
 // What bounds it (N = 128, 384 CTAs, FP32): instruction issue (56 % of the slots
 // of the average SM, the busiest of the 152 holds three of the 384 CTAs) and the
-// shared-memory pipe (52 %); 17.1 M warp instructions against 37.5 M for a kernel
+// shared-memory pipe (52 %); 17 M warp instructions against 37.5 M for a kernel
 // that formed every real transform and transposed the plane between the axes.
-// 30.7 us for the three terms at N = 128 (that kernel: 56.6), 8.2 at N = 64 (about
-// 30), 4.2 at N = 32 (27), 14.3 at N = 96 (five one-axis passes there: 133).  The
-// pair-blocked order of the planes gives 2.1 of the first, a copy of the code per
-// term cost 2 us (the warps waited for instructions), and 80 registers with three
-// resident CTAs run as fast as 127 with two.
+// 28.7 us for the three terms at N = 128 (that kernel: 56.6), 8.2 at N = 64 (about
+// 30), 4.2 at N = 32 (27), 12.3 at N = 96 (five one-axis passes there: 133).  The
+// pair-blocked order of the planes gives 2.1 of the first, index pairs within a lane
+// instead of shuffles 2.0 (N = 128; 2.0 of 14.3 at N = 96), a copy of the code per
+// term cost 2 (the warps waited for instructions), and 80 registers with three
+// resident CTAs run as fast as 128 with two.
 #pragma once
 
 #include <cooperative_groups.h>
@@ -299,6 +300,168 @@ __device__ __forceinline__ void mirror_put(C2<T> (&v)[Shape<N>::R], const C2<T> 
   }
 }
 
+// ------------------------------------------------------- mode pairs (k, N - k)
+// The transforms of real lines need FFT indices k and N - k together.  Where a
+// lane does an even number of DFT_M (NS), it takes residues s and R - s of the
+// index k = s + R k', so that every pair lies in one lane's registers and no
+// shuffle is needed: group g holds Z[s + R k'] in v[2 M g + k'] and Z[s' + R k'] in
+// v[2 M g + M + k'], s = g M + m, s' = R - s (lane 0, group 0: s = 0 and s' = R/2,
+// their own mirrors; pair_swap then puts each index's mirror where the other
+// lanes have it).  The inverse FFT starts from that layout with the DFT_M and
+// ends with the DFT_R, at index m + M j.  Where NS is odd, the natural layout and
+// shuffles between lanes m and M - m.
+template <int N>
+struct PairShape {
+  using S = Shape<N>;
+  static constexpr bool in_lane = S::NS % 2 == 0;
+  __device__ __forceinline__ static int s0(int g, int m) { return g * S::M + m; }
+  __device__ __forceinline__ static int s1(int g, int m) { return g == 0 && m == 0 ? S::R / 2 : S::R - g * S::M - m; }
+};
+// Lane 0, group 0, of in-lane pairs: a[k'] = Z[R k'], b[k'] = Z[R/2 + R k'].
+// Forward: upper half of a <- upper half of b; b[M-1-j] <- a[M-j], b[M-1] <- a[M/2].
+template <int M, typename T>
+__device__ __forceinline__ void pair_swap(C2<T>* a, C2<T>* b, bool lane0, bool back) {
+  C2<T> na[M / 2], nb[M / 2];
+#pragma unroll
+  for (int i = 0; i < M / 2; ++i) {
+    const int u = M / 2 + i;
+    if (!back) {
+      na[i] = b[u];
+      nb[i] = u + 1 < M ? a[u + 1] : a[M / 2];
+    } else {
+      na[i] = u == M / 2 ? b[M - 1] : b[u - 1];
+      nb[i] = a[u];
+    }
+  }
+#pragma unroll
+  for (int i = 0; i < M / 2; ++i) {
+    const int u = M / 2 + i;
+    a[u] = {lane0 ? na[i].x : a[u].x, lane0 ? na[i].y : a[u].y};
+    b[u] = {lane0 ? nb[i].x : b[u].x, lane0 ? nb[i].y : b[u].y};
+  }
+}
+
+// Forward FFT, z[m + M r] in v[r] -> the pair layout.
+template <int N, typename T, class Slots>
+__device__ __forceinline__ void fft_to_pairs(C2<T> (&v)[Shape<N>::R], C2<T>* P, const Slots& X, const C2<T>* tws,
+                                             int m) {
+  using S = Shape<N>;
+  constexpr int M = S::M, R = S::R;
+  if constexpr (!PairShape<N>::in_lane) {
+    team_fft<N, T>(v, P, X, tws, m);
+  } else {
+    dft<R>(v);
+    __syncwarp();
+#pragma unroll
+    for (int s = 0; s < R; ++s) {
+      C2<T> y = v[s];
+      if (s != 0) y = cmul(y, ldc(tws + s * M + m));
+      stc(P + X.at(s, m), y);
+    }
+    __syncwarp();
+#pragma unroll
+    for (int g = 0; g < S::NS / 2; ++g) {
+      const int s0 = PairShape<N>::s0(g, m), s1 = PairShape<N>::s1(g, m);
+      C2<T>* a = v + 2 * M * g;
+      C2<T>* b = a + M;
+#pragma unroll
+      for (int k = 0; k < M; ++k) {
+        a[k] = ldc(P + X.at(s0, k));
+        b[k] = ldc(P + X.at(s1, k));
+      }
+      dft<M>(a);
+      dft<M>(b);
+      if (g == 0) pair_swap<M>(a, b, m == 0, false);
+    }
+    __syncwarp();
+  }
+}
+// Forward FFT from the pair layout -> index m + M j in v[j].  twr[k R + s] =
+// exp(-2 pi i k s / N).
+template <int N, typename T, class Slots>
+__device__ __forceinline__ void fft_from_pairs(C2<T> (&v)[Shape<N>::R], C2<T>* P, const Slots& X, const C2<T>* tws,
+                                               const C2<T>* twr, int m) {
+  using S = Shape<N>;
+  constexpr int M = S::M, R = S::R;
+  if constexpr (!PairShape<N>::in_lane) {
+    team_fft<N, T>(v, P, X, tws, m);
+  } else {
+    __syncwarp();
+#pragma unroll
+    for (int g = 0; g < S::NS / 2; ++g) {
+      const int s0 = PairShape<N>::s0(g, m), s1 = PairShape<N>::s1(g, m);
+      C2<T>* a = v + 2 * M * g;
+      C2<T>* b = a + M;
+      if (g == 0) pair_swap<M>(a, b, m == 0, true);
+      dft<M>(a);
+      dft<M>(b);
+#pragma unroll
+      for (int k = 0; k < M; ++k) {
+        C2<T> x = a[k], y = b[k];
+        if (k != 0) {
+          x = cmul(x, ldc(twr + k * R + s0));
+          y = cmul(y, ldc(twr + k * R + s1));
+        }
+        stc(P + X.at(s0, k), x);
+        stc(P + X.at(s1, k), y);
+      }
+    }
+    __syncwarp();
+#pragma unroll
+    for (int s = 0; s < R; ++s) v[s] = ldc(P + X.at(s, m));
+    __syncwarp();
+    dft<R>(v);
+  }
+}
+// The lane's i-th index k < N/2 in the order of for_pairs, i < H.
+template <int N>
+__device__ __forceinline__ int pair_index(int i, int m) {
+  using S = Shape<N>;
+  if constexpr (PairShape<N>::in_lane) {
+    const int g = i / S::M, j = i % S::M;
+    return (j % 2 ? PairShape<N>::s1(g, m) : PairShape<N>::s0(g, m)) + S::R * (j / 2);
+  } else {
+    return m + S::M * i;
+  }
+}
+// f(i, k, self, Z_k, Z_(N-k)) for the lane's indices k < N/2; self: k = 0, with
+// Z_(N/2) in the place of Z_(N-k).  READ: the values come from v; WRITE: those
+// that f leaves go back to v.
+template <int N, bool READ, bool WRITE, typename T, class F>
+__device__ __forceinline__ void for_pairs(C2<T> (&v)[Shape<N>::R], int m, int partner, F&& f) {
+  using S = Shape<N>;
+  constexpr int M = S::M, R = S::R, H = S::H;
+  if constexpr (PairShape<N>::in_lane) {
+#pragma unroll
+    for (int g = 0; g < S::NS / 2; ++g) {
+      const int s0 = PairShape<N>::s0(g, m), s1 = PairShape<N>::s1(g, m);
+      C2<T>* a = v + 2 * M * g;
+      C2<T>* b = a + M;
+#pragma unroll
+      for (int j = 0; j < M / 2; ++j) {
+        f(g * M + 2 * j, s0 + R * j, g == 0 && j == 0 && m == 0, a[j], b[M - 1 - j]);
+        f(g * M + 2 * j + 1, s1 + R * j, false, b[j], a[M - 1 - j]);
+      }
+    }
+  } else {
+    C2<T> up[H];
+#pragma unroll
+    for (int j = 0; j < H; ++j) {
+      C2<T> z{}, g{};
+      if constexpr (READ) {
+        z = v[j];
+        g = mirror_fetch<N, T>(v, j, m, partner);
+      }
+      f(j, m + M * j, j == 0 && m == 0, z, g);
+      if constexpr (WRITE) {
+        v[j] = z;
+        up[j] = {__shfl_sync(0xffffffffu, g.x, partner), __shfl_sync(0xffffffffu, g.y, partner)};
+      }
+    }
+    if constexpr (WRITE) mirror_put<N, T>(v, up, m);
+  }
+}
+
 // 1 / d for d in [1e-8, 200]: in FP32 the hardware reciprocal (within 1 ulp)
 template <typename T>
 __device__ __forceinline__ T rcp(T d) {
@@ -361,7 +524,7 @@ struct Smem {
   using S = Shape<N>;
   static constexpr size_t scratch = S::CL > 1 ? sizeof(C2<T>) * S::TEAMS * N : 0;
   static constexpr size_t field = sizeof(C2<T>) * S::LL * N + scratch;
-  static constexpr size_t tables = sizeof(C2<T>) * (N + 2 * S::LINES) + sizeof(T) * S::LINES;
+  static constexpr size_t tables = sizeof(C2<T>) * (2 * N + 2 * S::LINES) + sizeof(T) * S::LINES;
   static constexpr size_t bytes = field + tables;
 };
 
@@ -379,10 +542,14 @@ __device__ __forceinline__ void term_plane(const T* in, T* out, const Term term,
   using S = Shape<N>;
   constexpr int M = S::M, R = S::R, H = S::H;
   C2<T>* tws = P + Smem<N, T>::field / sizeof(C2<T>);   // FFT twiddles [s][m]
-  C2<T>* qh = tws + N;                  // q_k / 2, k < N/2
+  C2<T>* twr = tws + N;                 // the same by [m][s]
+  C2<T>* qh = twr + N;                  // q_k / 2, k < N/2
   C2<T>* cy = qh + S::LINES;            // exp(i pi k / N), k < N/2
   T* sg = reinterpret_cast<T*>(cy + S::LINES);   // 4 sin^2(pi k / 2N), k < N/2
-  for (int e = threadIdx.x; e < N; e += S::THREADS) tws[e] = twg[2 * (e / M) * (e % M)];
+  for (int e = threadIdx.x; e < N; e += S::THREADS) {
+    tws[e] = twg[2 * (e / M) * (e % M)];
+    twr[e] = twg[2 * (e / R) * (e % R)];
+  }
   for (int e = threadIdx.x; e < S::LINES; e += S::THREADS) {
     const C2<T> q = qg[e];
     qh[e] = {T(0.5) * q.x, T(0.5) * q.y};
@@ -404,136 +571,115 @@ __device__ __forceinline__ void term_plane(const T* in, T* out, const Term term,
     if constexpr (S::CL > 1) cooperative_groups::this_cluster().sync();
     else __syncthreads();
   };
-  // the column pair n0, n0 + 1 of line l = m + M j
-  auto pair_at = [&](int j, int n0) -> C2<T>* {
-    const int l = m + M * j;
-    if constexpr (S::CL > 1) return lines[M * j / S::LL] + ((l % S::LL) * N + (n0 ^ line_sw<M>(l)));
+  // the column pair n0, n0 + 1 of line l
+  auto pair_at = [&](int l, int n0) -> C2<T>* {
+    if constexpr (S::CL > 1) return (l < S::LL ? lines[0] : lines[S::CL - 1]) + ((l % S::LL) * N + (n0 ^ line_sw<M>(l)));
     else return P + (l * N + (n0 ^ line_sw<M>(l)));
   };
   C2<T> v[R];
-  // One copy of the code of an FFT along x serves the forward and the inverse
-  // step (likewise along y): with a copy per step the warps wait for instructions.
+  // ---- along x: the rows of Makhoul positions 2p, 2p + 1 along y -> columns 2p, 2p + 1
 #pragma unroll 1
-  for (int back = 0; back < 2; ++back) {
-#pragma unroll 1
-    for (int rd = 0; rd < S::ROUNDS; ++rd) {
-      // the rows of Makhoul positions 2p, 2p + 1 along y <-> columns 2p, 2p + 1
-      const int n0 = 2 * (rank * S::LL + t + S::TEAMS * rd);
-      const int64_t at0 = (n0 / S::YB) * (N * S::YB) + m * S::YB + n0 % S::YB;
-      if (!back) {
-        const C2<T>* ra = reinterpret_cast<const C2<T>*>(in + at0);
-        const T fl = (n0 >= N / 2 && term.ys != signs.ys) ? T(-1) : T(1), fh = term.xs != signs.xs ? -fl : fl;
+  for (int rd = 0; rd < S::ROUNDS; ++rd) {
+    const int n0 = 2 * (rank * S::LL + t + S::TEAMS * rd);
+    const C2<T>* ra = reinterpret_cast<const C2<T>*>(in + (int64_t)(n0 / S::YB) * (N * S::YB) + m * S::YB + n0 % S::YB);
+    const T fl = (n0 >= N / 2 && term.ys != signs.ys) ? T(-1) : T(1), fh = term.xs != signs.xs ? -fl : fl;
 #pragma unroll
-        for (int r = 0; r < R; ++r) v[r] = cscale(ldc(ra + r * (M * S::YB / 2)), r < H ? fl : fh);
-        if (rd == 0) sync();   // tables (and the other CTA runs before its lines are written)
+    for (int r = 0; r < R; ++r) v[r] = cscale(ldc(ra + r * (M * S::YB / 2)), r < H ? fl : fh);
+    if (rd == 0) sync();   // tables (and the other CTA runs before its lines are written)
+    if constexpr (S::CL > 1) fft_to_pairs<N, T>(v, P, XScratch<N>{S::LL * N + t * N}, tws, m);
+    else fft_to_pairs<N, T>(v, P, XSlots<N>{n0}, tws, m);
+    for_pairs<N, true, false>(v, m, partner, [&](int, int l, bool self, C2<T> z, C2<T> g) {
+      const C2<T> q = ldc(qh + l);
+      C2<T> a = cmul(q, C2<T>{z.x + g.x, z.y - g.y}), b = cmul(q, C2<T>{z.y + g.y, g.x - z.x});
+      if (self) {   // the real modes 0 and N/2
+        a = {z.x, g.x};
+        b = {z.y, g.y};
+      }
+      C2<T>* at = pair_at(l, n0);   // the swizzle keeps pairs 2p, 2p + 1 together
+      if constexpr (sizeof(T) == 4) {
+        *reinterpret_cast<float4*>(at) = make_float4(a.x, a.y, b.x, b.y);
       } else {
-        // conj Z'_k = q conj(A + i B), conj Z'_(N-k) = conj(q) (A - i B)
-        C2<T> up[H];
-#pragma unroll
-        for (int j = 0; j < H; ++j) {
-          const C2<T>* at = pair_at(j, n0);
-          C2<T> a, b;
-          if constexpr (sizeof(T) == 4) {
-            const float4 f = *reinterpret_cast<const float4*>(at);
-            a = {f.x, f.y};
-            b = {f.z, f.w};
-          } else {
-            a = at[0];
-            b = at[1];
-          }
-          const C2<T> q = ldc(qh + m + M * j);
-          C2<T> lo = cmul(q, C2<T>{a.x - b.y, -(a.y + b.x)}), hi = cmul(conjg(q), C2<T>{a.x + b.y, a.y - b.x});
-          if (j == 0 && m == 0) {
-            lo = {T(0.5) * a.x, T(-0.5) * b.x};
-            hi = {T(0.5) * a.y, T(-0.5) * b.y};
-          }
-          v[j] = lo;
-          up[j] = {__shfl_sync(0xffffffffu, hi.x, partner), __shfl_sync(0xffffffffu, hi.y, partner)};
-        }
-        mirror_put<N, T>(v, up, m);
+        stc(at, a);
+        stc(at + 1, b);
       }
-      if constexpr (S::CL > 1) team_fft<N, T>(v, P, XScratch<N>{S::LL * N + t * N}, tws, m);
-      else team_fft<N, T>(v, P, XSlots<N>{n0}, tws, m);
-      if (!back) {
+    });
+  }
+  sync();
+  // ---- along y: transform, weight and inverse transform of line l in place
+#pragma unroll 1
+  for (int rd = 0; rd < S::ROUNDS; ++rd) {
+    const int tt = t + S::TEAMS * rd;
+    // the two teams of 8 lanes of a half warp take lines that differ in bit 1
+    const int ll = M == 8 ? ((tt & ~3) | ((tt & 1) << 1) | ((tt >> 1) & 1)) : tt, l = rank * S::LL + ll;
+    const YSlots<N> Y{ll * N, line_sw<M>(l)};
 #pragma unroll
-        for (int j = 0; j < H; ++j) {
-          const C2<T> g = mirror_fetch<N, T>(v, j, m, partner);
-          const C2<T> z = v[j], q = ldc(qh + m + M * j);
-          C2<T> a = cmul(q, C2<T>{z.x + g.x, z.y - g.y}), b = cmul(q, C2<T>{z.y + g.y, g.x - z.x});
-          if (j == 0 && m == 0) {   // the real modes 0 and N/2
-            a = {z.x, g.x};
-            b = {z.y, g.y};
-          }
-          C2<T>* at = pair_at(j, n0);   // the swizzle keeps pairs 2p, 2p + 1 together
-          if constexpr (sizeof(T) == 4) {
-            *reinterpret_cast<float4*>(at) = make_float4(a.x, a.y, b.x, b.y);
-          } else {
-            at[0] = a;
-            at[1] = b;
-          }
-        }
+    for (int r = 0; r < R; ++r) v[r] = ldc(P + (Y.base + ((m + M * r) ^ Y.sw)));
+    fft_to_pairs<N, T>(v, P, Y, tws, m);
+    // 4 sin^2 of the line's x modes l and N - l (line 0: 0 and N/2)
+    const T sl = sg[l];
+    const T axA = term.xs ? T(4) - sl : sl, axB = l ? (term.xs ? sl : T(4) - sl) : T(2);
+    LineW<T> W;
+    W.eA = axA + az;
+    W.eB = axB + az;
+    W.nA = term.nx ? axA : (term.ny ? T(0) : az);
+    W.nB = term.nx ? axB : (term.ny ? T(0) : az);
+    W.cy = term.ny ? T(1) : T(0);
+    W.f = T(0.5) * sc;   // twice a quarter: the inverse along x takes q / 2
+    for_pairs<N, true, true>(v, m, partner, [&](int, int k, bool self, C2<T>& z, C2<T>& p) {
+      const C2<T> c = ldc(cy + k);
+      const T sk = sg[k], sm = T(4) - sk;
+      T s, ds, tt2, dt;
+      W.pair(term.ys ? sm : sk, term.ys ? sk : sm, s, ds, tt2, dt);
+      // Z'_k = s Z + ds P* + c (t P + dt Z*), Z'_(N-k) = s P + ds Z* + c* (t Z + dt P*),
+      // conjugated for the inverse by a forward FFT
+      const C2<T> g = {tt2 * p.x + dt * z.x, tt2 * p.y - dt * z.y};
+      const C2<T> h = {tt2 * z.x + dt * p.x, tt2 * z.y - dt * p.y};
+      C2<T> lo = {s * z.x + ds * p.x + (c.x * g.x - c.y * g.y), ds * p.y - s * z.y - (c.x * g.y + c.y * g.x)};
+      C2<T> hi = {s * p.x + ds * z.x + (c.x * h.x + c.y * h.y), ds * z.y - s * p.y - (c.x * h.y - c.y * h.x)};
+      if (self) {   // indices 0 and N/2, each its own mirror
+        T wA, wB;
+        W.self(term.ys ? T(4) : T(0), wA, wB);
+        lo = {wA * z.x, -(wB * z.y)};
+        W.self(T(2), wA, wB);
+        hi = {wA * p.x, -(wB * p.y)};
+      }
+      z = lo;
+      p = hi;
+    });
+    fft_from_pairs<N, T>(v, P, Y, tws, twr, m);
+#pragma unroll
+    for (int j = 0; j < R; ++j) stc(P + (Y.base + ((m + M * j) ^ Y.sw)), conjg(v[j]));
+  }
+  sync();
+  // ---- along x back: columns 2p, 2p + 1 -> rows
+#pragma unroll 1
+  for (int rd = 0; rd < S::ROUNDS; ++rd) {
+    const int n0 = 2 * (rank * S::LL + t + S::TEAMS * rd);
+    // conj Z'_k = q conj(A + i B), conj Z'_(N-k) = conj(q) (A - i B)
+    for_pairs<N, false, true>(v, m, partner, [&](int, int l, bool self, C2<T>& lo, C2<T>& hi) {
+      const C2<T>* at = pair_at(l, n0);
+      C2<T> a, b;
+      if constexpr (sizeof(T) == 4) {
+        const float4 f = *reinterpret_cast<const float4*>(at);
+        a = {f.x, f.y};
+        b = {f.z, f.w};
       } else {
-        C2<T>* ra = reinterpret_cast<C2<T>*>(out + at0);
-#pragma unroll
-        for (int j = 0; j < R; ++j) stc(ra + j * (M * S::YB / 2), conjg(v[j]));
+        a = ldc(at);
+        b = ldc(at + 1);
       }
-    }
-    if (back) break;
-    sync();
-    // y: transform, weight and inverse transform of line l in place
-#pragma unroll 1
-    for (int rd = 0; rd < S::ROUNDS; ++rd) {
-      const int tt = t + S::TEAMS * rd;
-      // the two teams of 8 lanes of a half warp take lines that differ in bit 1
-      const int ll = M == 8 ? ((tt & ~3) | ((tt & 1) << 1) | ((tt >> 1) & 1)) : tt, l = rank * S::LL + ll;
-      const YSlots<N> Y{ll * N, line_sw<M>(l)};
-#pragma unroll
-      for (int r = 0; r < R; ++r) v[r] = ldc(P + (Y.base + ((m + M * r) ^ Y.sw)));
-#pragma unroll 1
-      for (int inv = 0; inv < 2; ++inv) {
-        team_fft<N, T>(v, P, Y, tws, m);
-        if (inv) break;
-        // 4 sin^2 of the line's x modes l and N - l (line 0: 0 and N/2)
-        const T sl = sg[l];
-        const T axA = term.xs ? T(4) - sl : sl, axB = l ? (term.xs ? sl : T(4) - sl) : T(2);
-        LineW<T> W;
-        W.eA = axA + az;
-        W.eB = axB + az;
-        W.nA = term.nx ? axA : (term.ny ? T(0) : az);
-        W.nB = term.nx ? axB : (term.ny ? T(0) : az);
-        W.cy = term.ny ? T(1) : T(0);
-        W.f = T(0.5) * sc;   // twice a quarter: the inverse along x takes q / 2
-        C2<T> up[H];
-#pragma unroll
-        for (int j = 0; j < H; ++j) {
-          const int k = m + M * j;
-          const C2<T> p = mirror_fetch<N, T>(v, j, m, partner);
-          const C2<T> z = v[j], c = ldc(cy + k);
-          const T sk = sg[k], sm = T(4) - sk;
-          T s, ds, tt2, dt;
-          W.pair(term.ys ? sm : sk, term.ys ? sk : sm, s, ds, tt2, dt);
-          // Z'_k = s Z + ds P* + c (t P + dt Z*), Z'_(N-k) = s P + ds Z* + c* (t Z + dt P*),
-          // conjugated for the inverse by a forward FFT
-          const C2<T> g = {tt2 * p.x + dt * z.x, tt2 * p.y - dt * z.y};
-          const C2<T> h = {tt2 * z.x + dt * p.x, tt2 * z.y - dt * p.y};
-          C2<T> lo = {s * z.x + ds * p.x + (c.x * g.x - c.y * g.y), ds * p.y - s * z.y - (c.x * g.y + c.y * g.x)};
-          C2<T> hi = {s * p.x + ds * z.x + (c.x * h.x + c.y * h.y), ds * z.y - s * p.y - (c.x * h.y - c.y * h.x)};
-          if (j == 0 && m == 0) {   // indices 0 and N/2, each its own mirror
-            T wA, wB;
-            W.self(term.ys ? T(4) : T(0), wA, wB);
-            lo = {wA * z.x, -(wB * z.y)};
-            W.self(T(2), wA, wB);
-            hi = {wA * p.x, -(wB * p.y)};
-          }
-          v[j] = lo;
-          up[j] = {__shfl_sync(0xffffffffu, hi.x, partner), __shfl_sync(0xffffffffu, hi.y, partner)};
-        }
-        mirror_put<N, T>(v, up, m);
+      const C2<T> q = ldc(qh + l);
+      lo = cmul(q, C2<T>{a.x - b.y, -(a.y + b.x)});
+      hi = cmul(conjg(q), C2<T>{a.x + b.y, a.y - b.x});
+      if (self) {
+        lo = {T(0.5) * a.x, T(-0.5) * b.x};
+        hi = {T(0.5) * a.y, T(-0.5) * b.y};
       }
+    });
+    if constexpr (S::CL > 1) fft_from_pairs<N, T>(v, P, XScratch<N>{S::LL * N + t * N}, tws, twr, m);
+    else fft_from_pairs<N, T>(v, P, XSlots<N>{n0}, tws, twr, m);
+    C2<T>* ra = reinterpret_cast<C2<T>*>(out + (int64_t)(n0 / S::YB) * (N * S::YB) + m * S::YB + n0 % S::YB);
 #pragma unroll
-      for (int j = 0; j < R; ++j) stc(P + (Y.base + ((m + M * j) ^ Y.sw)), conjg(v[j]));
-    }
-    sync();
+    for (int j = 0; j < R; ++j) stc(ra + j * (M * S::YB / 2), conjg(v[j]));
   }
   if constexpr (S::CL > 1) sync();   // the other CTA may still read this one's lines
 }

@@ -63,7 +63,7 @@ struct ZShape {
   static constexpr int BLOCKS = N * N / TILE;
   // two float tiles (N x TILE), over which the FFTs exchange, then the tables
   static constexpr size_t tile = sizeof(float) * N * TILE;
-  static constexpr size_t bytes = 2 * tile + sizeof(C2<float>) * (N + S::LINES);
+  static constexpr size_t bytes = 2 * tile + sizeof(C2<float>) * (2 * N + S::LINES);
   // resident CTAs per SM asked of the compiler (64 registers; 100 at N = 96, 24 values per lane)
   static constexpr int OCC = THREADS == 512 ? 2 : (THREADS == 256 ? 4 : (N == 96 ? 5 : 8));
 };
@@ -104,12 +104,15 @@ struct SlabArgs {
   double* partial[MAXB];
 };
 
-// Tables of a z kernel: FFT twiddles [s][m] and post-twiddles q_k, k < N/2.
+// Tables of a z kernel: FFT twiddles [s][m] and [m][s] and post-twiddles q_k, k < N/2.
 template <int N>
-__device__ __forceinline__ void z_tables(C2<float>* tws, C2<float>* qN, const C2<float>* __restrict__ twg,
-                                         const C2<float>* __restrict__ qg) {
+__device__ __forceinline__ void z_tables(C2<float>* tws, C2<float>* twr, C2<float>* qN,
+                                         const C2<float>* __restrict__ twg, const C2<float>* __restrict__ qg) {
   using S = plane::Shape<N>;
-  for (int e = threadIdx.x; e < N; e += ZShape<N>::THREADS) tws[e] = twg[2 * (e / S::M) * (e % S::M)];
+  for (int e = threadIdx.x; e < N; e += ZShape<N>::THREADS) {
+    tws[e] = twg[2 * (e / S::M) * (e % S::M)];
+    twr[e] = twg[2 * (e / S::R) * (e % S::R)];
+  }
   for (int e = threadIdx.x; e < S::LINES; e += ZShape<N>::THREADS) qN[e] = qg[e];
 }
 
@@ -145,7 +148,8 @@ k_cg_zfwd(const __grid_constant__ SlabArgs<MAXB> args, const C2<float>* __restri
   float* O3 = reinterpret_cast<float*>(smz);
   float* O1 = O3 + N * TILE;
   C2<float>* tws = P + N * TILE;
-  C2<float>* qN = tws + N;
+  C2<float>* twr = tws + N;
+  C2<float>* qN = twr + N;
   const int t = threadIdx.x / M, m = threadIdx.x % M, lane = threadIdx.x & 31;
   const int partner = (lane & ~(M - 1)) | ((M - m) & (M - 1));
   const int col0 = blockIdx.x * TILE;
@@ -184,35 +188,33 @@ k_cg_zfwd(const __grid_constant__ SlabArgs<MAXB> args, const C2<float>* __restri
       v[h + j] = {nv, h + j < H ? nv : -nv};
     }
   }
-  z_tables<N>(tws, qN, twg, qg);
+  z_tables<N>(tws, twr, qN, twg, qg);
   __syncthreads();
-  plane::team_fft<N, float>(v, P, z_slots<N>(t), tws, m);
+  plane::fft_to_pairs<N, float>(v, P, z_slots<N>(t), tws, m);
   float sx, sy;
   col_signs<N>(col0, sx, sy);
   const float s3 = sx * sy;
   // C + i S packed: q_k V_k = X_k - i X_(N-k) of both lines, k < N/2
   C2<float> oc[H], os[H];
-#pragma unroll
-  for (int j = 0; j < H; ++j) {
-    const C2<float> g = plane::mirror_fetch<N, float>(v, j, m, partner);
-    const C2<float> z = v[j], q0 = plane::ldc(qN + m + M * j);
+  plane::for_pairs<N, true, false>(v, m, partner, [&](int i, int k, bool self, C2<float> z, C2<float> g) {
+    const C2<float> q0 = plane::ldc(qN + k);
     const C2<float> qc = {0.5f * s3 * q0.x, 0.5f * s3 * q0.y}, qs = {0.5f * sy * q0.x, 0.5f * sy * q0.y};
-    oc[j] = cmul(qc, C2<float>{z.x + g.x, z.y - g.y});
-    os[j] = cmul(qs, C2<float>{z.y + g.y, g.x - z.x});
-    if (j == 0 && m == 0) {   // modes 0 and N/2 are real
+    oc[i] = cmul(qc, C2<float>{z.x + g.x, z.y - g.y});
+    os[i] = cmul(qs, C2<float>{z.y + g.y, g.x - z.x});
+    if (self) {   // modes 0 and N/2 are real
       constexpr float c4 = 0.70710678118654752440f;
-      oc[j] = {s3 * z.x, -(s3 * c4 * g.x)};
-      os[j] = {sy * z.y, -(sy * c4 * g.y)};
+      oc[i] = {s3 * z.x, -(s3 * c4 * g.x)};
+      os[i] = {sy * z.y, -(sy * c4 * g.y)};
     }
-  }
+  });
   __syncthreads();   // every team is through its exchange, which the tiles overlay
 #pragma unroll
-  for (int j = 0; j < H; ++j) {
-    const int k = m + M * j, kn = (j == 0 && m == 0) ? N / 2 : N - k;
-    O3[tile_at<N>(k, t)] = oc[j].x;
-    O3[tile_at<N>(kn, t)] = -oc[j].y;
-    O1[tile_at<N>(k, t)] = os[j].x;
-    O1[tile_at<N>(kn, t)] = -os[j].y;
+  for (int i = 0; i < H; ++i) {
+    const int k = plane::pair_index<N>(i, m), kn = k ? N - k : N / 2;
+    O3[tile_at<N>(k, t)] = oc[i].x;
+    O3[tile_at<N>(kn, t)] = -oc[i].y;
+    O1[tile_at<N>(k, t)] = os[i].x;
+    O1[tile_at<N>(kn, t)] = -os[i].y;
   }
   __syncthreads();
   float* __restrict__ z1 = args.z1[b];
@@ -298,7 +300,8 @@ k_cg_zinv(const __grid_constant__ SlabArgs<MAXB> args, const C2<float>* __restri
   float* O3 = reinterpret_cast<float*>(smi);
   float* O1 = O3 + N * TILE;
   C2<float>* tws = P + N * TILE;
-  C2<float>* qN = tws + N;
+  C2<float>* twr = tws + N;
+  C2<float>* qN = twr + N;
   const int t = threadIdx.x / M, m = threadIdx.x % M, lane = threadIdx.x & 31;
   const int partner = (lane & ~(M - 1)) | ((M - m) & (M - 1));
   const int col0 = blockIdx.x * TILE;
@@ -330,31 +333,27 @@ k_cg_zinv(const __grid_constant__ SlabArgs<MAXB> args, const C2<float>* __restri
       *reinterpret_cast<float4*>(O3 + at) = make_float4(s3 * f3[j].x, s3 * f3[j].y, s3 * f3[j].z, s3 * f3[j].w);
     }
   }
-  z_tables<N>(tws, qN, twg, qg);
+  z_tables<N>(tws, twr, qN, twg, qg);
   __syncthreads();
   // both inverse transforms of a column in one FFT: conj Z_k = q conj(A + i B),
   // conj Z_(N-k) = conj(q) (A - i B) with A = X_k - i X_(N-k) of the DCT-III input,
   // B of the DST-III input
-  C2<float> v[R], up[H];
-#pragma unroll
-  for (int j = 0; j < H; ++j) {
-    const int k = m + M * j, kn = (j == 0 && m == 0) ? N / 2 : N - k;
+  C2<float> v[R];
+  plane::for_pairs<N, false, true>(v, m, partner, [&](int, int k, bool self, C2<float>& lo, C2<float>& hi) {
+    const int kn = k ? N - k : N / 2;
     const float ax = O3[tile_at<N>(k, t)], ay = -O3[tile_at<N>(kn, t)];
     const float bx = O1[tile_at<N>(k, t)], by = -O1[tile_at<N>(kn, t)];
     const C2<float> q0 = plane::ldc(qN + k);
-    C2<float> lo = cmul(q0, C2<float>{ax - by, -(ay + bx)});
-    C2<float> hi = cmul(plane::conjg(q0), C2<float>{ax + by, ay - bx});
-    if (j == 0 && m == 0) {
+    lo = cmul(q0, C2<float>{ax - by, -(ay + bx)});
+    hi = cmul(plane::conjg(q0), C2<float>{ax + by, ay - bx});
+    if (self) {
       constexpr float c2 = 1.41421356237309504880f;
       lo = {ax, -bx};
       hi = {-(c2 * ay), c2 * by};
     }
-    v[j] = lo;
-    up[j] = {__shfl_sync(0xffffffffu, hi.x, partner), __shfl_sync(0xffffffffu, hi.y, partner)};
-  }
-  plane::mirror_put<N, float>(v, up, m);
+  });
   __syncthreads();   // the tiles are read; the exchange overlays them
-  plane::team_fft<N, float>(v, P, z_slots<N>(t), tws, m);
+  plane::fft_from_pairs<N, float>(v, P, z_slots<N>(t), tws, twr, m);
   // q = the two inverse transforms + c d + rank-one; d.q, r.r, r.q and q.q for
   // alpha and the expansion of the next r.r.  d.q and r.r (alpha, the stopping
   // test) exact to about 2^-48: every product split by FMA, all sums compensated;
