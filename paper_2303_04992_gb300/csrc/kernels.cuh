@@ -47,41 +47,53 @@ struct GridIx {
 };
 
 // ------------------------------------------------------------------ jumps
-// Jump values at every control point (Sec. 4.3).  One thread per fit row
-// (point y, component c'): the fitted value and surface derivatives
-// (d_1, d_2, d_11, d_12, d_22) of phi^(c') as a sequential sum over the row's
-// neighbours; then, per block of JB points, the 11 x 18 jump map from shared
-// memory (one output slot per task, input-major map rows).  All arithmetic is
-// FP64.  J is slot-major: J[s * n + y].
+// Jump values at every control point (Sec. 4.3).  Four threads per fit row
+// (point y, component c'), each every fourth of the row's neighbours: the fitted
+// value and surface derivatives (d_1, d_2, d_11, d_12, d_22) of phi^(c') as FP64
+// sums, added in a fixed order; then, per block of JB points, the 11 x 18 jump map
+// from shared memory (one output slot per task, input-major map rows).
+// J is slot-major: J[s * n + y].
 // The fit rows are interleaved by groups of 32 (a warp's rows): entry i of
 // row r at fit_off[r / 32] + 32 i + r % 32, weight k at fit_w[k ne + that],
 // rows padded to their group's longest with zero weights (column 0), so a
-// warp reads one entry of each of its rows with one coalesced load per array
-// and every row's sum is the one of its CSR order (the padding adds zeros).
-constexpr int JB = 32;                 // points per block (3 JB threads)
-__global__ void __launch_bounds__(3 * JB)
+// warp reads one entry of each of its rows with one coalesced load per array.
+// Bound by the FP64 pipe on large surfaces (46 M operations at 69304 points: 73 of
+// the 105 us it takes) and on small ones by the latency of a row's loads, a column
+// index and then the density value there: one thread per row (24 neighbours) took
+// 26 us at 4264 points and 61 at 17328, four take 15 and 43.
+constexpr int JB = 32;                 // points per block
+constexpr int JL = 4;                  // threads per fit row
+constexpr int J_THREADS = 3 * JB * JL;
+__global__ void __launch_bounds__(J_THREADS)
 k_jumps(const double* __restrict__ phi, const double* __restrict__ fpts, int64_t n,
         const int32_t* __restrict__ comp, const int32_t* __restrict__ pid,
         const int64_t* __restrict__ fit_off, const int32_t* __restrict__ fit_col,
         const double* __restrict__ fit_w, int64_t ne, const double* __restrict__ jmap,
         double* __restrict__ J) {
-  __shared__ double D[JB * 3][6];
+  __shared__ double part[JL][6][3 * JB];
+  __shared__ double D[3 * JB][6];
   const int64_t y0 = (int64_t)blockIdx.x * JB;
   {
-    const int t = threadIdx.x;                  // row 3 * (y - y0) + c'
-    const int64_t y = y0 + t / 3;
+    // warp w: rows 32 (w / JL) .. + 31 of the block, neighbours i = w mod JL, + JL, ...
+    const int w = threadIdx.x >> 5, l = w % JL, t = 32 * (w / JL) + (threadIdx.x & 31);   // row 3 (y - y0) + c'
     double acc[6] = {0, 0, 0, 0, 0, 0};
-    if (y < n) {
+    if (y0 + t / 3 < n) {
       const int64_t rr = 3 * y0 + t;
       const int64_t b = fit_off[rr >> 5], e = fit_off[(rr >> 5) + 1];
-      for (int64_t q = b + (rr & 31); q < e; q += 32) {
+#pragma unroll 2
+      for (int64_t q = b + (rr & 31) + 32 * l; q < e; q += 32 * JL) {
         const double v = phi[fit_col[q]];
 #pragma unroll
         for (int k = 0; k < 6; ++k) acc[k] += fit_w[k * ne + q] * v;
       }
     }
 #pragma unroll
-    for (int k = 0; k < 6; ++k) D[t][k] = acc[k];
+    for (int k = 0; k < 6; ++k) part[l][k][t] = acc[k];
+  }
+  __syncthreads();
+  for (int e = threadIdx.x; e < 6 * 3 * JB; e += J_THREADS) {
+    const int k = e / (3 * JB), t = e % (3 * JB);
+    D[t][k] = (part[0][k][t] + part[1][k][t]) + (part[2][k][t] + part[3][k][t]);
   }
   __syncthreads();
   // slot 0: the density itself at a primary point, its fitted value at a secondary one
@@ -93,7 +105,7 @@ k_jumps(const double* __restrict__ phi, const double* __restrict__ fpts, int64_t
     }
   }
   // slots 1..11: the jump map (input-major jmap[(y * 18 + q) * 11 + r])
-  for (int task = threadIdx.x; task < JB * 11; task += 3 * JB) {
+  for (int task = threadIdx.x; task < JB * 11; task += J_THREADS) {
     const int yl = task / 11, r = task - yl * 11;
     const int64_t y = y0 + yl;
     if (y >= n) continue;
@@ -821,23 +833,47 @@ __global__ void k_jumps_T(const double* __restrict__ Jbar, int64_t n, const int3
   }
 }
 
-// phibar[col] = Jbar[0][point of col] + sum over the fit entries reading col
-// of sum_s fit_w[s][q] Dbar[row][s]  (the surface fit transposed; q are the
-// entries' positions in the interleaved fit layout of k_jumps).
-__global__ void k_fit_T(const int64_t* __restrict__ ptr, const int32_t* __restrict__ q,
-                        const int32_t* __restrict__ rr, const double* __restrict__ fit_w, int64_t fit_nnz,
-                        const double* __restrict__ Dbar, const double* __restrict__ Jbar,
-                        const int64_t* __restrict__ prim_of, int64_t n_prim, double* __restrict__ out) {
-  for (int64_t col = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; col < n_prim;
-       col += (int64_t)gridDim.x * blockDim.x) {
-    double s = Jbar[prim_of[col]];
-    for (int64_t e = ptr[col]; e < ptr[col + 1]; ++e) {
-      const int64_t qe = q[e];
-      const double* D = Dbar + (size_t)rr[e] * 6;
+// The surface fit transposed, in two passes.  First every fit entry's share of its
+// column, E[pos] = sum_s fit_w[s][pos] Dbar[row][s], in the interleaved layout of
+// k_jumps, so that the weights (the bulk of the bytes) are read once and coalesced;
+// a gather of weights and Dbar per column entry read 8 of every 32 bytes it moved
+// (326 us on the star at N = 128; the two passes take a third of it).
+constexpr int FT_THREADS = 128;
+__global__ void __launch_bounds__(FT_THREADS)
+k_fit_entries_T(const int64_t* __restrict__ fit_off, int64_t rows, const double* __restrict__ fit_w, int64_t ne,
+                const double* __restrict__ Dbar, double* __restrict__ E) {
+  // a CTA takes one group of 32 rows, its warps every fourth entry of each
+  const int64_t g = blockIdx.x;
+  const int64_t row = 32 * g + (threadIdx.x & 31);
+  double D[6];
 #pragma unroll
-      for (int k = 0; k < 6; ++k) s += fit_w[k * fit_nnz + qe] * D[k];
-    }
-    out[col] = s;
+  for (int k = 0; k < 6; ++k) D[k] = row < rows ? Dbar[6 * row + k] : 0.0;
+  const int64_t end = fit_off[g + 1];
+#pragma unroll 2
+  for (int64_t q = fit_off[g] + threadIdx.x; q < end; q += FT_THREADS) {
+    double s = 0.0;
+#pragma unroll
+    for (int k = 0; k < 6; ++k) s += fit_w[k * ne + q] * D[k];
+    E[q] = s;
+  }
+}
+// Then phibar[col] = Jbar[0][point of col] + sum of E over the entries of col
+// (positions q, in a fixed order: eight lanes per column, every eighth entry each).
+constexpr int FT_LANES = 8;
+__global__ void k_fit_T(const int64_t* __restrict__ ptr, const int32_t* __restrict__ q, const double* __restrict__ E,
+                        const double* __restrict__ Jbar, const int64_t* __restrict__ prim_of, int64_t n_prim,
+                        double* __restrict__ out) {
+  const int l = threadIdx.x % FT_LANES;
+  const int64_t per = (int64_t)gridDim.x * (blockDim.x / FT_LANES);
+  // whole groups of lanes stay in the loop together
+  for (int64_t col = (int64_t)blockIdx.x * (blockDim.x / FT_LANES) + threadIdx.x / FT_LANES;
+       col < (n_prim + 31) / 32 * 32; col += per) {
+    double s = 0.0;
+    if (col < n_prim)
+      for (int64_t e = ptr[col] + l; e < ptr[col + 1]; e += FT_LANES) s += E[q[e]];
+#pragma unroll
+    for (int o = FT_LANES / 2; o > 0; o >>= 1) s += __shfl_xor_sync(0xffffffffu, s, o);
+    if (l == 0 && col < n_prim) out[col] = Jbar[prim_of[col]] + s;
   }
 }
 

@@ -169,7 +169,8 @@ struct kfbim_ctx {
   int64_t ta_n = 0, ca_n = 0;
   int64_t *d_ta_key = nullptr, *d_ta_ptr = nullptr, *d_ca_key = nullptr, *d_ca_ptr = nullptr,
           *d_ca_row = nullptr, *d_fa_ptr = nullptr;
-  int32_t *d_ta_q = nullptr, *d_fa_q = nullptr, *d_fa_rr = nullptr;
+  int32_t *d_ta_q = nullptr, *d_fa_q = nullptr;
+  double* d_fitE = nullptr;   // per fit entry: its share of its column in the transposed fit
   double *d_ta_w = nullptr, *d_ca_coef = nullptr, *d_Jbar = nullptr, *d_Dbar = nullptr;
   // counters of the current call
   int cg_iters = 0, refine_sweeps = 0, interface_solves = 0;
@@ -894,7 +895,7 @@ int interface_solve(kfbim_ctx* c, const double* phi, const double* fpts, const d
                     cudaStream_t s, bool need_p = true) {
   const int64_t n = c->n_all;
   const int at = prof_begin(c, s);
-  k_jumps<<<(unsigned)((n + JB - 1) / JB), 3 * JB, 0, s>>>(
+  k_jumps<<<(unsigned)((n + JB - 1) / JB), J_THREADS, 0, s>>>(
       phi, fpts, n, c->d_comp, c->d_pid, c->d_fit_off, c->d_fit_col, c->d_fit_w, c->fit_ell, c->d_jmap,
       c->J); ++g_launches;
   // fit rows (column index, six weights, the density value), the 11 x 18 jump
@@ -1109,21 +1110,17 @@ void adjoint_tables(kfbim_ctx* c) {
     c->d_ca_coef = upload(c, coef);
   }
   {  // fit entries by primary column
-    std::vector<std::vector<std::pair<int64_t, int64_t>>> bycol(std::max<int64_t>(1, t.n_prim));
-    for (int64_t rr = 0; rr + 1 < (int64_t)t.fit_ptr.size(); ++rr)
-      for (int64_t q = t.fit_ptr[rr]; q < t.fit_ptr[rr + 1]; ++q) bycol[t.fit_col[q]].emplace_back(q, rr);
+    std::vector<std::vector<int64_t>> bycol(std::max<int64_t>(1, t.n_prim));
+    for (int64_t q = 0; q < (int64_t)t.fit_col.size(); ++q) bycol[t.fit_col[q]].push_back(q);
     std::vector<int64_t> ptr{0};
-    std::vector<int32_t> qv, rv;
+    std::vector<int32_t> qv;
     for (int64_t col = 0; col < t.n_prim; ++col) {
-      for (const auto& pr : bycol[col]) {
-        qv.push_back(c->fit_pos[pr.first]);
-        rv.push_back((int32_t)pr.second);
-      }
+      for (const int64_t q : bycol[col]) qv.push_back(c->fit_pos[q]);
       ptr.push_back((int64_t)qv.size());
     }
     c->d_fa_ptr = upload(c, ptr);
     c->d_fa_q = upload(c, qv);
-    c->d_fa_rr = upload(c, rv);
+    c->d_fitE = dalloc<double>(c, (size_t)std::max<int64_t>(1, c->fit_ell));
   }
   c->d_Jbar = dalloc<double>(c, kSlots * c->n_all);
   c->d_Dbar = dalloc<double>(c, 18 * c->n_all);
@@ -1145,8 +1142,13 @@ int adjoint_tail(kfbim_ctx* c, double* out, cudaStream_t s) {
                                                        rbar, c->d_Jbar); ++g_launches;
   }
   k_jumps_T<<<grid_for(n), 256, 0, s>>>(c->d_Jbar, n, c->d_comp, c->d_pid, c->d_jmap, c->d_Dbar); ++g_launches;
-  k_fit_T<<<grid_for(c->n_prim), 256, 0, s>>>(c->d_fa_ptr, c->d_fa_q, c->d_fa_rr, c->d_fit_w, c->fit_ell, c->d_Dbar,
-                                               c->d_Jbar, c->d_prim_of, c->n_prim, out); ++g_launches;
+  const int64_t rows = 3 * n, groups = (rows + 31) / 32;
+  if (groups > 0) {
+    k_fit_entries_T<<<(unsigned)groups, FT_THREADS, 0, s>>>(c->d_fit_off, rows, c->d_fit_w, c->fit_ell, c->d_Dbar,
+                                                             c->d_fitE); ++g_launches;
+  }
+  k_fit_T<<<grid_for(c->n_prim * FT_LANES), 256, 0, s>>>(c->d_fa_ptr, c->d_fa_q, c->d_fitE, c->d_Jbar, c->d_prim_of,
+                                                          c->n_prim, out); ++g_launches;
   check_launch();
   return st;
 }
@@ -2013,7 +2015,7 @@ void interface_batch(kfbim_ctx* c, const std::vector<int>& act, const std::vecto
   const int64_t n = c->n_all;
   for (size_t q = 0; q < act.size(); ++q) {
     const kfbim_ctx::Slot& w = c->bs[act[q]];
-    k_jumps<<<(unsigned)((n + JB - 1) / JB), 3 * JB, 0, s>>>(
+    k_jumps<<<(unsigned)((n + JB - 1) / JB), J_THREADS, 0, s>>>(
         phi[q], fpts[q], n, c->d_comp, c->d_pid, c->d_fit_off, c->d_fit_col, c->d_fit_w, c->fit_ell,
         c->d_jmap, w.J);
     k_rhs_fill<<<grid_for(4 * c->N3), 256, 0, s>>>(fgrid[q], c->d_side[1], c->d_side[2], c->d_side[3],
@@ -2410,7 +2412,7 @@ int kfbim_jumps(kfbim_ctx* c, const double* phi, const double* fpts, double* Jou
     if (!phi || !Jout) return fail(c, KFBIM_E_INVALID, "kfbim_jumps: bad pointers");
     cudaStream_t s = (cudaStream_t)stream;
     const int64_t n = c->n_all;
-    k_jumps<<<(unsigned)((n + JB - 1) / JB), 3 * JB, 0, s>>>(
+    k_jumps<<<(unsigned)((n + JB - 1) / JB), J_THREADS, 0, s>>>(
         phi, fpts, n, c->d_comp, c->d_pid, c->d_fit_off, c->d_fit_col, c->d_fit_w, c->fit_ell, c->d_jmap,
         Jout); ++g_launches;
     check_launch();
