@@ -13,8 +13,8 @@
 // backwards Z_k = (c s, s' s + d), Z_(N-k) = (-c s, s' s - d) with c + i s' =
 // exp(i pi k / N), s = X_k + X_(N-k), d = X_(N-k) - X_k, and the inverse FFT is
 // z_n = x_2n + i x_(2n+1).  A lane ends a forward transform holding modes k and
-// N - k of its lines for k = m + M j < N/2, which is what the inverse starts from,
-// so the weight of a fused pass costs no exchange.
+// N - k of its lines (plane::for_pairs), which is what the inverse starts from, so
+// the weight of a fused pass costs no exchange.
 //
 // Lines go from global memory straight into the FFT registers and back: along y
 // and z a pair of lines is one vector per element and a warp's teams fill 32- to
@@ -62,13 +62,21 @@ struct Jobs {
 template <int N, typename T>
 struct LShape {
   using S = plane::Shape<N>;
-  static constexpr int TEAMS = 128 / S::M;                 // line pairs per CTA
-  static constexpr int THREADS = 128;
+  // FP64: the 512 CTAs of 128 threads of one field at N = 128 are 3.4 per SM, which
+  // the FP64 pipe (two lanes per SM and cycle) works through as four; 64 threads
+  static constexpr int THREADS = sizeof(T) == 8 ? 64 : 128;
+  static constexpr int TEAMS = THREADS / S::M;             // line pairs per CTA
   static constexpr int BLOCKS = (N * N / 2 + TEAMS - 1) / TEAMS;
-  static constexpr size_t bytes = sizeof(C2<T>) * ((size_t)TEAMS * N + N);
+  // FP32 at N = 256: a team of 16 lanes reads 16 rows of a pair at once, 16 bytes in
+  // each of 16 cache lines, and the L1's tag stage bounds the pass (85 % busy, 79 us
+  // per field along y or z against 30 along x); its CTA stages 64-byte rows instead
+  static constexpr bool STAGED = sizeof(T) == 4 && S::M == 16;
+  static constexpr int COLS = 2 * TEAMS;                   // lines per CTA
+  static constexpr size_t tile = STAGED ? sizeof(T) * N * COLS : 0;
+  static constexpr size_t bytes = sizeof(C2<T>) * ((size_t)TEAMS * N + 2 * N) + tile;
   // CTAs per SM asked of the compiler: 96 registers in FP32, 128 for the fused passes (168 at
   // N = 96, 24 values per lane), 255 in FP64
-  static constexpr int occ(bool fused) { return sizeof(T) == 8 ? 2 : (N == 96 ? 3 : (fused ? 4 : 5)); }
+  static constexpr int occ(bool fused) { return sizeof(T) == 8 ? 4 : (N == 96 ? 3 : (fused ? 4 : 5)); }
 };
 
 template <typename T, typename Tin>
@@ -111,6 +119,13 @@ __device__ __forceinline__ void st2(Tout* p, T a, T b, bool vec, bool acc = fals
   }
 }
 
+// a, negated where `neg` (by its sign bits: no FP64 instruction).
+template <typename T>
+__device__ __forceinline__ T flip(T a, bool neg) {
+  if constexpr (sizeof(T) == 4) return __uint_as_float(__float_as_uint(a) ^ (neg ? 0x80000000u : 0u));
+  else return __hiloint2double(__double2hiint(a) ^ (neg ? (int)0x80000000 : 0), __double2loint(a));
+}
+
 // The exchange slots of a team: as plane.cuh's along y, each team its own line.
 template <int N>
 __device__ __forceinline__ plane::YSlots<N> slots(int t) {
@@ -143,8 +158,61 @@ struct Weights {
   }
 };
 
+// The staged tile of a CTA: element i of line c at i COLS + (c ^ sw(i)) (pairs stay
+// together; rows 2 i and 2 i + 2 of a team's accesses on distinct banks).
+template <int COLS>
+__device__ __forceinline__ int tile_at(int i, int c) {
+  return i * COLS + (c ^ (2 * ((i >> 1) & (COLS / 2 - 1))));
+}
+template <int N, int COLS, int THREADS, typename T, typename Tin>
+__device__ __forceinline__ void tile_load(T* tile, const Tin* in, int64_t es) {
+  constexpr int Q = COLS / 4;
+  const bool wide = reinterpret_cast<uintptr_t>(in) % 16 == 0;   // a caller's field may not be
+#pragma unroll 8
+  for (int e = threadIdx.x; e < N * Q; e += THREADS) {
+    const int i = e / Q, c = (e % Q) * 4;
+    const Tin* p = in + (int64_t)i * es + c;
+    T v[4];
+    if (wide && sizeof(Tin) == 4) {
+      const float4 f = *reinterpret_cast<const float4*>(p);
+      v[0] = f.x; v[1] = f.y; v[2] = f.z; v[3] = f.w;
+    } else if (wide) {
+      const double2 f = reinterpret_cast<const double2*>(p)[0], g = reinterpret_cast<const double2*>(p)[1];
+      v[0] = to_work<T>(f.x); v[1] = to_work<T>(f.y); v[2] = to_work<T>(g.x); v[3] = to_work<T>(g.y);
+    } else {
+#pragma unroll
+      for (int k = 0; k < 4; ++k) v[k] = to_work<T>(p[k]);
+    }
+    *reinterpret_cast<float2*>(tile + tile_at<COLS>(i, c)) = make_float2(v[0], v[1]);
+    *reinterpret_cast<float2*>(tile + tile_at<COLS>(i, c + 2)) = make_float2(v[2], v[3]);
+  }
+}
+template <int N, int COLS, int THREADS, typename T, typename Tout>
+__device__ __forceinline__ void tile_store(const T* tile, Tout* out, int64_t es, bool acc) {
+  constexpr int Q = COLS / 4;
+  const bool wide = reinterpret_cast<uintptr_t>(out) % 16 == 0;
+#pragma unroll 4
+  for (int e = threadIdx.x; e < N * Q; e += THREADS) {
+    const int i = e / Q, c = (e % Q) * 4;
+    Tout* p = out + (int64_t)i * es + c;
+    const float2 a = *reinterpret_cast<const float2*>(tile + tile_at<COLS>(i, c));
+    const float2 b = *reinterpret_cast<const float2*>(tile + tile_at<COLS>(i, c + 2));
+    if constexpr (sizeof(Tout) == 8) {
+      st2<T>(p, a.x, a.y, true, acc);
+      st2<T>(p + 2, b.x, b.y, true, acc);
+    } else if (wide) {
+      *reinterpret_cast<float4*>(p) = make_float4(a.x, a.y, b.x, b.y);
+    } else {
+      p[0] = a.x;
+      p[1] = a.y;
+      p[2] = b.x;
+      p[3] = b.y;
+    }
+  }
+}
+
 template <typename Tin, typename T, typename Tout, int N, int OP, int MAXJ>
-__global__ void __launch_bounds__(128, (LShape<N, T>::occ(OP >= OP_F2I2)))
+__global__ void __launch_bounds__((LShape<N, T>::THREADS), (LShape<N, T>::occ(OP >= OP_F2I2)))
 k_lines(const __grid_constant__ Jobs<Tin, Tout, MAXJ> jobs, T h, T inv_mu, const C2<T>* __restrict__ twg,
         const C2<T>* __restrict__ qg, const T* __restrict__ s2) {
   using S = plane::Shape<N>;
@@ -155,7 +223,12 @@ k_lines(const __grid_constant__ Jobs<Tin, Tout, MAXJ> jobs, T h, T inv_mu, const
   extern __shared__ __align__(16) unsigned char sml[];
   C2<T>* P = reinterpret_cast<C2<T>*>(sml);
   C2<T>* tws = P + L::TEAMS * N;
-  for (int e = threadIdx.x; e < N; e += L::THREADS) tws[e] = twg[2 * (e / M) * (e % M)];
+  C2<T>* twr = tws + N;
+  constexpr bool pairs = plane::PairShape<N>::in_lane;
+  for (int e = threadIdx.x; e < N; e += L::THREADS) {
+    if (op_fwd1(OP) || op_fwd2(OP) || !pairs) tws[e] = twg[2 * (e / M) * (e % M)];
+    if ((op_inv1(OP) || op_inv2(OP)) && pairs) twr[e] = twg[2 * (e / R) * (e % R)];
+  }
   __syncthreads();
   const int t = threadIdx.x / M, m = threadIdx.x % M, lane = threadIdx.x & 31;
   const int partner = (lane & ~(M - 1)) | ((M - m) & (M - 1));
@@ -168,17 +241,27 @@ k_lines(const __grid_constant__ Jobs<Tin, Tout, MAXJ> jobs, T h, T inv_mu, const
   const int64_t ls = axis == 0 ? N : 1, es = axis == 0 ? 1 : (axis == 1 ? N : (int64_t)N * N);
   const Tin* in = job.in + base;
   Tout* out = job.out + base;
+  // along y and z at N = 256 the CTA's lines go through shared memory
+  constexpr bool STAGED = L::STAGED;
+  T* tile = reinterpret_cast<T*>(twr + N);
+  auto tp = [&](int i) { return tile + tile_at<L::COLS>(i, 2 * t); };   // element i of the pair
+  if constexpr (STAGED) {
+    if (axis != 0) {
+      tile_load<N, L::COLS, L::THREADS>(tile, in - 2 * t, es);
+      __syncthreads();
+    }
+  }
   const auto X = slots<N>(t);
   constexpr T half = T(0.5), r2 = T(1.41421356237309504880), ir2 = T(0.70710678118654752440);
-  // modes (k, N - k) of the two lines, k = m + M j; slot (0, N/2) for k = 0
+  // modes (k, N - k) of the two lines, k = k1(i); slot (0, N/2) for k = 0
   C2<T> A[H], B[H];
-  auto k2 = [&](int j) { return (j == 0 && m == 0) ? N / 2 : N - (m + M * j); };
+  auto k1 = [&](int i) { return plane::pair_index<N>(i, m); };
+  auto k2 = [&](int i) { return (i == 0 && m == 0) ? N / 2 : N - k1(i); };
   auto mode = [&](int k) { return dst ? N - 1 - k : k; };   // array index of DCT index k (F2, I2)
 
   // ------------------------------------------------------------- forward
   if constexpr (op_fwd2(OP)) {
     C2<T> v[R];
-    const T sg = dst ? T(-1) : T(1);
     if (axis == 0) {
 #pragma unroll
       for (int r = 0; r < H; ++r) {
@@ -186,32 +269,33 @@ k_lines(const __grid_constant__ Jobs<Tin, Tout, MAXJ> jobs, T h, T inv_mu, const
         const C2<T> a = ld2<T>(in + 2 * n, vec), b = ld2<T>(in + N + 2 * n, vec);
         v[r] = {a.x, b.x};
         // element 2n + 1 is position N - 1 - n: lane M - 1 - m, register R - 1 - r
-        v[R - 1 - r] = {sg * __shfl_xor_sync(0xffffffffu, a.y, M - 1), sg * __shfl_xor_sync(0xffffffffu, b.y, M - 1)};
+        v[R - 1 - r] = {flip(__shfl_xor_sync(0xffffffffu, a.y, M - 1), dst), flip(__shfl_xor_sync(0xffffffffu, b.y, M - 1), dst)};
       }
     } else {
 #pragma unroll
       for (int r = 0; r < R; ++r) {
         const int n = m + M * r;
         const int i = r < H ? 2 * n : 2 * (N - 1 - n) + 1;
-        v[r] = ld2<T>(in + (int64_t)i * es, vec);
-        if (r >= H) v[r] = plane::cscale(v[r], sg);
+        if constexpr (STAGED) v[r] = plane::ldc(reinterpret_cast<const C2<T>*>(tp(i)));
+        else v[r] = ld2<T>(in + (int64_t)i * es, vec);
+        if (r >= H) v[r] = {flip(v[r].x, dst), flip(v[r].y, dst)};
       }
     }
-    plane::team_fft<N, T>(v, P, X, tws, m);
-#pragma unroll
-    for (int j = 0; j < H; ++j) {
-      const C2<T> g = plane::mirror_fetch<N, T>(v, j, m, partner);
-      const C2<T> z = v[j], q0 = qg[m + M * j];
+    plane::fft_to_pairs<N, T>(v, P, X, tws, m);
+    plane::for_pairs<N, true, false>(v, m, partner, [&](int i, int k, bool self, C2<T> z, C2<T> g) {
+      const C2<T> q0 = qg[k];
       const C2<T> q = {half * q0.x, half * q0.y};
       C2<T> a = cmul(q, C2<T>{z.x + g.x, z.y - g.y}), b = cmul(q, C2<T>{z.y + g.y, g.x - z.x});
-      if (j == 0 && m == 0) {
+      if (self) {
         a = {z.x, -(ir2 * g.x)};
         b = {z.y, -(ir2 * g.y)};
       }
-      A[j] = {a.x, -a.y};   // X_k, X_(N-k)
-      B[j] = {b.x, -b.y};
-    }
+      A[i] = {a.x, -a.y};   // X_k, X_(N-k)
+      B[i] = {b.x, -b.y};
+    });
   } else if constexpr (op_fwd1(OP)) {
+#pragma unroll
+    for (int i = 0; i < H; ++i) B[i] = {T(0), T(0)};
 #pragma unroll 1
     for (int ab = 0; ab < 2; ++ab) {
       const Tin* x = in + ab * ls;
@@ -222,6 +306,7 @@ k_lines(const __grid_constant__ Jobs<Tin, Tout, MAXJ> jobs, T h, T inv_mu, const
         const int n = m + M * r;
         C2<T> a;
         if (axis == 0) a = ld2<T>(x + 2 * n, vec);
+        else if (STAGED) a = {tp(2 * n)[ab], tp(2 * n + 1)[ab]};
         else a = {to_work<T>(x[(int64_t)(2 * n) * es]), to_work<T>(x[(int64_t)(2 * n + 1) * es])};
         if (r == 0 && m == 0) a.x = T(0);
         v[r] = a;
@@ -235,23 +320,21 @@ k_lines(const __grid_constant__ Jobs<Tin, Tout, MAXJ> jobs, T h, T inv_mu, const
         const T im = __shfl_xor_sync(0xffffffffu, v[r].y, M - 1);
         v[R - 1 - r] = {-re, -im};
       }
-      plane::team_fft<N, T>(v, P, X, tws, m);
-#pragma unroll
-      for (int j = 0; j < H; ++j) {
-        const C2<T> g = plane::mirror_fetch<N, T>(v, j, m, partner);
-        const C2<T> z = v[j], w = twg[m + M * j];
+      plane::fft_to_pairs<N, T>(v, P, X, tws, m);
+      plane::for_pairs<N, true, false>(v, m, partner, [&](int i, int k, bool self, C2<T> z, C2<T> g) {
+        const C2<T> w = twg[k];
         // twice a and b: a = (.., z.y - g.y), b = (z.x - g.x, z.y + g.y)
         const T ia = T(0.25) * (z.y - g.y), wb = T(0.25) * (w.x * (z.x - g.x) - w.y * (z.y + g.y));
         C2<T> f = {wb - ia, wb + ia};
-        if (j == 0 && m == 0) f = {T(0), half * g.y};   // modes 0 and N/2
-        if (ab) B[j] = f;
-        else A[j] = f;
-      }
+        if (self) f = {T(0), half * g.y};   // modes 0 and N/2
+        A[i] = B[i];   // the first line's modes move on when the second's arrive
+        B[i] = f;
+      });
     }
   } else {   // inverse only: the modes come from memory
 #pragma unroll
     for (int j = 0; j < H; ++j) {
-      int ka = m + M * j, kb = k2(j);
+      int ka = k1(j), kb = k2(j);
       if constexpr (OP == OP_I2) {
         ka = mode(ka);
         kb = mode(kb);
@@ -261,7 +344,14 @@ k_lines(const __grid_constant__ Jobs<Tin, Tout, MAXJ> jobs, T h, T inv_mu, const
         a = {to_work<T>(in[ka]), to_work<T>(in[kb])};
         b = {to_work<T>(in[N + ka]), to_work<T>(in[N + kb])};
       } else {
-        const C2<T> e = ld2<T>(in + (int64_t)ka * es, vec), f = ld2<T>(in + (int64_t)kb * es, vec);
+        C2<T> e, f;
+        if constexpr (STAGED) {
+          e = plane::ldc(reinterpret_cast<const C2<T>*>(tp(ka)));
+          f = plane::ldc(reinterpret_cast<const C2<T>*>(tp(kb)));
+        } else {
+          e = ld2<T>(in + (int64_t)ka * es, vec);
+          f = ld2<T>(in + (int64_t)kb * es, vec);
+        }
         a = {e.x, f.x};
         b = {e.y, f.y};
       }
@@ -315,7 +405,7 @@ k_lines(const __grid_constant__ Jobs<Tin, Tout, MAXJ> jobs, T h, T inv_mu, const
   if constexpr (fused) {
 #pragma unroll
     for (int j = 0; j < H; ++j) {
-      int ka = m + M * j, kb = k2(j);
+      int ka = k1(j), kb = k2(j);
       if constexpr (OP == OP_F2I2) {
         ka = mode(ka);
         kb = mode(kb);
@@ -331,21 +421,17 @@ k_lines(const __grid_constant__ Jobs<Tin, Tout, MAXJ> jobs, T h, T inv_mu, const
   if constexpr (op_inv2(OP)) {
     // both lines in one FFT: conj Z_k = q conj(a + i b), conj Z_(N-k) = conj(q) (a - i b)
     // with a = X_k - i X_(N-k) of line A, b of line B
-    C2<T> v[R], up[H];
-#pragma unroll
-    for (int j = 0; j < H; ++j) {
-      const C2<T> a = {A[j].x, -A[j].y}, b = {B[j].x, -B[j].y}, q = qg[m + M * j];
-      C2<T> lo = cmul(q, C2<T>{a.x - b.y, -(a.y + b.x)});
-      C2<T> hi = cmul(plane::conjg(q), C2<T>{a.x + b.y, a.y - b.x});
-      if (j == 0 && m == 0) {
+    C2<T> v[R];
+    plane::for_pairs<N, false, true>(v, m, partner, [&](int i, int k, bool self, C2<T>& lo, C2<T>& hi) {
+      const C2<T> a = {A[i].x, -A[i].y}, b = {B[i].x, -B[i].y}, q = qg[k];
+      lo = cmul(q, C2<T>{a.x - b.y, -(a.y + b.x)});
+      hi = cmul(plane::conjg(q), C2<T>{a.x + b.y, a.y - b.x});
+      if (self) {
         lo = {a.x, -b.x};
         hi = {r2 * A[0].y, -(r2 * B[0].y)};
       }
-      v[j] = lo;
-      up[j] = {__shfl_sync(0xffffffffu, hi.x, partner), __shfl_sync(0xffffffffu, hi.y, partner)};
-    }
-    plane::mirror_put<N, T>(v, up, m);
-    plane::team_fft<N, T>(v, P, X, tws, m);
+    });
+    plane::fft_from_pairs<N, T>(v, P, X, tws, twr, m);
     const T sc = T(1) / T(N), so = (OP == OP_I2 || OP == OP_F2I2) && dst ? -sc : sc;
     const bool weighted = OP == OP_I2 && job.wmode != W_NONE;
 #pragma unroll
@@ -374,28 +460,31 @@ k_lines(const __grid_constant__ Jobs<Tin, Tout, MAXJ> jobs, T h, T inv_mu, const
           e = {e.x * w1, e.y * u1};
           o = {o.x * w2, o.y * u2};
         }
-        st2<T>(out + (int64_t)(2 * n) * es, e.x, e.y, vec, acc);
-        st2<T>(out + (int64_t)io * es, o.x, o.y, vec, acc);
+        if constexpr (STAGED) {
+          plane::stc(reinterpret_cast<C2<T>*>(tp(2 * n)), e);
+          plane::stc(reinterpret_cast<C2<T>*>(tp(io)), o);
+        } else {
+          st2<T>(out + (int64_t)(2 * n) * es, e.x, e.y, vec, acc);
+          st2<T>(out + (int64_t)io * es, o.x, o.y, vec, acc);
+        }
       }
     }
   } else if constexpr (op_inv1(OP)) {
 #pragma unroll 1
     for (int ab = 0; ab < 2; ++ab) {
-      C2<T> v[R], up[H];
-#pragma unroll
-      for (int j = 0; j < H; ++j) {
-        const C2<T> f = ab ? B[j] : A[j], w = twg[m + M * j];   // exp(-i pi k / N)
+      C2<T> v[R];
+      plane::for_pairs<N, false, true>(v, m, partner, [&](int i, int k, bool self, C2<T>& lo, C2<T>& hi) {
+        const C2<T> f = A[i], w = twg[k];   // exp(-i pi k / N)
+        A[i] = B[i];
         const T s = f.x + f.y, d = f.y - f.x, cs = w.x * s, ss = -(w.y * s);
-        C2<T> lo = {cs, -(ss + d)}, hi = {-cs, d - ss};   // conjugated
-        if (j == 0 && m == 0) {
+        lo = {cs, -(ss + d)};   // conjugated
+        hi = {-cs, d - ss};
+        if (self) {
           lo = {T(0), T(0)};
           hi = {T(0), T(-2) * f.y};
         }
-        v[j] = lo;
-        up[j] = {__shfl_sync(0xffffffffu, hi.x, partner), __shfl_sync(0xffffffffu, hi.y, partner)};
-      }
-      plane::mirror_put<N, T>(v, up, m);
-      plane::team_fft<N, T>(v, P, X, tws, m);
+      });
+      plane::fft_from_pairs<N, T>(v, P, X, tws, twr, m);
       Tout* x = out + ab * ls;
       const T sc = T(1) / T(N);
       const bool weighted = OP == OP_I1 && job.wmode != W_NONE;
@@ -412,6 +501,9 @@ k_lines(const __grid_constant__ Jobs<Tin, Tout, MAXJ> jobs, T h, T inv_mu, const
         }
         if (axis == 0) {
           st2<T>(x + 2 * n, e, o, vec);
+        } else if (STAGED) {
+          tp(2 * n)[ab] = e;
+          tp(2 * n + 1)[ab] = o;
         } else {
           x[(int64_t)(2 * n) * es] = e;
           x[(int64_t)(2 * n + 1) * es] = o;
@@ -421,7 +513,7 @@ k_lines(const __grid_constant__ Jobs<Tin, Tout, MAXJ> jobs, T h, T inv_mu, const
   } else {   // forward only: the modes go to memory
 #pragma unroll
     for (int j = 0; j < H; ++j) {
-      int ka = m + M * j, kb = k2(j);
+      int ka = k1(j), kb = k2(j);
       if constexpr (OP == OP_F2) {
         ka = mode(ka);
         kb = mode(kb);
@@ -439,9 +531,20 @@ k_lines(const __grid_constant__ Jobs<Tin, Tout, MAXJ> jobs, T h, T inv_mu, const
         out[N + ka] = b.x;
         out[N + kb] = b.y;
       } else {
-        st2<T>(out + (int64_t)ka * es, a.x, b.x, vec);
-        st2<T>(out + (int64_t)kb * es, a.y, b.y, vec);
+        if constexpr (STAGED) {
+          plane::stc(reinterpret_cast<C2<T>*>(tp(ka)), C2<T>{a.x, b.x});
+          plane::stc(reinterpret_cast<C2<T>*>(tp(kb)), C2<T>{a.y, b.y});
+        } else {
+          st2<T>(out + (int64_t)ka * es, a.x, b.x, vec);
+          st2<T>(out + (int64_t)kb * es, a.y, b.y, vec);
+        }
       }
+    }
+  }
+  if constexpr (STAGED) {
+    if (axis != 0) {
+      __syncthreads();
+      tile_store<N, L::COLS, L::THREADS>(tile, out - 2 * t, es, acc);
     }
   }
 }

@@ -77,3 +77,20 @@ def test_transform_matches_dense(solver, kind, axis):
         solver.transform_f32(kind, axis, xin, out, backend=1, wmode=wmode, wc=wc)
         got = out.double().reshape(N, N, N)
         assert float((got - want).abs().max()) < TOL * float(want.abs().max()), (wmode, off)
+
+
+@pytest.mark.parametrize("comp", [1, 2, 3])
+def test_poisson_matches_dense(solver, comp):
+    """The fused pass (DST-I, weight, inverse DST-I in one kernel) between plain FP64 passes: 1e-12, a few
+    thousand roundings of the largest value."""
+    N, c = solver.N, comp - 1
+    r = torch.randn(N, N, N, dtype=torch.float64, device="cuda",
+                    generator=torch.Generator(device="cuda").manual_seed(comp))
+    u = torch.zeros(N ** 3, dtype=torch.float64, device="cuda")
+    solver.poisson(comp, r.reshape(-1), u)
+    F = [torch.from_numpy(matrix(5 if a == c else 3, N)).cuda() for a in range(3)]
+    B = [torch.from_numpy(matrix(6 if a == c else 4, N)).cuda() for a in range(3)]
+    w = torch.from_numpy(np.ascontiguousarray(weight(N, 2, c, solver.h, 1.0).transpose(2, 1, 0))).cuda()
+    v = torch.einsum("ck,bj,ai,kji->cba", F[2], F[1], F[0], r) * w
+    want = torch.einsum("kc,jb,ia,cba->kji", B[2], B[1], B[0], v).reshape(-1)
+    assert float((u - want).abs().max()) < 1e-12 * float(want.abs().max())
