@@ -34,8 +34,9 @@ __device__ __forceinline__ double block_sum(double v, double* sh) {
 // transform passes of S d return immediately.
 struct CGScalars {
   double rr, bb, stop, dq, alpha, beta, sumd, rank1, cdiag;
-  int done, iters;
+  int done, iters;   // done: 1 converged, 2 (slab form) stopped at the cap of a device-side loop
   unsigned int ticket[3];
+  int idle;          // slab form: done before the current iteration began
 };
 
 // Device-side loop of a CG run captured as a conditional graph: the loop's

@@ -13,7 +13,15 @@
 namespace kfbim {
 
 constexpr int RED_THREADS = 256;
-constexpr int RED_BLOCKS = 1216;  // 8 x 152 SMs
+constexpr int RED_BLOCKS = 1216;  // at most: 8 x 152 SMs
+// Blocks of a reduction over n values: at least four values per thread, since the
+// block and grid sums cost more than the values (FP64 shuffles and adds, one atomic
+// per block): one value per thread took the FP64 CG's vector kernels 13 us each at
+// N = 64.
+inline int red_blocks(int64_t n) {
+  const int64_t b = (n + 4 * RED_THREADS - 1) / (4 * RED_THREADS);
+  return (int)(b < 1 ? 1 : (b > RED_BLOCKS ? RED_BLOCKS : b));
+}
 
 // Index arithmetic of the N^3 grid fields, flat index x = (k N + j) N + i:
 // shifts when N is a power of two (lg = log2 N), divisions otherwise (lg < 0,

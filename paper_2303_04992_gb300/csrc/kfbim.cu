@@ -288,12 +288,12 @@ struct Tw<float> {
   static const float* s2(kfbim_ctx* c) { return c->d_s2f; }
 };
 
-// Reduction partials per batch slot: RED_BLOCKS for the staged CG kernels,
-// four per block of the slab iteration's k_cg_zinv (4 x 512 at N = 128, 4 x 2048
-// at N = 256).
+// Reduction partials per batch slot: RED_BLOCKS for the staged CG kernels, the
+// slab iteration's reduction memory.
 size_t run_partials(const kfbim_ctx* c) {
-  return std::max((size_t)2 * RED_BLOCKS, (size_t)c->N * c->N / 8);
+  return std::max((size_t)2 * RED_BLOCKS, (slab_reduce_slots(c->N) + 1) / 2 * 2);
 }
+
 // One transform pass of a stage: input, output, axis, first transform,
 // second transform, spectral weight, weight component, accumulate flag, and
 // the done flag of the CG run the pass belongs to (nullable).
@@ -587,9 +587,10 @@ double read_scalar(kfbim_ctx* c, const double* dptr, cudaStream_t s) {
 
 template <typename Ta, typename Tb>
 void dot(kfbim_ctx* c, const Ta* x, const Tb* y, int64_t n, double* out, double scale, cudaStream_t s) {
-  k_dot_partial<Ta, Tb><<<RED_BLOCKS, RED_THREADS, 0, s>>>(x, y, n, c->partial); ++g_launches;
+  const int nb = red_blocks(n);
+  k_dot_partial<Ta, Tb><<<nb, RED_THREADS, 0, s>>>(x, y, n, c->partial); ++g_launches;
   check_launch();
-  k_sum_partials<<<1, RED_THREADS, 0, s>>>(c->partial, RED_BLOCKS, scale, out); ++g_launches;
+  k_sum_partials<<<1, RED_THREADS, 0, s>>>(c->partial, nb, scale, out); ++g_launches;
   check_launch();
 }
 
@@ -638,9 +639,9 @@ void cg_iteration(kfbim_ctx* c, const CgWs<T>& w, cudaStream_t s, const CgLoop& 
   }
   schur_apply3<T>(c, w.d, w.q, w.q2, w.q3, w.T6, s, &c->cgs->done);
   const int at = prof_begin(c, s);
-  k_cg_alpha<T><<<RED_BLOCKS, RED_THREADS, 0, s>>>(w.d, w.q, w.q2, w.q3, n, c->cgs, c->partial); ++g_launches;
-  k_cg_update<T><<<RED_BLOCKS, RED_THREADS, 0, s>>>(w.x, w.r, w.d, w.q, n, c->cgs, c->partial); ++g_launches;
-  k_cg_direction<T><<<RED_BLOCKS, RED_THREADS, 0, s>>>(w.d, w.r, n, c->cgs, c->partial, loop); ++g_launches;
+  k_cg_alpha<T><<<red_blocks(n), RED_THREADS, 0, s>>>(w.d, w.q, w.q2, w.q3, n, c->cgs, c->partial); ++g_launches;
+  k_cg_update<T><<<red_blocks(n), RED_THREADS, 0, s>>>(w.x, w.r, w.d, w.q, n, c->cgs, c->partial); ++g_launches;
+  k_cg_direction<T><<<red_blocks(n), RED_THREADS, 0, s>>>(w.d, w.r, n, c->cgs, c->partial, loop); ++g_launches;
   // values moved: alpha 5 N^3 (d, q, q2, q3 read, q written), update 6, direction 3
   prof_end(c, s, at, KFBIM_KCLASS_CG_VECTOR, 3, 14.0 * n * sizeof(T));
   check_launch();
@@ -670,6 +671,7 @@ cudaGraphExec_t cg_graph(kfbim_ctx* c, const CgWs<T>& w) {
   // capture stream with the done flag raised does nothing but configure them
   const int one = 1;
   CK(cudaMemcpyAsync(&c->cgs->done, &one, sizeof(int), cudaMemcpyHostToDevice, c->cap_stream));
+  CK(cudaMemcpyAsync(&c->cgs->idle, &one, sizeof(int), cudaMemcpyHostToDevice, c->cap_stream));
   const int64_t before = g_launches;
   cg_iteration<T>(c, w, c->cap_stream);
   CK(cudaStreamSynchronize(c->cap_stream));
@@ -710,12 +712,18 @@ cudaGraphExec_t cg_graph(kfbim_ctx* c, const CgWs<T>& w) {
   return c->cg_exec[slot];
 }
 
+// Trips of a device-side loop that ran `iters` CG iterations: the staged form stops
+// in its last iteration (one trip at least), the slab form in the one after it.
+int loop_trips(const kfbim_ctx* c, int iters, int slot) {
+  return slot == Slot<float>::v && c->slab ? iters + 1 : std::max(1, iters);
+}
+
 // A CG run's scalars as the host reads them: counters and status.
 int cg_result(kfbim_ctx* c, const CGScalars& h, int slot, bool loop) {
   c->cg_iters += h.iters;
-  if (loop) g_launches += (int64_t)std::max(1, h.iters) * c->cg_graph_kernels[slot];   // one trip at least
+  if (loop) g_launches += (int64_t)loop_trips(c, h.iters, slot) * c->cg_graph_kernels[slot];
   if (!std::isfinite(h.rr)) return KFBIM_E_NONFINITE;
-  return h.done ? KFBIM_OK : KFBIM_E_NOCONV;
+  return h.done == 1 ? KFBIM_OK : KFBIM_E_NOCONV;
 }
 
 // The grid scalars in one copy (waits for the stream).
@@ -753,7 +761,7 @@ int cg(kfbim_ctx* c, const T* b, const SlabRhs* rhs, const CgWs<T>& w, double to
     CK(cudaMemsetAsync(w.x, 0, n * sizeof(T), s));
     CK(cudaMemcpyAsync(w.r, b, n * sizeof(T), cudaMemcpyDeviceToDevice, s));
     CK(cudaMemcpyAsync(w.d, b, n * sizeof(T), cudaMemcpyDeviceToDevice, s));
-    k_cg_init<T><<<RED_BLOCKS, RED_THREADS, 0, s>>>(b, n, c->cgs, tol * tol, rank1, c->cpen, c->partial,
+    k_cg_init<T><<<red_blocks(n), RED_THREADS, 0, s>>>(b, n, c->cgs, tol * tol, rank1, c->cpen, c->partial,
                                                      &c->gs->active);
     ++g_launches;
   }
@@ -837,7 +845,7 @@ int grid_solve_mixed(kfbim_ctx* c, cudaStream_t s, bool need_p) {
   double* resf = c->t1;            // FP64 residual [rf (3 fields) | rg]
   double* resg = c->t1 + 3 * N3;
   double* gmean = &c->gs->gmean;
-  k_rhs_moments<<<RED_BLOCKS, RED_THREADS, 0, s>>>(c->rhs, N3, c->navier ? 0 : 1, c->partial, &c->gs->ticket, gmean,
+  k_rhs_moments<<<red_blocks(4 * N3), RED_THREADS, 0, s>>>(c->rhs, N3, c->navier ? 0 : 1, c->partial, &c->gs->ticket, gmean,
                                                     &c->gs->ref2); ++g_launches;
   check_launch();
   int status = KFBIM_OK;
@@ -1731,7 +1739,7 @@ std::vector<SlabCg> slab_batch_runs(kfbim_ctx* c, const std::vector<int>& slots)
 // slots skip them.
 __global__ void k_cg_mark_idle(CGScalars* s, int nslot, unsigned long long active) {
   const int b = threadIdx.x;
-  if (b < nslot && !((active >> b) & 1ull)) s[b].done = 1;
+  if (b < nslot && !((active >> b) & 1ull)) s[b].done = s[b].idle = 1;
 }
 
 // The batched slab CG of all bcap slots as a conditional while loop: one
@@ -1822,7 +1830,7 @@ void cg_batch(kfbim_ctx* c, const std::vector<int>& act, const std::vector<const
     CK(cudaMemsetAsync(w.x, 0, n * sizeof(float), s));
     CK(cudaMemcpyAsync(w.r, w.fu, n * sizeof(float), cudaMemcpyDeviceToDevice, s));
     CK(cudaMemcpyAsync(w.d, w.fu, n * sizeof(float), cudaMemcpyDeviceToDevice, s));
-    k_cg_init<float><<<RED_BLOCKS, RED_THREADS, 0, s>>>(w.fu, n, &c->bcgs[b], rhs[k].tol2, rank1, c->cpen,
+    k_cg_init<float><<<red_blocks(n), RED_THREADS, 0, s>>>(w.fu, n, &c->bcgs[b], rhs[k].tol2, rank1, c->cpen,
                                                          c->partial, nullptr);
     ++g_launches;
   }
@@ -1841,7 +1849,7 @@ void cg_batch(kfbim_ctx* c, const std::vector<int>& act, const std::vector<const
     std::memcpy(h.data(), c->bpinned, sizeof(CGScalars) * c->bcap);
     if (exec) {
       int trips = 1;
-      for (int b : act) trips = std::max(trips, h[b].iters);
+      for (int b : act) trips = std::max(trips, loop_trips(c, h[b].iters, Slot<float>::v));
       g_launches += (int64_t)trips * c->bcg_kernels;
     }
     std::vector<int> run;
@@ -1851,7 +1859,7 @@ void cg_batch(kfbim_ctx* c, const std::vector<int>& act, const std::vector<const
     }
     if (run.empty() || launched >= c->opt.cg_max) break;
     // the CG vector updates of every running instance in one launch per step,
-    // RED_BLOCKS blocks per instance (the single-run reduction order)
+    // the blocks of a single run per instance (its reduction order)
     CgBatchArgs<float> A{};
     for (size_t k = 0; k < run.size(); ++k) {
       const kfbim_ctx::Slot& w = c->bs[run[k]];
@@ -1864,7 +1872,7 @@ void cg_batch(kfbim_ctx* c, const std::vector<int>& act, const std::vector<const
       A.s[k] = &c->bcgs[run[k]];
       A.partial[k] = c->bpartial + run_partials(c) * run[k];
     }
-    const dim3 grid(RED_BLOCKS, (unsigned)run.size());
+    const dim3 grid(red_blocks(n), (unsigned)run.size());
     if (c->slab) {
       // the three slab kernels of all running instances, one launch each per
       // iteration (blockIdx.y = instance; the single-run arithmetic)
@@ -1918,7 +1926,7 @@ void grid_solve_batch(kfbim_ctx* c, const std::vector<int>& act, cudaStream_t s,
   auto ticket = [&](int b) { return reinterpret_cast<unsigned int*>(c->bscal + 8 * b + 6); };
   for (int b : act) {
     const kfbim_ctx::Slot& w = c->bs[b];
-    k_rhs_moments<<<RED_BLOCKS, RED_THREADS, 0, s>>>(w.rhs, N3, c->navier ? 0 : 1, c->partial, ticket(b),
+    k_rhs_moments<<<red_blocks(4 * N3), RED_THREADS, 0, s>>>(w.rhs, N3, c->navier ? 0 : 1, c->partial, ticket(b),
                                                       c->bscal + 8 * b, c->bscal + 8 * b + 1);
     ++g_launches;
   }

@@ -6,6 +6,17 @@
 
 namespace kfbim {
 
+size_t slab_reduce_slots(int N) {
+  switch (N) {
+    case 256: return slab::ZShape<256>::REDUCE;
+    case 128: return slab::ZShape<128>::REDUCE;
+    case 96: return slab::ZShape<96>::REDUCE;
+    case 64: return slab::ZShape<64>::REDUCE;
+    case 32: return slab::ZShape<32>::REDUCE;
+    default: return 0;
+  }
+}
+
 bool slab_supported(int N) { return N == 32 || N == 64 || N == 96 || N == 128 || N == 256; }
 
 namespace {
@@ -56,7 +67,7 @@ slab::SlabArgs<MAXB> make_args(const SlabCg* runs, int nrun) {
 }
 
 // Kernel `which` of the iteration: 0 k_cg_zfwd, 1 k_cg_terms, 2 k_cg_zinv; 3 is
-// k_cg_fin, the update still pending when a run stops.
+// k_cg_fin, the end of a run.
 template <int N, int MAXB>
 void launch_nb(int which, const slab::SlabArgs<MAXB>& args, const SlabCg& t, int nrun, const CgLoop& loop,
                cudaStream_t st) {
@@ -64,7 +75,7 @@ void launch_nb(int which, const slab::SlabArgs<MAXB>& args, const SlabCg& t, int
   using V = slab::Conv<N>;
   switch (which) {
     case 0:
-      slab::k_cg_zfwd<N, MAXB><<<dim3(Z::BLOCKS, nrun), Z::THREADS, Z::bytes, st>>>(args, t.tw, t.qN);
+      slab::k_cg_zfwd<N, MAXB><<<dim3(Z::BLOCKS, nrun), Z::THREADS, Z::bytes, st>>>(args, t.tw, t.qN, loop);
       break;
     case 1:
       if constexpr (plane::Shape<N>::CL > 1)
@@ -75,7 +86,7 @@ void launch_nb(int which, const slab::SlabArgs<MAXB>& args, const SlabCg& t, int
             args, t.tw, t.qN, t.s2, t.inv_mu);
       break;
     case 2:
-      slab::k_cg_zinv<N, MAXB><<<dim3(Z::BLOCKS, nrun), Z::THREADS, Z::bytes, st>>>(args, t.tw, t.qN, loop);
+      slab::k_cg_zinv<N, MAXB><<<dim3(Z::BLOCKS, nrun), Z::THREADS, Z::bytes, st>>>(args, t.tw, t.qN);
       break;
     default:
       slab::k_cg_fin<N, MAXB><<<dim3(V::BLOCKS, nrun), V::THREADS, V::bytes, st>>>(args);

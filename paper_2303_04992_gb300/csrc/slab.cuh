@@ -13,7 +13,9 @@
 // The vector update of iteration k waits for alpha_k, which is known only
 // once the reduction of d.q over the whole grid is done, so it is carried
 // into the first kernel of iteration k + 1, which touches every element
-// anyway; the next r.r (for beta and the stopping test) then comes from its
+// anyway (and whose CTAs each merge the blocks' sums of iteration k while their
+// vectors load: a last block that merged them took 4 us at the end of every
+// iteration); the next r.r (for beta and the stopping test) then comes from its
 // expansion
 //   |r - alpha q|^2 = r.r - 2 alpha r.q + alpha^2 q.q
 // with r.r, r.q and q.q summed beside d.q over the stored vectors.  r.r is
@@ -22,14 +24,16 @@
 // carried on from one iteration to the next those errors would add up to
 // about 1e-7 of the first r.r, far above a stopping level of 1e-11 of it.
 // One CG iteration:
-//   k_cg_zfwd   x += alpha d, r -= alpha q (pending update), d = r + beta d,
-//               Z1 = S_z d, Z3 = C_z d, sum(d)          (4 reads, 5 writes)
+//   k_cg_zfwd   alpha, the next r.r, beta; x += alpha d, r -= alpha q (pending
+//               update), d = r + beta d, Z1 = S_z d, Z3 = C_z d, sum(d)
+//                                                       (4 reads, 5 writes)
 //   k_cg_terms  W1, W2 from Z1, W3 from Z3             (3 reads, 3 writes)
-//   k_cg_zinv   q = S_z^-1 (W1 + W2) + C_z^-1 W3 + c d + rank-one; d.q, r.r,
-//               r.q, q.q; alpha, the next r.r, beta     (5 reads, 1 write)
+//   k_cg_zinv   q = S_z^-1 (W1 + W2) + C_z^-1 W3 + c d + rank-one; the blocks'
+//               sums of d.q, r.r, r.q, q.q              (5 reads, 1 write)
 // i.e. 21 N^3 values moved per iteration, against 28 for the transform
-// passes of Schur apply run one axis at a time plus 14 for the CG vectors;
-// k_cg_fin applies the last pending update once the run stops.
+// passes of Schur apply run one axis at a time plus 14 for the CG vectors.  The
+// k_cg_zfwd that finds the run converged applies the pending update of x and marks
+// it done; the kernels after it do nothing.
 //
 // Orders.  Along every axis position n is Makhoul's (v_n = x_2n, v_(N-1-n) =
 // x_(2n+1)), so a line's FFT input is contiguous and DST-II is DCT-II with the
@@ -64,6 +68,15 @@ struct ZShape {
   // two float tiles (N x TILE), over which the FFTs exchange, then the tables
   static constexpr size_t tile = sizeof(float) * N * TILE;
   static constexpr size_t bytes = 2 * tile + sizeof(C2<float>) * (2 * N + S::LINES);
+  // blocks whose sums of k_cg_zinv are merged into one part by the last of them,
+  // so that no CTA of k_cg_zfwd reads more than 16 KB of parts
+  static constexpr int GROUP = BLOCKS > 512 ? BLOCKS / 256 : 1;
+  static constexpr int PARTS = BLOCKS / GROUP;
+  // a run's reduction memory, in float2: the parts (of four sums), the blocks' sums of d,
+  // the blocks' sums of a group, the groups' tickets
+  static constexpr int SUMD = 4 * PARTS, BLOCK_SUMS = SUMD + BLOCKS;
+  static constexpr int TICKETS = BLOCK_SUMS + (GROUP > 1 ? 4 * BLOCKS : 0);
+  static constexpr int REDUCE = TICKETS + (GROUP > 1 ? PARTS : 0);
   // resident CTAs per SM asked of the compiler (64 registers; 100 at N = 96, 24 values per lane)
   static constexpr int OCC = THREADS == 512 ? 2 : (THREADS == 256 ? 4 : (N == 96 ? 5 : 8));
 };
@@ -126,23 +139,67 @@ __device__ __forceinline__ void col_signs(int col0, float& sx, float& sy) {
   sy = y >= N / 2 ? -1.f : 1.f;
 }
 
-// The pending update x += alpha d, r -= alpha q (nothing pending in the first
-// iteration, where x is not read either: it starts at zero); d = r + beta d;
-// Z1 = DST-II_z d (negated at odd y), Z3 = DCT-II_z d (negated at odd x and at
-// odd y); sumd = sum d.  One column per team of M lanes.
+// The scalars of an iteration from the parts of the k_cg_zinv before it (PARTS each
+// of d.q, r.r, r.q, q.q), merged in a fixed order: every CTA computes the same
+// values.  One warp per sum, and one thread for the FP64 arithmetic (by all threads
+// of a CTA it alone took 6 us per iteration at N = 128).
+struct CgStep {
+  double alpha, rr;     // rr: |r - alpha q|^2 by its expansion
+  float a, beta;        // alpha, beta in FP32
+};
+template <int N, int THREADS>
+__device__ __forceinline__ void cg_step(const float2* __restrict__ part, double* sums, CgStep* c) {
+  constexpr int WARPS = THREADS / 32, P = ZShape<N>::PARTS;
+  const int w = threadIdx.x >> 5, lane = threadIdx.x & 31;
+#pragma unroll
+  for (int j = w; j < 4; j += WARPS) {
+    CgAcc<float> g;
+#pragma unroll 8
+    for (int e = lane; e < P; e += 32) {
+      const float2 p = part[j * P + e];
+      g.merge(p.x, p.y);
+    }
+    warp_merge(g);
+    if (lane == 0) sums[j] = g.value();
+  }
+  __syncthreads();
+  if (threadIdx.x == 0) {
+    const double dq = sums[0], rr = sums[1];
+    const double alpha = (dq != 0.0) ? rr / dq : 0.0;
+    const double r1 = rr - 2.0 * alpha * sums[2] + alpha * alpha * sums[3];
+    c->alpha = alpha;
+    c->rr = r1;
+    c->a = float(alpha);
+    c->beta = (rr != 0.0) ? float(r1 / rr) : 0.f;
+  }
+  __syncthreads();
+}
+
+// alpha, beta and the stopping test of the iteration before; its update x += alpha
+// d, r -= alpha q (nothing pending in the first iteration; x starts at zero and is
+// read from the third on); d = r + beta d; Z1 = DST-II_z d (negated at odd y), Z3 =
+// DCT-II_z d (negated at odd x and at odd y); sum d.  A run that has converged or
+// reached its cap only gets the update of x.  One column per team of M lanes.
 // Bound by the loads' latency (the fields live in the L2 at N <= 128): no
 // barrier stands between the loads and the FFT, whose inputs they are.
 template <int N, int MAXB>
 __global__ void __launch_bounds__(ZShape<N>::THREADS, ZShape<N>::OCC)
 k_cg_zfwd(const __grid_constant__ SlabArgs<MAXB> args, const C2<float>* __restrict__ twg,
-          const C2<float>* __restrict__ qg) {
+          const C2<float>* __restrict__ qg, const CgLoop loop) {
   using S = plane::Shape<N>;
   using Z = ZShape<N>;
   constexpr int M = S::M, R = S::R, H = S::H, TILE = Z::TILE;
   __shared__ float2 sh[32];
+  __shared__ double sums[4];
+  __shared__ CgStep step;
   const int b = blockIdx.y;
   CGScalars* s = args.s[b];
-  if (s->done) return;
+  // idle: done before this iteration (set by k_cg_start and k_cg_zinv; `done` is
+  // written by this kernel and may be seen half-way)
+  if (s->idle) {
+    if (blockIdx.x == 0 && threadIdx.x == 0) loop_idle(loop);
+    return;
+  }
   extern __shared__ __align__(16) unsigned char smz[];
   C2<float>* P = reinterpret_cast<C2<float>*>(smz);
   float* O3 = reinterpret_cast<float*>(smz);
@@ -154,7 +211,6 @@ k_cg_zfwd(const __grid_constant__ SlabArgs<MAXB> args, const C2<float>* __restri
   const int partner = (lane & ~(M - 1)) | ((M - m) & (M - 1));
   const int col0 = blockIdx.x * TILE;
   const int its = s->iters;
-  const float a = float(s->alpha), beta = float(s->beta);
   const int64_t e0 = (int64_t)(col0 + t) * M + m;
   constexpr int64_t ES = (int64_t)N * N * M;   // from one element of a lane to the next
   float* __restrict__ x = args.xs[b] + e0;
@@ -164,6 +220,8 @@ k_cg_zfwd(const __grid_constant__ SlabArgs<MAXB> args, const C2<float>* __restri
   CgAcc<float> acc[1];
   C2<float> v[R];
   constexpr int HALF = R / 2;   // loads in flight per array
+  float a = 0.f, beta = 0.f;
+  bool stop = false;
 #pragma unroll
   for (int h = 0; h < R; h += HALF) {
     float rv[HALF], dv[HALF], xv[HALF], qv[HALF];
@@ -174,6 +232,19 @@ k_cg_zfwd(const __grid_constant__ SlabArgs<MAXB> args, const C2<float>* __restri
       xv[j] = its > 1 ? x[(h + j) * ES] : 0.f;
       qv[j] = its ? q[(h + j) * ES] : 0.f;
     }
+    if (h == 0 && its) {   // while the vectors load
+      cg_step<N, Z::THREADS>(reinterpret_cast<const float2*>(args.partial[b]), sums, &step);
+      a = step.a;
+      beta = step.beta;
+      const bool done = !(step.rr > s->stop), cap = loop.maxit > 0 && its >= loop.maxit;
+      stop = done || cap;
+      if (blockIdx.x == 0 && threadIdx.x == 0) {
+        s->alpha = step.alpha;
+        s->rr = step.rr;
+        if (stop) s->done = done ? 1 : 2;
+        loop_step(loop, done, its);
+      }
+    }
 #pragma unroll
     for (int j = 0; j < HALF; ++j) {
       if (its) {
@@ -182,12 +253,13 @@ k_cg_zfwd(const __grid_constant__ SlabArgs<MAXB> args, const C2<float>* __restri
         r[(h + j) * ES] = rv[j];
       }
       const float nv = rv[j] + beta * dv[j];
-      d[(h + j) * ES] = nv;
+      if (!stop) d[(h + j) * ES] = nv;
       acc[0].add(nv);
       // the DCT-II (real) and DST-II (imaginary) inputs of one line
       v[h + j] = {nv, h + j < H ? nv : -nv};
     }
   }
+  if (stop) return;
   z_tables<N>(tws, twr, qN, twg, qg);
   __syncthreads();
   plane::fft_to_pairs<N, float>(v, P, z_slots<N>(t), tws, m);
@@ -227,7 +299,8 @@ k_cg_zfwd(const __grid_constant__ SlabArgs<MAXB> args, const C2<float>* __restri
   }
   // the block's part of sum(d); k_cg_terms merges the parts
   block_merge<1>(acc, sh);
-  if (threadIdx.x == 0) reinterpret_cast<float2*>(args.partial[b])[blockIdx.x] = make_float2(acc[0].s, acc[0].c);
+  if (threadIdx.x == 0)
+    (reinterpret_cast<float2*>(args.partial[b]) + Z::SUMD)[blockIdx.x] = make_float2(acc[0].s, acc[0].c);
 }
 
 // sum(d) from the blocks' parts of k_cg_zfwd, in block order, by one CTA.
@@ -251,7 +324,7 @@ __device__ __forceinline__ void terms_body(const SlabArgs<MAXB>& args, int unit,
   if (args.s[b]->done) return;
   extern __shared__ __align__(16) unsigned char smx[];
   if (unit == 3 * N - 1 && rank == 0)
-    merge_sumd<N, plane::Shape<N>::THREADS>(reinterpret_cast<const float2*>(args.partial[b]), args.s[b]);
+    merge_sumd<N, plane::Shape<N>::THREADS>(reinterpret_cast<const float2*>(args.partial[b]) + ZShape<N>::SUMD, args.s[b]);
   const int term = unit % 3, k = unit / 3;
   const int64_t off = (int64_t)k * N * N;
   const float* in = (term == 2 ? args.z3[b] : args.z1[b]) + off;
@@ -278,13 +351,12 @@ k_cg_terms_cl(const __grid_constant__ SlabArgs<MAXB> args, const C2<float>* __re
   terms_body<N, MAXB>(args, blockIdx.x / 2, blockIdx.x % 2, twg, qg, s2g, inv_mu);
 }
 
-// q = DST-III_z (W1 + W2) + DCT-III_z W3 + cdiag d + rank1 sumd; d.q, r.r, r.q,
-// q.q; alpha, the next r.r and beta, done once that r.r <= stop.  Columns as
-// k_cg_zfwd; W1 comes negated at odd y, W2 at odd x, W3 at both.
+// q = DST-III_z (W1 + W2) + DCT-III_z W3 + cdiag d + rank1 sumd; the blocks' sums of
+// d.q, r.r, r.q and q.q.  Columns as k_cg_zfwd; W1 comes negated at odd y, W2 at odd x, W3 at both.
 template <int N, int MAXB>
 __global__ void __launch_bounds__(ZShape<N>::THREADS, ZShape<N>::OCC)
 k_cg_zinv(const __grid_constant__ SlabArgs<MAXB> args, const C2<float>* __restrict__ twg,
-          const C2<float>* __restrict__ qg, const CgLoop loop) {
+          const C2<float>* __restrict__ qg) {
   using S = plane::Shape<N>;
   using Z = ZShape<N>;
   constexpr int M = S::M, R = S::R, H = S::H, TILE = Z::TILE;
@@ -292,7 +364,7 @@ k_cg_zinv(const __grid_constant__ SlabArgs<MAXB> args, const C2<float>* __restri
   const int b = blockIdx.y;
   CGScalars* s = args.s[b];
   if (s->done) {
-    if (blockIdx.x == 0 && threadIdx.x == 0) loop_idle(loop);
+    if (blockIdx.x == 0 && threadIdx.x == 0) s->idle = 1;
     return;
   }
   extern __shared__ __align__(16) unsigned char smi[];
@@ -393,22 +465,38 @@ k_cg_zinv(const __grid_constant__ SlabArgs<MAXB> args, const C2<float>* __restri
       acc[3].add(qq);
     }
   }
-  double sum[4];
-  if (last_block_merge<4>(acc, reinterpret_cast<float2*>(args.partial[b]), &s->ticket[0], sh, sum) &&
-      threadIdx.x == 0) {
-    const double dq = sum[0], rr = sum[1];
-    const double al = (dq != 0.0) ? rr / dq : 0.0;
-    const double rr1 = rr - 2.0 * al * sum[2] + al * al * sum[3];   // |r - alpha q|^2
-    s->dq = dq;
-    s->alpha = al;
-    s->beta = (rr != 0.0) ? rr1 / rr : 0.0;
-    s->rr = rr1;
-    const int its = s->iters + 1;
-    const bool done = !(rr1 > s->stop);
-    s->iters = its;
-    if (done) s->done = 1;
-    loop_step(loop, done, its);
+  // the block's (or its group's) part
+  float2* part = reinterpret_cast<float2*>(args.partial[b]);
+  block_merge<4>(acc, sh);
+  if constexpr (Z::GROUP == 1) {
+    if (threadIdx.x == 0) {
+#pragma unroll
+      for (int j = 0; j < 4; ++j) part[j * Z::PARTS + blockIdx.x] = make_float2(acc[j].s, acc[j].c);
+    }
+  } else {
+    if (threadIdx.x == 0) {
+      float2* own = part + Z::BLOCK_SUMS + 4 * blockIdx.x;
+#pragma unroll
+      for (int j = 0; j < 4; ++j) own[j] = make_float2(acc[j].s, acc[j].c);
+      __threadfence();
+      const int g = blockIdx.x / Z::GROUP;
+      unsigned int* ticket = reinterpret_cast<unsigned int*>(part + Z::TICKETS + g);
+      if (atomicAdd(ticket, 1u) == Z::GROUP - 1) {   // the group's last block: its blocks in order
+        __threadfence();
+        CgAcc<float> m[4];
+        for (int k = 0; k < Z::GROUP; ++k)
+#pragma unroll
+          for (int j = 0; j < 4; ++j) {
+            const float2 p = __ldcg(part + Z::BLOCK_SUMS + 4 * (g * Z::GROUP + k) + j);
+            m[j].merge(p.x, p.y);
+          }
+#pragma unroll
+        for (int j = 0; j < 4; ++j) part[j * Z::PARTS + g] = make_float2(m[j].s, m[j].c);
+        *ticket = 0u;
+      }
+    }
   }
+  if (blockIdx.x == 0 && threadIdx.x == 0) s->iters += 1;
 }
 
 // ------------------------------------------------ natural <-> slab order
@@ -440,9 +528,11 @@ __global__ void __launch_bounds__(Conv<N>::THREADS) k_to_slab(const float* __res
   using V = Conv<N>;
   extern __shared__ float smc[];
   const int blk = blockIdx.x;
+#pragma unroll 8
   for (int e = threadIdx.x; e < V::ROWS * N; e += V::THREADS) smc[(e / N) * V::RS + e % N] = in[V::row(blk, e / N) + e % N];
   __syncthreads();
   float* o = out + V::base(blk);
+#pragma unroll 8
   for (int e = threadIdx.x; e < V::ROWS * N; e += V::THREADS) o[e] = smc[(e % V::ROWS) * V::RS + V::nat(e / V::ROWS)];
 }
 template <int N>
@@ -451,8 +541,10 @@ __global__ void __launch_bounds__(Conv<N>::THREADS) k_from_slab(const float* __r
   extern __shared__ float smc[];
   const int blk = blockIdx.x;
   const float* i = in + V::base(blk);
+#pragma unroll 8
   for (int e = threadIdx.x; e < V::ROWS * N; e += V::THREADS) smc[(e % V::ROWS) * V::RS + V::nat(e / V::ROWS)] = i[e];
   __syncthreads();
+#pragma unroll 8
   for (int e = threadIdx.x; e < V::ROWS * N; e += V::THREADS) out[V::row(blk, e / N) + e % N] = smc[(e / N) * V::RS + e % N];
 }
 
@@ -483,6 +575,7 @@ k_cg_start(const __grid_constant__ SlabArgs<MAXB> args, const __grid_constant__ 
   const double* __restrict__ gm = st.gm[run];
   const float *__restrict__ b1 = st.b1[run], *__restrict__ b2 = st.b2[run], *__restrict__ b3 = st.b3[run];
   CgAcc<float> acc[1];
+#pragma unroll 8
   for (int e = threadIdx.x; e < V::ROWS * N; e += V::THREADS) {
     const int64_t at = V::row(blk, e / N) + e % N;
     // FP32 sums of the FP64 g rounded once (by integer operations)
@@ -492,41 +585,55 @@ k_cg_start(const __grid_constant__ SlabArgs<MAXB> args, const __grid_constant__ 
   }
   __syncthreads();
   float* __restrict__ o = args.r[run] + V::base(blk);
+#pragma unroll 8
   for (int e = threadIdx.x; e < V::ROWS * N; e += V::THREADS) o[e] = smc[(e % V::ROWS) * V::RS + V::nat(e / V::ROWS)];
+  if constexpr (ZShape<N>::GROUP > 1) {   // the tickets of k_cg_zinv's groups
+    if (blk == 0)
+      for (int e = threadIdx.x; e < ZShape<N>::PARTS; e += V::THREADS)
+        *reinterpret_cast<unsigned int*>(reinterpret_cast<float2*>(args.partial[run]) + ZShape<N>::TICKETS + e) = 0u;
+  }
   double sum[1];
   if (last_block_merge<1>(acc, reinterpret_cast<float2*>(args.partial[run]), &s->ticket[1], sh, sum) &&
       threadIdx.x == 0) {
     s->rr = sum[0];
     s->bb = sum[0];
     s->stop = st.tol2[run] * sum[0];
-    s->alpha = 0.0;
-    s->beta = 0.0;
     s->rank1 = rank1;
     s->cdiag = cdiag;
     s->iters = 0;
-    s->done = (sum[0] > s->stop) ? 0 : 1;
+    s->done = s->idle = (sum[0] > s->stop) ? 0 : 1;
     if (active && !s->done) atomicAdd(active, 1);
   }
 }
 
-// End of a run: x = xs + alpha d, the update still pending when it stopped, in
-// natural order (x = 0 when no iteration ran).
+// End of a run: x in natural order (0 when no iteration ran); a run that the host
+// stopped before k_cg_zfwd saw its end still has an update pending.
 template <int N, int MAXB>
 __global__ void __launch_bounds__(Conv<N>::THREADS) k_cg_fin(const __grid_constant__ SlabArgs<MAXB> args) {
   using V = Conv<N>;
   extern __shared__ float smc[];
+  __shared__ double sums[4];
+  __shared__ CgStep step;
   const int run = blockIdx.y, blk = blockIdx.x;
   const CGScalars* s = args.s[run];
-  const float a = float(s->alpha);
   const int its = s->iters;
   const float* __restrict__ xs = args.xs[run] + V::base(blk);
+  float a = 0.f;
+  const bool pending = its && !s->done;
+  if (pending) {
+    cg_step<N, V::THREADS>(reinterpret_cast<const float2*>(args.partial[run]), sums, &step);
+    a = step.a;
+  }
   const float* __restrict__ d = args.d[run] + V::base(blk);
+#pragma unroll 8
   for (int e = threadIdx.x; e < V::ROWS * N; e += V::THREADS) {
-    const float x0 = its > 1 ? xs[e] : 0.f;
-    smc[(e % V::ROWS) * V::RS + V::nat(e / V::ROWS)] = its ? x0 + a * d[e] : 0.f;
+    float x0 = its > (pending ? 1 : 0) ? xs[e] : 0.f;
+    if (pending) x0 += a * d[e];
+    smc[(e % V::ROWS) * V::RS + V::nat(e / V::ROWS)] = x0;
   }
   __syncthreads();
   float* __restrict__ x = args.x[run];
+#pragma unroll 8
   for (int e = threadIdx.x; e < V::ROWS * N; e += V::THREADS) x[V::row(blk, e / N) + e % N] = smc[(e / N) * V::RS + e % N];
 }
 

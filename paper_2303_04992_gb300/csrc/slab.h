@@ -16,8 +16,8 @@ struct C2;
 // term results w1, w2 (N^3 floats each); the FP32 transform tables (full-circle
 // twiddles exp(-2 pi i t / 2N), t < 2N; post-twiddles exp(-i pi k / 2N), k < N;
 // the eigenvalue table 4 sin^2 of the DCT (N) and DST (N) modes), 1/mu, the
-// device scalars and the reduction partials (at least 4 N^2 / 16 slots of
-// eight bytes: k_cg_zinv stores four FP32 pairs per block).
+// device scalars and the reduction memory (slab_reduce_slots(N) slots of eight
+// bytes).
 struct SlabCg {
   int N;
   float *x, *xs, *r, *d, *q, *z1, *z3, *w1, *w2;
@@ -35,6 +35,7 @@ constexpr int kSlabBatchMax = 64;
 // Grids the slab iteration covers: N / 2 complex lines of N numbers (a whole
 // plane) fit in the shared memory of one CTA, at N = 256 of a cluster of two.
 bool slab_supported(int N);
+size_t slab_reduce_slots(int N);
 // Raises the kernels' dynamic shared-memory limits on the current device.
 cudaError_t slab_prepare(int N);
 
@@ -57,13 +58,13 @@ int slab_cg_start(const SlabCg* runs, int nrun, const SlabRhs* rhs, double rank1
                   cudaStream_t st);
 // One CG iteration of the runs (a no-op on the device for a run whose s->done is
 // set); each run's arithmetic and reduction order are those of a single run.
-// Each iteration leaves its own vector update (x += alpha d, r -= alpha q)
-// pending for the next one, so a run that has stopped needs slab_cg_finish
-// before x is read.
+// Each iteration leaves its own vector update (x += alpha d, r -= alpha q), its
+// stopping test and its scalars for the next one's first kernel, so a run ends in
+// an iteration that does nothing more.
 // loop: the device-side loop the iteration is the body of (captured graphs).
 int slab_cg_iteration(const SlabCg* runs, int nrun, const CgLoop& loop, cudaStream_t st);
-// x = xs + alpha d in natural order, the update still pending when the run
-// stopped (whether by done or by an iteration cap).
+// x in natural order, with the update still pending when the host stopped
+// launching iterations, if any.
 int slab_cg_finish(const SlabCg* runs, int nrun, cudaStream_t st);
 // One kernel of the iteration (0 k_cg_zfwd, 1 k_cg_terms, 2 k_cg_zinv; 3 the
 // finishing update) of a single run, for per-kernel timing.
