@@ -74,9 +74,13 @@ struct LShape {
   static constexpr int COLS = 2 * TEAMS;                   // lines per CTA
   static constexpr size_t tile = STAGED ? sizeof(T) * N * COLS : 0;
   static constexpr size_t bytes = sizeof(C2<T>) * ((size_t)TEAMS * N + 2 * N) + tile;
-  // CTAs per SM asked of the compiler: 96 registers in FP32, 128 for the fused passes (168 at
-  // N = 96, 24 values per lane), 255 in FP64
-  static constexpr int occ(bool fused) { return sizeof(T) == 8 ? 4 : (N == 96 ? 3 : (fused ? 4 : 5)); }
+  // CTAs per SM asked of the compiler.  FP32: 96 registers, 128 where two lines' modes are
+  // held beside the FFT (168 at N = 96, 24 values per lane).  FP64: 128 registers for a plain
+  // pass (the 1024 CTAs of one field at N = 128 resident at once), 168 and 255.
+  static constexpr int occ(int op) {
+    if (sizeof(T) == 8) return N == 96 || op == OP_F1I2 ? 4 : (op == OP_F2 || op == OP_I2 ? 8 : 6);
+    return N == 96 ? 3 : (op == OP_F1I2 ? 4 : 5);
+  }
 };
 
 template <typename T, typename Tin>
@@ -212,7 +216,7 @@ __device__ __forceinline__ void tile_store(const T* tile, Tout* out, int64_t es,
 }
 
 template <typename Tin, typename T, typename Tout, int N, int OP, int MAXJ>
-__global__ void __launch_bounds__((LShape<N, T>::THREADS), (LShape<N, T>::occ(OP >= OP_F2I2)))
+__global__ void __launch_bounds__((LShape<N, T>::THREADS), (LShape<N, T>::occ(OP)))
 k_lines(const __grid_constant__ Jobs<Tin, Tout, MAXJ> jobs, T h, T inv_mu, const C2<T>* __restrict__ twg,
         const C2<T>* __restrict__ qg, const T* __restrict__ s2) {
   using S = plane::Shape<N>;
@@ -253,15 +257,14 @@ k_lines(const __grid_constant__ Jobs<Tin, Tout, MAXJ> jobs, T h, T inv_mu, const
   }
   const auto X = slots<N>(t);
   constexpr T half = T(0.5), r2 = T(1.41421356237309504880), ir2 = T(0.70710678118654752440);
-  // modes (k, N - k) of the two lines, k = k1(i); slot (0, N/2) for k = 0
-  C2<T> A[H], B[H];
+  // the lane's modes (k, N - k), k = k1(i); slot (0, N/2) for k = 0
   auto k1 = [&](int i) { return plane::pair_index<N>(i, m); };
   auto k2 = [&](int i) { return (i == 0 && m == 0) ? N / 2 : N - k1(i); };
   auto mode = [&](int k) { return dst ? N - 1 - k : k; };   // array index of DCT index k (F2, I2)
+  constexpr bool fused = OP == OP_F2I2 || OP == OP_F1I1 || OP == OP_F1I2;
 
-  // ------------------------------------------------------------- forward
-  if constexpr (op_fwd2(OP)) {
-    C2<T> v[R];
+  // ---- the steps of a pass; A, B: modes (k, N - k) of the two lines
+  auto load2 = [&](C2<T>(&v)[R]) {   // both lines, Makhoul's order
     if (axis == 0) {
 #pragma unroll
       for (int r = 0; r < H; ++r) {
@@ -269,7 +272,8 @@ k_lines(const __grid_constant__ Jobs<Tin, Tout, MAXJ> jobs, T h, T inv_mu, const
         const C2<T> a = ld2<T>(in + 2 * n, vec), b = ld2<T>(in + N + 2 * n, vec);
         v[r] = {a.x, b.x};
         // element 2n + 1 is position N - 1 - n: lane M - 1 - m, register R - 1 - r
-        v[R - 1 - r] = {flip(__shfl_xor_sync(0xffffffffu, a.y, M - 1), dst), flip(__shfl_xor_sync(0xffffffffu, b.y, M - 1), dst)};
+        v[R - 1 - r] = {flip(__shfl_xor_sync(0xffffffffu, a.y, M - 1), dst),
+                        flip(__shfl_xor_sync(0xffffffffu, b.y, M - 1), dst)};
       }
     } else {
 #pragma unroll
@@ -281,263 +285,278 @@ k_lines(const __grid_constant__ Jobs<Tin, Tout, MAXJ> jobs, T h, T inv_mu, const
         if (r >= H) v[r] = {flip(v[r].x, dst), flip(v[r].y, dst)};
       }
     }
-    plane::fft_to_pairs<N, T>(v, P, X, tws, m);
-    plane::for_pairs<N, true, false>(v, m, partner, [&](int i, int k, bool self, C2<T> z, C2<T> g) {
-      const C2<T> q0 = qg[k];
-      const C2<T> q = {half * q0.x, half * q0.y};
-      C2<T> a = cmul(q, C2<T>{z.x + g.x, z.y - g.y}), b = cmul(q, C2<T>{z.y + g.y, g.x - z.x});
-      if (self) {
-        a = {z.x, -(ir2 * g.x)};
-        b = {z.y, -(ir2 * g.y)};
-      }
-      A[i] = {a.x, -a.y};   // X_k, X_(N-k)
-      B[i] = {b.x, -b.y};
-    });
-  } else if constexpr (op_fwd1(OP)) {
+  };
+  auto load1 = [&](C2<T>(&v)[R], int ab) {   // one line, packed odd extension
+    const Tin* x = in + ab * ls;
+    // z_n = x_2n + i x_(2n+1) (x_0 is the wall: 0), z_(N-n) = -x_2n - i x_(2n-1)
 #pragma unroll
-    for (int i = 0; i < H; ++i) B[i] = {T(0), T(0)};
-#pragma unroll 1
-    for (int ab = 0; ab < 2; ++ab) {
-      const Tin* x = in + ab * ls;
-      C2<T> v[R];
-      // z_n = x_2n + i x_(2n+1) (x_0 is the wall: 0), z_(N-n) = -x_2n - i x_(2n-1)
-#pragma unroll
-      for (int r = 0; r < H; ++r) {
-        const int n = m + M * r;
-        C2<T> a;
-        if (axis == 0) a = ld2<T>(x + 2 * n, vec);
-        else if (STAGED) a = {tp(2 * n)[ab], tp(2 * n + 1)[ab]};
-        else a = {to_work<T>(x[(int64_t)(2 * n) * es]), to_work<T>(x[(int64_t)(2 * n + 1) * es])};
-        if (r == 0 && m == 0) a.x = T(0);
-        v[r] = a;
-      }
-#pragma unroll
-      for (int r = 0; r < H; ++r) {
-        // position n = m + M (R - 1 - r): x_2n' of n' = N - n at lane M - m, register r (lane 0:
-        // register r + 1, zero for n' = N/2), x_(2n'-1) at lane M - 1 - m, register r
-        const T nx = r + 1 < H ? v[r + 1].x : T(0);
-        const T re = __shfl_sync(0xffffffffu, m ? v[r].x : nx, partner);
-        const T im = __shfl_xor_sync(0xffffffffu, v[r].y, M - 1);
-        v[R - 1 - r] = {-re, -im};
-      }
-      plane::fft_to_pairs<N, T>(v, P, X, tws, m);
-      plane::for_pairs<N, true, false>(v, m, partner, [&](int i, int k, bool self, C2<T> z, C2<T> g) {
-        const C2<T> w = twg[k];
-        // twice a and b: a = (.., z.y - g.y), b = (z.x - g.x, z.y + g.y)
-        const T ia = T(0.25) * (z.y - g.y), wb = T(0.25) * (w.x * (z.x - g.x) - w.y * (z.y + g.y));
-        C2<T> f = {wb - ia, wb + ia};
-        if (self) f = {T(0), half * g.y};   // modes 0 and N/2
-        A[i] = B[i];   // the first line's modes move on when the second's arrive
-        B[i] = f;
-      });
+    for (int r = 0; r < H; ++r) {
+      const int n = m + M * r;
+      C2<T> a;
+      if (axis == 0) a = ld2<T>(x + 2 * n, vec);
+      else if (STAGED) a = {tp(2 * n)[ab], tp(2 * n + 1)[ab]};
+      else a = {to_work<T>(x[(int64_t)(2 * n) * es]), to_work<T>(x[(int64_t)(2 * n + 1) * es])};
+      if (r == 0 && m == 0) a.x = T(0);
+      v[r] = a;
     }
-  } else {   // inverse only: the modes come from memory
 #pragma unroll
-    for (int j = 0; j < H; ++j) {
-      int ka = k1(j), kb = k2(j);
-      if constexpr (OP == OP_I2) {
-        ka = mode(ka);
-        kb = mode(kb);
-      }
-      C2<T> a, b;
-      if (axis == 0) {
-        a = {to_work<T>(in[ka]), to_work<T>(in[kb])};
-        b = {to_work<T>(in[N + ka]), to_work<T>(in[N + kb])};
-      } else {
-        C2<T> e, f;
-        if constexpr (STAGED) {
-          e = plane::ldc(reinterpret_cast<const C2<T>*>(tp(ka)));
-          f = plane::ldc(reinterpret_cast<const C2<T>*>(tp(kb)));
-        } else {
-          e = ld2<T>(in + (int64_t)ka * es, vec);
-          f = ld2<T>(in + (int64_t)kb * es, vec);
-        }
-        a = {e.x, f.x};
-        b = {e.y, f.y};
-      }
-      if (OP == OP_I1 && j == 0 && m == 0) a.x = b.x = T(0);   // DST-I has no mode 0
-      A[j] = a;
-      B[j] = b;
-    }
-  }
-
-  // -------------------------------------------------------------- weight
-  Weights<T, N> WA, WB;
-  constexpr bool fused = OP == OP_F2I2 || OP == OP_F1I1 || OP == OP_F1I2;
-  if (fused || job.wmode != W_NONE) {
-    auto setup = [&](int ln) {
-      Weights<T, N> w;
-      w.s2 = s2;
-      w.h = h;
-      w.inv_mu = inv_mu;
-      w.wmode = job.wmode;
-      w.own = job.wc == axis;
-      w.kind = w.own ? 0 : 1;
-      // the two other axes' mode indices and their kinds (component axis 0, else 1)
-      const int hi = ln / N, lo = ln % N;
-      const int ax1 = axis == 0 ? 1 : 0, ax2 = axis == 2 ? 1 : 2;   // lo runs along ax1, hi along ax2
-      const T v1 = s2[(job.wc == ax1 ? 0 : 1) * N + lo], v2 = s2[(job.wc == ax2 ? 0 : 1) * N + hi];
-      w.rest = v1 + v2;
-      w.num = w.own ? T(0) : (job.wc == ax1 ? w.numer(v1, lo == 0) : w.numer(v2, hi == 0));
-      return w;
-    };
-    WA = setup(line);
-    WB = setup(line + 1);
-  }
-  // the weights of modes a1, a2 of both lines: one reciprocal for the four (products of
-  // 4 sin^2 sums, 1e-4 .. 12 each)
-  auto weigh = [&](int a1, int a2, T& w1, T& w2, T& u1, T& u2) {
-    T d1, d2, e1, e2;
-    const T n1 = WA.at(a1, d1), n2 = WA.at(a2, d2), o1 = WB.at(a1, e1), o2 = WB.at(a2, e2);
-    if constexpr (sizeof(T) == 4) {
-      w1 = n1 * plane::rcp(d1);
-      w2 = n2 * plane::rcp(d2);
-      u1 = o1 * plane::rcp(e1);
-      u2 = o2 * plane::rcp(e2);
-    } else {
-      const T d = d1 * d2, e = e1 * e2, r = T(1) / (d * e), rd = e * r, re = d * r;
-      w1 = n1 * (d2 * rd);
-      w2 = n2 * (d1 * rd);
-      u1 = o1 * (e2 * re);
-      u2 = o2 * (e1 * re);
+    for (int r = 0; r < H; ++r) {
+      // position n = m + M (R - 1 - r): x_2n' of n' = N - n at lane M - m, register r (lane 0:
+      // register r + 1, zero for n' = N/2), x_(2n'-1) at lane M - 1 - m, register r
+      const T nx = r + 1 < H ? v[r + 1].x : T(0);
+      const T re = __shfl_sync(0xffffffffu, m ? v[r].x : nx, partner);
+      const T im = __shfl_xor_sync(0xffffffffu, v[r].y, M - 1);
+      v[R - 1 - r] = {-re, -im};
     }
   };
-  if constexpr (fused) {
-#pragma unroll
-    for (int j = 0; j < H; ++j) {
-      int ka = k1(j), kb = k2(j);
-      if constexpr (OP == OP_F2I2) {
-        ka = mode(ka);
-        kb = mode(kb);
-      }
-      T w1, w2, u1, u2;
-      weigh(ka, kb, w1, w2, u1, u2);
-      A[j] = {A[j].x * w1, A[j].y * w2};
-      B[j] = {B[j].x * u1, B[j].y * u2};
+  auto modes2 = [&](int k, bool self, C2<T> z, C2<T> g, C2<T>& A, C2<T>& B) {
+    const C2<T> q0 = qg[k];
+    const C2<T> q = {half * q0.x, half * q0.y};
+    C2<T> a = cmul(q, C2<T>{z.x + g.x, z.y - g.y}), b = cmul(q, C2<T>{z.y + g.y, g.x - z.x});
+    if (self) {
+      a = {z.x, -(ir2 * g.x)};
+      b = {z.y, -(ir2 * g.y)};
     }
-  }
-
-  // ------------------------------------------------------------- inverse
-  if constexpr (op_inv2(OP)) {
-    // both lines in one FFT: conj Z_k = q conj(a + i b), conj Z_(N-k) = conj(q) (a - i b)
-    // with a = X_k - i X_(N-k) of line A, b of line B
-    C2<T> v[R];
-    plane::for_pairs<N, false, true>(v, m, partner, [&](int i, int k, bool self, C2<T>& lo, C2<T>& hi) {
-      const C2<T> a = {A[i].x, -A[i].y}, b = {B[i].x, -B[i].y}, q = qg[k];
-      lo = cmul(q, C2<T>{a.x - b.y, -(a.y + b.x)});
-      hi = cmul(plane::conjg(q), C2<T>{a.x + b.y, a.y - b.x});
-      if (self) {
-        lo = {a.x, -b.x};
-        hi = {r2 * A[0].y, -(r2 * B[0].y)};
-      }
-    });
-    plane::fft_from_pairs<N, T>(v, P, X, tws, twr, m);
-    const T sc = T(1) / T(N), so = (OP == OP_I2 || OP == OP_F2I2) && dst ? -sc : sc;
+    A = {a.x, -a.y};   // X_k, X_(N-k)
+    B = {b.x, -b.y};
+  };
+  auto modes1 = [&](int k, bool self, C2<T> z, C2<T> g) {
+    const C2<T> w = twg[k];
+    // four times Im a and Re(w b) over two: a = (.., z.y - g.y), b = (z.x - g.x, z.y + g.y)
+    const T ia = T(0.25) * (z.y - g.y), wb = T(0.25) * (w.x * (z.x - g.x) - w.y * (z.y + g.y));
+    C2<T> f = {wb - ia, wb + ia};
+    if (self) f = {T(0), half * g.y};   // modes 0 and N/2
+    return f;
+  };
+  // the inverse FFT's input, conjugated: conj Z_k = q conj(a + i b), conj Z_(N-k) = conj(q) (a - i b)
+  // with a = X_k - i X_(N-k) of line A, b of line B
+  auto back2 = [&](int k, bool self, C2<T> A, C2<T> B, C2<T>& lo, C2<T>& hi) {
+    const C2<T> a = {A.x, -A.y}, b = {B.x, -B.y}, q = qg[k];
+    lo = cmul(q, C2<T>{a.x - b.y, -(a.y + b.x)});
+    hi = cmul(plane::conjg(q), C2<T>{a.x + b.y, a.y - b.x});
+    if (self) {
+      lo = {a.x, -b.x};
+      hi = {r2 * A.y, -(r2 * B.y)};
+    }
+  };
+  auto back1 = [&](int k, bool self, C2<T> f, C2<T>& lo, C2<T>& hi) {
+    const C2<T> w = twg[k];   // exp(-i pi k / N)
+    const T s = f.x + f.y, d = f.y - f.x, cs = w.x * s, ss = -(w.y * s);
+    lo = {cs, -(ss + d)};
+    hi = {-cs, d - ss};
+    if (self) {
+      lo = {T(0), T(0)};
+      hi = {T(0), T(-2) * f.y};
+    }
+  };
+  // weights of line ln
+  auto weights = [&](int ln) {
+    Weights<T, N> w;
+    w.s2 = s2;
+    w.h = h;
+    w.inv_mu = inv_mu;
+    w.wmode = job.wmode;
+    w.own = job.wc == axis;
+    w.kind = w.own ? 0 : 1;
+    // the two other axes' mode indices and their kinds (component axis 0, else 1)
+    const int hi = ln / N, lo = ln % N;
+    const int ax1 = axis == 0 ? 1 : 0, ax2 = axis == 2 ? 1 : 2;   // lo runs along ax1, hi along ax2
+    const T v1 = s2[(job.wc == ax1 ? 0 : 1) * N + lo], v2 = s2[(job.wc == ax2 ? 0 : 1) * N + hi];
+    w.rest = v1 + v2;
+    w.num = w.own ? T(0) : (job.wc == ax1 ? w.numer(v1, lo == 0) : w.numer(v2, hi == 0));
+    return w;
+  };
+  // a mode pair (array indices ka, kb) times its weights; FP64: one reciprocal for the two
+  // (products of 4 sin^2 sums, 1e-4 .. 12 each)
+  auto weigh = [&](const Weights<T, N>& W, int ka, int kb, C2<T>& f) {
+    T d1, d2;
+    const T n1 = W.at(ka, d1), n2 = W.at(kb, d2);
+    if constexpr (sizeof(T) == 4) {
+      f = {f.x * (n1 * plane::rcp(d1)), f.y * (n2 * plane::rcp(d2))};
+    } else {
+      const T r = T(1) / (d1 * d2);
+      f = {f.x * (n1 * (d2 * r)), f.y * (n2 * (d1 * r))};
+    }
+  };
+  auto store2 = [&](const C2<T>(&v)[R]) {
+    // v holds the conjugate: line A in the real, minus line B in the imaginary part; element
+    // 2n here, element 2n + 1 at position N - 1 - n
+    const T sc = T(1) / T(N);
+    const bool neg = OP != OP_F1I2 && dst;
     const bool weighted = OP == OP_I2 && job.wmode != W_NONE;
 #pragma unroll
     for (int j = 0; j < H; ++j) {
       const int n = m + M * j;
-      // v holds the conjugate: line A in the real, minus line B in the imaginary part;
-      // element 2n here, element 2n + 1 at position N - 1 - n
-      C2<T> e = {sc * v[j].x, -(sc * v[j].y)};
+      // along x the odd element comes from the mirror lane: A and B of elements 2n, 2n + 1
+      const int io = axis == 0 ? 2 * n + 1 : 2 * ((M - 1 - m) + M * j) + 1;
+      C2<T> o = v[R - 1 - j];
+      if (axis == 0) o = {__shfl_xor_sync(0xffffffffu, o.x, M - 1), __shfl_xor_sync(0xffffffffu, o.y, M - 1)};
+      C2<T> fa = {sc * v[j].x, flip(sc * o.x, neg)}, fb = {-(sc * v[j].y), flip(sc * o.y, !neg)};
+      if (weighted) {
+        weigh(weights(line), 2 * n, io, fa);
+        weigh(weights(line + 1), 2 * n, io, fb);
+      }
       if (axis == 0) {
-        C2<T> o = {so * __shfl_xor_sync(0xffffffffu, v[R - 1 - j].x, M - 1),
-                   -(so * __shfl_xor_sync(0xffffffffu, v[R - 1 - j].y, M - 1))};
-        if (weighted) {
-          T w1, w2, u1, u2;
-          weigh(2 * n, 2 * n + 1, w1, w2, u1, u2);
-          e = {e.x * w1, e.y * u1};
-          o = {o.x * w2, o.y * u2};
-        }
-        st2<T>(out + 2 * n, e.x, o.x, vec, acc);
-        st2<T>(out + N + 2 * n, e.y, o.y, vec, acc);
+        st2<T>(out + 2 * n, fa.x, fa.y, vec, acc);
+        st2<T>(out + N + 2 * n, fb.x, fb.y, vec, acc);
+      } else if constexpr (STAGED) {
+        plane::stc(reinterpret_cast<C2<T>*>(tp(2 * n)), C2<T>{fa.x, fb.x});
+        plane::stc(reinterpret_cast<C2<T>*>(tp(io)), C2<T>{fa.y, fb.y});
       } else {
-        C2<T> o = {so * v[R - 1 - j].x, -(so * v[R - 1 - j].y)};
-        const int io = 2 * ((M - 1 - m) + M * j) + 1;   // register R - 1 - j: position N - 1 - (io / 2)
-        if (weighted) {
-          T w1, w2, u1, u2;
-          weigh(2 * n, io, w1, w2, u1, u2);
-          e = {e.x * w1, e.y * u1};
-          o = {o.x * w2, o.y * u2};
-        }
-        if constexpr (STAGED) {
-          plane::stc(reinterpret_cast<C2<T>*>(tp(2 * n)), e);
-          plane::stc(reinterpret_cast<C2<T>*>(tp(io)), o);
-        } else {
-          st2<T>(out + (int64_t)(2 * n) * es, e.x, e.y, vec, acc);
-          st2<T>(out + (int64_t)io * es, o.x, o.y, vec, acc);
-        }
+        st2<T>(out + (int64_t)(2 * n) * es, fa.x, fb.x, vec, acc);
+        st2<T>(out + (int64_t)io * es, fa.y, fb.y, vec, acc);
       }
     }
-  } else if constexpr (op_inv1(OP)) {
-#pragma unroll 1
-    for (int ab = 0; ab < 2; ++ab) {
-      C2<T> v[R];
-      plane::for_pairs<N, false, true>(v, m, partner, [&](int i, int k, bool self, C2<T>& lo, C2<T>& hi) {
-        const C2<T> f = A[i], w = twg[k];   // exp(-i pi k / N)
-        A[i] = B[i];
-        const T s = f.x + f.y, d = f.y - f.x, cs = w.x * s, ss = -(w.y * s);
-        lo = {cs, -(ss + d)};   // conjugated
-        hi = {-cs, d - ss};
-        if (self) {
-          lo = {T(0), T(0)};
-          hi = {T(0), T(-2) * f.y};
-        }
-      });
-      plane::fft_from_pairs<N, T>(v, P, X, tws, twr, m);
-      Tout* x = out + ab * ls;
-      const T sc = T(1) / T(N);
-      const bool weighted = OP == OP_I1 && job.wmode != W_NONE;
-#pragma unroll
-      for (int j = 0; j < H; ++j) {
-        const int n = m + M * j;
-        T e = sc * v[j].x, o = -(sc * v[j].y);
-        if (j == 0 && m == 0) e = T(0);
-        if (weighted) {
-          T w1, w2, u1, u2;
-          weigh(2 * n, 2 * n + 1, w1, w2, u1, u2);
-          e *= ab ? u1 : w1;
-          o *= ab ? u2 : w2;
-        }
-        if (axis == 0) {
-          st2<T>(x + 2 * n, e, o, vec);
-        } else if (STAGED) {
-          tp(2 * n)[ab] = e;
-          tp(2 * n + 1)[ab] = o;
-        } else {
-          x[(int64_t)(2 * n) * es] = e;
-          x[(int64_t)(2 * n + 1) * es] = o;
-        }
-      }
-    }
-  } else {   // forward only: the modes go to memory
+  };
+  auto store1 = [&](const C2<T>(&v)[R], int ab) {
+    Tout* x = out + ab * ls;
+    const T sc = T(1) / T(N);
+    const bool weighted = OP == OP_I1 && job.wmode != W_NONE;
 #pragma unroll
     for (int j = 0; j < H; ++j) {
-      int ka = k1(j), kb = k2(j);
-      if constexpr (OP == OP_F2) {
-        ka = mode(ka);
-        kb = mode(kb);
-      }
-      C2<T> a = A[j], b = B[j];
-      if (job.wmode != W_NONE) {
-        T w1, w2, u1, u2;
-        weigh(ka, kb, w1, w2, u1, u2);
-        a = {a.x * w1, a.y * w2};
-        b = {b.x * u1, b.y * u2};
-      }
+      const int n = m + M * j;
+      C2<T> f = {sc * v[j].x, -(sc * v[j].y)};
+      if (j == 0 && m == 0) f.x = T(0);
+      if (weighted) weigh(weights(line + ab), 2 * n, 2 * n + 1, f);
       if (axis == 0) {
-        out[ka] = a.x;
-        out[kb] = a.y;
-        out[N + ka] = b.x;
-        out[N + kb] = b.y;
+        st2<T>(x + 2 * n, f.x, f.y, vec);
+      } else if (STAGED) {
+        tp(2 * n)[ab] = f.x;
+        tp(2 * n + 1)[ab] = f.y;
       } else {
-        if constexpr (STAGED) {
-          plane::stc(reinterpret_cast<C2<T>*>(tp(ka)), C2<T>{a.x, b.x});
-          plane::stc(reinterpret_cast<C2<T>*>(tp(kb)), C2<T>{a.y, b.y});
-        } else {
-          st2<T>(out + (int64_t)ka * es, a.x, b.x, vec);
-          st2<T>(out + (int64_t)kb * es, a.y, b.y, vec);
-        }
+        x[(int64_t)(2 * n) * es] = f.x;
+        x[(int64_t)(2 * n + 1) * es] = f.y;
+      }
+    }
+  };
+  auto fwd_store = [&](int i, C2<T> a, C2<T> b, int ka, int kb) {   // modes of both lines to memory
+    if (job.wmode != W_NONE) {
+      weigh(weights(line), ka, kb, a);
+      weigh(weights(line + 1), ka, kb, b);
+    }
+    if (axis == 0) {
+      out[ka] = a.x;
+      out[kb] = a.y;
+      out[N + ka] = b.x;
+      out[N + kb] = b.y;
+    } else if constexpr (STAGED) {
+      plane::stc(reinterpret_cast<C2<T>*>(tp(ka)), C2<T>{a.x, b.x});
+      plane::stc(reinterpret_cast<C2<T>*>(tp(kb)), C2<T>{a.y, b.y});
+    } else {
+      st2<T>(out + (int64_t)ka * es, a.x, b.x, vec);
+      st2<T>(out + (int64_t)kb * es, a.y, b.y, vec);
+    }
+  };
+  auto load_modes = [&](int ka, int kb, C2<T>& a, C2<T>& b) {
+    if (axis == 0) {
+      a = {to_work<T>(in[ka]), to_work<T>(in[kb])};
+      b = {to_work<T>(in[N + ka]), to_work<T>(in[N + kb])};
+    } else {
+      C2<T> e, f;
+      if constexpr (STAGED) {
+        e = plane::ldc(reinterpret_cast<const C2<T>*>(tp(ka)));
+        f = plane::ldc(reinterpret_cast<const C2<T>*>(tp(kb)));
+      } else {
+        e = ld2<T>(in + (int64_t)ka * es, vec);
+        f = ld2<T>(in + (int64_t)kb * es, vec);
+      }
+      a = {e.x, f.x};
+      b = {e.y, f.y};
+    }
+  };
+
+  // ---- the passes
+  C2<T> v[R];
+  if constexpr (OP == OP_F2) {
+    load2(v);
+    plane::fft_to_pairs<N, T>(v, P, X, tws, m);
+    plane::for_pairs<N, true, false>(v, m, partner, [&](int i, int k, bool self, C2<T> z, C2<T> g) {
+      C2<T> A, B;
+      modes2(k, self, z, g, A, B);
+      fwd_store(i, A, B, mode(k), mode(self ? N / 2 : N - k));
+    });
+  } else if constexpr (OP == OP_F2I2) {
+    load2(v);
+    plane::fft_to_pairs<N, T>(v, P, X, tws, m);
+    const Weights<T, N> WA = weights(line), WB = weights(line + 1);
+    plane::for_pairs<N, true, true>(v, m, partner, [&](int, int k, bool self, C2<T>& z, C2<T>& g) {
+      C2<T> A, B;
+      modes2(k, self, z, g, A, B);
+      const int ka = mode(k), kb = mode(self ? N / 2 : N - k);
+      weigh(WA, ka, kb, A);
+      weigh(WB, ka, kb, B);
+      back2(k, self, A, B, z, g);
+    });
+    plane::fft_from_pairs<N, T>(v, P, X, tws, twr, m);
+    store2(v);
+  } else if constexpr (OP == OP_I2) {
+    C2<T> A[H], B[H];   // every mode is read before any output is written (in place)
+#pragma unroll
+    for (int i = 0; i < H; ++i) load_modes(mode(k1(i)), mode(k2(i)), A[i], B[i]);
+    plane::for_pairs<N, false, true>(v, m, partner, [&](int i, int k, bool self, C2<T>& lo, C2<T>& hi) {
+      back2(k, self, A[i], B[i], lo, hi);
+    });
+    plane::fft_from_pairs<N, T>(v, P, X, tws, twr, m);
+    store2(v);
+  } else if constexpr (OP == OP_F1I1) {
+#pragma unroll 1
+    for (int ab = 0; ab < 2; ++ab) {
+      load1(v, ab);
+      plane::fft_to_pairs<N, T>(v, P, X, tws, m);
+      const Weights<T, N> W = weights(line + ab);
+      plane::for_pairs<N, true, true>(v, m, partner, [&](int, int k, bool self, C2<T>& z, C2<T>& g) {
+        C2<T> f = modes1(k, self, z, g);
+        weigh(W, k, self ? N / 2 : N - k, f);
+        back1(k, self, f, z, g);
+      });
+      plane::fft_from_pairs<N, T>(v, P, X, tws, twr, m);
+      store1(v, ab);
+    }
+  } else {
+    // A, B: the lines' modes, the first line's moving on to A when the second's arrive in B
+    C2<T> A[H], B[H];
+    if constexpr (OP == OP_I1) {
+#pragma unroll
+      for (int i = 0; i < H; ++i) {
+        load_modes(k1(i), k2(i), A[i], B[i]);
+        if (i == 0 && m == 0) A[i].x = B[i].x = T(0);   // DST-I has no mode 0
+      }
+    } else {
+#pragma unroll
+      for (int i = 0; i < H; ++i) B[i] = {T(0), T(0)};
+#pragma unroll 1
+      for (int ab = 0; ab < 2; ++ab) {
+        load1(v, ab);
+        plane::fft_to_pairs<N, T>(v, P, X, tws, m);
+        plane::for_pairs<N, true, false>(v, m, partner, [&](int i, int k, bool self, C2<T> z, C2<T> g) {
+          A[i] = B[i];
+          B[i] = modes1(k, self, z, g);
+        });
+      }
+    }
+    if constexpr (OP == OP_F1) {
+#pragma unroll
+      for (int i = 0; i < H; ++i) fwd_store(i, A[i], B[i], k1(i), k2(i));
+    } else if constexpr (OP == OP_F1I2) {
+      const Weights<T, N> WA = weights(line), WB = weights(line + 1);
+      plane::for_pairs<N, false, true>(v, m, partner, [&](int i, int k, bool self, C2<T>& lo, C2<T>& hi) {
+        const int kb = self ? N / 2 : N - k;
+        weigh(WA, k, kb, A[i]);
+        weigh(WB, k, kb, B[i]);
+        back2(k, self, A[i], B[i], lo, hi);
+      });
+      plane::fft_from_pairs<N, T>(v, P, X, tws, twr, m);
+      store2(v);
+    } else {
+      static_assert(OP == OP_I1, "the seven operations");
+#pragma unroll 1
+      for (int ab = 0; ab < 2; ++ab) {
+        plane::for_pairs<N, false, true>(v, m, partner, [&](int i, int k, bool self, C2<T>& lo, C2<T>& hi) {
+          back1(k, self, A[i], lo, hi);
+          A[i] = B[i];
+        });
+        plane::fft_from_pairs<N, T>(v, P, X, tws, twr, m);
+        store1(v, ab);
       }
     }
   }
