@@ -58,14 +58,15 @@ struct Shape {
   static constexpr int NS = R / M;                               // DFT_M per lane
   static constexpr int H = R / 2;
   static constexpr int LINES = N / 2;
-  // CTAs per plane: the 256 KB of a plane at N = 256 take two CTAs of a cluster,
-  // each with half of the lines, half of the row pairs and the other's lines
-  // through distributed shared memory
-  static constexpr int CL = N == 256 ? 2 : 1;
+  // CTAs per plane: the 256 KB of a plane at N = 256 take the four CTAs of a
+  // cluster, each with a quarter of the lines and of the row pairs and the others'
+  // lines through distributed shared memory (two CTAs fit a plane as well, but only
+  // one of them an SM, where nothing then runs during its waits)
+  static constexpr int CL = N == 256 ? 4 : 1;
   static constexpr int LL = LINES / CL;                          // lines and row pairs per CTA
   static constexpr int ROUNDS = N >= 128 ? 2 : 1;                // FFTs per team and axis step
   static constexpr int TEAMS = LL / ROUNDS;
-  static constexpr int THREADS = TEAMS * M;                      // 512, 256, 192, 256, 64
+  static constexpr int THREADS = TEAMS * M;                      // N = 256: 256; 256, 192, 256, 64
   static constexpr int YB = 2 * (32 / M);                        // y positions of one warp's row pairs
   static_assert(R % M == 0, "four-step split");
 };
@@ -235,7 +236,7 @@ struct XSlots {   // along x
   }
 };
 template <int N>
-struct XScratch {   // along x on two CTAs, whose columns are not whole: a buffer of the team
+struct XScratch {   // along x on a cluster, whose CTAs' columns are not whole: a buffer of the team
   using S = Shape<N>;
   int base;
   __device__ __forceinline__ int at(int s, int v) const { return base + s * S::M + (v ^ (s & (S::M - 1))); }
@@ -534,7 +535,7 @@ struct Smem {
 // instead the signs of `signs` (so that two terms can share an input).
 // az: the plane's 4 sin^2 along z; sc: 1 / (mu N^2).
 // twg: exp(-pi i t / N), t < 2N; qg: exp(-pi i k / 2N); s2: 4 sin^2(pi a / 2N), a < N.
-// Called by all threads of the CTA (of both CTAs of the cluster; rank: this one's).
+// Called by all threads of the CTA (of every CTA of the cluster; rank: this one's).
 template <int N, typename T>
 __device__ __forceinline__ void term_plane(const T* in, T* out, const Term term, const Term signs, T az, T sc,
                                            C2<T>* P, const C2<T>* __restrict__ twg, const C2<T>* __restrict__ qg,
@@ -571,9 +572,10 @@ __device__ __forceinline__ void term_plane(const T* in, T* out, const Term term,
     if constexpr (S::CL > 1) cooperative_groups::this_cluster().sync();
     else __syncthreads();
   };
-  // the column pair n0, n0 + 1 of line l
-  auto pair_at = [&](int l, int n0) -> C2<T>* {
-    if constexpr (S::CL > 1) return (l < S::LL ? lines[0] : lines[S::CL - 1]) + ((l % S::LL) * N + (n0 ^ line_sw<M>(l)));
+  // the column pair n0, n0 + 1 of line l, the lane's i-th index
+  auto pair_at = [&](int i, int l, int n0) -> C2<T>* {
+    static_assert(S::CL == 1 || !PairShape<N>::in_lane, "i gives the owner of line m + M i");
+    if constexpr (S::CL > 1) return lines[M * i / S::LL] + ((l % S::LL) * N + (n0 ^ line_sw<M>(l)));
     else return P + (l * N + (n0 ^ line_sw<M>(l)));
   };
   C2<T> v[R];
@@ -585,17 +587,17 @@ __device__ __forceinline__ void term_plane(const T* in, T* out, const Term term,
     const T fl = (n0 >= N / 2 && term.ys != signs.ys) ? T(-1) : T(1), fh = term.xs != signs.xs ? -fl : fl;
 #pragma unroll
     for (int r = 0; r < R; ++r) v[r] = cscale(ldc(ra + r * (M * S::YB / 2)), r < H ? fl : fh);
-    if (rd == 0) sync();   // tables (and the other CTA runs before its lines are written)
+    if (rd == 0) sync();   // tables (and the others run before their lines are written)
     if constexpr (S::CL > 1) fft_to_pairs<N, T>(v, P, XScratch<N>{S::LL * N + t * N}, tws, m);
     else fft_to_pairs<N, T>(v, P, XSlots<N>{n0}, tws, m);
-    for_pairs<N, true, false>(v, m, partner, [&](int, int l, bool self, C2<T> z, C2<T> g) {
+    for_pairs<N, true, false>(v, m, partner, [&](int i, int l, bool self, C2<T> z, C2<T> g) {
       const C2<T> q = ldc(qh + l);
       C2<T> a = cmul(q, C2<T>{z.x + g.x, z.y - g.y}), b = cmul(q, C2<T>{z.y + g.y, g.x - z.x});
       if (self) {   // the real modes 0 and N/2
         a = {z.x, g.x};
         b = {z.y, g.y};
       }
-      C2<T>* at = pair_at(l, n0);   // the swizzle keeps pairs 2p, 2p + 1 together
+      C2<T>* at = pair_at(i, l, n0);   // the swizzle keeps pairs 2p, 2p + 1 together
       if constexpr (sizeof(T) == 4) {
         *reinterpret_cast<float4*>(at) = make_float4(a.x, a.y, b.x, b.y);
       } else {
@@ -656,8 +658,8 @@ __device__ __forceinline__ void term_plane(const T* in, T* out, const Term term,
   for (int rd = 0; rd < S::ROUNDS; ++rd) {
     const int n0 = 2 * (rank * S::LL + t + S::TEAMS * rd);
     // conj Z'_k = q conj(A + i B), conj Z'_(N-k) = conj(q) (A - i B)
-    for_pairs<N, false, true>(v, m, partner, [&](int, int l, bool self, C2<T>& lo, C2<T>& hi) {
-      const C2<T>* at = pair_at(l, n0);
+    for_pairs<N, false, true>(v, m, partner, [&](int i, int l, bool self, C2<T>& lo, C2<T>& hi) {
+      const C2<T>* at = pair_at(i, l, n0);
       C2<T> a, b;
       if constexpr (sizeof(T) == 4) {
         const float4 f = *reinterpret_cast<const float4*>(at);
@@ -681,7 +683,7 @@ __device__ __forceinline__ void term_plane(const T* in, T* out, const Term term,
 #pragma unroll
     for (int j = 0; j < R; ++j) stc(ra + j * (M * S::YB / 2), conjg(v[j]));
   }
-  if constexpr (S::CL > 1) sync();   // the other CTA may still read this one's lines
+  if constexpr (S::CL > 1) sync();   // the others may still read this CTA's lines
 }
 
 }  // namespace plane

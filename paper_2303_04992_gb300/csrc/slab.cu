@@ -79,7 +79,7 @@ void launch_nb(int which, const slab::SlabArgs<MAXB>& args, const SlabCg& t, int
       break;
     case 1:
       if constexpr (plane::Shape<N>::CL > 1)
-        slab::k_cg_terms_cl<N, MAXB><<<dim3(2 * 3 * N, nrun), plane::Shape<N>::THREADS,
+        slab::k_cg_terms_cl<N, MAXB><<<dim3(plane::Shape<N>::CL * 3 * N, nrun), plane::Shape<N>::THREADS,
                                        plane::Smem<N, float>::bytes, st>>>(args, t.tw, t.qN, t.s2, t.inv_mu);
       else
         slab::k_cg_terms<N, MAXB><<<dim3(3 * N, nrun), plane::Shape<N>::THREADS, plane::Smem<N, float>::bytes, st>>>(

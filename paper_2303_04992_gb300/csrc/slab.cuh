@@ -77,8 +77,9 @@ struct ZShape {
   static constexpr int SUMD = 4 * PARTS, BLOCK_SUMS = SUMD + BLOCKS;
   static constexpr int TICKETS = BLOCK_SUMS + (GROUP > 1 ? 4 * BLOCKS : 0);
   static constexpr int REDUCE = TICKETS + (GROUP > 1 ? PARTS : 0);
-  // resident CTAs per SM asked of the compiler (64 registers; 100 at N = 96, 24 values per lane)
-  static constexpr int OCC = THREADS == 512 ? 2 : (THREADS == 256 ? 4 : (N == 96 ? 5 : 8));
+  // resident CTAs per SM asked of the compiler (64 registers; 100 at N = 96, 24 values per lane;
+  // 128 on the small grids, which have few CTAs)
+  static constexpr int OCC = THREADS == 512 ? 2 : (THREADS == 256 ? 4 : (N == 96 ? 5 : 4));
 };
 
 // Element (z mode k, column l) of a tile at k TILE + (l ^ tile_sw(k)): the lanes of
@@ -219,7 +220,7 @@ k_cg_zfwd(const __grid_constant__ SlabArgs<MAXB> args, const C2<float>* __restri
   const float* __restrict__ q = args.q[b] + e0;
   CgAcc<float> acc[1];
   C2<float> v[R];
-  constexpr int HALF = R / 2;   // loads in flight per array
+  constexpr int HALF = R > 8 ? R / 2 : R;   // loads in flight per array
   float a = 0.f, beta = 0.f;
   bool stop = false;
 #pragma unroll
@@ -341,14 +342,15 @@ k_cg_terms(const __grid_constant__ SlabArgs<MAXB> args, const C2<float>* __restr
            const C2<float>* __restrict__ qg, const float* __restrict__ s2g, float inv_mu) {
   terms_body<N, MAXB>(args, blockIdx.x, 0, twg, qg, s2g, inv_mu);
 }
-// The same with a plane on a cluster of two CTAs (N = 256): 270 us, bound by
-// issue and shared memory with its 16 warps per SM; the five one-axis stages it
-// replaces took 1.16 ms of a staged CG iteration of 1.32 ms (now 0.47 ms).
+// The same with a plane on a cluster (N = 256): 235 us as four CTAs of 256 threads,
+// two clusters' CTAs per SM (272 us as two CTAs of 512), bound by issue and shared
+// memory; the five one-axis stages it replaces took 1.16 ms of a staged CG
+// iteration of 1.32 ms (now 0.42 ms).
 template <int N, int MAXB>
-__global__ void __cluster_dims__(2, 1, 1) __launch_bounds__(plane::Shape<N>::THREADS, 1)
+__global__ void __cluster_dims__(plane::Shape<N>::CL, 1, 1) __launch_bounds__(plane::Shape<N>::THREADS, 2)
 k_cg_terms_cl(const __grid_constant__ SlabArgs<MAXB> args, const C2<float>* __restrict__ twg,
               const C2<float>* __restrict__ qg, const float* __restrict__ s2g, float inv_mu) {
-  terms_body<N, MAXB>(args, blockIdx.x / 2, blockIdx.x % 2, twg, qg, s2g, inv_mu);
+  terms_body<N, MAXB>(args, blockIdx.x / plane::Shape<N>::CL, blockIdx.x % plane::Shape<N>::CL, twg, qg, s2g, inv_mu);
 }
 
 // q = DST-III_z (W1 + W2) + DCT-III_z W3 + cdiag d + rank1 sumd; the blocks' sums of
