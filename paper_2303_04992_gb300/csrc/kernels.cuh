@@ -9,6 +9,7 @@
 
 #include "cg_common.cuh"
 #include "fastcvt.h"
+#include "fixsum.h"
 
 namespace kfbim {
 
@@ -51,6 +52,13 @@ struct GridIx {
       k = (int)(q / N);
       j = (int)(q - (int64_t)k * N);
     }
+  }
+  __device__ __forceinline__ void unflat32(int x, int& i, int& j, int& k) const {
+    const unsigned q = lg >= 0 ? (unsigned)x >> lg : (unsigned)x / (unsigned)N;
+    const unsigned z = lg >= 0 ? q >> lg : q / (unsigned)N;
+    i = x - (int)q * N;
+    j = (int)(q - z * N);
+    k = (int)z;
   }
 };
 
@@ -244,68 +252,75 @@ __global__ void k_f_minus_gp(const double* __restrict__ f, const double* __restr
 // (Stokes: c = 0; Navier: the mean is 0 and c = 1/(lambda + mu)), and its norm
 // r2 = |rf|^2 + |rg|^2 for the refinement's stopping test (compensated FP32 squares
 // of the values rounded to FP32: about 1e-7 relative), which a pass of its own over
-// the stored residual took 17 us for at N = 128.
-__global__ void k_mac_residual(const double* __restrict__ f, const double* __restrict__ g,
-                               const double* __restrict__ gmean, const double* __restrict__ u,
-                               const double* __restrict__ p, GridIx gx, double h, double mu, double cpen,
-                               double* __restrict__ rf, double* __restrict__ rg, double* __restrict__ partial,
-                               unsigned int* ticket, double* __restrict__ r2) {
-  __shared__ float2 sh[32];
+// the stored residual took 17 us for at N = 128.  Bound by the FP64
+// pipe (two lanes per SM and cycle) at seven to nine operations per value, 180 us at
+// N = 128: the velocities' neighbour sums are 64-bit integer sums (fixsum.h), closer
+// than FP64 additions, and leave it three per value, while the divergence stays on
+// it (all four fields in integers: 121 us, bound by their instructions).  A warp
+// takes the four fields of its points in turn and its neighbours begin with other
+// ones, so that both pipes stay busy: 108 us, and 0.82 ms for 1.32 ms at N = 256.
+constexpr int MAC_OCC = 4;
+inline int mac_blocks(int64_t n3) {   // one wave
+  return (int)std::min<int64_t>((n3 + RED_THREADS - 1) / RED_THREADS, 152 * MAC_OCC);
+}
+template <int C>
+__device__ __forceinline__ double mac_row(const double* __restrict__ f, const double* __restrict__ g, double gm,
+                                          const double* __restrict__ u, const double* __restrict__ p, int N, int N3,
+                                          int x, const int (&id)[3], double ih, double c_lap, double cpen) {
+  const int st[3] = {1, N, N * N};
+  if constexpr (C < 3) {
+    if (id[C] == 0) return 0.0;
+    const uint64_t* uc = reinterpret_cast<const uint64_t*>(u) + (int64_t)C * N3 + x;
+    const uint64_t u0 = uc[0], ghost = u0 ^ 0x8000000000000000ull;
+    uint64_t lo[3], hi[3];
+    int E = max(kFixMin, fix_exp(u0));
+#pragma unroll
+    for (int b = 0; b < 3; ++b) {
+      // along the field's own axis the walls hold zeros, along the others the wall's
+      // ghost is minus the first interior value
+      lo[b] = id[b] >= (b == C ? 2 : 1) ? uc[-st[b]] : (b == C ? 0ull : ghost);
+      hi[b] = id[b] + 1 <= N - 1 ? uc[st[b]] : (b == C ? 0ull : ghost);
+      E = max(E, max(fix_exp(lo[b]), fix_exp(hi[b])));
+    }
+    const double rest = fma(-ih, p[x] - p[x - st[C]], f[(int64_t)C * N3 + x]);
+    int64_t sum = -6 * fix_of(u0, E);
+#pragma unroll
+    for (int b = 0; b < 3; ++b) sum += fix_of(lo[b], E) + fix_of(hi[b], E);
+    return fma(-c_lap, fix_value(sum, E), rest);   // f - dp / h - c_lap (sum - 6 u0)
+  } else {
+    double d[3];
+#pragma unroll
+    for (int b = 0; b < 3; ++b) {
+      const double* ub = u + (int64_t)b * N3 + x;
+      const double lo = id[b] >= 1 ? ub[0] : 0.0, hi = id[b] + 1 <= N - 1 ? ub[st[b]] : 0.0;
+      d[b] = hi - lo;
+    }
+    return fma(-ih, (d[0] + d[1]) + d[2], fma(-cpen, p[x], g[x] - gm));
+  }
+}
+
+__global__ void __launch_bounds__(RED_THREADS, MAC_OCC)
+k_mac_residual(const double* __restrict__ f, const double* __restrict__ g, const double* __restrict__ gmean,
+               const double* __restrict__ u, const double* __restrict__ p, GridIx gx, double h, double mu, double cpen,
+               double* __restrict__ rf, double* __restrict__ rg, double* __restrict__ partial,
+               unsigned int* __restrict__ ticket, double* __restrict__ r2) {
+  __shared__ float2 sh[RED_THREADS / 32];
   CgAcc<float> acc[1];
-  const int N = gx.N;
-  const int64_t N3 = gx.n3();
-  const double ih = 1.0 / h, c_lap = -mu / (h * h);
-  const double gm = gmean[0];
-  // FP64 throughput is the bound here (a small fraction of the FP32 rate on
-  // this GPU): the six neighbours are summed first and scaled once
-  for (int64_t e = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; e < 4 * N3;
-       e += (int64_t)gridDim.x * blockDim.x) {
-    int64_t x;
-    const int c = gx.field(e, x);
+  const int N = gx.N, N3 = (int)gx.n3();
+  const double ih = 1.0 / h, c_lap = -mu / (h * h), gm = gmean[0];
+  const int first = (threadIdx.x >> 5) + (threadIdx.x >> 7) * 2;
+  for (int x = blockIdx.x * blockDim.x + threadIdx.x; x < N3; x += gridDim.x * blockDim.x) {
     int id[3];
-    gx.unflat(x, id[0], id[1], id[2]);
-    if (c < 3) {
-      const int nrm = c == 0 ? id[0] : (c == 1 ? id[1] : id[2]);
-      if (nrm == 0) { rf[e] = 0.0; continue; }
-      const double* uc = u + (int64_t)c * N3;
-      const double u0 = uc[x];
-      double pair[3];
-#pragma unroll
-      for (int b = 0; b < 3; ++b) {
-        const int64_t st = gx.stride(b);
-        const int ib = b == 0 ? id[0] : (b == 1 ? id[1] : id[2]);
-        double um, up;
-        if (b == c) {
-          um = (ib - 1 >= 1) ? uc[x - st] : 0.0;
-          up = (ib + 1 <= N - 1) ? uc[x + st] : 0.0;
-        } else {
-          um = (ib > 0) ? uc[x - st] : -u0;
-          up = (ib < N - 1) ? uc[x + st] : -u0;
-        }
-        pair[b] = up + um;
-      }
-      // nine FP64 operations per value: five adds for the neighbours, the
-      // centre by one FMA, the pressure difference and two FMAs for
-      // rf = f - dp / h - c_lap (sum - 6 u0)
-      const double lap = fma(-6.0, u0, (pair[0] + pair[1]) + pair[2]);
-      const double dp = p[x] - p[x - gx.stride(c)];
-      const double v = fma(-c_lap, lap, fma(-ih, dp, f[e]));
-      rf[e] = v;
-      const float vf = f64_to_f32(v);
-      acc[0].add_prod(vf, vf);
-    } else {
-      double dif[3];
-#pragma unroll
-      for (int b = 0; b < 3; ++b) {
-        const int64_t st = gx.stride(b);
-        const int ib = b == 0 ? id[0] : (b == 1 ? id[1] : id[2]);
-        const double* ub = u + (int64_t)b * N3;
-        const double lo = (ib >= 1) ? ub[x] : 0.0;
-        const double hi = (ib + 1 <= N - 1) ? ub[x + st] : 0.0;
-        dif[b] = hi - lo;
-      }
-      const double v = fma(-ih, (dif[0] + dif[1]) + dif[2], fma(-cpen, p[x], g[x] - gm));
-      rg[x] = v;
+    gx.unflat32(x, id[0], id[1], id[2]);
+#pragma unroll 1
+    for (int it = 0; it < 4; ++it) {
+      const int c = (first + it) & 3;
+      double v;
+      if (c == 0) v = mac_row<0>(f, g, gm, u, p, N, N3, x, id, ih, c_lap, cpen);
+      else if (c == 1) v = mac_row<1>(f, g, gm, u, p, N, N3, x, id, ih, c_lap, cpen);
+      else if (c == 2) v = mac_row<2>(f, g, gm, u, p, N, N3, x, id, ih, c_lap, cpen);
+      else v = mac_row<3>(f, g, gm, u, p, N, N3, x, id, ih, c_lap, cpen);
+      (c < 3 ? rf + (int64_t)c * N3 : rg)[x] = v;
       const float vf = f64_to_f32(v);
       acc[0].add_prod(vf, vf);
     }

@@ -874,7 +874,7 @@ int grid_solve_mixed(kfbim_ctx* c, cudaStream_t s, bool need_p) {
     recover_velocity(c, c->fu, c->u, w.T6, first, s);
     if (!c->fp32_only) {   // FP32: one correction solve, no FP64 residual
       const int at = prof_begin(c, s);
-      k_mac_residual<<<grid_for(4 * N3), 256, 0, s>>>(f, g, gmean, c->u, c->p, c->gix(), c->h, c->mu, c->cpen, resf, resg,
+      k_mac_residual<<<mac_blocks(N3), RED_THREADS, 0, s>>>(f, g, gmean, c->u, c->p, c->gix(), c->h, c->mu, c->cpen, resf, resg,
                                                        c->partial, &c->gs->ticket, &c->gs->r2); ++g_launches;
       // reads f, g, u, p (8 N^3 doubles), writes rf, rg (4 N^3)
       prof_end(c, s, at, KFBIM_KCLASS_MAC_RESIDUAL, 1, 12.0 * N3 * sizeof(double));
@@ -1989,7 +1989,7 @@ void grid_solve_batch(kfbim_ctx* c, const std::vector<int>& act, cudaStream_t s,
     if (c->fp32_only) break;   // FP32: one correction solve, no FP64 residual
     for (int b : live) {
       const kfbim_ctx::Slot& w = c->bs[b];
-      k_mac_residual<<<grid_for(4 * N3), 256, 0, s>>>(w.rhs, w.rhs + 3 * N3, c->bscal + 8 * b, w.u, w.p,
+      k_mac_residual<<<mac_blocks(N3), RED_THREADS, 0, s>>>(w.rhs, w.rhs + 3 * N3, c->bscal + 8 * b, w.u, w.p,
                                                       c->gix(), c->h, c->mu, c->cpen, w.res, w.res + 3 * N3, c->partial,
                                                       ticket(b), c->bscal + 8 * b + 2);
       ++g_launches;
