@@ -211,7 +211,7 @@ def measured_peaks():
     return 6800.0, "fallback"
 
 
-PASS_SOURCES = {"fft": ("transforms.cuh", "plane.cuh", "lines.cuh"),
+PASS_SOURCES = {"fft": ("transforms.cuh", "plane.cuh", "lines.cuh", "overlap.cuh"),
                  "tensor": ("transforms.cuh", "transforms2.cuh", "tc_pass.cuh")}
 
 
@@ -260,7 +260,7 @@ def ncu_traffic_slab(workload):
         return None
     txt = open(p).read()
     h = hashlib.sha256()
-    for f in ("slab.cuh", "cg_common.cuh", "plane.cuh"):
+    for f in ("slab.cuh", "cg_common.cuh", "plane.cuh", "overlap.cuh"):
         h.update(open(os.path.join(ROOT, "paper_2303_04992_gb300", "csrc", f), "rb").read())
     m = re.search(r"kernel_source_sha256_12:\s*([0-9a-f]+)", txt)
     t = re.search(r"dram_bytes_per_launch:\s*([0-9.eE+]+)", txt)

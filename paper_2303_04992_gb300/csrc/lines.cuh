@@ -28,6 +28,7 @@
 #include <stdint.h>
 
 #include "fastcvt.h"
+#include "overlap.cuh"
 #include "plane.cuh"
 #include "transforms.cuh"
 
@@ -223,7 +224,6 @@ k_lines(const __grid_constant__ Jobs<Tin, Tout, MAXJ> jobs, T h, T inv_mu, const
   using L = LShape<N, T>;
   constexpr int M = S::M, R = S::R, H = S::H;
   const Job<Tin, Tout>& job = jobs.j[blockIdx.y];
-  if (job.skip && *job.skip) return;
   extern __shared__ __align__(16) unsigned char sml[];
   C2<T>* P = reinterpret_cast<C2<T>*>(sml);
   C2<T>* tws = P + L::TEAMS * N;
@@ -233,6 +233,9 @@ k_lines(const __grid_constant__ Jobs<Tin, Tout, MAXJ> jobs, T h, T inv_mu, const
     if (op_fwd1(OP) || op_fwd2(OP) || !pairs) tws[e] = twg[2 * (e / M) * (e % M)];
     if ((op_inv1(OP) || op_inv2(OP)) && pairs) twr[e] = twg[2 * (e / R) * (e % R)];
   }
+  overlap_wait();
+  overlap_trigger();
+  if (job.skip && *job.skip) return;
   __syncthreads();
   const int t = threadIdx.x / M, m = threadIdx.x % M, lane = threadIdx.x & 31;
   const int partner = (lane & ~(M - 1)) | ((M - m) & (M - 1));

@@ -13,8 +13,8 @@ cudaError_t lines_launch_op(const lines::Jobs<Tin, Tout, MAXJ>& jobs, int njobs,
   auto kern = lines::k_lines<Tin, T, Tout, N, OP, MAXJ>;
   const cudaError_t e = raise_dynamic_smem(reinterpret_cast<const void*>(kern), L::bytes);
   if (e != cudaSuccess) return e;
-  kern<<<dim3((unsigned)L::BLOCKS, (unsigned)njobs), L::THREADS, L::bytes, s>>>(jobs, h, inv_mu, tw, qN, s2);
-  return cudaGetLastError();
+  return launch_overlapped(sizeof(T) == 4 && N <= 128, kern, dim3((unsigned)L::BLOCKS, (unsigned)njobs), L::THREADS, L::bytes, s, jobs, h, inv_mu,
+                           tw, qN, s2);
 }
 
 template <int N, typename Tin, typename T, typename Tout, int MAXJ>

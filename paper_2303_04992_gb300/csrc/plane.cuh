@@ -529,19 +529,13 @@ struct Smem {
   static constexpr size_t bytes = field + tables;
 };
 
-// One term on one plane: `in` and `out` are planes in the slab order (below;
-// they may be the same).  Where an axis takes DST-II
-// the field's odd nodes along it are negated in `in` and in `out`; `in` carries
-// instead the signs of `signs` (so that two terms can share an input).
-// az: the plane's 4 sin^2 along z; sc: 1 / (mu N^2).
+// The tables of term_plane behind the field in shared memory.
 // twg: exp(-pi i t / N), t < 2N; qg: exp(-pi i k / 2N); s2: 4 sin^2(pi a / 2N), a < N.
-// Called by all threads of the CTA (of every CTA of the cluster; rank: this one's).
 template <int N, typename T>
-__device__ __forceinline__ void term_plane(const T* in, T* out, const Term term, const Term signs, T az, T sc,
-                                           C2<T>* P, const C2<T>* __restrict__ twg, const C2<T>* __restrict__ qg,
-                                           const T* __restrict__ s2, int rank = 0) {
+__device__ __forceinline__ void term_tables(C2<T>* P, const C2<T>* __restrict__ twg, const C2<T>* __restrict__ qg,
+                                            const T* __restrict__ s2) {
   using S = Shape<N>;
-  constexpr int M = S::M, R = S::R, H = S::H;
+  constexpr int M = S::M, R = S::R;
   C2<T>* tws = P + Smem<N, T>::field / sizeof(C2<T>);   // FFT twiddles [s][m]
   C2<T>* twr = tws + N;                 // the same by [m][s]
   C2<T>* qh = twr + N;                  // q_k / 2, k < N/2
@@ -557,6 +551,25 @@ __device__ __forceinline__ void term_plane(const T* in, T* out, const Term term,
     cy[e] = conjg(twg[e]);
     sg[e] = s2[e];
   }
+}
+
+// One term on one plane: `in` and `out` are planes in the slab order (below;
+// they may be the same).  Where an axis takes DST-II
+// the field's odd nodes along it are negated in `in` and in `out`; `in` carries
+// instead the signs of `signs` (so that two terms can share an input).
+// az: the plane's 4 sin^2 along z; sc: 1 / (mu N^2).
+// P: Smem<N, T>, its tables filled (term_tables; a barrier follows here).
+// Called by all threads of the CTA (of every CTA of the cluster; rank: this one's).
+template <int N, typename T>
+__device__ __forceinline__ void term_plane(const T* in, T* out, const Term term, const Term signs, T az, T sc,
+                                           C2<T>* P, int rank = 0) {
+  using S = Shape<N>;
+  constexpr int M = S::M, R = S::R, H = S::H;
+  C2<T>* tws = P + Smem<N, T>::field / sizeof(C2<T>);   // FFT twiddles [s][m]
+  C2<T>* twr = tws + N;                 // the same by [m][s]
+  C2<T>* qh = twr + N;                  // q_k / 2, k < N/2
+  C2<T>* cy = qh + S::LINES;            // exp(i pi k / N), k < N/2
+  T* sg = reinterpret_cast<T*>(cy + S::LINES);   // 4 sin^2(pi k / 2N), k < N/2
   const int t = threadIdx.x / M, m = threadIdx.x % M;
   const int lane = threadIdx.x & 31;
   const int partner = (lane & ~(M - 1)) | ((M - m) & (M - 1));

@@ -66,6 +66,11 @@ slab::SlabArgs<MAXB> make_args(const SlabCg* runs, int nrun) {
   return a;
 }
 
+// Launches that overlap the kernel before them: where the measurements in overlap.cuh
+// show a gain.
+template <int N>
+constexpr bool kOverlap = N <= 128;
+
 // Kernel `which` of the iteration: 0 k_cg_zfwd, 1 k_cg_terms, 2 k_cg_zinv; 3 is
 // k_cg_fin, the end of a run.
 template <int N, int MAXB>
@@ -79,14 +84,16 @@ void launch_nb(int which, const slab::SlabArgs<MAXB>& args, const SlabCg& t, int
       break;
     case 1:
       if constexpr (plane::Shape<N>::CL > 1)
-        slab::k_cg_terms_cl<N, MAXB><<<dim3(plane::Shape<N>::CL * 3 * N, nrun), plane::Shape<N>::THREADS,
-                                       plane::Smem<N, float>::bytes, st>>>(args, t.tw, t.qN, t.s2, t.inv_mu);
+        (void)launch_overlapped(kOverlap<N>, slab::k_cg_terms_cl<N, MAXB>, dim3(plane::Shape<N>::CL * 3 * N, nrun),
+                                plane::Shape<N>::THREADS, plane::Smem<N, float>::bytes, st, args, t.tw, t.qN, t.s2,
+                                t.inv_mu);
       else
-        slab::k_cg_terms<N, MAXB><<<dim3(3 * N, nrun), plane::Shape<N>::THREADS, plane::Smem<N, float>::bytes, st>>>(
-            args, t.tw, t.qN, t.s2, t.inv_mu);
+        (void)launch_overlapped(kOverlap<N>, slab::k_cg_terms<N, MAXB>, dim3(3 * N, nrun), plane::Shape<N>::THREADS,
+                                plane::Smem<N, float>::bytes, st, args, t.tw, t.qN, t.s2, t.inv_mu);
       break;
     case 2:
-      slab::k_cg_zinv<N, MAXB><<<dim3(Z::BLOCKS, nrun), Z::THREADS, Z::bytes, st>>>(args, t.tw, t.qN);
+      (void)launch_overlapped(kOverlap<N>, slab::k_cg_zinv<N, MAXB>, dim3(Z::BLOCKS, nrun), Z::THREADS, Z::bytes, st, args, t.tw,
+                              t.qN);
       break;
     default:
       slab::k_cg_fin<N, MAXB><<<dim3(V::BLOCKS, nrun), V::THREADS, V::bytes, st>>>(args);

@@ -52,6 +52,7 @@
 
 #include "cg_common.cuh"
 #include "fastcvt.h"
+#include "overlap.cuh"
 #include "plane.cuh"
 
 namespace kfbim {
@@ -195,6 +196,7 @@ k_cg_zfwd(const __grid_constant__ SlabArgs<MAXB> args, const C2<float>* __restri
   __shared__ CgStep step;
   const int b = blockIdx.y;
   CGScalars* s = args.s[b];
+  overlap_trigger();
   // idle: done before this iteration (set by k_cg_start and k_cg_zinv; `done` is
   // written by this kernel and may be seen half-way)
   if (s->idle) {
@@ -322,8 +324,11 @@ __device__ __forceinline__ void terms_body(const SlabArgs<MAXB>& args, int unit,
                                            const C2<float>* __restrict__ twg, const C2<float>* __restrict__ qg,
                                            const float* __restrict__ s2g, float inv_mu) {
   const int b = blockIdx.y;
-  if (args.s[b]->done) return;
   extern __shared__ __align__(16) unsigned char smx[];
+  plane::term_tables<N, float>(reinterpret_cast<C2<float>*>(smx), twg, qg, s2g);
+  overlap_wait();
+  overlap_trigger();
+  if (args.s[b]->done) return;
   if (unit == 3 * N - 1 && rank == 0)
     merge_sumd<N, plane::Shape<N>::THREADS>(reinterpret_cast<const float2*>(args.partial[b]) + ZShape<N>::SUMD, args.s[b]);
   const int term = unit % 3, k = unit / 3;
@@ -333,8 +338,7 @@ __device__ __forceinline__ void terms_body(const SlabArgs<MAXB>& args, int unit,
   // 4 sin^2 along z: DCT-II mode k (term 3), DST-II mode N - 1 - k (terms 1, 2)
   const float az = term == 2 ? s2g[k] : s2g[2 * N - 1 - k];
   plane::term_plane<N, float>(in, out, plane::term_of(term), plane::term_of(term == 2 ? 2 : 0), az,
-                              inv_mu * (1.0f / ((float)N * N)), reinterpret_cast<C2<float>*>(smx), twg, qg, s2g,
-                              rank);
+                              inv_mu * (1.0f / ((float)N * N)), reinterpret_cast<C2<float>*>(smx), rank);
 }
 template <int N, int MAXB>
 __global__ void __launch_bounds__(plane::Shape<N>::THREADS, 2)
@@ -365,10 +369,6 @@ k_cg_zinv(const __grid_constant__ SlabArgs<MAXB> args, const C2<float>* __restri
   __shared__ float2 sh[4 * 32];
   const int b = blockIdx.y;
   CGScalars* s = args.s[b];
-  if (s->done) {
-    if (blockIdx.x == 0 && threadIdx.x == 0) s->idle = 1;
-    return;
-  }
   extern __shared__ __align__(16) unsigned char smi[];
   C2<float>* P = reinterpret_cast<C2<float>*>(smi);
   float* O3 = reinterpret_cast<float*>(smi);
@@ -376,6 +376,12 @@ k_cg_zinv(const __grid_constant__ SlabArgs<MAXB> args, const C2<float>* __restri
   C2<float>* tws = P + N * TILE;
   C2<float>* twr = tws + N;
   C2<float>* qN = twr + N;
+  z_tables<N>(tws, twr, qN, twg, qg);
+  overlap_wait();
+  if (s->done) {
+    if (blockIdx.x == 0 && threadIdx.x == 0) s->idle = 1;
+    return;
+  }
   const int t = threadIdx.x / M, m = threadIdx.x % M, lane = threadIdx.x & 31;
   const int partner = (lane & ~(M - 1)) | ((M - m) & (M - 1));
   const int col0 = blockIdx.x * TILE;
@@ -407,7 +413,6 @@ k_cg_zinv(const __grid_constant__ SlabArgs<MAXB> args, const C2<float>* __restri
       *reinterpret_cast<float4*>(O3 + at) = make_float4(s3 * f3[j].x, s3 * f3[j].y, s3 * f3[j].z, s3 * f3[j].w);
     }
   }
-  z_tables<N>(tws, twr, qN, twg, qg);
   __syncthreads();
   // both inverse transforms of a column in one FFT: conj Z_k = q conj(A + i B),
   // conj Z_(N-k) = conj(q) (A - i B) with A = X_k - i X_(N-k) of the DCT-III input,
