@@ -253,7 +253,7 @@ SLAB_CLASSES = ("cg_zfwd", "cg_xy", "cg_zinv", "cg_update")
 
 
 def ncu_traffic_slab(workload):
-    """DRAM bytes per launch of k_cg_xy from the committed ncu summary, if it
+    """DRAM bytes per launch of k_cg_terms from the committed ncu summary, if it
     was taken on the current slab source (else None)."""
     p = os.path.join(ROOT, "profiles", "cg_xy_%s.md" % workload)
     if not os.path.exists(p):
@@ -272,7 +272,7 @@ def ncu_traffic_slab(workload):
 def roofline_line(kernels, kprof, N3, cg_iters, args, peak, peak_kind):
     """The roofline object of the bench line.  Dominant kernel: the one with
     the largest share of the step.  For the slab CG the algorithmic bytes per
-    launch are the byte model's figure for the work the kernel does: k_cg_xy
+    launch are the byte model's figure for the work the kernel does: k_cg_terms
     does the middle pass of the Schur apply on all three terms (6 N^3 b); the
     whole CG iteration (three kernels, plus each run's closing update spread
     over its iterations) is reported beside it against 27 N^3 b."""
@@ -497,7 +497,7 @@ def c4_grids_leg(args, flush, stream, dev):
         st = s.last_stats
         out["star%d" % n] = {"instances": B, "solves_per_s": round(B * 1e3 / ms, 4), "ms_per_batch": round(ms, 2),
                              "gmres_iters_max": max(x["gmres_iters"] for x in st),
-                             "slab_cg": n in (32, 64, 128)}
+                             "slab_cg": n in (32, 64, 96, 128, 256)}
         s.close()
     return out
 

@@ -380,8 +380,8 @@ typedef enum {
                                        z transforms (9 N^3 floats) */
   KFBIM_KCLASS_CG_XY = 3,           /* slab CG: xy planes of the three terms (6 N^3 floats) */
   KFBIM_KCLASS_CG_ZINV = 4,         /* slab CG: inverse z transforms, d.q, r.r, r.q, q.q (6 N^3 floats) */
-  KFBIM_KCLASS_CG_UPDATE = 5,       /* slab CG: the x update still pending when a run stops
-                                       (3 N^3 floats, once per CG run) */
+  KFBIM_KCLASS_CG_UPDATE = 5,       /* slab CG: x back in natural order when a run stops
+                                       (2 N^3 floats, once per CG run) */
   KFBIM_KCLASS_CG_VECTOR = 6,       /* staged CG: the three vector kernels (14 N^3 values) */
   KFBIM_KCLASS_MAC_RESIDUAL = 7,    /* MIXED refinement: FP64 MAC residual (12 N^3 doubles) */
   KFBIM_KCLASS_JUMPS = 8,           /* jump evaluation (fit rows, jump maps, jumps) */
