@@ -353,15 +353,15 @@ void launch_jobs(kfbim_ctx* c, const Job* list, int nj, cudaStream_t s, const in
             reinterpret_cast<uintptr_t>(j.out) % (2 * sizeof(Tout)) == 0;
   }
   const int op = line_op(list[0].t0, list[0].t1);
-  const T h = T(c->h), im = T(1.0 / c->mu);
+  const lines::Scales<T> sc{T(1.0 / c->mu), T(c->h * c->h / c->mu), T(-c->h / c->mu)};
   const auto *tw = Tw<T>::twc(c), *q = Tw<T>::q(c);
   const T* s2 = Tw<T>::s2(c);
   switch (c->N) {
-    case 256: CK((lines_launch<256, Tin, T, Tout, MAXJ>(op, jobs, nj, h, im, tw, q, s2, s))); break;
-    case 128: CK((lines_launch<128, Tin, T, Tout, MAXJ>(op, jobs, nj, h, im, tw, q, s2, s))); break;
-    case 96: CK((lines_launch<96, Tin, T, Tout, MAXJ>(op, jobs, nj, h, im, tw, q, s2, s))); break;
-    case 64: CK((lines_launch<64, Tin, T, Tout, MAXJ>(op, jobs, nj, h, im, tw, q, s2, s))); break;
-    default: CK((lines_launch<32, Tin, T, Tout, MAXJ>(op, jobs, nj, h, im, tw, q, s2, s)));
+    case 256: CK((lines_launch<256, Tin, T, Tout, MAXJ>(op, jobs, nj, sc, tw, q, s2, s))); break;
+    case 128: CK((lines_launch<128, Tin, T, Tout, MAXJ>(op, jobs, nj, sc, tw, q, s2, s))); break;
+    case 96: CK((lines_launch<96, Tin, T, Tout, MAXJ>(op, jobs, nj, sc, tw, q, s2, s))); break;
+    case 64: CK((lines_launch<64, Tin, T, Tout, MAXJ>(op, jobs, nj, sc, tw, q, s2, s))); break;
+    default: CK((lines_launch<32, Tin, T, Tout, MAXJ>(op, jobs, nj, sc, tw, q, s2, s)));
   }
   ++g_launches;
 }

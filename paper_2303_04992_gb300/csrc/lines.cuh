@@ -138,6 +138,13 @@ __device__ __forceinline__ plane::YSlots<N> slots(int t) {
   return {t * N, M == 16 ? 0 : (M == 8 ? (t & 1) << 3 : (t & 3) << 2)};
 }
 
+// The constant factors of the spectral weights, each rounded once from FP64: 1 / mu
+// (W_SCHUR), h^2 / mu (W_POISSON), -h / mu (W_RHS).
+template <typename T>
+struct Scales {
+  T schur, poisson, rhs;
+};
+
 // Weights of a pass (the factors of spectral_weight2): 4 sin^2 of the line's two
 // other modes, of the mode along the pass's axis, and the numerator.
 template <typename T, int N>
@@ -148,13 +155,13 @@ struct Weights {
   int kind;     // 0: the pass's axis takes DCT / DST-I modes, 1: DST-II modes
   int wmode;
   bool own;     // the weight's component axis is the pass's axis
-  T h, inv_mu;
+  Scales<T> sc;
   // numerator for component mode value v = 4 sin^2 (zero for mode 0 of a face basis)
   __device__ __forceinline__ T numer(T v, bool zero) const {
-    if (wmode == W_SCHUR) return v * inv_mu;
+    if (wmode == W_SCHUR) return v * sc.schur;
     if (zero) return T(0);
-    if (wmode == W_POISSON) return h * h * inv_mu;
-    return -h * inv_mu * sqrt(v);   // -2 h sin(a), v = 4 sin^2(a)
+    if (wmode == W_POISSON) return sc.poisson;
+    return sc.rhs * sqrt(v);   // -2 h sin(a), v = 4 sin^2(a)
   }
   __device__ __forceinline__ T at(int a, T& den) const {
     const T v = s2[kind * N + a];
@@ -218,7 +225,7 @@ __device__ __forceinline__ void tile_store(const T* tile, Tout* out, int64_t es,
 
 template <typename Tin, typename T, typename Tout, int N, int OP, int MAXJ>
 __global__ void __launch_bounds__((LShape<N, T>::THREADS), (LShape<N, T>::occ(OP)))
-k_lines(const __grid_constant__ Jobs<Tin, Tout, MAXJ> jobs, T h, T inv_mu, const C2<T>* __restrict__ twg,
+k_lines(const __grid_constant__ Jobs<Tin, Tout, MAXJ> jobs, const Scales<T> scales, const C2<T>* __restrict__ twg,
         const C2<T>* __restrict__ qg, const T* __restrict__ s2) {
   using S = plane::Shape<N>;
   using L = LShape<N, T>;
@@ -356,8 +363,7 @@ k_lines(const __grid_constant__ Jobs<Tin, Tout, MAXJ> jobs, T h, T inv_mu, const
   auto weights = [&](int ln) {
     Weights<T, N> w;
     w.s2 = s2;
-    w.h = h;
-    w.inv_mu = inv_mu;
+    w.sc = scales;
     w.wmode = job.wmode;
     w.own = job.wc == axis;
     w.kind = w.own ? 0 : 1;
@@ -369,17 +375,14 @@ k_lines(const __grid_constant__ Jobs<Tin, Tout, MAXJ> jobs, T h, T inv_mu, const
     w.num = w.own ? T(0) : (job.wc == ax1 ? w.numer(v1, lo == 0) : w.numer(v2, hi == 0));
     return w;
   };
-  // a mode pair (array indices ka, kb) times its weights; FP64: one reciprocal for the two
-  // (products of 4 sin^2 sums, 1e-4 .. 12 each)
+  // a mode pair (array indices ka, kb) times its weights, the reciprocals correctly rounded.
+  // FP64: one reciprocal of the product of the two denominators is 1 % of an FP64 matvec
+  // faster and adds 3 % to the error of a Poisson solve (N = 64: 5.96e-16 against 5.80e-16)
   auto weigh = [&](const Weights<T, N>& W, int ka, int kb, C2<T>& f) {
     T d1, d2;
     const T n1 = W.at(ka, d1), n2 = W.at(kb, d2);
-    if constexpr (sizeof(T) == 4) {
-      f = {f.x * (n1 * plane::rcp(d1)), f.y * (n2 * plane::rcp(d2))};
-    } else {
-      const T r = T(1) / (d1 * d2);
-      f = {f.x * (n1 * (d2 * r)), f.y * (n2 * (d1 * r))};
-    }
+    if constexpr (sizeof(T) == 4) f = {f.x * (n1 * __frcp_rn(d1)), f.y * (n2 * __frcp_rn(d2))};
+    else f = {f.x * (n1 * __drcp_rn(d1)), f.y * (n2 * __drcp_rn(d2))};
   };
   auto store2 = [&](const C2<T>(&v)[R]) {
     // v holds the conjugate: line A in the real, minus line B in the imaginary part; element

@@ -25,7 +25,7 @@ cudaError_t raise_dynamic_smem(const void* kern, size_t bytes);
 // cudaErrorInvalidValue for a combination that has no kernel (plain DST-I passes
 // of a batch).
 template <int N, typename Tin, typename T, typename Tout, int MAXJ>
-cudaError_t lines_launch(int op, const lines::Jobs<Tin, Tout, MAXJ>& jobs, int njobs, T h, T inv_mu,
+cudaError_t lines_launch(int op, const lines::Jobs<Tin, Tout, MAXJ>& jobs, int njobs, const lines::Scales<T>& sc,
                          const C2<T>* tw, const C2<T>* qN, const T* s2, cudaStream_t s);
 
 }  // namespace kfbim

@@ -7,21 +7,21 @@
 namespace kfbim {
 
 template <int N, int OP, typename Tin, typename T, typename Tout, int MAXJ>
-cudaError_t lines_launch_op(const lines::Jobs<Tin, Tout, MAXJ>& jobs, int njobs, T h, T inv_mu, const C2<T>* tw,
-                            const C2<T>* qN, const T* s2, cudaStream_t s) {
+cudaError_t lines_launch_op(const lines::Jobs<Tin, Tout, MAXJ>& jobs, int njobs, const lines::Scales<T>& sc,
+                            const C2<T>* tw, const C2<T>* qN, const T* s2, cudaStream_t s) {
   using L = lines::LShape<N, T>;
   auto kern = lines::k_lines<Tin, T, Tout, N, OP, MAXJ>;
   const cudaError_t e = raise_dynamic_smem(reinterpret_cast<const void*>(kern), L::bytes);
   if (e != cudaSuccess) return e;
-  return launch_overlapped(sizeof(T) == 4 && N <= 128, kern, dim3((unsigned)L::BLOCKS, (unsigned)njobs), L::THREADS, L::bytes, s, jobs, h, inv_mu,
-                           tw, qN, s2);
+  return launch_overlapped(sizeof(T) == 4 && N <= 128, kern, dim3((unsigned)L::BLOCKS, (unsigned)njobs), L::THREADS,
+                           L::bytes, s, jobs, sc, tw, qN, s2);
 }
 
 template <int N, typename Tin, typename T, typename Tout, int MAXJ>
-cudaError_t lines_launch(int op, const lines::Jobs<Tin, Tout, MAXJ>& jobs, int njobs, T h, T inv_mu,
+cudaError_t lines_launch(int op, const lines::Jobs<Tin, Tout, MAXJ>& jobs, int njobs, const lines::Scales<T>& sc,
                          const C2<T>* tw, const C2<T>* qN, const T* s2, cudaStream_t s) {
 #define KFBIM_LINES_OP(OP) \
-  case OP: return lines_launch_op<N, OP, Tin, T, Tout, MAXJ>(jobs, njobs, h, inv_mu, tw, qN, s2, s)
+  case OP: return lines_launch_op<N, OP, Tin, T, Tout, MAXJ>(jobs, njobs, sc, tw, qN, s2, s)
   if constexpr (sizeof(Tout) > sizeof(T)) {
     switch (op) {
       KFBIM_LINES_OP(lines::OP_I2);
@@ -57,8 +57,8 @@ cudaError_t lines_launch(int op, const lines::Jobs<Tin, Tout, MAXJ>& jobs, int n
 
 #define KFBIM_LINES_INSTANTIATE_ONE(N, TIN, T, TOUT, MAXJ)                                                    \
   template cudaError_t kfbim::lines_launch<N, TIN, T, TOUT, MAXJ>(                                            \
-      int, const kfbim::lines::Jobs<TIN, TOUT, MAXJ>&, int, T, T, const kfbim::C2<T>*, const kfbim::C2<T>*, \
-      const T*, cudaStream_t);
+      int, const kfbim::lines::Jobs<TIN, TOUT, MAXJ>&, int, const kfbim::lines::Scales<T>&,                 \
+      const kfbim::C2<T>*, const kfbim::C2<T>*, const T*, cudaStream_t);
 #define KFBIM_LINES_INSTANTIATE(N)                                                  \
   KFBIM_LINES_INSTANTIATE_ONE(N, double, double, double, kfbim::kLineJobs)          \
   KFBIM_LINES_INSTANTIATE_ONE(N, double, float, float, kfbim::kLineJobs)            \

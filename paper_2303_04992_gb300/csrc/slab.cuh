@@ -337,8 +337,11 @@ __device__ __forceinline__ void terms_body(const SlabArgs<MAXB>& args, int unit,
   float* out = (term == 0 ? args.w1[b] : (term == 1 ? args.w2[b] : args.z3[b])) + off;
   // 4 sin^2 along z: DCT-II mode k (term 3), DST-II mode N - 1 - k (terms 1, 2)
   const float az = term == 2 ? s2g[k] : s2g[2 * N - 1 - k];
+  // 1 / N per inverse transform, as the one-axis passes scale: at N = 96 the rounding of
+  // 1 / 96 offsets part of the FFT constants' (operator error 2.1e-7 with 1 / N^2 rounded once)
+  constexpr float invN = 1.0f / N;
   plane::term_plane<N, float>(in, out, plane::term_of(term), plane::term_of(term == 2 ? 2 : 0), az,
-                              inv_mu * (1.0f / ((float)N * N)), reinterpret_cast<C2<float>*>(smx), rank);
+                              inv_mu * (invN * invN), reinterpret_cast<C2<float>*>(smx), rank);
 }
 template <int N, int MAXB>
 __global__ void __launch_bounds__(plane::Shape<N>::THREADS, 2)
