@@ -366,7 +366,10 @@ __global__ void k_dot_partial(const Ta* __restrict__ x, const Tb* __restrict__ y
 // solve in one pass: gmean = mean(g) (0 unless `stokes`), ref2 = |f|^2 + |g - gmean|^2.
 // |f|^2 sums compensated FP32 squares of the values rounded to FP32 by integer
 // operations (about 1e-7 relative, without FP64 instructions per element); the
-// two moments of g are FP64.  The last block merges the blocks' parts in order.
+// two moments of g are FP64 and, where the mean is removed, those of g - g[0], so that
+// |g - gmean|^2 does not cancel where g is a large constant and a small rest (g is zero
+// away from the boundary, g[0] too: the shift then costs nothing).  The last block
+// merges the blocks' parts in order.
 constexpr int MOMENT_DOUBLES = 3;   // partial doubles per block
 __global__ void k_rhs_moments(const double* __restrict__ rhs, int64_t n3, int stokes, double* __restrict__ partial,
                               unsigned int* ticket, double* __restrict__ gmean, double* __restrict__ ref2) {
@@ -381,8 +384,9 @@ __global__ void k_rhs_moments(const double* __restrict__ rhs, int64_t n3, int st
     a[0].add_prod(v, v);
   }
   const double* __restrict__ g = rhs + 3 * n3;
+  const double g0 = stokes ? g[0] : 0.0;
   for (int64_t e = t0; e < n3; e += step) {
-    const double v = g[e];
+    const double v = g0 != 0.0 ? g[e] - g0 : g[e];
     s1 += v;
     s2 = fma(v, v, s2);
   }
@@ -414,7 +418,7 @@ __global__ void k_rhs_moments(const double* __restrict__ rhs, int64_t n3, int st
   s2 = block_sum<double>(s2, sh);
   if (threadIdx.x == 0) {
     const double m = stokes ? s1 / (double)n3 : 0.0;
-    *gmean = m;
+    *gmean = g0 + m;
     *ref2 = t[0].value() + fmax(s2 - m * s1, 0.0);
     *ticket = 0u;
   }
