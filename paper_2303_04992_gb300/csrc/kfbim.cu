@@ -27,6 +27,7 @@
 
 #include "internal.h"
 #include "kernels.cuh"
+#include "roots.h"
 #include "transforms.cuh"
 #include "transforms2.cuh"
 #include "lines.h"
@@ -1345,18 +1346,15 @@ void fill_tables(kfbim_ctx* c) {
   std::vector<C2<double>> tw(N), q(N);
   std::vector<C2<float>> tw32(N), q32(N);
   for (int k = 0; k < N; ++k) {
-    const double a = M_PI * (double)k / (double)N;
-    tw[k] = {std::cos(a), -std::sin(a)};
-    const double b = 0.5 * a;
-    q[k] = {std::cos(b), -std::sin(b)};
+    unit_root(k, N, &tw[k].x, &tw[k].y);
+    unit_root(k, 2 * N, &q[k].x, &q[k].y);
     tw32[k] = {(float)tw[k].x, (float)tw[k].y};
     q32[k] = {(float)q[k].x, (float)q[k].y};
   }
   std::vector<C2<double>> twc(2 * N);
   std::vector<C2<float>> twc32(2 * N);
   for (int k = 0; k < 2 * N; ++k) {
-    const double a = M_PI * (double)k / (double)N;
-    twc[k] = {std::cos(a), -std::sin(a)};
+    unit_root(k, N, &twc[k].x, &twc[k].y);
     twc32[k] = {(float)twc[k].x, (float)twc[k].y};
   }
   c->d_twc64 = upload(c, twc);
