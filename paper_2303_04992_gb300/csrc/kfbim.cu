@@ -767,14 +767,15 @@ int cg(kfbim_ctx* c, const T* b, const SlabRhs* rhs, const CgWs<T>& w, double to
     ++g_launches;
   }
   check_launch();
-  // the update a slab run left pending when it stopped
-  auto finish = [&] {
+  // the end of a slab run, with the update it left pending if the host stopped it
+  auto finish = [&](bool pending) {
     if constexpr (std::is_same<T, float>::value) {
       if (!slab) return;
       const int at = prof_begin(c, s);
       const SlabCg a = slab_run(c, w);
       g_launches += slab_cg_finish(&a, 1, s);
-      prof_end(c, s, at, KFBIM_KCLASS_CG_UPDATE, 1, (double)kSlabValues[3] * c->N3 * sizeof(float));
+      prof_end(c, s, at, KFBIM_KCLASS_CG_UPDATE, 1,
+               (double)(kSlabValues[3] + (pending ? 1 : 0)) * c->N3 * sizeof(float));
       check_launch();
     }
   };
@@ -782,13 +783,13 @@ int cg(kfbim_ctx* c, const T* b, const SlabRhs* rhs, const CgWs<T>& w, double to
   if (loop) CK(cudaGraphLaunch(exec, s));
   if (loop && deferred) {
     *deferred = true;
-    finish();
+    finish(false);
     return KFBIM_OK;
   }
   for (int launched = 0;; launched += kCgGraphIters) {
     const CGScalars h = read_grid_scalars(c, s).cg;
     if (loop || !std::isfinite(h.rr) || h.done || launched >= maxit) {
-      finish();
+      finish(!h.done && h.iters > 0);
       return cg_result(c, h, slot, loop);
     }
     if (graphs) {

@@ -69,9 +69,9 @@ int slab_cg_finish(const SlabCg* runs, int nrun, cudaStream_t st);
 // One kernel of the iteration (0 k_cg_zfwd, 1 k_cg_terms, 2 k_cg_zinv; 3 the
 // finishing update) of a single run, for per-kernel timing.
 int slab_launch(int which, const SlabCg& a, cudaStream_t st);
-// Algorithmic bytes each kernel moves (FP32 values read and written, with
-// an update pending): 9, 6, 6 and 3 N^3 floats.
-constexpr int kSlabValues[4] = {9, 6, 6, 3};
+// Algorithmic bytes each kernel moves: 9, 6, 6 and 2 N^3 floats read and written (the
+// last reads d as well where the host stopped the run with an update pending).
+constexpr int kSlabValues[4] = {9, 6, 6, 2};
 // q = S d (the three spectral terms plus s->cdiag d plus s->rank1 sum(d)), d and
 // q in natural order, with s->iters = 0, s->beta = 0 and s->done = 0.
 int slab_schur_apply(const SlabCg& a, const float* d, float* q, cudaStream_t st);
