@@ -110,15 +110,10 @@ __device__ __forceinline__ C2<T> csub(C2<T> a, C2<T> b) {
     return {a.x - b.x, a.y - b.y};
   }
 }
-// a s, packed in FP32
-template <typename T>
-__device__ __forceinline__ C2<T> cscale(C2<T> a, T s) {
-  if constexpr (sizeof(T) == 4) {
-    const float2 r = __fmul2_rn(make_float2(a.x, a.y), make_float2(s, s));
-    return {r.x, r.y};
-  } else {
-    return {a.x * s, a.y * s};
-  }
+// a s, packed
+__device__ __forceinline__ C2<float> cscale(C2<float> a, float s) {
+  const float2 r = __fmul2_rn(make_float2(a.x, a.y), make_float2(s, s));
+  return {r.x, r.y};
 }
 
 // b exp(-2 pi i j / L) for a compile-time j (forward twiddles): quarter turns
@@ -463,16 +458,11 @@ __device__ __forceinline__ void for_pairs(C2<T> (&v)[Shape<N>::R], int m, int pa
   }
 }
 
-// 1 / d for a sum d of three 4 sin^2, in [1e-4, 12]: in FP32 the hardware reciprocal (within 1 ulp)
-template <typename T>
-__device__ __forceinline__ T rcp(T d) {
-  if constexpr (sizeof(T) == 4) {
-    float r;
-    asm("rcp.approx.ftz.f32 %0, %1;" : "=f"(r) : "f"(d));
-    return r;
-  } else {
-    return T(1) / d;
-  }
+// 1 / d for a sum d of three 4 sin^2, in [1e-4, 12]: the hardware reciprocal (within 1 ulp)
+__device__ __forceinline__ float rcp(float d) {
+  float r;
+  asm("rcp.approx.ftz.f32 %0, %1;" : "=f"(r) : "f"(d));
+  return r;
 }
 
 // One term of the Schur operator, uniform over a CTA.  The axis `term` takes
@@ -493,56 +483,55 @@ __device__ __forceinline__ Term term_of(int term) { return {term != 0, term != 1
 // relative in the 2-norm on white noise (mu = 0.7): 1.88e-7, 2.01e-7, 1.87e-7, 2.14e-7,
 // 2.42e-7 at N = 32, 64, 96, 128, 256; real transforms with correctly rounded reciprocals,
 // one axis at a time: 2.12e-7, 2.12e-7, 1.94e-7, 2.21e-7, 2.62e-7.
-template <typename T>
 struct LineW {
-  T eA, eB, nA, nB, cy, f;
+  float eA, eB, nA, nB, cy, f;
   // ay, ay2: 4 sin^2 at k and N - k
-  __device__ __forceinline__ void pair(T ay, T ay2, T& s, T& ds, T& t, T& dt) const {
-    const T y1 = cy * ay, y2 = cy * ay2;
+  __device__ __forceinline__ void pair(float ay, float ay2, float& s, float& ds, float& t, float& dt) const {
+    const float y1 = cy * ay, y2 = cy * ay2;
     // the weights (over f) of A and B at k and N - k
-    const T u1 = (nA + y1) * rcp(eA + ay), u2 = (nA + y2) * rcp(eA + ay2);
-    const T v1 = (nB + y1) * rcp(eB + ay), v2 = (nB + y2) * rcp(eB + ay2);
-    const T sA = u1 + u2, sB = v1 + v2, tA = u1 - u2, tB = v1 - v2;
+    const float u1 = (nA + y1) * rcp(eA + ay), u2 = (nA + y2) * rcp(eA + ay2);
+    const float v1 = (nB + y1) * rcp(eB + ay), v2 = (nB + y2) * rcp(eB + ay2);
+    const float sA = u1 + u2, sB = v1 + v2, tA = u1 - u2, tB = v1 - v2;
     s = f * (sA + sB);
     ds = f * (sA - sB);
     t = f * (tA + tB);
     dt = f * (tA - tB);
   }
   // the weights of A and B at an index that is its own mirror (k = 0 and N/2)
-  __device__ __forceinline__ void self(T ay, T& wA, T& wB) const {
-    wA = T(4) * f * (nA + cy * ay) * rcp(eA + ay);
-    wB = T(4) * f * (nB + cy * ay) * rcp(eB + ay);
+  __device__ __forceinline__ void self(float ay, float& wA, float& wB) const {
+    wA = 4.f * f * (nA + cy * ay) * rcp(eA + ay);
+    wB = 4.f * f * (nB + cy * ay) * rcp(eB + ay);
   }
 };
 
-template <int N, typename T>
+template <int N>
 struct Smem {
   using S = Shape<N>;
-  static constexpr size_t scratch = S::CL > 1 ? sizeof(C2<T>) * S::TEAMS * N : 0;
-  static constexpr size_t field = sizeof(C2<T>) * S::LL * N + scratch;
-  static constexpr size_t tables = sizeof(C2<T>) * (2 * N + 2 * S::LINES) + sizeof(T) * S::LINES;
+  static constexpr size_t scratch = S::CL > 1 ? sizeof(C2<float>) * S::TEAMS * N : 0;
+  static constexpr size_t field = sizeof(C2<float>) * S::LL * N + scratch;
+  static constexpr size_t tables = sizeof(C2<float>) * (2 * N + 2 * S::LINES) + sizeof(float) * S::LINES;
   static constexpr size_t bytes = field + tables;
 };
 
 // The tables of term_plane behind the field in shared memory.
 // twg: exp(-pi i t / N), t < 2N; qg: exp(-pi i k / 2N); s2: 4 sin^2(pi a / 2N), a < N.
-template <int N, typename T>
-__device__ __forceinline__ void term_tables(C2<T>* P, const C2<T>* __restrict__ twg, const C2<T>* __restrict__ qg,
-                                            const T* __restrict__ s2) {
+template <int N>
+__device__ __forceinline__ void term_tables(C2<float>* P, const C2<float>* __restrict__ twg,
+                                            const C2<float>* __restrict__ qg, const float* __restrict__ s2) {
   using S = Shape<N>;
   constexpr int M = S::M, R = S::R;
-  C2<T>* tws = P + Smem<N, T>::field / sizeof(C2<T>);   // FFT twiddles [s][m]
-  C2<T>* twr = tws + N;                 // the same by [m][s]
-  C2<T>* qh = twr + N;                  // q_k / 2, k < N/2
-  C2<T>* cy = qh + S::LINES;            // exp(i pi k / N), k < N/2
-  T* sg = reinterpret_cast<T*>(cy + S::LINES);   // 4 sin^2(pi k / 2N), k < N/2
+  C2<float>* tws = P + Smem<N>::field / sizeof(C2<float>);   // FFT twiddles [s][m]
+  C2<float>* twr = tws + N;                 // the same by [m][s]
+  C2<float>* qh = twr + N;                  // q_k / 2, k < N/2
+  C2<float>* cy = qh + S::LINES;            // exp(i pi k / N), k < N/2
+  float* sg = reinterpret_cast<float*>(cy + S::LINES);   // 4 sin^2(pi k / 2N), k < N/2
   for (int e = threadIdx.x; e < N; e += S::THREADS) {
     tws[e] = twg[2 * (e / M) * (e % M)];
     twr[e] = twg[2 * (e / R) * (e % R)];
   }
   for (int e = threadIdx.x; e < S::LINES; e += S::THREADS) {
-    const C2<T> q = qg[e];
-    qh[e] = {T(0.5) * q.x, T(0.5) * q.y};
+    const C2<float> q = qg[e];
+    qh[e] = {0.5f * q.x, 0.5f * q.y};
     cy[e] = conjg(twg[e]);
     sg[e] = s2[e];
   }
@@ -553,23 +542,23 @@ __device__ __forceinline__ void term_tables(C2<T>* P, const C2<T>* __restrict__ 
 // the field's odd nodes along it are negated in `in` and in `out`; `in` carries
 // instead the signs of `signs` (so that two terms can share an input).
 // az: the plane's 4 sin^2 along z; sc: 1 / (mu N^2).
-// P: Smem<N, T>, its tables filled (term_tables; a barrier follows here).
+// P: Smem<N>, its tables filled (term_tables; a barrier follows here).
 // Called by all threads of the CTA (of every CTA of the cluster; rank: this one's).
-template <int N, typename T>
-__device__ __forceinline__ void term_plane(const T* in, T* out, const Term term, const Term signs, T az, T sc,
-                                           C2<T>* P, int rank = 0) {
+template <int N>
+__device__ __forceinline__ void term_plane(const float* in, float* out, const Term term, const Term signs, float az,
+                                           float sc, C2<float>* P, int rank = 0) {
   using S = Shape<N>;
   constexpr int M = S::M, R = S::R, H = S::H;
-  C2<T>* tws = P + Smem<N, T>::field / sizeof(C2<T>);   // FFT twiddles [s][m]
-  C2<T>* twr = tws + N;                 // the same by [m][s]
-  C2<T>* qh = twr + N;                  // q_k / 2, k < N/2
-  C2<T>* cy = qh + S::LINES;            // exp(i pi k / N), k < N/2
-  T* sg = reinterpret_cast<T*>(cy + S::LINES);   // 4 sin^2(pi k / 2N), k < N/2
+  C2<float>* tws = P + Smem<N>::field / sizeof(C2<float>);   // FFT twiddles [s][m]
+  C2<float>* twr = tws + N;                 // the same by [m][s]
+  C2<float>* qh = twr + N;                  // q_k / 2, k < N/2
+  C2<float>* cy = qh + S::LINES;            // exp(i pi k / N), k < N/2
+  float* sg = reinterpret_cast<float*>(cy + S::LINES);   // 4 sin^2(pi k / 2N), k < N/2
   const int t = threadIdx.x / M, m = threadIdx.x % M;
   const int lane = threadIdx.x & 31;
   const int partner = (lane & ~(M - 1)) | ((M - m) & (M - 1));
   // the lines of CTA c of the cluster (all lines without one)
-  C2<T>* lines[S::CL];
+  C2<float>* lines[S::CL];
   if constexpr (S::CL > 1) {
 #pragma unroll
     for (int c = 0; c < S::CL; ++c) lines[c] = cooperative_groups::this_cluster().map_shared_rank(P, c);
@@ -581,37 +570,33 @@ __device__ __forceinline__ void term_plane(const T* in, T* out, const Term term,
     else __syncthreads();
   };
   // the column pair n0, n0 + 1 of line l, the lane's i-th index
-  auto pair_at = [&](int i, int l, int n0) -> C2<T>* {
+  auto pair_at = [&](int i, int l, int n0) -> C2<float>* {
     static_assert(S::CL == 1 || !PairShape<N>::in_lane, "i gives the owner of line m + M i");
     if constexpr (S::CL > 1) return lines[M * i / S::LL] + ((l % S::LL) * N + (n0 ^ line_sw<M>(l)));
     else return P + (l * N + (n0 ^ line_sw<M>(l)));
   };
-  C2<T> v[R];
+  C2<float> v[R];
   // ---- along x: the rows of Makhoul positions 2p, 2p + 1 along y -> columns 2p, 2p + 1
 #pragma unroll 1
   for (int rd = 0; rd < S::ROUNDS; ++rd) {
     const int n0 = 2 * (rank * S::LL + t + S::TEAMS * rd);
-    const C2<T>* ra = reinterpret_cast<const C2<T>*>(in + (int64_t)(n0 / S::YB) * (N * S::YB) + m * S::YB + n0 % S::YB);
-    const T fl = (n0 >= N / 2 && term.ys != signs.ys) ? T(-1) : T(1), fh = term.xs != signs.xs ? -fl : fl;
+    const C2<float>* ra =
+        reinterpret_cast<const C2<float>*>(in + (int64_t)(n0 / S::YB) * (N * S::YB) + m * S::YB + n0 % S::YB);
+    const float fl = (n0 >= N / 2 && term.ys != signs.ys) ? -1.f : 1.f, fh = term.xs != signs.xs ? -fl : fl;
 #pragma unroll
     for (int r = 0; r < R; ++r) v[r] = cscale(ldc(ra + r * (M * S::YB / 2)), r < H ? fl : fh);
     if (rd == 0) sync();   // tables (and the others run before their lines are written)
-    if constexpr (S::CL > 1) fft_to_pairs<N, T>(v, P, XScratch<N>{S::LL * N + t * N}, tws, m);
-    else fft_to_pairs<N, T>(v, P, XSlots<N>{n0}, tws, m);
-    for_pairs<N, true, false>(v, m, partner, [&](int i, int l, bool self, C2<T> z, C2<T> g) {
-      const C2<T> q = ldc(qh + l);
-      C2<T> a = cmul(q, C2<T>{z.x + g.x, z.y - g.y}), b = cmul(q, C2<T>{z.y + g.y, g.x - z.x});
+    if constexpr (S::CL > 1) fft_to_pairs<N, float>(v, P, XScratch<N>{S::LL * N + t * N}, tws, m);
+    else fft_to_pairs<N, float>(v, P, XSlots<N>{n0}, tws, m);
+    for_pairs<N, true, false>(v, m, partner, [&](int i, int l, bool self, C2<float> z, C2<float> g) {
+      const C2<float> q = ldc(qh + l);
+      C2<float> a = cmul(q, C2<float>{z.x + g.x, z.y - g.y}), b = cmul(q, C2<float>{z.y + g.y, g.x - z.x});
       if (self) {   // the real modes 0 and N/2
         a = {z.x, g.x};
         b = {z.y, g.y};
       }
-      C2<T>* at = pair_at(i, l, n0);   // the swizzle keeps pairs 2p, 2p + 1 together
-      if constexpr (sizeof(T) == 4) {
-        *reinterpret_cast<float4*>(at) = make_float4(a.x, a.y, b.x, b.y);
-      } else {
-        stc(at, a);
-        stc(at + 1, b);
-      }
+      C2<float>* at = pair_at(i, l, n0);   // the swizzle keeps pairs 2p, 2p + 1 together
+      *reinterpret_cast<float4*>(at) = make_float4(a.x, a.y, b.x, b.y);
     });
   }
   sync();
@@ -624,39 +609,39 @@ __device__ __forceinline__ void term_plane(const T* in, T* out, const Term term,
     const YSlots<N> Y{ll * N, line_sw<M>(l)};
 #pragma unroll
     for (int r = 0; r < R; ++r) v[r] = ldc(P + (Y.base + ((m + M * r) ^ Y.sw)));
-    fft_to_pairs<N, T>(v, P, Y, tws, m);
+    fft_to_pairs<N, float>(v, P, Y, tws, m);
     // 4 sin^2 of the line's x modes l and N - l (line 0: 0 and N/2)
-    const T sl = sg[l];
-    const T axA = term.xs ? T(4) - sl : sl, axB = l ? (term.xs ? sl : T(4) - sl) : T(2);
-    LineW<T> W;
+    const float sl = sg[l];
+    const float axA = term.xs ? 4.f - sl : sl, axB = l ? (term.xs ? sl : 4.f - sl) : 2.f;
+    LineW W;
     W.eA = axA + az;
     W.eB = axB + az;
-    W.nA = term.nx ? axA : (term.ny ? T(0) : az);
-    W.nB = term.nx ? axB : (term.ny ? T(0) : az);
-    W.cy = term.ny ? T(1) : T(0);
-    W.f = T(0.5) * sc;   // twice a quarter: the inverse along x takes q / 2
-    for_pairs<N, true, true>(v, m, partner, [&](int, int k, bool self, C2<T>& z, C2<T>& p) {
-      const C2<T> c = ldc(cy + k);
-      const T sk = sg[k], sm = T(4) - sk;
-      T s, ds, tt2, dt;
+    W.nA = term.nx ? axA : (term.ny ? 0.f : az);
+    W.nB = term.nx ? axB : (term.ny ? 0.f : az);
+    W.cy = term.ny ? 1.f : 0.f;
+    W.f = 0.5f * sc;   // twice a quarter: the inverse along x takes q / 2
+    for_pairs<N, true, true>(v, m, partner, [&](int, int k, bool self, C2<float>& z, C2<float>& p) {
+      const C2<float> c = ldc(cy + k);
+      const float sk = sg[k], sm = 4.f - sk;
+      float s, ds, tt2, dt;
       W.pair(term.ys ? sm : sk, term.ys ? sk : sm, s, ds, tt2, dt);
       // Z'_k = s Z + ds P* + c (t P + dt Z*), Z'_(N-k) = s P + ds Z* + c* (t Z + dt P*),
       // conjugated for the inverse by a forward FFT
-      const C2<T> g = {tt2 * p.x + dt * z.x, tt2 * p.y - dt * z.y};
-      const C2<T> h = {tt2 * z.x + dt * p.x, tt2 * z.y - dt * p.y};
-      C2<T> lo = {s * z.x + ds * p.x + (c.x * g.x - c.y * g.y), ds * p.y - s * z.y - (c.x * g.y + c.y * g.x)};
-      C2<T> hi = {s * p.x + ds * z.x + (c.x * h.x + c.y * h.y), ds * z.y - s * p.y - (c.x * h.y - c.y * h.x)};
+      const C2<float> g = {tt2 * p.x + dt * z.x, tt2 * p.y - dt * z.y};
+      const C2<float> h = {tt2 * z.x + dt * p.x, tt2 * z.y - dt * p.y};
+      C2<float> lo = {s * z.x + ds * p.x + (c.x * g.x - c.y * g.y), ds * p.y - s * z.y - (c.x * g.y + c.y * g.x)};
+      C2<float> hi = {s * p.x + ds * z.x + (c.x * h.x + c.y * h.y), ds * z.y - s * p.y - (c.x * h.y - c.y * h.x)};
       if (self) {   // indices 0 and N/2, each its own mirror
-        T wA, wB;
-        W.self(term.ys ? T(4) : T(0), wA, wB);
+        float wA, wB;
+        W.self(term.ys ? 4.f : 0.f, wA, wB);
         lo = {wA * z.x, -(wB * z.y)};
-        W.self(T(2), wA, wB);
+        W.self(2.f, wA, wB);
         hi = {wA * p.x, -(wB * p.y)};
       }
       z = lo;
       p = hi;
     });
-    fft_from_pairs<N, T>(v, P, Y, tws, twr, m);
+    fft_from_pairs<N, float>(v, P, Y, tws, twr, m);
 #pragma unroll
     for (int j = 0; j < R; ++j) stc(P + (Y.base + ((m + M * j) ^ Y.sw)), conjg(v[j]));
   }
@@ -666,28 +651,22 @@ __device__ __forceinline__ void term_plane(const T* in, T* out, const Term term,
   for (int rd = 0; rd < S::ROUNDS; ++rd) {
     const int n0 = 2 * (rank * S::LL + t + S::TEAMS * rd);
     // conj Z'_k = q conj(A + i B), conj Z'_(N-k) = conj(q) (A - i B)
-    for_pairs<N, false, true>(v, m, partner, [&](int i, int l, bool self, C2<T>& lo, C2<T>& hi) {
-      const C2<T>* at = pair_at(i, l, n0);
-      C2<T> a, b;
-      if constexpr (sizeof(T) == 4) {
-        const float4 f = *reinterpret_cast<const float4*>(at);
-        a = {f.x, f.y};
-        b = {f.z, f.w};
-      } else {
-        a = ldc(at);
-        b = ldc(at + 1);
-      }
-      const C2<T> q = ldc(qh + l);
-      lo = cmul(q, C2<T>{a.x - b.y, -(a.y + b.x)});
-      hi = cmul(conjg(q), C2<T>{a.x + b.y, a.y - b.x});
+    for_pairs<N, false, true>(v, m, partner, [&](int i, int l, bool self, C2<float>& lo, C2<float>& hi) {
+      const C2<float>* at = pair_at(i, l, n0);
+      const float4 f = *reinterpret_cast<const float4*>(at);
+      const C2<float> a = {f.x, f.y}, b = {f.z, f.w};
+      const C2<float> q = ldc(qh + l);
+      lo = cmul(q, C2<float>{a.x - b.y, -(a.y + b.x)});
+      hi = cmul(conjg(q), C2<float>{a.x + b.y, a.y - b.x});
       if (self) {
-        lo = {T(0.5) * a.x, T(-0.5) * b.x};
-        hi = {T(0.5) * a.y, T(-0.5) * b.y};
+        lo = {0.5f * a.x, -0.5f * b.x};
+        hi = {0.5f * a.y, -0.5f * b.y};
       }
     });
-    if constexpr (S::CL > 1) fft_from_pairs<N, T>(v, P, XScratch<N>{S::LL * N + t * N}, tws, twr, m);
-    else fft_from_pairs<N, T>(v, P, XSlots<N>{n0}, tws, twr, m);
-    C2<T>* ra = reinterpret_cast<C2<T>*>(out + (int64_t)(n0 / S::YB) * (N * S::YB) + m * S::YB + n0 % S::YB);
+    if constexpr (S::CL > 1) fft_from_pairs<N, float>(v, P, XScratch<N>{S::LL * N + t * N}, tws, twr, m);
+    else fft_from_pairs<N, float>(v, P, XSlots<N>{n0}, tws, twr, m);
+    C2<float>* ra =
+        reinterpret_cast<C2<float>*>(out + (int64_t)(n0 / S::YB) * (N * S::YB) + m * S::YB + n0 % S::YB);
 #pragma unroll
     for (int j = 0; j < R; ++j) stc(ra + j * (M * S::YB / 2), conjg(v[j]));
   }

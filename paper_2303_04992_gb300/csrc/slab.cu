@@ -29,8 +29,8 @@ cudaError_t raise(K kern, size_t bytes) {
 template <int N, int MAXB>
 cudaError_t prepare_nb() {
   cudaError_t e;
-  if constexpr (plane::Shape<N>::CL > 1) e = raise(slab::k_cg_terms_cl<N, MAXB>, plane::Smem<N, float>::bytes);
-  else e = raise(slab::k_cg_terms<N, MAXB>, plane::Smem<N, float>::bytes);
+  if constexpr (plane::Shape<N>::CL > 1) e = raise(slab::k_cg_terms_cl<N, MAXB>, plane::Smem<N>::bytes);
+  else e = raise(slab::k_cg_terms<N, MAXB>, plane::Smem<N>::bytes);
   if (e == cudaSuccess) e = raise(slab::k_cg_zfwd<N, MAXB>, slab::ZShape<N>::bytes);
   if (e == cudaSuccess) e = raise(slab::k_cg_zinv<N, MAXB>, slab::ZShape<N>::bytes);
   if (e == cudaSuccess) e = raise(slab::k_cg_start<N, MAXB>, slab::Conv<N>::bytes);
@@ -85,11 +85,11 @@ void launch_nb(int which, const slab::SlabArgs<MAXB>& args, const SlabCg& t, int
     case 1:
       if constexpr (plane::Shape<N>::CL > 1)
         (void)launch_overlapped(kOverlap<N>, slab::k_cg_terms_cl<N, MAXB>, dim3(plane::Shape<N>::CL * 3 * N, nrun),
-                                plane::Shape<N>::THREADS, plane::Smem<N, float>::bytes, st, args, t.tw, t.qN, t.s2,
+                                plane::Shape<N>::THREADS, plane::Smem<N>::bytes, st, args, t.tw, t.qN, t.s2,
                                 t.inv_mu);
       else
         (void)launch_overlapped(kOverlap<N>, slab::k_cg_terms<N, MAXB>, dim3(3 * N, nrun), plane::Shape<N>::THREADS,
-                                plane::Smem<N, float>::bytes, st, args, t.tw, t.qN, t.s2, t.inv_mu);
+                                plane::Smem<N>::bytes, st, args, t.tw, t.qN, t.s2, t.inv_mu);
       break;
     case 2:
       (void)launch_overlapped(kOverlap<N>, slab::k_cg_zinv<N, MAXB>, dim3(Z::BLOCKS, nrun), Z::THREADS, Z::bytes, st, args, t.tw,

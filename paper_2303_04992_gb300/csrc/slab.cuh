@@ -325,7 +325,7 @@ __device__ __forceinline__ void terms_body(const SlabArgs<MAXB>& args, int unit,
                                            const float* __restrict__ s2g, float inv_mu) {
   const int b = blockIdx.y;
   extern __shared__ __align__(16) unsigned char smx[];
-  plane::term_tables<N, float>(reinterpret_cast<C2<float>*>(smx), twg, qg, s2g);
+  plane::term_tables<N>(reinterpret_cast<C2<float>*>(smx), twg, qg, s2g);
   overlap_wait();
   overlap_trigger();
   if (args.s[b]->done) return;
@@ -340,7 +340,7 @@ __device__ __forceinline__ void terms_body(const SlabArgs<MAXB>& args, int unit,
   // 1 / N per inverse transform, as the one-axis passes scale: at N = 96 the rounding of
   // 1 / 96 offsets part of the FFT constants' (operator error 2.1e-7 with 1 / N^2 rounded once)
   constexpr float invN = 1.0f / N;
-  plane::term_plane<N, float>(in, out, plane::term_of(term), plane::term_of(term == 2 ? 2 : 0), az,
+  plane::term_plane<N>(in, out, plane::term_of(term), plane::term_of(term == 2 ? 2 : 0), az,
                               inv_mu * (invN * invN), reinterpret_cast<C2<float>*>(smx), rank);
 }
 template <int N, int MAXB>
