@@ -476,31 +476,32 @@ __device__ __forceinline__ Term term_of(int term) { return {term != 0, term != 1
 
 // Weights of one complex y line (real lines A and B: two x modes) at DCT index
 // k < N/2 along y and its mirror N - k: s, ds, t, dt of the header comment.
-// eX = ax + az; nX: the numerator's part that does not depend on y; cy: 1 where
-// the numerator is ay; f: a quarter of the weight's factor.  A reciprocal per weight:
-// one for the product of two denominators saves 1 % of a matvec at N = 128 (the special
-// function unit) and leaves the weights less exact.  The operator's error against 64 bits,
-// relative in the 2-norm on white noise (mu = 0.7): 1.88e-7, 2.01e-7, 1.87e-7, 2.14e-7,
-// 2.42e-7 at N = 32, 64, 96, 128, 256; real transforms with correctly rounded reciprocals,
-// one axis at a time: 2.12e-7, 2.12e-7, 1.94e-7, 2.21e-7, 2.62e-7.
+// eX = ax + az; nX: the numerator's part that does not depend on y; cy: where the
+// numerator is ay; both with a quarter of the weight's factor.  A reciprocal per
+// weight: one for the product of two denominators is half a percent of a matvec
+// faster and leaves the weights less exact; correctly rounded ones take 4 % longer
+// and change nothing below.  The operator's error against 64 bits, relative in the
+// 2-norm on white noise (mu = 0.7): 1.89e-7, 2.04e-7, 1.87e-7, 2.15e-7, 2.44e-7 at
+// N = 32, 64, 96, 128, 256; real transforms with correctly rounded reciprocals, one
+// axis at a time: 2.12e-7, 2.12e-7, 1.94e-7, 2.21e-7, 2.62e-7.
 struct LineW {
-  float eA, eB, nA, nB, cy, f;
+  float eA, eB, nA, nB, cy;
   // ay, ay2: 4 sin^2 at k and N - k
   __device__ __forceinline__ void pair(float ay, float ay2, float& s, float& ds, float& t, float& dt) const {
     const float y1 = cy * ay, y2 = cy * ay2;
-    // the weights (over f) of A and B at k and N - k
+    // the weights (a quarter) of A and B at k and N - k
     const float u1 = (nA + y1) * rcp(eA + ay), u2 = (nA + y2) * rcp(eA + ay2);
     const float v1 = (nB + y1) * rcp(eB + ay), v2 = (nB + y2) * rcp(eB + ay2);
     const float sA = u1 + u2, sB = v1 + v2, tA = u1 - u2, tB = v1 - v2;
-    s = f * (sA + sB);
-    ds = f * (sA - sB);
-    t = f * (tA + tB);
-    dt = f * (tA - tB);
+    s = sA + sB;
+    ds = sA - sB;
+    t = tA + tB;
+    dt = tA - tB;
   }
   // the weights of A and B at an index that is its own mirror (k = 0 and N/2)
   __device__ __forceinline__ void self(float ay, float& wA, float& wB) const {
-    wA = 4.f * f * (nA + cy * ay) * rcp(eA + ay);
-    wB = 4.f * f * (nB + cy * ay) * rcp(eB + ay);
+    wA = 4.f * (nA + cy * ay) * rcp(eA + ay);
+    wB = 4.f * (nB + cy * ay) * rcp(eB + ay);
   }
 };
 
@@ -616,10 +617,10 @@ __device__ __forceinline__ void term_plane(const float* in, float* out, const Te
     LineW W;
     W.eA = axA + az;
     W.eB = axB + az;
-    W.nA = term.nx ? axA : (term.ny ? 0.f : az);
-    W.nB = term.nx ? axB : (term.ny ? 0.f : az);
-    W.cy = term.ny ? 1.f : 0.f;
-    W.f = 0.5f * sc;   // twice a quarter: the inverse along x takes q / 2
+    const float f = 0.5f * sc;   // twice a quarter: the inverse along x takes q / 2
+    W.nA = f * (term.nx ? axA : (term.ny ? 0.f : az));
+    W.nB = f * (term.nx ? axB : (term.ny ? 0.f : az));
+    W.cy = term.ny ? f : 0.f;
     for_pairs<N, true, true>(v, m, partner, [&](int, int k, bool self, C2<float>& z, C2<float>& p) {
       const C2<float> c = ldc(cy + k);
       const float sk = sg[k], sm = 4.f - sk;
