@@ -166,7 +166,7 @@ typedef struct {
 } kfbim_options;
 
 /* Kernels of the FP32 transforms of MIXED contexts.
- * The Schur CG (Sec. 4.2, the dominant cost) runs, for N = 32, 64, 96 and 128,
+ * The Schur CG (Sec. 4.2, the dominant cost) runs, for N = 32, 64, 96, 128 and 256,
  * as three kernels per iteration: the pending vector update and the transforms
  * along z of the CG direction, one CTA per spectral term and (x, y) plane for
  * the rest of the three terms in shared memory, and the inverse transforms along
@@ -349,7 +349,7 @@ int kfbim_solve_adjoint(kfbim_ctx* ctx, const double* ubar_dev, double* gbar_dev
  * and CG iteration per instance).
  * MIXED contexts run the instances in lockstep: every FFT stage is one launch
  * for all instances still iterating, each Schur CG of the batch (N = 32, 64,
- * 96, 128) is one launch of a CUDA graph whose conditional while loop runs the
+ * 96, 128, 256) is one launch of a CUDA graph whose conditional while loop runs the
  * three slab kernels of every instance until all are done, and GMRES reads
  * its host scalars once per iteration for the whole batch.  FP64 contexts solve the instances one
  * after another.  The first call with a larger B than before allocates the
@@ -381,7 +381,8 @@ typedef enum {
   KFBIM_KCLASS_CG_XY = 3,           /* slab CG: xy planes of the three terms (6 N^3 floats) */
   KFBIM_KCLASS_CG_ZINV = 4,         /* slab CG: inverse z transforms, d.q, r.r, r.q, q.q (6 N^3 floats) */
   KFBIM_KCLASS_CG_UPDATE = 5,       /* slab CG: x back in natural order when a run stops
-                                       (2 N^3 floats, once per CG run) */
+                                       (2 N^3 floats, once per CG run; 3 where the host
+                                       stopped it with an update pending) */
   KFBIM_KCLASS_CG_VECTOR = 6,       /* staged CG: the three vector kernels (14 N^3 values) */
   KFBIM_KCLASS_MAC_RESIDUAL = 7,    /* MIXED refinement: FP64 MAC residual (12 N^3 doubles) */
   KFBIM_KCLASS_JUMPS = 8,           /* jump evaluation (fit rows, jump maps, jumps) */

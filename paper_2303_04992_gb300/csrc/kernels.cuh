@@ -258,7 +258,8 @@ __global__ void k_f_minus_gp(const double* __restrict__ f, const double* __restr
 // than FP64 additions, and leave it three per value, while the divergence stays on
 // it (all four fields in integers: 121 us, bound by their instructions).  A warp
 // takes the four fields of its points in turn and its neighbours begin with other
-// ones, so that both pipes stay busy: 108 us, and 0.82 ms for 1.32 ms at N = 256.
+// ones, so that both pipes stay busy (FP64 62 %, issue 54 %): 104 us, and 0.80 ms for
+// 1.32 ms at N = 256.
 constexpr int MAC_OCC = 4;
 inline int mac_blocks(int64_t n3) {   // one wave
   return (int)std::min<int64_t>((n3 + RED_THREADS - 1) / RED_THREADS, 152 * MAC_OCC);

@@ -26,16 +26,16 @@
 // columns x the teams of a half warp), the exchange along y (runs of M), the
 // 16-byte column pairs (M lines) and the line accesses free of bank conflicts.
 //
-// What bounds it (N = 128, 384 CTAs, FP32): instruction issue (56 % of the slots
+// What bounds it (N = 128, 384 CTAs, FP32): instruction issue (59 % of the slots
 // of the average SM, the busiest of the 152 holds three of the 384 CTAs) and the
-// shared-memory pipe (52 %); 17 M warp instructions against 37.5 M for a kernel
+// shared-memory pipe (50 %); 16.6 M warp instructions against 37.5 M for a kernel
 // that formed every real transform and transposed the plane between the axes.
-// 28.7 us for the three terms at N = 128 (that kernel: 56.6), 8.2 at N = 64 (about
-// 30), 4.2 at N = 32 (27), 12.3 at N = 96 (five one-axis passes there: 133).  The
-// pair-blocked order of the planes gives 2.1 of the first, index pairs within a lane
-// instead of shuffles 2.0 (N = 128; 2.0 of 14.3 at N = 96), a copy of the code per
-// term cost 2 (the warps waited for instructions), and 80 registers with three
-// resident CTAs run as fast as 128 with two.
+// Between events, which add about 3 us: 25.3 us for the three terms at N = 128 (that
+// kernel: 56.6), 9.5 at N = 64 (about 30), 7.2 at N = 32 (27), 13.4 at N = 96 (five
+// one-axis passes there: 133).  Of that the pair-blocked order of the planes gave 2.1 at
+// N = 128, index pairs within a lane instead of shuffles 2.0 (at N = 96 as much), a copy
+// of the code per term cost 2 (the warps waited for instructions), and 80 registers with
+// three resident CTAs ran as fast as 128 with two.
 #pragma once
 
 #include <cooperative_groups.h>

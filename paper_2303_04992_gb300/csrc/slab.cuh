@@ -350,9 +350,9 @@ k_cg_terms(const __grid_constant__ SlabArgs<MAXB> args, const C2<float>* __restr
   terms_body<N, MAXB>(args, blockIdx.x, 0, twg, qg, s2g, inv_mu);
 }
 // The same with a plane on a cluster (N = 256): 235 us as four CTAs of 256 threads,
-// two clusters' CTAs per SM (272 us as two CTAs of 512), bound by issue and shared
-// memory; the five one-axis stages it replaces took 1.16 ms of a staged CG
-// iteration of 1.32 ms (now 0.42 ms).
+// two clusters' CTAs per SM (272 us as two CTAs of 512); issue 42 %, shared memory
+// 38 % busy, the rest the waits of 16 warps per SM.  The five one-axis stages it
+// replaces took 1.16 ms of a staged CG iteration of 1.32 ms (now 0.42 ms).
 template <int N, int MAXB>
 __global__ void __cluster_dims__(plane::Shape<N>::CL, 1, 1) __launch_bounds__(plane::Shape<N>::THREADS, 2)
 k_cg_terms_cl(const __grid_constant__ SlabArgs<MAXB> args, const C2<float>* __restrict__ twg,

@@ -12,8 +12,8 @@ struct CgLoop;
 template <typename T>
 struct C2;
 
-// One CG run's buffers: the solution x in natural order; xs, r, d, q (slab order), the z-transformed fields z1, z3 and the
-// term results w1, w2 (N^3 floats each); the FP32 transform tables (full-circle
+// One CG run's buffers: the solution x in natural order; xs, r, d, q (slab order), the
+// z-transformed fields z1, z3 and the term results w1, w2 (N^3 floats each); the FP32 transform tables (full-circle
 // twiddles exp(-2 pi i t / 2N), t < 2N; post-twiddles exp(-i pi k / 2N), k < N;
 // the eigenvalue table 4 sin^2 of the DCT (N) and DST (N) modes), 1/mu, the
 // device scalars and the reduction memory (slab_reduce_slots(N) slots of eight
@@ -33,7 +33,7 @@ struct SlabCg {
 constexpr int kSlabBatchMax = 64;
 
 // Grids the slab iteration covers: N / 2 complex lines of N numbers (a whole
-// plane) fit in the shared memory of one CTA, at N = 256 of a cluster of two.
+// plane) fit in the shared memory of one CTA, at N = 256 of a cluster of four.
 bool slab_supported(int N);
 size_t slab_reduce_slots(int N);
 // Raises the kernels' dynamic shared-memory limits on the current device.
@@ -73,7 +73,8 @@ int slab_launch(int which, const SlabCg& a, cudaStream_t st);
 // last reads d as well where the host stopped the run with an update pending).
 constexpr int kSlabValues[4] = {9, 6, 6, 2};
 // q = S d (the three spectral terms plus s->cdiag d plus s->rank1 sum(d)), d and
-// q in natural order, with s->iters = 0, s->beta = 0 and s->done = 0.
+// q in natural order, with s->iters = 0, s->beta = 0 and s->done = 0.  At N = 256 the
+// tickets in the reduction memory must be zero, as slab_cg_start leaves them.
 int slab_schur_apply(const SlabCg& a, const float* d, float* q, cudaStream_t st);
 
 }  // namespace kfbim
