@@ -11,9 +11,8 @@ the per-step CUDA events.
 
 Printed JSON line (rank 0): value = solves/s over all ranks (MIXED precision),
 the FP64 path's solves/s beside it, the relative difference of the MIXED
-density from the FP64 one, the roofline of the dominant kernel (the FP32
-transform passes, timed with CUDA events around each launch in a second run
-of the same steps), the oracle CPU baseline, e2e through kfbim_solve_host with
+density from the FP64 one, the roofline of the dominant kernel (timed with CUDA
+events around each launch in a second run of the same steps), the oracle CPU baseline, e2e through kfbim_solve_host with
 host buffers, the kernel-launch count and the SM clocks sampled during the
 timed region; beside them, the autotuner's choice of transform kernels, one
 adjoint (gradient) solve on the same data, and a batch of 16 instances in one
@@ -211,29 +210,33 @@ def measured_peaks():
     return 6800.0, "fallback"
 
 
-PASS_SOURCES = {"fft": ("transforms.cuh", "plane.cuh", "lines.cuh", "overlap.cuh"),
-                 "tensor": ("transforms.cuh", "transforms2.cuh", "tc_pass.cuh")}
+CSRC = os.path.join(ROOT, "paper_2303_04992_gb300", "csrc")
+# Kernel of each timed class; the sources of the slab CG's, over which the hash in
+# their ncu summary is taken.
+CLASS_KERNEL = {"cg_xy": "k_cg_terms", "cg_zfwd": "k_cg_zfwd", "cg_zinv": "k_cg_zinv", "cg_update": "k_cg_fin",
+                "transform_fp32": "k_lines", "transform_fp64": "k_lines", "mac_residual": "k_mac_residual",
+                "jumps": "k_jumps"}
+SLAB_SOURCES = ("slab.cuh", "cg_common.cuh", "plane.cuh", "overlap.cuh")
 
 
-def kernel_source_hash(kind="fft"):
+def kernel_source_hash():
     h = hashlib.sha256()
-    for f in PASS_SOURCES[kind]:
-        h.update(open(os.path.join(ROOT, "paper_2303_04992_gb300", "csrc", f), "rb").read())
+    for f in SLAB_SOURCES:
+        h.update(open(os.path.join(CSRC, f), "rb").read())
     return h.hexdigest()[:12]
 
 
-def ncu_traffic(workload, kind="fft"):
-    """DRAM bytes per launch of the FP32 transform pass (FFT or tensor-core
-    kernel) from the committed ncu summary, if it was taken on the current
-    kernel source (else None)."""
-    name = "axis_pass_fp32_%s.md" if kind == "fft" else "tc_pass_fp32_%s.md"
-    p = os.path.join(ROOT, "profiles", name % workload)
+def ncu_traffic(kernel, workload):
+    """DRAM bytes per launch of a slab CG kernel from the committed ncu summary
+    profiles/slab_cg_<workload>.md (a line "<kernel> dram_bytes_per_launch: B"), if it was
+    taken on the current kernel source (else None)."""
+    p = os.path.join(ROOT, "profiles", "slab_cg_%s.md" % workload)
     if not os.path.exists(p):
         return None
     txt = open(p).read()
     m = re.search(r"kernel_source_sha256_12:\s*([0-9a-f]+)", txt)
-    t = re.search(r"dram_bytes_per_launch:\s*([0-9.eE+]+)", txt)
-    if not m or not t or m.group(1) != kernel_source_hash(kind):
+    t = re.search(r"%s dram_bytes_per_launch:\s*([0-9.eE+]+)" % re.escape(kernel), txt)
+    if not m or not t or m.group(1) != kernel_source_hash():
         return None
     return float(t.group(1))
 
@@ -250,23 +253,7 @@ MODEL_SCHUR_VALUES = 20
 MODEL_CG_VECTOR_VALUES = 7
 MODEL_MIDDLE_PASS_VALUES = 6
 SLAB_CLASSES = ("cg_zfwd", "cg_xy", "cg_zinv", "cg_update")
-
-
-def ncu_traffic_slab(workload):
-    """DRAM bytes per launch of k_cg_terms from the committed ncu summary, if it
-    was taken on the current slab source (else None)."""
-    p = os.path.join(ROOT, "profiles", "cg_xy_%s.md" % workload)
-    if not os.path.exists(p):
-        return None
-    txt = open(p).read()
-    h = hashlib.sha256()
-    for f in ("slab.cuh", "cg_common.cuh", "plane.cuh", "overlap.cuh"):
-        h.update(open(os.path.join(ROOT, "paper_2303_04992_gb300", "csrc", f), "rb").read())
-    m = re.search(r"kernel_source_sha256_12:\s*([0-9a-f]+)", txt)
-    t = re.search(r"dram_bytes_per_launch:\s*([0-9.eE+]+)", txt)
-    if not m or not t or m.group(1) != h.hexdigest()[:12]:
-        return None
-    return float(t.group(1))
+BUILD_CG_VALUES = 21   # what the slab kernels read and write per iteration: 9, 6 and 6 N^3
 
 
 def roofline_line(kernels, kprof, N3, cg_iters, args, peak, peak_kind):
@@ -275,26 +262,26 @@ def roofline_line(kernels, kprof, N3, cg_iters, args, peak, peak_kind):
     launch are the byte model's figure for the work the kernel does: k_cg_terms
     does the middle pass of the Schur apply on all three terms (6 N^3 b); the
     whole CG iteration (three kernels, plus each run's closing update spread
-    over its iterations) is reported beside it against 27 N^3 b."""
+    over its iterations) is reported beside it against 27 N^3 b and against the
+    21 N^3 b that the kernels read and write."""
     dom = max(kernels, key=lambda k: kernels[k]["share_of_step"])
     kd = kernels[dom]
     line = {"bound": "hbm", "peak": peak, "unit": "GB/s", "peak_source": peak_kind,
-            "kernel": dom, "avg_launch_us": kd["avg_launch_us"], "launches_per_step": kd["launches_per_step"],
-            "share_of_step": kd["share_of_step"], "build_bytes_per_launch": kd["build_bytes_per_launch"],
+            "kernel": CLASS_KERNEL.get(dom, dom), "avg_launch_us": kd["avg_launch_us"],
+            "launches_per_step": kd["launches_per_step"], "share_of_step": kd["share_of_step"],
+            "build_bytes_per_launch": kd["build_bytes_per_launch"],
             "achieved_build_bytes": kd["achieved_gbs_build_bytes"]}
     if dom == "cg_xy":
         model = MODEL_MIDDLE_PASS_VALUES * N3 * MODEL_B
         line["model"] = "three-pass byte model: middle pass of S d on three fields, 6 N^3 b, b = 4"
-        line["traffic"] = ncu_traffic_slab(args.workload)
     elif dom in ("transform_fp32", "transform_fp64"):
         # one one-axis pass of one field: 2 N^3 b per job, at the launch's jobs
         model = kd["build_bytes_per_launch"]
         line["model"] = "one-axis pass: N^3 values read and written per job"
-        line["traffic"] = ncu_traffic(args.workload, "fft")
     else:
         model = kd["build_bytes_per_launch"]
         line["model"] = "values read and written once"
-        line["traffic"] = None
+    line["traffic"] = ncu_traffic(line["kernel"], args.workload)
     achieved = model / (kd["avg_launch_us"] * 1e-6) / 1e9
     line["algorithmic_bytes_per_launch"] = model
     line["achieved"] = round(achieved, 1)
@@ -306,7 +293,10 @@ def roofline_line(kernels, kprof, N3, cg_iters, args, peak, peak_kind):
         line["cg_iteration"] = {"us": round(it_us, 3), "model_bytes": bytes_it,
                                 "achieved": round(bytes_it / (it_us * 1e-6) / 1e9, 1),
                                 "frac": round(bytes_it / (it_us * 1e-6) / 1e9 / peak, 4),
-                                "model": "three-pass byte model: 27 N^3 b per CG iteration (S d 20, vectors 7)"}
+                                "model": "three-pass byte model: 27 N^3 b per CG iteration (S d 20, vectors 7)",
+                                "build_bytes": BUILD_CG_VALUES * N3 * MODEL_B,
+                                "achieved_build_bytes": round(BUILD_CG_VALUES * N3 * MODEL_B / (it_us * 1e-6) / 1e9,
+                                                              1)}
     return line
 
 
