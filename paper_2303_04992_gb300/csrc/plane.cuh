@@ -28,7 +28,7 @@
 //
 // What bounds it (N = 128, 384 CTAs, FP32): instruction issue (59 % of the slots
 // of the average SM, the busiest of the 152 holds three of the 384 CTAs) and the
-// shared-memory pipe (50 %); 16.6 M warp instructions against 37.5 M for a kernel
+// shared-memory pipe (51 %); 16.5 M warp instructions against 37.5 M for a kernel
 // that formed every real transform and transposed the plane between the axes.
 // Between events, which add about 3 us: 25.3 us for the three terms at N = 128 (that
 // kernel: 56.6), 9.5 at N = 64 (about 30), 7.2 at N = 32 (27), 13.4 at N = 96 (five
